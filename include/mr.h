@@ -117,7 +117,9 @@ typedef enum {
 } mr_mode;
 
 typedef enum {
-  MR_KM_FP32 = 0,         /* FP32 SIMT distances, exact re-check of near ties */
+  MR_KM_FP32 = 0,         /* the library picks the distance pass: split operands on the
+                             tensor cores where they cover the shape, else FP32 SIMT;
+                             exact re-check of near ties */
   MR_KM_BF16_TC = 1,      /* BF16 tensor-core distance GEMM (tcgen05, FP32
                              accumulate) on split operands x = hi + lo (three
                              BF16 products), FP32 then FP64 re-check of near

@@ -105,19 +105,62 @@ __device__ __forceinline__ void top2lb_merge(uint32_t& a1, uint32_t& a2, uint32_
   la = g3;
 }
 
-// Centroid norms: cn[k] = ||c_k||^2 (FP32, sequential FMA); cmax[0] = max ||c_k||.
-__global__ void km_prep_kernel(const float* __restrict__ c, uint32_t k, uint32_t d, float* __restrict__ cn,
-                               unsigned int* cmax_bits, long long* sums, unsigned long long* counts, uint32_t* nflag) {
+// Start of a job: the current centroids are the initial ones, the counters
+// and statistics are zero, and center[j] is the mean of the initial centroids'
+// coordinate j (0 where that is not finite), the shift the tensor-core pass
+// applies to points and centroids alike.  One CTA per 32 dimensions.
+constexpr int SETUP_THREADS = 1024;
+__global__ void __launch_bounds__(SETUP_THREADS) km_setup_kernel(const float* __restrict__ init, uint32_t k,
+                                                                 uint32_t d, float* __restrict__ c,
+                                                                 float* __restrict__ center, uint32_t* nflag,
+                                                                 unsigned long long* stats) {
+  __shared__ double red[SETUP_THREADS / 32][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t j = blockIdx.x * 32 + lane;
+  double s = 0.0;
+  if (j < d)
+    for (uint32_t i = w; i < k; i += SETUP_THREADS / 32) {
+      const float v = init[(uint64_t)i * d + j];
+      c[(uint64_t)i * d + j] = v;
+      s += (double)v;
+    }
+  red[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && j < d) {
+    for (int i = 1; i < SETUP_THREADS / 32; ++i) s += red[i][lane];
+    const float m = (float)(s / (double)k);
+    center[j] = isfinite(m) ? m : 0.f;
+  }
+  if (blockIdx.x == 0 && threadIdx.x < 8) nflag[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 4) stats[threadIdx.x] = 0;
+}
+
+// Centroid norms, one warp per centroid: cn[k] = ||c_k - center||^2 (FP32
+// FMAs; center null: no shift) and cmax[0] = max ||c_k - center||.  Also
+// clears the iteration's counters.  (With one thread per centroid, whose row
+// reads are strided, this took 11 us at K = 256, D = 64 and 20 us at K = 512,
+// D = 128.)
+__global__ void km_prep_kernel(const float* __restrict__ c, uint32_t k, uint32_t d, const float* __restrict__ center,
+                               float* __restrict__ cn, unsigned int* cmax_bits, long long* sums,
+                               unsigned long long* counts, uint32_t* nflag) {
   pdl_wait();
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = tid; i < (uint64_t)k; i += nth) {
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint64_t i = tid >> 5; i < (uint64_t)k; i += nth >> 5) {
     float s = 0.f;
-    for (uint32_t j = 0; j < d; ++j) s = fmaf(c[i * d + j], c[i * d + j], s);
-    cn[i] = s;
-    atomicMax(cmax_bits, __float_as_uint(sqrtf(s)));
+    for (uint32_t j = lane; j < d; j += 32) {
+      const float v = center ? __fsub_rn(c[i * d + j], center[j]) : c[i * d + j];
+      s = fmaf(v, v, s);
+    }
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      cn[i] = s;
+      atomicMax(cmax_bits, __float_as_uint(sqrtf(s)));
+    }
   }
-  for (uint64_t i = tid; i < (uint64_t)k * d; i += nth) sums[i] = 0;
+  if (sums)
+    for (uint64_t i = tid; i < (uint64_t)k * d; i += nth) sums[i] = 0;
   for (uint64_t i = tid; i < (uint64_t)k; i += nth) counts[i] = 0;
   if (tid < 2) nflag[tid] = 0;
   if (tid == 2) nflag[4] = 0;  // pair list
@@ -344,6 +387,22 @@ __device__ __forceinline__ float warp_dist32(const float* __restrict__ xp, const
   return s;
 }
 
+// Fixed-point exponent s (at most 60): the largest with max|x| 2^s < 2^39 and
+// max|x| 2^s n < 2^62, so every q = rint(x 2^s) fits 40 bits (the update's
+// hi/lo split) and no sum of n of them can overflow int64.  s may be
+// negative for very large inputs; x 2^s then rounds only where it is far
+// below 1/2, and rounds to 0 either way.  (max|x| = f 2^e with f < 1, so
+// s <= 39 - e holds; n lowers it by at most 8 more.)
+__device__ __forceinline__ int fx_shift_of(float m, uint32_t n) {
+  if (!(m > 0.f)) return 60;
+  const double lim = fmin(ldexp(1.0, 39), ldexp(1.0, 62) / (double)n);
+  int e;
+  frexpf(m, &e);
+  int s = 39 - e < 60 ? 39 - e : 60;
+  while (s > -200 && ldexp((double)m, s) >= lim) --s;
+  return s;
+}
+
 // Exact choice between two centroids for the listed points (pairs whose
 // other centroids are already ruled out), four pairs per warp: lanes 8g ..
 // 8g + 7 take pair g, each lane dimensions s, s + 8, ... of the point and of
@@ -354,10 +413,15 @@ __device__ __forceinline__ float warp_dist32(const float* __restrict__ xp, const
 // stage's list (deferred, ndef), which km_fp64_stage_kernel then settles
 // with all such points in parallel (the FP64 pipe of this GPU is narrow:
 // done here, a few such points kept a few SMs busy long after the rest had
-// finished).  stat[0] counts the pairs.
-__global__ void km_pair_kernel(const float* __restrict__ x, uint32_t d, const float* __restrict__ c,
+// finished).  stat[0] counts the pairs.  With maxabs not null (the first
+// iteration, whose distance pass or a pass before it found max |x|) one thread
+// also sets the update's fixed-point exponent.
+__global__ void km_pair_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c,
                                const uint2* __restrict__ pairs, const uint32_t* npairs, int32_t* assign,
-                               unsigned long long* stat, uint32_t* deferred, uint32_t* ndef) {
+                               unsigned long long* stat, uint32_t* deferred, uint32_t* ndef,
+                               const unsigned int* maxabs, int* shift) {
+  pdl_wait();
+  if (maxabs && blockIdx.x == 0 && threadIdx.x == 0) *shift = fx_shift_of(__uint_as_float(*maxabs), n);
   const uint32_t np = *npairs;
   const int lane = threadIdx.x & 31, grp = lane >> 3, sl = lane & 7;
   const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -642,21 +706,6 @@ __global__ void km_maxabs_kernel(const float* __restrict__ x, uint64_t cnt, unsi
   for (uint64_t i = done + tid; i < cnt; i += nth) m = max(m, __float_as_uint(fabsf(x[i])));
   for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) atomicMax(out, m);
-}
-
-// Fixed-point exponent s (at most 60): the largest with max|x| 2^s < 2^39 and
-// max|x| 2^s n < 2^62, so every q = rint(x 2^s) fits 40 bits (the update's
-// hi/lo split) and no sum of n of them can overflow int64.  s may be
-// negative for very large inputs; x 2^s then rounds only where it is far
-// below 1/2, and rounds to 0 either way.
-__global__ void km_scale_kernel(const unsigned int* maxabs, uint32_t n, int* shift) {
-  const float m = __uint_as_float(*maxabs);
-  int s = 60;
-  if (m > 0.f) {
-    const double lim = fmin(ldexp(1.0, 39), ldexp(1.0, 62) / (double)n);
-    while (s > -200 && (double)m * ldexp(1.0, s) >= lim) --s;
-  }
-  *shift = s;
 }
 
 __device__ __forceinline__ uint32_t cluster_of(const int32_t* assign, uint64_t i, uint32_t k) {
@@ -1325,24 +1374,19 @@ inline uint64_t a256(uint64_t x) { return (x + 255) & ~255ull; }
 
 }  // namespace
 
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, int precision) {
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k) {
   uint64_t b = 0;
   b += a256((uint64_t)k * d * 4);      // cent
   b += a256((uint64_t)n * 4 + 16);     // assign (+16: the update copies ids in 16-byte units)
   b += a256((uint64_t)k * d * 8);      // sums
   b += a256((uint64_t)k * 8);          // counts
-  b += a256(4 * 8);                    // stats
-  b += a256((uint64_t)n * 4);          // flagged
-  b += a256(8 * 4);                    // counters: nflag[2], maxabs, cmax, pairs
+  b += 256;                            // stats, counters (nflag, maxabs, cmax, pairs), shift
+  b += a256((uint64_t)n * 4);          // points to re-check; the sorted update's permutation
   b += a256((uint64_t)n * 8);          // pair list
   b += a256((uint64_t)n * 4);          // FP64 stage list
-  b += a256((uint64_t)k * 4 * 2);      // cnorm (||c||^2) + spare
-  b += a256(16);                       // shift
+  b += a256((uint64_t)k * 4);          // ||c||^2
+  b += a256((uint64_t)d * 4);          // center
   b += a256((uint64_t)k * 4);          // per-cluster write cursor
-  if (precision != MR_KM_FP32) {
-    b += a256((uint64_t)n * 4);        // second flag list
-    b += a256((uint64_t)k * d * 2 * 2);  // bf16 centroids (hi, lo)
-  }
   if (local_sums_fit(d, k)) b += a256((uint64_t)LS_MAX_CTAS * k * d * 8);  // per-CTA partial sums
   return (size_t)b;
 }
@@ -1355,22 +1399,17 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes) {
   b.assign = reinterpret_cast<int32_t*>(take(n * 4 + 16));
   b.sums = reinterpret_cast<long long*>(take(k * d * 8));
   b.counts = reinterpret_cast<unsigned long long*>(take(k * 8));
-  b.stats = reinterpret_cast<unsigned long long*>(take(32));
+  uint8_t* ctl = take(256);
+  b.stats = reinterpret_cast<unsigned long long*>(ctl);
+  b.nflag = reinterpret_cast<uint32_t*>(ctl + 64);
+  b.maxabs = reinterpret_cast<unsigned int*>(b.nflag + 2);
+  b.shift = reinterpret_cast<int*>(ctl + 128);
   b.flagged = reinterpret_cast<uint32_t*>(take(n * 4));
-  b.nflag = reinterpret_cast<uint32_t*>(take(32));
   b.pairs = reinterpret_cast<uint2*>(take(n * 8));
   b.deferred = reinterpret_cast<uint32_t*>(take(n * 4));
-  b.maxabs = reinterpret_cast<unsigned int*>(b.nflag + 2);
-  b.cnorm = reinterpret_cast<float*>(take(k * 8));
-  b.cent_bf16_norm = nullptr;
-  int* shift = reinterpret_cast<int*>(take(16));
+  b.cnorm = reinterpret_cast<float*>(take(k * 4));
+  b.center = reinterpret_cast<float*>(take(d * 4));
   b.kcursor = reinterpret_cast<uint32_t*>(take(k * 4));
-  b.fx_shift = 0;
-  b.xnorm = reinterpret_cast<float*>(shift);  // holds the device-side shift
-  if (b.precision != MR_KM_FP32) {
-    b.cent_bf16_norm = reinterpret_cast<float*>(take(n * 4));  // second flag list
-    b.cb = reinterpret_cast<uint16_t*>(take(k * d * 4));
-  }
   b.part = local_sums_fit(d, k) ? reinterpret_cast<long long*>(take((uint64_t)LS_MAX_CTAS * k * d * 8)) : nullptr;
   if ((uint64_t)(q - p) > bytes) return cudaErrorInvalidValue;
   return cudaSuccess;
@@ -1385,18 +1424,23 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
                           cudaStream_t s, float* out_c, int32_t* out_a, unsigned long long* out_s, uint64_t* nk) {
   cudaError_t e;
   const uint32_t n = b.n, d = b.d, k = b.k;
-  int* shift = reinterpret_cast<int*>(b.xnorm);
+  int* shift = b.shift;
   unsigned int* cmax_bits = b.nflag + 3;
-  if ((e = cudaMemcpyAsync(b.cent, init, (size_t)k * d * 4, cudaMemcpyDeviceToDevice, s)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(b.stats, 0, 32, s)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(b.nflag, 0, 32, s)) != cudaSuccess) return e;
-  // the fixed-point scale needs max |x|: a pass of its own for the FP32
+  km_setup_kernel<<<(d + 31) / 32, SETUP_THREADS, 0, s>>>(init, k, d, b.cent, b.center, b.nflag, b.stats);
+  ++*nk;
+  // The distance pass only has to settle the clear cases (every near tie is
+  // re-checked), so an FP32 job takes the tensor-core pass on split operands
+  // wherever that covers its shape: the assignments are the FP64 definition's
+  // either way.  At 200,003 x 37, K = 100 the pass takes 32 us instead of 156
+  // and the whole ten-round call 0.91 ms instead of 2.11.  A context that has set a wait limit or stops
+  // the copies (diagnostics of the pipelined passes) keeps FP32 jobs on the
+  // SIMT pass, which waits on nothing.
+  const bool tc = b.precision != MR_KM_FP32 || (km_tc_supported(d, k) && b.polls < 0 && b.stop_copies == 0);
+  // the fixed-point scale needs max |x|: a pass of its own for the SIMT
   // path; the tensor-core pass finds it while converting the first iteration
-  const bool tc = b.precision != MR_KM_FP32;
   if (!tc) {
     km_maxabs_kernel<<<di.sms * 4, 256, 0, s>>>(x, (uint64_t)n * d, b.maxabs);
-    km_scale_kernel<<<1, 1, 0, s>>>(b.maxabs, n, shift);
-    *nk += 2;
+    ++*nk;
   }
   const int asm_bytes = (DC_MAX * CS_LD + DC_MAX * XS_LD) * 4;
   if ((e = cudaFuncSetAttribute(km_assign_fp32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1469,35 +1513,33 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   for (uint32_t it = 0; it < iters; ++it) {
     // kernels that follow another kernel of this job on the stream start
     // while it drains (programmatic dependent launch; each waits first)
-    if (it == 0)
-      km_prep_kernel<<<64, 256, 0, s>>>(b.cent, k, d, b.cnorm, cmax_bits, b.sums, b.counts, b.nflag);
-    else if ((e = launch_pdl(km_prep_kernel, dim3(64), dim3(256), 0, s, (const float*)b.cent, k, d, b.cnorm, cmax_bits,
-                             b.sums, b.counts, b.nflag)) != cudaSuccess)
+    const unsigned pgrid = k < 8 * 64 ? (k + 7) / 8 : 64;
+    if ((e = launch_pdl(km_prep_kernel, dim3(pgrid), dim3(256), 0, s, (const float*)b.cent, k, d,
+                        tc ? (const float*)b.center : (const float*)nullptr, b.cnorm, cmax_bits,
+                        local ? (long long*)nullptr : b.sums, b.counts, b.nflag)) != cudaSuccess)
       return e;
-    if (b.precision != MR_KM_FP32) {
+    if (tc) {
       if ((e = launch_kmeans_tc_assign(x, n, d, b.cent, k, b, di, s, nk, it == 0)) != cudaSuccess) return e;
-      if (it == 0) {
-        km_scale_kernel<<<1, 1, 0, s>>>(b.maxabs, n, shift);
-        ++*nk;
-      }
     } else {
       if ((e = kt_begin(b.kt, s)) != cudaSuccess) return e;
       (k <= 256 ? km_assign_fp32_kernel<true> : km_assign_fp32_kernel<false>)<<<agrid, KM_THREADS, asm_bytes, s>>>(
-          x, n, d, b.cent, k, b.cnorm, cmax_bits, nullptr, nullptr, b.assign, b.flagged, b.nflag, b.pairs,
+          x, n, d, b.cent, k, b.cnorm, cmax_bits, nullptr, nullptr, b.assign, b.flagged, b.nflag + 1, b.pairs,
           b.nflag + 4, nullptr);
       if ((e = cudaGetLastError()) != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;
       ++*nk;
     }
     // one warp per pair, latency-bound: a full SM of warps (32 registers a thread)
-    km_pair_kernel<<<di.sms * 8, 256, 0, s>>>(x, d, b.cent, b.pairs, b.nflag + 4, b.assign, b.stats, b.deferred,
-                                              b.nflag + 5);
+    if ((e = launch_pdl(km_pair_kernel, dim3(di.sms * 8), dim3(256), 0, s, x, n, d, (const float*)b.cent,
+                        (const uint2*)b.pairs, (const uint32_t*)(b.nflag + 4), b.assign, b.stats, b.deferred,
+                        b.nflag + 5, it == 0 ? (const unsigned int*)b.maxabs : (const unsigned int*)nullptr,
+                        shift)) != cudaSuccess)
+      return e;
     ++*nk;
-    // the points neither pass could decide: from the tensor-core pass its
-    // list (re-checked straight away with FP32 direct differences; the points
-    // where those leave more than one candidate go to the FP64 stage), from
-    // the FP32 pass its own
-    const uint32_t* rl = b.precision != MR_KM_FP32 ? reinterpret_cast<const uint32_t*>(b.cent_bf16_norm) : b.flagged;
-    const uint32_t* rn = b.precision != MR_KM_FP32 ? b.nflag + 1 : b.nflag;
+    // the points the distance pass could not decide are re-checked straight
+    // away with FP32 direct differences; the points where those leave more
+    // than one candidate go to the FP64 stage
+    const uint32_t* rl = b.flagged;
+    const uint32_t* rn = b.nflag + 1;
     if (rc_smem)
       e = launch_pdl(km_recheck_fp64_smem_kernel, dim3(di.sms * rc_per_sm), dim3(512), (size_t)rc_bytes, s, x, d,
                      (const float*)b.cent, k, rl, rn, b.assign, b.stats, b.deferred, b.nflag + 5);

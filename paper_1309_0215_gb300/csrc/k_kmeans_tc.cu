@@ -38,7 +38,13 @@
 // exact BF16 products is charged (products + 8) * 2^-21 ||x|| ||c|| (four
 // times the round-to-nearest bound, allowing truncating adders), and the FP32
 // norms and the final fma/add (D + 8) * 2^-24 (||x|| + ||c||)^2 (Higham,
-// eq. 3.5).  The keys hold d~ truncated to 16 mantissa bits (t <= d~ <
+// eq. 3.5).  Points and centroids are first shifted by the mean m of the
+// initial centroids, x' = fl(x - m) and c' = fl(c - m): distances do not
+// change, but the bounds then scale with the spread of the data, not with
+// its offset from zero.  Each subtraction is correctly rounded, so x' - c'
+// differs from x - c by at most 2^-24 (||x'|| + ||c'||) and its square by at
+// most twice that times (||x'|| + ||c'||): (D + 12) in place of (D + 8)
+// covers it, and x, c stand for x', c' in all of the bounds here.  The keys hold d~ truncated to 16 mantissa bits (t <= d~ <
 // t (1 + 2^-15)), so with G = 2E + 2^-14 t_1: if t_2 - t_1 > max(1e-3 t_1, G)
 // the tensor-core winner is the exact winner.  Otherwise, if b_3 - t_1 > G,
 // where b_3 is a lower bound of every key but the top two, every other
@@ -214,7 +220,7 @@ __device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 12
 template <int TERMS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, uint32_t k,
-                    const float* __restrict__ cnorm, const unsigned int* cmax_bits, int32_t* __restrict__ assign,
+                    const float* __restrict__ center, const float* __restrict__ cnorm, const unsigned int* cmax_bits, int32_t* __restrict__ assign,
                     uint32_t* __restrict__ list, uint32_t* nlist, uint2* __restrict__ pairs, uint32_t* npairs,
                     unsigned long long* timeouts, float* dbg, long long polls, uint32_t stop_copies,
                     unsigned int* maxabs) {
@@ -251,14 +257,16 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // everything read from here on was written by earlier kernels of the job
+  pdl_wait();
   // centroid operands (rows >= k and dims >= d are zero) and norms
   for (uint32_t t = threadIdx.x; t < npad * (KD / 2); t += blockDim.x) {
     const uint32_t row = t / (KD / 2), pr = t % (KD / 2);
     const uint32_t d0 = 2 * pr;
     float a = 0.f, b = 0.f;
     if (row < k) {
-      if (d0 < d) a = c[(uint64_t)row * d + d0];
-      if (d0 + 1 < d) b = c[(uint64_t)row * d + d0 + 1];
+      if (d0 < d) a = __fsub_rn(c[(uint64_t)row * d + d0], center[d0]);
+      if (d0 + 1 < d) b = __fsub_rn(c[(uint64_t)row * d + d0 + 1], center[d0 + 1]);
     }
     uint32_t hi, lo;
     split2(a, b, hi, lo);
@@ -285,6 +293,9 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
     const int cw = warp - CVT_WARP0;
     const int col = lane & 15, rsub = lane >> 4;
     const bool vec = d == KD && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
+    float mv[4];  // the shift of this lane's four dimensions
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mv[j] = 4u * col + j < d ? center[4 * col + j] : 0.f;
     unsigned int mabs = 0;  // bits of max |x| over the values this thread converts (non-negative floats order as ints)
     for (uint32_t i = 0;; ++i) {
       const uint32_t tile = blockIdx.x + i * gridDim.x;
@@ -332,6 +343,10 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
           if (maxabs)
             mabs = max(mabs, max(max(__float_as_uint(fabsf(v[q].x)), __float_as_uint(fabsf(v[q].y))),
                                  max(__float_as_uint(fabsf(v[q].z)), __float_as_uint(fabsf(v[q].w)))));
+          v[q].x = __fsub_rn(v[q].x, mv[0]);
+          v[q].y = __fsub_rn(v[q].y, mv[1]);
+          v[q].z = __fsub_rn(v[q].z, mv[2]);
+          v[q].w = __fsub_rn(v[q].w, mv[3]);
           float ss = fmaf(v[q].w, v[q].w, fmaf(v[q].z, v[q].z, fmaf(v[q].y, v[q].y, v[q].x * v[q].x)));
           ss += __shfl_xor_sync(0xffffffffu, ss, 8);
           ss += __shfl_xor_sync(0xffffffffu, ss, 4);
@@ -434,7 +449,7 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
     const int fw = warp - FIN_WARP0;
     const float eps_sum = TERMS == 3 ? (3.05f * 1.52587890625e-05f + (float)(3 * KD + 8) * 4.76837158203125e-07f)
                                      : (2.f * 3.90625e-03f + 1.52587890625e-05f + (float)(KD + 8) * 4.76837158203125e-07f);
-    const float eps32 = 1.01f * (float)(d + 8) * 5.9604644775390625e-08f;
+    const float eps32 = 1.01f * (float)(d + 12) * 5.9604644775390625e-08f;
     for (uint32_t i = 0;; ++i) {
       const uint32_t tile = blockIdx.x + i * gridDim.x;
       if (tile >= ntiles) break;
@@ -475,7 +490,8 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
         if (p < n) {
           const float d1 = key_dist(g1), d2 = key_dist(g2), d3 = key_dist(g3);
           const float xn = sqrtf(nxv[h]);
-          const float e = 2.f * eps_sum * xn * cmax + eps32 * (xn + cmax) * (xn + cmax);
+          // (1e-36: the products of tiny values may be flushed to zero)
+          const float e = 2.f * eps_sum * xn * cmax + eps32 * (xn + cmax) * (xn + cmax) + 1e-36f;
           // keys under-state a distance by less than 2^-15 of it (2^-14 allowed)
           const float gap = 2.f * e + 6.103515625e-05f * d1;
           if (g1 < 0) flag = true;  // a negative smallest distance: re-check
@@ -580,8 +596,8 @@ size_t km_tc_smem_bytes() { return sizeof(TcSmem) + 1024; }
 // Raw launch: list/nlist receive the points to re-check, pairs/npairs the
 // two-candidate points; maxabs (when not null) receives the bits of max |x|.
 cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
-                                const float* cnorm, const unsigned int* cmax_bits, int32_t* assign, uint32_t* list,
-                                uint32_t* nlist, uint2* pairs, uint32_t* npairs, unsigned long long* timeouts,
+                                const float* center, const float* cnorm, const unsigned int* cmax_bits,
+                                int32_t* assign, uint32_t* list, uint32_t* nlist, uint2* pairs, uint32_t* npairs, unsigned long long* timeouts,
                                 float* dbg, int grid, cudaStream_t s, long long polls, uint32_t stop_copies,
                                 unsigned int* maxabs) {
   const int smem = (int)km_tc_smem_bytes();
@@ -590,16 +606,17 @@ cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t 
     if ((e = cudaFuncSetAttribute(km_tc_assign_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
         cudaSuccess)
       return e;
-    km_tc_assign_kernel<3><<<grid, TC_THREADS, smem, s>>>(x, n, d, c, k, cnorm, cmax_bits, assign, list, nlist,
-                                                           pairs, npairs, timeouts, dbg, polls, stop_copies, maxabs);
+    return launch_pdl(km_tc_assign_kernel<3>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
+                      cnorm, cmax_bits, assign, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
+                      maxabs);
   } else {
     if ((e = cudaFuncSetAttribute(km_tc_assign_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
         cudaSuccess)
       return e;
-    km_tc_assign_kernel<1><<<grid, TC_THREADS, smem, s>>>(x, n, d, c, k, cnorm, cmax_bits, assign, list, nlist,
-                                                           pairs, npairs, timeouts, dbg, polls, stop_copies, maxabs);
+    return launch_pdl(km_tc_assign_kernel<1>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
+                      cnorm, cmax_bits, assign, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
+                      maxabs);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
@@ -607,12 +624,11 @@ cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, cons
   const uint32_t ntiles = (n + TM - 1) / TM;
   uint32_t grid = ntiles < (uint32_t)di.sms ? ntiles : (uint32_t)di.sms;
   if (b.grid_cap && grid > b.grid_cap) grid = b.grid_cap;
-  uint32_t* list = reinterpret_cast<uint32_t*>(b.cent_bf16_norm);
   const int terms = b.precision == MR_KM_BF16X1_TC ? 1 : 3;
   cudaError_t e = kt_begin(b.kt, s);
   if (e != cudaSuccess) return e;
-  e = launch_km_tc_kernel(terms, x, n, d, c, k, b.cnorm, b.nflag + 3, b.assign, list, b.nflag + 1, b.pairs,
-                          b.nflag + 4, b.stats + 3, nullptr, (int)grid, s, b.polls < 0 ? SPIN_LIMIT : b.polls,
+  e = launch_km_tc_kernel(terms, x, n, d, c, k, b.center, b.cnorm, b.nflag + 3, b.assign, b.flagged, b.nflag + 1,
+                          b.pairs, b.nflag + 4, b.stats + 3, nullptr, (int)grid, s, b.polls < 0 ? SPIN_LIMIT : b.polls,
                           b.stop_copies, maxabs ? b.maxabs : nullptr);
   if (e != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;
   ++*nk;

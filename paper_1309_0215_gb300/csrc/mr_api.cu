@@ -383,7 +383,7 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
       // result: centroids [K*D] f32 | assignments [N] i32 | pad to 8 | stats [4] u64
       const uint64_t res_bytes = km_stats_offset(K, D, N) + 32;
       const uint64_t res = align256(res_bytes);
-      const uint64_t scr = align256(km_scratch_bytes(N, D, K, (int)d.km_precision));
+      const uint64_t scr = align256(km_scratch_bytes(N, D, K));
       const uint64_t init_bytes = d.input_on_device ? 0 : align256((uint64_t)K * D * 4);
       mr_status st = dev_alloc(c, res + scr + init_bytes, &j->slab);
       if (st) return st;

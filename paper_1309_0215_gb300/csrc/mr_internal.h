@@ -143,25 +143,22 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 struct KmBuffers {
   uint32_t n = 0, d = 0, k = 0;
   float* cent = nullptr;        // [k][d] current centroids (FP32 state)
-  float* cent_bf16_norm = nullptr;
   int32_t* assign = nullptr;    // [n]
   long long* sums = nullptr;    // [k][d] fixed-point sums
   unsigned long long* counts = nullptr;  // [k]
   unsigned long long* stats = nullptr;   // [4]
-  uint32_t* flagged = nullptr;  // [n] indices of points to re-check
-  uint32_t* nflag = nullptr;    // [8] counters: [0] FP64 list, [1] FP32 list, [2] max|x| bits, [3] max||c|| bits, [4] pairs,
+  uint32_t* flagged = nullptr;  // [n] points to re-check; later the sorted update's permutation
+  uint32_t* nflag = nullptr;    // [8] counters: [1] points to re-check, [2] max|x| bits, [3] max||c|| bits, [4] pairs,
                                 //     [5] points deferred to the FP64 stage
   uint32_t* deferred = nullptr; // [n] points whose choice needs the FP64 definition
   uint2* pairs = nullptr;       // [n] {point, k1 | k2 << 16}: exact choice between two centroids
-  float* xnorm = nullptr;       // [n] ||x||
-  float* cnorm = nullptr;       // [k] ||c|| and ||c||^2
-  uint16_t* xb = nullptr;       // BF16 copy of the points [n][d]
-  uint16_t* cb = nullptr;       // BF16 centroids [k][d]
+  float* cnorm = nullptr;       // [k] ||c||^2 (of the shifted centroids on the tensor-core path)
+  float* center = nullptr;      // [d] the shift
   unsigned int* maxabs = nullptr;  // [1] bits of max |x|
+  int* shift = nullptr;         // [1] fixed-point scale exponent
   uint32_t* kcursor = nullptr;  // [k] counting-sort write cursors
   long long* part = nullptr;    // [CTAs][k][d] partial sums of the local-array update (nullptr: sort path)
   KTimer* kt = nullptr;         // times the distance pass of each iteration
-  int fx_shift = 32;            // fixed-point scale exponent
   int precision = 0;
   // diagnostics (mr_set_option): polls of a bounded device wait (< 0: the
   // default), cap on the CTAs of the persistent kernels (0: none), tiles the
@@ -170,7 +167,7 @@ struct KmBuffers {
   uint32_t grid_cap = 0;
   uint32_t stop_copies = 0;
 };
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, int precision);
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k);
 cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes);
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,
                           cudaStream_t s, float* out_cent, int32_t* out_assign, unsigned long long* out_stats,

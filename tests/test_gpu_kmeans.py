@@ -304,3 +304,19 @@ def test_kmeans_full_size_bf16_matches_fp32_path(mr):
     assert np.array_equal(a16, a32)
     assert np.array_equal(c16, c32)
     assert int(st[3]) == 0
+
+
+@pytest.mark.parametrize("n,d,k", [(1_999, 64, 256), (2_001, 63, 255), (1_153, 1, 1), (1_281, 2, 9)])
+@pytest.mark.parametrize("offset,scale", [(0.0, 1.0), (1000.0, 1.0), (-3e6, 1e4), (0.0, 1e-15), (1e15, 1e15)])
+def test_kmeans_fp32_on_the_tensor_cores(mr, n, d, k, offset, scale):
+    """FP32 jobs that take the tensor-core pass, at the edges of its shapes and
+    with data far from the origin, tiny and huge: one round from the same
+    centroids gives the oracle's assignments and centroids."""
+    x, _, _ = synth.kmeans_points(n, d, max(1, min(k, 32)), seed=n + d)
+    x = (x * np.float32(scale) + np.float32(offset)).astype(np.float32)
+    init = synth.kmeans_init(x, k, seed=n)
+    c_ref, a_ref = oracle.kmeans(x, init, 1)
+    c, a, stats = _run(mr, x, init, 1, 0)
+    assert np.array_equal(a, a_ref)
+    assert _rel_err(c, c_ref) <= TOL
+    assert int(stats[3]) == 0
