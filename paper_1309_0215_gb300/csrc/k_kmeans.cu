@@ -112,8 +112,8 @@ __device__ __forceinline__ void top2lb_merge(uint32_t& a1, uint32_t& a2, uint32_
 constexpr int SETUP_THREADS = 1024;
 __global__ void __launch_bounds__(SETUP_THREADS) km_setup_kernel(const float* __restrict__ init, uint32_t k,
                                                                  uint32_t d, float* __restrict__ c,
-                                                                 float* __restrict__ center, uint32_t* nflag,
-                                                                 unsigned long long* stats) {
+                                                                 float* __restrict__ center, long long* sums,
+                                                                 uint32_t* nflag, unsigned long long* stats) {
   __shared__ double red[SETUP_THREADS / 32][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t j = blockIdx.x * 32 + lane;
@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(SETUP_THREADS) km_setup_kernel(const float* __
     for (uint32_t i = w; i < k; i += SETUP_THREADS / 32) {
       const float v = init[(uint64_t)i * d + j];
       c[(uint64_t)i * d + j] = v;
+      if (sums) sums[(uint64_t)i * d + j] = 0;
       s += (double)v;
     }
   red[w][lane] = s;
@@ -135,52 +136,19 @@ __global__ void __launch_bounds__(SETUP_THREADS) km_setup_kernel(const float* __
   if (blockIdx.x == 0 && threadIdx.x < 4) stats[threadIdx.x] = 0;
 }
 
-// Centroid norms, one warp per centroid: cn[k] = ||c_k - center||^2 (FP32
-// FMAs; center null: no shift) and cmax[0] = max ||c_k - center||.  Also
-// clears the iteration's counters.  (With one thread per centroid, whose row
-// reads are strided, this took 11 us at K = 256, D = 64 and 20 us at K = 512,
-// D = 128.)
-__global__ void km_prep_kernel(const float* __restrict__ c, uint32_t k, uint32_t d, const float* __restrict__ center,
-                               float* __restrict__ cn, unsigned int* cmax_bits, long long* sums,
-                               unsigned long long* counts, uint32_t* nflag) {
-  pdl_wait();
-  const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
-  const uint32_t lane = threadIdx.x & 31;
-  for (uint64_t i = tid >> 5; i < (uint64_t)k; i += nth >> 5) {
-    float s = 0.f;
-    for (uint32_t j = lane; j < d; j += 32) {
-      const float v = center ? __fsub_rn(c[i * d + j], center[j]) : c[i * d + j];
-      s = fmaf(v, v, s);
-    }
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      cn[i] = s;
-      atomicMax(cmax_bits, __float_as_uint(sqrtf(s)));
-    }
-  }
-  if (sums)
-    for (uint64_t i = tid; i < (uint64_t)k * d; i += nth) sums[i] = 0;
-  for (uint64_t i = tid; i < (uint64_t)k; i += nth) counts[i] = 0;
-  if (tid < 2) nflag[tid] = 0;
-  if (tid == 2) nflag[4] = 0;  // pair list
-  if (tid == 3) nflag[5] = 0;  // FP64 stage list
-}
-
 // FP32 assignment.  A CTA processes tiles of 64 points; warp w owns points
 // 8w..8w+7 of the tile, lane l owns centroids l + 32 j (j < 8) of each chunk
 // of up to 256 centroids.  Dot products accumulate over dimension chunks
 // staged in shared memory (points transposed [dim][point], centroids
 // [dim][centroid]).  When K <= 256 and D <= 64 the centroids are loaded once
-// per CTA.  idx != nullptr restricts the pass to the listed points.
+// per CTA.
 // KEYS (K <= 256): selection by packed keys (top-2 plus a lower bound of
 // the other keys); else a float top-3 with indices.
 template <bool KEYS>
 __global__ void __launch_bounds__(KM_THREADS, 2)
 km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, uint32_t k,
-                      const float* __restrict__ cn, const unsigned int* cmax_bits, const uint32_t* idx,
-                      const uint32_t* nidx, int32_t* __restrict__ assign, uint32_t* flagged, uint32_t* nflag,
-                      uint2* __restrict__ pairs, uint32_t* npairs, unsigned long long* stat) {
+                      const float* __restrict__ cn, const unsigned int* cmax_bits, int32_t* __restrict__ assign,
+                      uint32_t* flagged, uint32_t* nflag, uint2* __restrict__ pairs, uint32_t* npairs) {
   extern __shared__ float km_sm[];
   const int dc = d < DC_MAX ? (int)d : DC_MAX;
   const int kc = k < KC_MAX ? (int)k : KC_MAX;
@@ -188,13 +156,11 @@ km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const
   float* xs = km_sm + DC_MAX * CS_LD;  // [dc][XS_LD]
   __shared__ float nx_s[TP];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t npts = idx ? *nidx : n;
+  const uint32_t npts = n;
   const bool resident = k <= KC_MAX && d <= DC_MAX;
   const bool vec4 = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   const float cmax = __uint_as_float(*cmax_bits);
   const float eps = 1.01f * (float)(d + 8) * 5.9604645e-8f;  // 2^-24
-  if (idx && blockIdx.x == 0 && threadIdx.x == 0 && stat) atomicAdd(stat, (unsigned long long)npts);
-  if ((uint64_t)blockIdx.x * TP >= npts) return;  // no tile for this CTA (a short list)
 
   auto load_c = [&](uint32_t k0, uint32_t d0) {
     for (int t = threadIdx.x; t < kc * dc; t += KM_THREADS) {
@@ -240,7 +206,7 @@ km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const
           const uint32_t pi = p0 + pp;
           float v[4] = {0.f, 0.f, 0.f, 0.f};
           if (pi < npts) {
-            const uint32_t p = idx ? idx[pi] : pi;
+            const uint32_t p = pi;
             const float* row = x + (uint64_t)p * d + d0 + dd;
             if (vec4 && dd + 4 <= dlim) {
               const float4 q = __ldg(reinterpret_cast<const float4*>(row));
@@ -344,7 +310,7 @@ km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const
     const uint32_t pi = p0 + warp * 8 + lane;
     bool flag = false, pair = false;
     if (lane < 8 && pi < npts) {
-      const uint32_t p = idx ? idx[pi] : pi;
+      const uint32_t p = pi;
       const float nxv = sqrtf(nx_s[warp * 8 + lane]);
       const float e = eps * (nxv + cmax) * (nxv + cmax);
       const float gap = 2.f * e + (KEYS ? 6.103515625e-05f * fmaxf(mt.d1, 0.f) : 0.f);
@@ -359,7 +325,7 @@ km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const
       if (lane == 0) base = atomicAdd(npairs, (uint32_t)__popc(pm));
       base = __shfl_sync(0xffffffffu, base, 0);
       if (pair) {
-        const uint32_t p = idx ? idx[pi] : pi;
+        const uint32_t p = pi;
         pairs[base + __popc(pm & ((1u << lane) - 1))] = make_uint2(p, (uint32_t)mt.k1 | ((uint32_t)mt.k2 << 16));
       }
     }
@@ -369,22 +335,11 @@ km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const
       if (lane == 0) base = atomicAdd(nflag, (uint32_t)__popc(fm));
       base = __shfl_sync(0xffffffffu, base, 0);
       if (flag) {
-        const uint32_t p = idx ? idx[pi] : pi;
+        const uint32_t p = pi;
         flagged[base + __popc(fm & ((1u << lane) - 1))] = p;
       }
     }
   }
-}
-
-__device__ __forceinline__ float warp_dist32(const float* __restrict__ xp, const float* __restrict__ cp, uint32_t d,
-                                             int lane) {
-  float s = 0.f;
-  for (uint32_t j = lane; j < d; j += 32) {
-    const float t = xp[j] - cp[j];
-    s = fmaf(t, t, s);
-  }
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
 }
 
 // Fixed-point exponent s (at most 60): the largest with max|x| 2^s < 2^39 and
@@ -403,288 +358,273 @@ __device__ __forceinline__ int fx_shift_of(float m, uint32_t n) {
   return s;
 }
 
-// Exact choice between two centroids for the listed points (pairs whose
-// other centroids are already ruled out), four pairs per warp: lanes 8g ..
-// 8g + 7 take pair g, each lane dimensions s, s + 8, ... of the point and of
-// both centroid rows, so a warp has four points' rows in flight at once.
-// FP32 direct differences first: their relative error is at most g for any
-// summation order (as in the re-check below), so a ratio beyond widen
-// decides the exact order; closer pairs (and NaNs) are appended to the FP64
-// stage's list (deferred, ndef), which km_fp64_stage_kernel then settles
-// with all such points in parallel (the FP64 pipe of this GPU is narrow:
-// done here, a few such points kept a few SMs busy long after the rest had
-// finished).  stat[0] counts the pairs.  With maxabs not null (the first
-// iteration, whose distance pass or a pass before it found max |x|) one thread
-// also sets the update's fixed-point exponent.
-__global__ void km_pair_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c,
-                               const uint2* __restrict__ pairs, const uint32_t* npairs, int32_t* assign,
-                               unsigned long long* stat, uint32_t* deferred, uint32_t* ndef,
-                               const unsigned int* maxabs, int* shift) {
-  pdl_wait();
-  if (maxabs && blockIdx.x == 0 && threadIdx.x == 0) *shift = fx_shift_of(__uint_as_float(*maxabs), n);
-  const uint32_t np = *npairs;
-  const int lane = threadIdx.x & 31, grp = lane >> 3, sl = lane & 7;
-  const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  if (w0 == 0 && lane == 0 && stat) atomicAdd(stat, (unsigned long long)np);
+// ------------------------------------------------- settling the near ties
+// One kernel settles what the distance pass left open.
+//
+// Points with two candidates (pairs, eight lanes each): FP32 direct
+// differences to both centroids.  Their relative error is at most g =
+// gamma_{D+3} for any summation order (Higham, eq. 3.5 on a sum of squares),
+// so a ratio beyond widen decides the exact order.
+//
+// Listed points, in batches of SET_RP per CTA: FP32 direct differences to every
+// centroid, one thread per centroid and all the batch's points at once: the
+// points lie in shared memory dimension by dimension (one broadcast 16-byte
+// read gives four points' coordinates), the centroids come from a transposed
+// copy in coalesced reads that serve the whole batch, and two points go into
+// each packed FP32 instruction.  Only the two smallest distances matter: when
+// the second is beyond widen times the first, the first is the FP64 winner.
+//
+// A point that FP32 cannot decide is settled by the definition in FP64 on the
+// spot, by its whole CTA: the candidates are the centroids whose FP32
+// distance is within the bound of the smallest; the products (x_j - c_j)^2,
+// separately rounded, for all dimensions of a chunk of candidates at once
+// (the FP64 pipe is narrow on this GPU), and one thread per candidate adding
+// them with the dimensions in order.  The lowest index wins an exact tie;
+// all-NaN distances give index 0, as the definition.
+//
+// Bounded by the FP32 pipe for long lists (2 K D operations a listed point)
+// and by latency for short ones.  As three launches (pairs, a re-check with the
+// centroids staged in each CTA's shared memory and one warp per point, a
+// kernel for the FP64 points) this took 15 + 56 + 20 us at 4M x 64, K = 256
+// (181K pairs, 22K listed points, 100 FP64 points); now 43 us.  For K x D
+// beyond shared memory the re-check went warp by warp over the centroids: 531
+// of 576 us at 250,000 x 128, K = 512; now 55 us.
+// stat[0] counts the points re-checked, stat[1] those settled in FP64.
+constexpr int SET_RP = 16;        // listed points per batch
+constexpr int SET_LD = SET_RP + 4;  // row stride of the staged points (16-byte rows)
+constexpr int SET_T_MAX = 256;
+constexpr uint32_t SET_PROD = 2048;  // doubles of product scratch
+inline int set_threads(uint32_t k) { return k >= 225 ? 256 : (int)((k + 31) / 32 < 2 ? 64 : (k + 31) / 32 * 32); }
+inline size_t set_smem(uint32_t d, uint32_t k) {
+  const size_t stage = (size_t)d * SET_LD * 4, prod = (size_t)SET_PROD * 8;
+  return (stage > prod ? stage : prod) + (size_t)d * 4 + (size_t)k * 8;
+}
+__device__ __forceinline__ float rel_bound_widen(uint32_t d) {
   const float g = 1.01f * (float)(d + 8) * 5.9604644775390625e-08f;
-  const float widen = (1.f + g) / (1.f - g) * (1.f + 4.f * 5.9604644775390625e-08f);
-  for (uint64_t f0 = 4 * w0; f0 < np; f0 += 4 * nw) {
-    const uint64_t f = f0 + (uint64_t)grp;
-    const bool live = f < np;
-    const uint2 e = live ? pairs[f] : make_uint2(0u, 0u);
-    const uint32_t k1 = e.y & 0xffffu, k2 = e.y >> 16;
-    const float* xp = x + (uint64_t)e.x * d;
-    const float* c1 = c + (uint64_t)k1 * d;
-    const float* c2 = c + (uint64_t)k2 * d;
-    float f1 = 0.f, f2 = 0.f;
-    if (live)
-      for (uint32_t j = (uint32_t)sl; j < d; j += 8) {
-        const float xv = xp[j];
-        const float t1 = xv - c1[j], t2 = xv - c2[j];
-        f1 = fmaf(t1, t1, f1);
-        f2 = fmaf(t2, t2, f2);
-      }
-#pragma unroll
-    for (int o = 4; o; o >>= 1) {
-      f1 += __shfl_xor_sync(0xffffffffu, f1, o);
-      f2 += __shfl_xor_sync(0xffffffffu, f2, o);
-    }
-    if (live && sl == 0) {
-      if (f2 > f1 * widen) assign[e.x] = (int32_t)k1;
-      else if (f1 > f2 * widen) assign[e.x] = (int32_t)k2;
-      else deferred[atomicAdd(ndef, 1u)] = e.x;
-    }
-  }
+  return (1.f + g) / (1.f - g) * (1.f + 4.f * 5.9604644775390625e-08f);
+}
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  return (unsigned long long)__float_as_uint(a) | ((unsigned long long)__float_as_uint(b) << 32);
+}
+// a += (x - c)^2 for two points at once (nc = {-c, -c}); x + (-c) rounds as x - c
+__device__ __forceinline__ void sqdiff2(unsigned long long& a, unsigned long long x, unsigned long long nc) {
+  unsigned long long t;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(x), "l"(nc));
+  asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(a) : "l"(t));
 }
 
-// Exact FP64 argmin for the listed points, one warp per point.  Pass 1:
-// FP32 distance to every centroid with the lanes spread over the dimensions
-// (coalesced centroid rows, warp-sum; the bound below holds for any order),
-// keeping the smallest.  Pass 2: in FP64, separately rounded subtract,
-// multiply and add with the dimensions in order, only for the centroids whose
-// FP32 distance is within the relative error bound of that minimum (one lane
-// per such centroid).
-__global__ void km_recheck_fp64_kernel(const float* __restrict__ x, uint32_t d, const float* __restrict__ c, uint32_t k,
-                                       const uint32_t* flagged, const uint32_t* nflag, int32_t* assign,
-                                       unsigned long long* stat) {
-  pdl_wait();
-  const uint32_t nf = *nflag;
-  const int lane = threadIdx.x & 31;
-  const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  // every listed point is checked in FP32 and then in FP64 (stat[0], stat[1])
-  if (w0 == 0 && lane == 0 && stat) {
-    atomicAdd(stat, (unsigned long long)nf);
-    atomicAdd(stat + 1, (unsigned long long)nf);
-  }
-  const float g = 1.01f * (float)(d + 8) * 5.9604644775390625e-08f;
-  const float widen = (1.f + g) / (1.f - g) * (1.f + 4.f * 5.9604644775390625e-08f);
-  for (uint64_t f = w0; f < nf; f += nw) {
-    const uint32_t p = flagged[f];
-    const float* xp = x + (uint64_t)p * d;
-    float m32 = INFINITY;
-    for (uint32_t kk = 0; kk < k; ++kk) m32 = fminf(m32, warp_dist32(xp, c + (uint64_t)kk * d, d, lane));
-    const float lim = m32 * widen;
-    double best = INFINITY;
-    int bk = 0x7fffffff;
-    for (uint32_t k0 = 0; k0 < k; k0 += 32) {
-      // candidates of this group of 32 centroids, then one lane per candidate
-      uint32_t cand = 0;
-      for (uint32_t t = 0; t < 32 && k0 + t < k; ++t) {
-        const float s32 = warp_dist32(xp, c + (uint64_t)(k0 + t) * d, d, lane);
-        if (s32 <= lim || m32 != m32) cand |= 1u << t;
-      }
-      if ((cand >> lane) & 1u) {
-        const uint32_t kk = k0 + lane;
-        const float* cp = c + (uint64_t)kk * d;
-        double s64 = 0.0;
-        for (uint32_t j = 0; j < d; ++j) {
-          const double t = __dsub_rn((double)xp[j], (double)cp[j]);
-          s64 = __dadd_rn(s64, __dmul_rn(t, t));
-        }
-        if (s64 < best) best = s64, bk = (int)kk;  // kk increases per lane: the lowest index keeps a tie
-      }
-    }
-    for (int o = 16; o; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
-      if (ob < best || (ob == best && ok < bk)) best = ob, bk = ok;
-    }
-    if (lane == 0) assign[p] = bk == 0x7fffffff ? 0 : bk;  // all-NaN distances: index 0, as the definition
-  }
-}
+struct SettleShared {
+  uint32_t m1[SET_T_MAX / 32][SET_RP], k1[SET_T_MAX / 32][SET_RP], m2[SET_T_MAX / 32][SET_RP];
+  uint32_t open[SET_T_MAX / 8 > SET_RP ? SET_T_MAX / 8 : SET_RP];  // points of the batch left to FP64
+  uint32_t nopen, ncand;
+  float red_f[SET_T_MAX / 32];
+  double red_d[SET_T_MAX / 32];
+  int red_k[SET_T_MAX / 32];
+};
 
-// The same re-check with the centroids staged in shared memory (row stride
-// D or D + 1 floats, whichever is odd: lanes reading different rows at one
-// column hit different banks).  Lane l owns centroids l, l+32, ... (at most KLANE of them): one
-// pass computes their FP32 distances into registers and the warp takes the
-// minimum; a point with more than one candidate within the bound goes to
-// the FP64 stage's list (deferred, ndef).
-constexpr int KLANE = 8;  // K <= 256
-// Points are handed out in contiguous ranges of at least RC_MIN per CTA, so
-// only as many CTAs stage the centroids as there is work for (the lists are
-// a few thousand points).  stat[0] counts the listed points (all checked in
-// FP32).
-constexpr uint32_t RC_MIN = 64;
-__global__ void km_recheck_fp64_smem_kernel(const float* __restrict__ x, uint32_t d, const float* __restrict__ c,
-                                            uint32_t k, const uint32_t* flagged, const uint32_t* nflag,
-                                            int32_t* assign, unsigned long long* stat, uint32_t* deferred,
-                                            uint32_t* ndef) {
-  pdl_wait();
-  extern __shared__ float cs[];  // [k][d | 1]
-  const uint32_t nf = *nflag;
-  const uint32_t per = max(RC_MIN, (nf + gridDim.x - 1) / gridDim.x);
-  const uint64_t f_lo = (uint64_t)blockIdx.x * per;
-  const uint64_t f_hi = f_lo + per < nf ? f_lo + per : nf;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && stat) atomicAdd(stat, (unsigned long long)nf);
-  if (f_lo >= nf) return;  // no work for this CTA: no staging either
-  const uint32_t ld = d | 1;
-  for (uint32_t t = threadIdx.x; t < k * d; t += blockDim.x) cs[(t / d) * ld + (t % d)] = c[t];
+// The FP64 definition for point p, by the whole CTA (all threads call this).
+__device__ void settle_fp64(const float* __restrict__ x, uint32_t d, const float* __restrict__ c,
+                            const float* __restrict__ ct, uint32_t k, uint32_t p, int32_t* assign, double* prod,
+                            float* xs, float* dist, uint32_t* cand, SettleShared& S) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const float widen = rel_bound_widen(d);
+  const uint32_t cc = max(1u, min(SET_PROD / d, blockDim.x));  // candidates per product chunk (d <= 1024)
+  const float* xp = x + (uint64_t)p * d;
+  __syncthreads();  // the shared arrays' previous use is over
+  for (uint32_t j = threadIdx.x; j < d; j += blockDim.x) xs[j] = xp[j];
+  if (threadIdx.x == 0) S.ncand = 0;
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const uint32_t wpb = blockDim.x >> 5;
-  const float g = 1.01f * (float)(d + 8) * 5.9604644775390625e-08f;
-  const float widen = (1.f + g) / (1.f - g) * (1.f + 4.f * 5.9604644775390625e-08f);
-  for (uint64_t f = f_lo + (threadIdx.x >> 5); f < f_hi; f += wpb) {
-    const uint32_t p = flagged[f];
-    const float* xp = x + (uint64_t)p * d;
-    float dist[KLANE];
-#pragma unroll
-    for (int q = 0; q < KLANE; ++q) dist[q] = 0.f;
+  float m = INFINITY;
+  for (uint32_t kk = threadIdx.x; kk < k; kk += blockDim.x) {
+    float s32 = 0.f;
     for (uint32_t j = 0; j < d; ++j) {
-      const float xv = __ldg(xp + j);
-#pragma unroll
-      for (int q = 0; q < KLANE; ++q) {
-        const uint32_t kk = lane + 32 * q;
-        if (kk < k) {
-          const float t = xv - cs[kk * ld + j];
-          dist[q] = fmaf(t, t, dist[q]);
-        }
+      const float t = xs[j] - __ldg(ct + (uint64_t)j * k + kk);
+      s32 = fmaf(t, t, s32);
+    }
+    dist[kk] = s32;
+    m = fminf(m, s32);
+  }
+  for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) S.red_f[warp] = m;
+  __syncthreads();
+  float m32 = S.red_f[0];
+  for (int w = 1; w < nw; ++w) m32 = fminf(m32, S.red_f[w]);
+  const float lim = m32 * widen;
+  for (uint32_t kk = threadIdx.x; kk < k; kk += blockDim.x)
+    if (dist[kk] <= lim || m32 != m32) cand[atomicAdd(&S.ncand, 1u)] = kk;
+  __syncthreads();
+  const uint32_t nc = S.ncand;
+  double best = INFINITY;
+  int bk = 0x7fffffff;
+  for (uint32_t c0 = 0; c0 < nc; c0 += cc) {
+    const uint32_t cn = nc - c0 < cc ? nc - c0 : cc;
+    for (uint32_t ci = warp; ci < cn; ci += nw) {
+      const float* cp = c + (uint64_t)cand[c0 + ci] * d;
+      for (uint32_t j = lane; j < d; j += 32) {
+        const double t = __dsub_rn((double)xs[j], (double)__ldg(cp + j));
+        prod[ci * d + j] = __dmul_rn(t, t);
       }
     }
-    float m32 = INFINITY;
-#pragma unroll
-    for (int q = 0; q < KLANE; ++q)
-      if (lane + 32 * q < k) m32 = fminf(m32, dist[q]);
-    for (int o = 16; o; o >>= 1) m32 = fminf(m32, __shfl_xor_sync(0xffffffffu, m32, o));
-    const float lim = m32 * widen;
-    // one candidate within the bound: it is the argmin, no FP64 needed
-    uint32_t ncand = 0;
-    int first = -1;
-#pragma unroll
-    for (int q = 0; q < KLANE; ++q) {
-      const uint32_t kk = lane + 32 * q;
-      const bool cq = kk < k && (dist[q] <= lim || m32 != m32);
-      if (cq && first < 0) first = (int)kk;
-      ncand += (uint32_t)__popc(__ballot_sync(0xffffffffu, cq));
+    __syncthreads();
+    if (threadIdx.x < cn) {
+      double s64 = 0.0;
+      for (uint32_t j = 0; j < d; ++j) s64 = __dadd_rn(s64, prod[threadIdx.x * d + j]);
+      const int kk = (int)cand[c0 + threadIdx.x];
+      if (s64 < best || (s64 == best && kk < bk)) best = s64, bk = kk;
     }
-    if (ncand == 1) {
-      if (first >= 0) assign[p] = first;
-    } else if (lane == 0) {
-      deferred[atomicAdd(ndef, 1u)] = p;
-    }
+    __syncthreads();
+  }
+  for (int o = 16; o; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
+    if (ob < best || (ob == best && ok < bk)) best = ob, bk = ok;
+  }
+  if (lane == 0) S.red_d[warp] = best, S.red_k[warp] = bk;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < nw; ++w)
+      if (S.red_d[w] < best || (S.red_d[w] == best && S.red_k[w] < bk)) best = S.red_d[w], bk = S.red_k[w];
+    assign[p] = bk == 0x7fffffff ? 0 : bk;
   }
 }
 
-// The FP64 stage: the exact argmin of each point the pair and re-check passes
-// deferred, one CTA per point (all of them at once: there are tens to a few
-// hundred per iteration).  FP32 direct differences to every centroid (one
-// thread per centroid), the block minimum, the candidates within the
-// relative bound of it; then the definition in FP64 for the candidates only:
-// the products (x_j - c_j)^2, separately rounded, for all dimensions of a
-// chunk of candidates at once, and one thread per candidate adding them with
-// the dimensions in order, so the FP64 pipe (narrow on this GPU) runs 2
-// instructions per (candidate, dimension) spread over the block and one
-// dependent chain of D adds per chunk.  The lowest index wins an exact tie;
-// all-NaN distances give index 0, as the definition.  stat[1] counts the points.
-constexpr int F64_THREADS = 256;
-constexpr uint32_t F64_PROD = 8192;  // doubles of product scratch
-inline size_t fp64_stage_smem(uint32_t d, uint32_t k) {
-  return (size_t)F64_PROD * 8 + (size_t)d * 4 + (size_t)k * 8 + 64;
-}
-__global__ void __launch_bounds__(F64_THREADS) km_fp64_stage_kernel(const float* __restrict__ x, uint32_t d,
-                                                                    const float* __restrict__ c, uint32_t k,
-                                                                    const uint32_t* list, const uint32_t* nlist,
-                                                                    int32_t* assign, unsigned long long* stat) {
+// MULTI: more centroids than threads, so each thread keeps a running top-2.
+// With maxabs not null (the first iteration, whose distance pass or a pass
+// before it found max |x|) one thread also sets the update's exponent.
+template <bool MULTI>
+__global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
+    const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, const float* __restrict__ ct,
+    uint32_t k, const uint2* __restrict__ pairs, const uint32_t* npairs, const uint32_t* __restrict__ list,
+    const uint32_t* nlist, int32_t* assign, unsigned long long* stat, const unsigned int* maxabs, int* shift,
+    unsigned int* cmax_next) {
   pdl_wait();
-  extern __shared__ __align__(16) unsigned char f64_sm[];
-  double* prod = reinterpret_cast<double*>(f64_sm);   // [cc][d]
-  float* xs = reinterpret_cast<float*>(prod + F64_PROD);  // [d]
+  extern __shared__ __align__(16) unsigned char set_sm[];
+  __shared__ SettleShared S;
+  const size_t stage = (size_t)d * SET_LD * 4;
+  float* xt = reinterpret_cast<float*>(set_sm);       // [d][SET_LD] staged points, or
+  double* prod = reinterpret_cast<double*>(set_sm);   // [cc][d] FP64 products
+  float* xs = reinterpret_cast<float*>(set_sm + (stage > SET_PROD * 8 ? stage : SET_PROD * 8));  // [d]
   float* dist = xs + d;                               // [k]
   uint32_t* cand = reinterpret_cast<uint32_t*>(dist + k);  // [k]
-  __shared__ float red_f[F64_THREADS / 32];
-  __shared__ double red_d[F64_THREADS / 32];
-  __shared__ int red_k[F64_THREADS / 32];
-  __shared__ uint32_t ncand;
-  const uint32_t nf = *nlist;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && stat) atomicAdd(stat + 1, (unsigned long long)nf);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float g = 1.01f * (float)(d + 8) * 5.9604644775390625e-08f;
-  const float widen = (1.f + g) / (1.f - g) * (1.f + 4.f * 5.9604644775390625e-08f);
-  // candidates per product chunk (d <= 1024: at least 8), one summing thread each
-  const uint32_t cc = F64_PROD / d < (uint32_t)F64_THREADS ? F64_PROD / d : (uint32_t)F64_THREADS;
-  for (uint32_t f = blockIdx.x; f < nf; f += gridDim.x) {
-    const uint32_t p = list[f];
-    const float* xp = x + (uint64_t)p * d;
-    __syncthreads();  // the previous point's use of the shared arrays is over
-    for (uint32_t j = threadIdx.x; j < d; j += F64_THREADS) xs[j] = xp[j];
-    if (threadIdx.x == 0) ncand = 0;
-    __syncthreads();
-    float m = INFINITY;
-    for (uint32_t kk = threadIdx.x; kk < k; kk += F64_THREADS) {
-      const float* cp = c + (uint64_t)kk * d;
-      float s32 = 0.f;
-      for (uint32_t j = 0; j < d; ++j) {
-        const float t = xs[j] - __ldg(cp + j);
-        s32 = fmaf(t, t, s32);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t np = *npairs, nf = *nlist;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (maxabs) *shift = fx_shift_of(__uint_as_float(*maxabs), n);
+    *cmax_next = 0;  // the next iteration's max ||c||
+    if (np + nf) atomicAdd(stat, (unsigned long long)np + nf);
+  }
+  const float widen = rel_bound_widen(d);
+  const uint32_t ppb = blockDim.x >> 3;  // pairs per batch
+  const uint64_t rb = ((uint64_t)nf + SET_RP - 1) / SET_RP, nb = rb + ((uint64_t)np + ppb - 1) / ppb;
+  unsigned long long settled = 0;  // thread 0: points settled in FP64
+  for (uint64_t b = blockIdx.x; b < nb; b += gridDim.x) {
+    __syncthreads();  // the previous batch's shared arrays are no longer read
+    if (threadIdx.x == 0) S.nopen = 0;
+    if (b < rb) {
+      const uint32_t f0 = (uint32_t)b * SET_RP;
+      const uint32_t cnt = nf - f0 < (uint32_t)SET_RP ? nf - f0 : (uint32_t)SET_RP;
+      for (uint32_t r = warp; r < (uint32_t)SET_RP; r += nw) {
+        const float* xp = x + (uint64_t)list[f0 + (r < cnt ? r : 0)] * d;
+        for (uint32_t j = lane; j < d; j += 32) xt[j * SET_LD + r] = xp[j];
       }
-      dist[kk] = s32;
-      m = fminf(m, s32);
-    }
-    for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) red_f[warp] = m;
-    __syncthreads();
-    float m32 = red_f[0];
-    for (int w = 1; w < F64_THREADS / 32; ++w) m32 = fminf(m32, red_f[w]);
-    const float lim = m32 * widen;
-    for (uint32_t kk = threadIdx.x; kk < k; kk += F64_THREADS)
-      if (dist[kk] <= lim || m32 != m32) cand[atomicAdd(&ncand, 1u)] = kk;
-    __syncthreads();
-    const uint32_t nc = ncand;
-    double best = INFINITY;
-    int bk = 0x7fffffff;
-    for (uint32_t c0 = 0; c0 < nc; c0 += cc) {
-      const uint32_t cn = nc - c0 < cc ? nc - c0 : cc;
-      for (uint32_t ci = warp; ci < cn; ci += F64_THREADS / 32) {
-        const float* cp = c + (uint64_t)cand[c0 + ci] * d;
-        for (uint32_t j = lane; j < d; j += 32) {
-          const double t = __dsub_rn((double)xs[j], (double)__ldg(cp + j));
-          prod[ci * d + j] = __dmul_rn(t, t);
+      __syncthreads();
+      uint32_t b1[MULTI ? SET_RP : 1], bi[MULTI ? SET_RP : 1], b2[MULTI ? SET_RP : 1];
+      if (MULTI) {
+#pragma unroll
+        for (int r = 0; r < (MULTI ? SET_RP : 1); ++r) b1[r] = b2[r] = 0x7F800000u, bi[r] = 0;
+      }
+      unsigned long long acc[SET_RP / 2];
+      for (uint32_t kk = threadIdx.x; MULTI ? kk - threadIdx.x < k : kk == threadIdx.x; kk += blockDim.x) {
+#pragma unroll
+        for (int q = 0; q < SET_RP / 2; ++q) acc[q] = 0ull;
+        if (kk < k) {
+#pragma unroll 2
+          for (uint32_t j = 0; j < d; ++j) {
+            const float cv = -__ldg(ct + (uint64_t)j * k + kk);
+            const unsigned long long nc = pack2(cv, cv);
+            const ulonglong2* row = reinterpret_cast<const ulonglong2*>(xt + j * SET_LD);
+#pragma unroll
+            for (int q = 0; q < SET_RP / 4; ++q) {
+              const ulonglong2 v = row[q];
+              sqdiff2(acc[2 * q], v.x, nc);
+              sqdiff2(acc[2 * q + 1], v.y, nc);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < SET_RP / 2; ++q) acc[q] = 0x7F8000007F800000ull;  // no centroid: +inf
+        }
+        if (MULTI) {
+#pragma unroll
+          for (int r = 0; r < (MULTI ? SET_RP : 1); ++r) {
+            const uint32_t v = (uint32_t)(acc[r >> 1] >> (32 * (r & 1)));
+            if (v < b1[r]) b2[r] = b1[r], b1[r] = v, bi[r] = kk;
+            else b2[r] = min(b2[r], v);
+          }
+        }
+      }
+      // distances are non-negative (or NaN, above every other), so their bits order like them
+#pragma unroll
+      for (int r = 0; r < SET_RP; ++r) {
+        const uint32_t v = MULTI ? b1[MULTI ? r : 0] : (uint32_t)(acc[r >> 1] >> (32 * (r & 1)));
+        const uint32_t m1 = __reduce_min_sync(0xffffffffu, v);
+        const int lead = __ffs(__ballot_sync(0xffffffffu, v == m1)) - 1;
+        const uint32_t m2 =
+            __reduce_min_sync(0xffffffffu, lane == lead ? (MULTI ? b2[MULTI ? r : 0] : 0x7F800000u) : v);
+        if (lane == lead) {
+          S.m1[warp][r] = m1;
+          S.m2[warp][r] = m2;
+          S.k1[warp][r] = MULTI ? bi[MULTI ? r : 0] : threadIdx.x;
         }
       }
       __syncthreads();
-      if (threadIdx.x < cn) {
-        double s64 = 0.0;
-        for (uint32_t j = 0; j < d; ++j) s64 = __dadd_rn(s64, prod[threadIdx.x * d + j]);
-        const int kk = (int)cand[c0 + threadIdx.x];
-        if (s64 < best || (s64 == best && kk < bk)) best = s64, bk = kk;
+      if (threadIdx.x < cnt) {
+        const uint32_t r = threadIdx.x;
+        uint32_t m1 = S.m1[0][r], k1 = S.k1[0][r], m2 = S.m2[0][r];
+        for (int w = 1; w < nw; ++w) {
+          const uint32_t o1 = S.m1[w][r];
+          if (o1 < m1) m2 = min(m1, S.m2[w][r]), m1 = o1, k1 = S.k1[w][r];
+          else m2 = min(m2, o1);
+        }
+        const uint32_t p = list[f0 + r];
+        if (__uint_as_float(m2) > __uint_as_float(m1) * widen) assign[p] = (int32_t)k1;
+        else S.open[atomicAdd(&S.nopen, 1u)] = p;
       }
+    } else {
       __syncthreads();
+      const uint64_t f = (b - rb) * ppb + (threadIdx.x >> 3);
+      const uint32_t sl = threadIdx.x & 7;
+      const bool live = f < np;
+      const uint2 e = live ? pairs[f] : make_uint2(0u, 0u);
+      const uint32_t k1 = e.y & 0xffffu, k2 = e.y >> 16;
+      const float* xp = x + (uint64_t)e.x * d;
+      const float* c1 = c + (uint64_t)k1 * d;
+      const float* c2 = c + (uint64_t)k2 * d;
+      float f1 = 0.f, f2 = 0.f;
+      if (live)
+        for (uint32_t j = sl; j < d; j += 8) {
+          const float xv = xp[j];
+          const float t1 = xv - c1[j], t2 = xv - c2[j];
+          f1 = fmaf(t1, t1, f1);
+          f2 = fmaf(t2, t2, f2);
+        }
+#pragma unroll
+      for (int o = 4; o; o >>= 1) {
+        f1 += __shfl_xor_sync(0xffffffffu, f1, o);
+        f2 += __shfl_xor_sync(0xffffffffu, f2, o);
+      }
+      if (live && sl == 0) {
+        if (f2 > f1 * widen) assign[e.x] = (int32_t)k1;
+        else if (f1 > f2 * widen) assign[e.x] = (int32_t)k2;
+        else S.open[atomicAdd(&S.nopen, 1u)] = e.x;
+      }
     }
-    for (int o = 16; o; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
-      if (ob < best || (ob == best && ok < bk)) best = ob, bk = ok;
-    }
-    if (lane == 0) red_d[warp] = best, red_k[warp] = bk;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < F64_THREADS / 32; ++w)
-        if (red_d[w] < best || (red_d[w] == best && red_k[w] < bk)) best = red_d[w], bk = red_k[w];
-      assign[p] = bk == 0x7fffffff ? 0 : bk;
-    }
+    const uint32_t no = S.nopen;
+    for (uint32_t i = 0; i < no; ++i) settle_fp64(x, d, c, ct, k, S.open[i], assign, prod, xs, dist, cand, S);
+    settled += no;
   }
+  if (threadIdx.x == 0 && settled) atomicAdd(stat + 1, settled);
 }
 
 // max |x| over all coordinates (as float bits; non-negative floats order like ints)
@@ -1303,47 +1243,67 @@ __global__ void __launch_bounds__(WS_THREADS, 1) km_window_sum_kernel(const floa
     if (C[i]) atomicAdd(counts + i, (unsigned long long)C[i]);
 }
 
-// Sum of the g partials of each element (warp w of a CTA adds partials w,
-// w + 8, ... of 32 consecutive elements), then the centroid as in
-// km_finalize_kernel.
+// The centroids of the next round, one CTA per centroid: the sum of the g
+// partials of each dimension (or the sums of the sorted update), c_k =
+// (sum_k * 2^-s) / count_k in FP64, rounded to FP32 (an empty cluster keeps
+// c_k), and what the next distance pass and re-check need of them: the shifted
+// norm cn[k] = ||c_k - center||^2 (FP32 FMAs; center null: no shift), the
+// largest norm, the transposed copy ct and cleared counters.  first: only the
+// latter, for the initial centroids.
 constexpr int RF_THREADS = 256;
-__global__ void __launch_bounds__(RF_THREADS) km_reduce_finalize_kernel(const long long* __restrict__ part,
-                                                                        uint32_t g, float* c, uint32_t k, uint32_t d,
-                                                                        const unsigned long long* counts,
-                                                                        const int* shift, unsigned int* cmax_bits) {
+__global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long* __restrict__ part, uint32_t g,
+                                                                 long long* sums, float* c, uint32_t k, uint32_t d,
+                                                                 unsigned long long* counts, const int* shift,
+                                                                 const float* __restrict__ center,
+                                                                 float* __restrict__ cn, unsigned int* cmax,
+                                                                 float* __restrict__ ct, uint32_t* nflag,
+                                                                 uint32_t first) {
   pdl_wait();
   __shared__ long long red[RF_THREADS / 32][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint64_t kd = (uint64_t)k * d;
-  const uint64_t e = (uint64_t)blockIdx.x * 32 + lane;
-  long long a = 0;
-  if (e < kd) {
+  const uint64_t kd = (uint64_t)k * d, kk = blockIdx.x, row = kk * d;
+  const unsigned long long cnt = first ? 0 : counts[kk];
+  const double inv = cnt ? ldexp(1.0, -*shift) : 0.0;
+  float nrm = 0.f;
+  __syncthreads();  // every thread has read the count that is cleared below
+  for (uint32_t j0 = 0; j0 < d; j0 += 32) {
+    const uint32_t j = j0 + lane;
+    long long a = 0;
+    if (cnt && part) {
+      if (j < d) {
 #pragma unroll 4
-    for (uint32_t j = w; j < g; j += RF_THREADS / 32) a += part[(uint64_t)j * kd + e];
-  }
-  red[w][lane] = a;
-  __syncthreads();
-  if (w == 0) {
+        for (uint32_t q = w; q < g; q += RF_THREADS / 32) a += part[(uint64_t)q * kd + row + j];
+      }
+      __syncthreads();  // the previous dimensions' sums have been read
+      red[w][lane] = a;
+      __syncthreads();
+    }
+    if (w == 0 && j < d) {
+      if (cnt) {
+        if (part) {
 #pragma unroll
-    for (int i = 1; i < RF_THREADS / 32; ++i) a += red[i][lane];
-    if (e < kd) {
-      const unsigned long long cnt = counts[e / d];
-      if (cnt) c[e] = (float)(((double)a * ldexp(1.0, -*shift)) / (double)cnt);
+          for (int i = 1; i < RF_THREADS / 32; ++i) a += red[i][lane];
+        } else {
+          a = sums[row + j];
+        }
+      }
+      const float v = cnt ? (float)(((double)a * inv) / (double)cnt) : c[row + j];
+      if (cnt) c[row + j] = v;
+      if (!part && !first) sums[row + j] = 0;
+      ct[(uint64_t)j * k + kk] = v;
+      const float t = center ? __fsub_rn(v, center[j]) : v;
+      nrm = fmaf(t, t, nrm);
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *cmax_bits = 0;
-}
-
-// c_k = (sum_k * 2^-s) / count_k in FP64, rounded to FP32; empty clusters keep c_k.
-__global__ void km_finalize_kernel(float* c, uint32_t k, uint32_t d, const long long* sums,
-                                   const unsigned long long* counts, const int* shift, unsigned int* cmax_bits) {
-  const double inv = ldexp(1.0, -*shift);
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (uint64_t)k * d;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const unsigned long long cnt = counts[i / d];
-    if (cnt) c[i] = (float)(((double)sums[i] * inv) / (double)cnt);
+  if (w == 0) {
+    for (int o = 16; o; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+    if (lane == 0) {
+      cn[kk] = nrm;
+      atomicMax(cmax, __float_as_uint(sqrtf(nrm)));
+      counts[kk] = 0;
+      if (kk == 0) nflag[1] = nflag[4] = 0;  // points to re-check, pairs
+    }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *cmax_bits = 0;
 }
 
 __global__ void km_finish_kernel(const float* c, uint64_t kd, float* out_c, const int32_t* assign, uint32_t n,
@@ -1383,9 +1343,9 @@ size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k) {
   b += 256;                            // stats, counters (nflag, maxabs, cmax, pairs), shift
   b += a256((uint64_t)n * 4);          // points to re-check; the sorted update's permutation
   b += a256((uint64_t)n * 8);          // pair list
-  b += a256((uint64_t)n * 4);          // FP64 stage list
   b += a256((uint64_t)k * 4);          // ||c||^2
   b += a256((uint64_t)d * 4);          // center
+  b += a256((uint64_t)k * d * 4);      // transposed centroids
   b += a256((uint64_t)k * 4);          // per-cluster write cursor
   if (local_sums_fit(d, k)) b += a256((uint64_t)LS_MAX_CTAS * k * d * 8);  // per-CTA partial sums
   return (size_t)b;
@@ -1406,9 +1366,9 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes) {
   b.shift = reinterpret_cast<int*>(ctl + 128);
   b.flagged = reinterpret_cast<uint32_t*>(take(n * 4));
   b.pairs = reinterpret_cast<uint2*>(take(n * 8));
-  b.deferred = reinterpret_cast<uint32_t*>(take(n * 4));
   b.cnorm = reinterpret_cast<float*>(take(k * 4));
   b.center = reinterpret_cast<float*>(take(d * 4));
+  b.ct = reinterpret_cast<float*>(take(k * d * 4));
   b.kcursor = reinterpret_cast<uint32_t*>(take(k * 4));
   b.part = local_sums_fit(d, k) ? reinterpret_cast<long long*>(take((uint64_t)LS_MAX_CTAS * k * d * 8)) : nullptr;
   if ((uint64_t)(q - p) > bytes) return cudaErrorInvalidValue;
@@ -1418,17 +1378,16 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes) {
 bool km_tc_supported(uint32_t d, uint32_t k);
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
-                                    KmBuffers& b, const DevInfo& di, cudaStream_t s, uint64_t* nk, bool maxabs);
+                                    KmBuffers& b, const unsigned int* cmax, const DevInfo& di, cudaStream_t s,
+                                    uint64_t* nk, bool maxabs);
 
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,
                           cudaStream_t s, float* out_c, int32_t* out_a, unsigned long long* out_s, uint64_t* nk) {
   cudaError_t e;
   const uint32_t n = b.n, d = b.d, k = b.k;
   int* shift = b.shift;
-  unsigned int* cmax_bits = b.nflag + 3;
-  km_setup_kernel<<<(d + 31) / 32, SETUP_THREADS, 0, s>>>(init, k, d, b.cent, b.center, b.nflag, b.stats);
-  ++*nk;
-  // The distance pass only has to settle the clear cases (every near tie is
+  auto cmax_of = [&](uint32_t it) { return b.nflag + 6 + (it & 1); };  // max ||c||, one word per parity of the round
+    // The distance pass only has to settle the clear cases (every near tie is
   // re-checked), so an FP32 job takes the tensor-core pass on split operands
   // wherever that covers its shape: the assignments are the FP64 definition's
   // either way.  At 200,003 x 37, K = 100 the pass takes 32 us instead of 156
@@ -1436,12 +1395,6 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   // the copies (diagnostics of the pipelined passes) keeps FP32 jobs on the
   // SIMT pass, which waits on nothing.
   const bool tc = b.precision != MR_KM_FP32 || (km_tc_supported(d, k) && b.polls < 0 && b.stop_copies == 0);
-  // the fixed-point scale needs max |x|: a pass of its own for the SIMT
-  // path; the tensor-core pass finds it while converting the first iteration
-  if (!tc) {
-    km_maxabs_kernel<<<di.sms * 4, 256, 0, s>>>(x, (uint64_t)n * d, b.maxabs);
-    ++*nk;
-  }
   const int asm_bytes = (DC_MAX * CS_LD + DC_MAX * XS_LD) * 4;
   if ((e = cudaFuncSetAttribute(km_assign_fp32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 asm_bytes)) != cudaSuccess ||
@@ -1494,66 +1447,52 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   if (b.grid_cap && ls_grid > b.grid_cap) ls_grid = b.grid_cap;
   if (ls_grid < 1) ls_grid = 1;
   const long long polls = b.polls < 0 ? pipe::SPIN_LIMIT : b.polls;
-  const int rc_bytes = (int)((uint64_t)k * (d + 1) * 4);
-  const bool rc_smem = k <= 32 * KLANE && rc_bytes <= di.smem_optin;
-  // as many re-check CTAs per SM as the centroid copies allow (at most 3: 48 warps)
-  int rc_per_sm = rc_smem ? (di.smem_optin + 1024) / (rc_bytes + 1024) : 1;
-  rc_per_sm = rc_per_sm < 1 ? 1 : (rc_per_sm > 3 ? 3 : rc_per_sm);
-  if (rc_smem &&
-      (e = cudaFuncSetAttribute(km_recheck_fp64_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rc_bytes)) !=
-          cudaSuccess)
-    return e;
-  const int f64_bytes = (int)fp64_stage_smem(d, k);
-  if ((e = cudaFuncSetAttribute(km_fp64_stage_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, f64_bytes)) !=
+  const int set_t = set_threads(k);
+  const size_t set_bytes = set_smem(d, k);
+  auto set_kernel = k > (uint32_t)set_t ? km_settle_kernel<true> : km_settle_kernel<false>;
+  if ((e = cudaFuncSetAttribute(set_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes)) !=
       cudaSuccess)
     return e;
   const uint32_t ntiles = (n + TP - 1) / TP;
   uint32_t agrid = ntiles < (uint32_t)di.sms * 2 ? ntiles : (uint32_t)di.sms * 2;
   if (b.grid_cap && agrid > b.grid_cap) agrid = b.grid_cap;
+  km_setup_kernel<<<(d + 31) / 32, SETUP_THREADS, 0, s>>>(init, k, d, b.cent, b.center,
+                                                          local ? nullptr : b.sums, b.nflag, b.stats);
+  ++*nk;
+  // the fixed-point scale needs max |x|: a pass of its own for the SIMT
+  // path; the tensor-core pass finds it while converting the first iteration
+  if (!tc) {
+    km_maxabs_kernel<<<di.sms * 4, 256, 0, s>>>(x, (uint64_t)n * d, b.maxabs);
+    ++*nk;
+  }
+  const float* center = tc ? b.center : nullptr;
+  auto finalize = [&](uint32_t it, bool first) {
+    ++*nk;
+    return launch_pdl(km_finalize_kernel, dim3(k), dim3(RF_THREADS), 0, s,
+                      local ? (const long long*)b.part : (const long long*)nullptr, ls_grid, b.sums, b.cent, k, d,
+                      b.counts, (const int*)shift, center, b.cnorm, cmax_of(it), b.ct, b.nflag, first ? 1u : 0u);
+  };
+  if ((e = finalize(0, true)) != cudaSuccess) return e;
   for (uint32_t it = 0; it < iters; ++it) {
     // kernels that follow another kernel of this job on the stream start
     // while it drains (programmatic dependent launch; each waits first)
-    const unsigned pgrid = k < 8 * 64 ? (k + 7) / 8 : 64;
-    if ((e = launch_pdl(km_prep_kernel, dim3(pgrid), dim3(256), 0, s, (const float*)b.cent, k, d,
-                        tc ? (const float*)b.center : (const float*)nullptr, b.cnorm, cmax_bits,
-                        local ? (long long*)nullptr : b.sums, b.counts, b.nflag)) != cudaSuccess)
-      return e;
     if (tc) {
-      if ((e = launch_kmeans_tc_assign(x, n, d, b.cent, k, b, di, s, nk, it == 0)) != cudaSuccess) return e;
+      if ((e = launch_kmeans_tc_assign(x, n, d, b.cent, k, b, cmax_of(it), di, s, nk, it == 0)) != cudaSuccess)
+        return e;
     } else {
       if ((e = kt_begin(b.kt, s)) != cudaSuccess) return e;
       (k <= 256 ? km_assign_fp32_kernel<true> : km_assign_fp32_kernel<false>)<<<agrid, KM_THREADS, asm_bytes, s>>>(
-          x, n, d, b.cent, k, b.cnorm, cmax_bits, nullptr, nullptr, b.assign, b.flagged, b.nflag + 1, b.pairs,
-          b.nflag + 4, nullptr);
+          x, n, d, b.cent, k, b.cnorm, cmax_of(it), b.assign, b.flagged, b.nflag + 1, b.pairs, b.nflag + 4);
       if ((e = cudaGetLastError()) != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;
       ++*nk;
     }
-    // one warp per pair, latency-bound: a full SM of warps (32 registers a thread)
-    if ((e = launch_pdl(km_pair_kernel, dim3(di.sms * 8), dim3(256), 0, s, x, n, d, (const float*)b.cent,
-                        (const uint2*)b.pairs, (const uint32_t*)(b.nflag + 4), b.assign, b.stats, b.deferred,
-                        b.nflag + 5, it == 0 ? (const unsigned int*)b.maxabs : (const unsigned int*)nullptr,
-                        shift)) != cudaSuccess)
+    if ((e = launch_pdl(set_kernel, dim3(di.sms * (2048 / set_t < 8 ? 2048 / set_t : 8)), dim3(set_t), set_bytes, s, x,
+                        n, d, (const float*)b.cent, (const float*)b.ct, k, (const uint2*)b.pairs,
+                        (const uint32_t*)(b.nflag + 4), (const uint32_t*)b.flagged, (const uint32_t*)(b.nflag + 1),
+                        b.assign, b.stats, it == 0 ? (const unsigned int*)b.maxabs : (const unsigned int*)nullptr,
+                        shift, cmax_of(it + 1))) != cudaSuccess)
       return e;
     ++*nk;
-    // the points the distance pass could not decide are re-checked straight
-    // away with FP32 direct differences; the points where those leave more
-    // than one candidate go to the FP64 stage
-    const uint32_t* rl = b.flagged;
-    const uint32_t* rn = b.nflag + 1;
-    if (rc_smem)
-      e = launch_pdl(km_recheck_fp64_smem_kernel, dim3(di.sms * rc_per_sm), dim3(512), (size_t)rc_bytes, s, x, d,
-                     (const float*)b.cent, k, rl, rn, b.assign, b.stats, b.deferred, b.nflag + 5);
-    else
-      e = launch_pdl(km_recheck_fp64_kernel, dim3(di.sms * 4), dim3(256), 0, s, x, d, (const float*)b.cent, k, rl, rn,
-                     b.assign, b.stats);
-    if (e != cudaSuccess) return e;
-    // the FP64 stage: the points the pair and re-check passes left to the
-    // definition, one CTA each, all at once
-    if ((e = launch_pdl(km_fp64_stage_kernel, dim3(di.sms * 2), dim3(F64_THREADS), (size_t)f64_bytes, s, x, d,
-                        (const float*)b.cent, k, (const uint32_t*)b.deferred, (const uint32_t*)(b.nflag + 5), b.assign,
-                        b.stats)) != cudaSuccess)
-      return e;
-    *nk += 2;  // re-check, FP64 stage
     if (local) {  // update with local arrays
       if (wsum)
         e = launch_pdl(ws_kernel, dim3(ls_grid),
@@ -1567,12 +1506,8 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
         e = launch_pdl(km_local_sum_kernel, dim3(ls_grid), dim3(LS_THREADS), (size_t)ls_bytes, s, x, n, d, k,
                        (const int32_t*)b.assign, (const int*)shift, b.part, b.counts);
       if (e != cudaSuccess) return e;
-      if ((e = launch_pdl(km_reduce_finalize_kernel, dim3((unsigned)(((uint64_t)k * d + 31) / 32)), dim3(RF_THREADS),
-                          0, s, (const long long*)b.part, ls_grid, b.cent, k, d, (const unsigned long long*)b.counts,
-                          (const int*)shift, cmax_bits)) != cudaSuccess)
-        return e;
-      *nk += 3;  // prep, update, reduction
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      ++*nk;
+      if ((e = finalize(it + 1, false)) != cudaSuccess) return e;
       continue;
     }
     // update: counting sort of the points by cluster, then run-wise sums
@@ -1584,9 +1519,8 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
     // after the scatter, kcursor[c] is one past the last position of cluster c
     km_sum_kernel<<<(unsigned)((sum_warps * 32 + 255) / 256), 256, 0, s>>>(x, n, d, k, b.kcursor, b.flagged, shift,
                                                                            b.sums);
-    km_finalize_kernel<<<64, 256, 0, s>>>(b.cent, k, d, b.sums, b.counts, shift, cmax_bits);
-    *nk += 6;  // prep, count, offsets, scatter, sums, finalize
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    *nk += 4;  // count, offsets, scatter, sums
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = finalize(it + 1, false)) != cudaSuccess) return e;
   }
   if ((e = launch_pdl(km_finish_kernel, dim3(di.sms * 4), dim3(256), 0, s, (const float*)b.cent, (uint64_t)k * d,
                       out_c, (const int32_t*)b.assign, n, out_a, (const unsigned long long*)b.stats, out_s, iters)) !=

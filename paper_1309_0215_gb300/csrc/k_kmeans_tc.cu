@@ -620,14 +620,15 @@ cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t 
 }
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
-                                    KmBuffers& b, const DevInfo& di, cudaStream_t s, uint64_t* nk, bool maxabs) {
+                                    KmBuffers& b, const unsigned int* cmax, const DevInfo& di, cudaStream_t s,
+                                    uint64_t* nk, bool maxabs) {
   const uint32_t ntiles = (n + TM - 1) / TM;
   uint32_t grid = ntiles < (uint32_t)di.sms ? ntiles : (uint32_t)di.sms;
   if (b.grid_cap && grid > b.grid_cap) grid = b.grid_cap;
   const int terms = b.precision == MR_KM_BF16X1_TC ? 1 : 3;
   cudaError_t e = kt_begin(b.kt, s);
   if (e != cudaSuccess) return e;
-  e = launch_km_tc_kernel(terms, x, n, d, c, k, b.center, b.cnorm, b.nflag + 3, b.assign, b.flagged, b.nflag + 1,
+  e = launch_km_tc_kernel(terms, x, n, d, c, k, b.center, b.cnorm, cmax, b.assign, b.flagged, b.nflag + 1,
                           b.pairs, b.nflag + 4, b.stats + 3, nullptr, (int)grid, s, b.polls < 0 ? SPIN_LIMIT : b.polls,
                           b.stop_copies, maxabs ? b.maxabs : nullptr);
   if (e != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;

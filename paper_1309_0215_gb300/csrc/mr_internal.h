@@ -148,12 +148,12 @@ struct KmBuffers {
   unsigned long long* counts = nullptr;  // [k]
   unsigned long long* stats = nullptr;   // [4]
   uint32_t* flagged = nullptr;  // [n] points to re-check; later the sorted update's permutation
-  uint32_t* nflag = nullptr;    // [8] counters: [1] points to re-check, [2] max|x| bits, [3] max||c|| bits, [4] pairs,
-                                //     [5] points deferred to the FP64 stage
-  uint32_t* deferred = nullptr; // [n] points whose choice needs the FP64 definition
+  uint32_t* nflag = nullptr;    // [8] counters: [1] points to re-check, [2] max|x| bits, [4] pairs, [6], [7] max||c||
+                                //     bits of even and odd rounds
   uint2* pairs = nullptr;       // [n] {point, k1 | k2 << 16}: exact choice between two centroids
   float* cnorm = nullptr;       // [k] ||c||^2 (of the shifted centroids on the tensor-core path)
   float* center = nullptr;      // [d] the shift
+  float* ct = nullptr;          // [d][k] transposed centroids
   unsigned int* maxabs = nullptr;  // [1] bits of max |x|
   int* shift = nullptr;         // [1] fixed-point scale exponent
   uint32_t* kcursor = nullptr;  // [k] counting-sort write cursors
