@@ -220,7 +220,7 @@ __device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 12
 template <int TERMS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, uint32_t k,
-                    const float* __restrict__ center, const float* __restrict__ cnorm, const unsigned int* cmax_bits, int32_t* __restrict__ assign,
+                    const float* __restrict__ center, const float* __restrict__ cnorm, const unsigned int* cmax_bits, uint32_t* __restrict__ assign, uint32_t* nchg,
                     uint32_t* __restrict__ list, uint32_t* nlist, uint2* __restrict__ pairs, uint32_t* npairs,
                     unsigned long long* timeouts, float* dbg, long long polls, uint32_t stop_copies,
                     unsigned int* maxabs) {
@@ -450,11 +450,18 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
     const float eps_sum = TERMS == 3 ? (3.05f * 1.52587890625e-05f + (float)(3 * KD + 8) * 4.76837158203125e-07f)
                                      : (2.f * 3.90625e-03f + 1.52587890625e-05f + (float)(KD + 8) * 4.76837158203125e-07f);
     const float eps32 = 1.01f * (float)(d + 12) * 5.9604644775390625e-08f;
+    uint32_t moved = 0;  // this lane's points that changed cluster
     for (uint32_t i = 0;; ++i) {
       const uint32_t tile = blockIdx.x + i * gridDim.x;
       if (tile >= ntiles) break;
       const int b = (int)(i & 1);
       const uint32_t v = i >> 1;
+      uint32_t was[FIN_QUADS];  // the points' words, loaded while the tile is in the pipeline
+#pragma unroll
+      for (int h = 0; h < FIN_QUADS; ++h) {
+        const uint32_t p = tile * TM + (uint32_t)((fw * FIN_QUADS + h) * 32 + lane);
+        was[h] = nchg && p < n ? assign[p] & 0xffffu : 0u;
+      }
       const bool okx = mbar_wait(&S.xfull[b], v & 1, err, polls);
       if (!__all_sync(0xffffffffu, okx)) break;
       int o1[FIN_QUADS][QUARTERS], o2[FIN_QUADS][QUARTERS], ol[FIN_QUADS][QUARTERS];
@@ -495,7 +502,12 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
           // keys under-state a distance by less than 2^-15 of it (2^-14 allowed)
           const float gap = 2.f * e + 6.103515625e-05f * d1;
           if (g1 < 0) flag = true;  // a negative smallest distance: re-check
-          else if (d2 - d1 > fmaxf(1e-3f * d1, gap)) assign[p] = g1 & 0xFF;
+          else if (d2 - d1 > fmaxf(1e-3f * d1, gap)) {
+            const uint32_t now = (uint32_t)g1 & 0xFFu;
+            const uint32_t old = nchg ? was[h] : now;
+            assign[p] = km_word(now, old);
+            moved += now != old;
+          }
           else if (d3 - d1 > gap) pair = true;  // only the top two can be the exact minimum
           else flag = true;
         }
@@ -517,6 +529,8 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
         }
       }
     }
+    moved = __reduce_add_sync(0xffffffffu, moved);
+    if (lane == 0 && moved) atomicAdd(nchg, moved);
   } else {
     // ------------------------------------------------------------- epilogue
     // Warp e reads TMEM lane quadrant e % 4 (rows 32 (e % 4) ..) and column
@@ -593,11 +607,12 @@ bool km_tc_supported(uint32_t d, uint32_t k) { return d >= 1 && d <= KD && k >= 
 
 size_t km_tc_smem_bytes() { return sizeof(TcSmem) + 1024; }
 
-// Raw launch: list/nlist receive the points to re-check, pairs/npairs the
+// Raw launch: nchg (null in a job's first round, whose words hold nothing yet)
+// counts the points that changed cluster; list/nlist receive the points to re-check, pairs/npairs the
 // two-candidate points; maxabs (when not null) receives the bits of max |x|.
 cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                 const float* center, const float* cnorm, const unsigned int* cmax_bits,
-                                int32_t* assign, uint32_t* list, uint32_t* nlist, uint2* pairs, uint32_t* npairs, unsigned long long* timeouts,
+                                uint32_t* assign, uint32_t* nchg, uint32_t* list, uint32_t* nlist, uint2* pairs, uint32_t* npairs, unsigned long long* timeouts,
                                 float* dbg, int grid, cudaStream_t s, long long polls, uint32_t stop_copies,
                                 unsigned int* maxabs) {
   const int smem = (int)km_tc_smem_bytes();
@@ -607,28 +622,28 @@ cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t 
         cudaSuccess)
       return e;
     return launch_pdl(km_tc_assign_kernel<3>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
-                      cnorm, cmax_bits, assign, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
+                      cnorm, cmax_bits, assign, nchg, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
                       maxabs);
   } else {
     if ((e = cudaFuncSetAttribute(km_tc_assign_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
         cudaSuccess)
       return e;
     return launch_pdl(km_tc_assign_kernel<1>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
-                      cnorm, cmax_bits, assign, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
+                      cnorm, cmax_bits, assign, nchg, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
                       maxabs);
   }
 }
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
-                                    KmBuffers& b, const unsigned int* cmax, const DevInfo& di, cudaStream_t s,
-                                    uint64_t* nk, bool maxabs) {
+                                    KmBuffers& b, const unsigned int* cmax, uint32_t* nchg, const DevInfo& di,
+                                    cudaStream_t s, uint64_t* nk, bool maxabs) {
   const uint32_t ntiles = (n + TM - 1) / TM;
   uint32_t grid = ntiles < (uint32_t)di.sms ? ntiles : (uint32_t)di.sms;
   if (b.grid_cap && grid > b.grid_cap) grid = b.grid_cap;
   const int terms = b.precision == MR_KM_BF16X1_TC ? 1 : 3;
   cudaError_t e = kt_begin(b.kt, s);
   if (e != cudaSuccess) return e;
-  e = launch_km_tc_kernel(terms, x, n, d, c, k, b.center, b.cnorm, cmax, b.assign, b.flagged, b.nflag + 1,
+  e = launch_km_tc_kernel(terms, x, n, d, c, k, b.center, b.cnorm, cmax, b.assign, nchg, b.flagged, b.nflag + 1,
                           b.pairs, b.nflag + 4, b.stats + 3, nullptr, (int)grid, s, b.polls < 0 ? SPIN_LIMIT : b.polls,
                           b.stop_copies, maxabs ? b.maxabs : nullptr);
   if (e != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;

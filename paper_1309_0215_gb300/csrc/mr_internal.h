@@ -138,18 +138,25 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// An assignment word holds the point's cluster (low half) and the cluster it
+// had when the sums were last updated (high half; K <= 4096).
+__device__ __forceinline__ uint32_t km_word(uint32_t now, uint32_t summed) { return now | (summed << 16); }
+// Both, for indexing: a word that a timed-out pass left unwritten counts as cluster 0.
+__device__ __forceinline__ uint32_t km_now(uint32_t w, uint32_t k) { return (w & 0xffffu) < k ? w & 0xffffu : 0u; }
+__device__ __forceinline__ uint32_t km_summed(uint32_t w, uint32_t k) { return (w >> 16) < k ? w >> 16 : 0u; }
 #endif
 
 struct KmBuffers {
   uint32_t n = 0, d = 0, k = 0;
   float* cent = nullptr;        // [k][d] current centroids (FP32 state)
-  int32_t* assign = nullptr;    // [n]
+  uint32_t* assign = nullptr;   // [n] assignment words (km_word)
   long long* sums = nullptr;    // [k][d] fixed-point sums
-  unsigned long long* counts = nullptr;  // [k]
+  unsigned long long* counts = nullptr;  // [k] cluster sizes, then [k] those a full update counts
   unsigned long long* stats = nullptr;   // [4]
   uint32_t* flagged = nullptr;  // [n] points to re-check; later the sorted update's permutation
-  uint32_t* nflag = nullptr;    // [8] counters: [1] points to re-check, [2] max|x| bits, [4] pairs, [6], [7] max||c||
-                                //     bits of even and odd rounds
+  uint32_t* nflag = nullptr;    // [8] counters: [1] points to re-check, [2] max|x| bits, [4] pairs; of even and odd
+                                //     rounds: [0], [5] points that changed cluster, [6], [7] max||c|| bits
   uint2* pairs = nullptr;       // [n] {point, k1 | k2 << 16}: exact choice between two centroids
   float* cnorm = nullptr;       // [k] ||c||^2 (of the shifted centroids on the tensor-core path)
   float* center = nullptr;      // [d] the shift

@@ -320,3 +320,31 @@ def test_kmeans_fp32_on_the_tensor_cores(mr, n, d, k, offset, scale):
     assert np.array_equal(a, a_ref)
     assert _rel_err(c, c_ref) <= TOL
     assert int(stats[3]) == 0
+
+
+@pytest.mark.parametrize("n,d,k", [
+    (30_001, 64, 40),     # window-sorted update, 8-byte loads
+    (30_001, 21, 9),      # window-sorted update, one dimension per lane
+    (12_001, 96, 16),     # row-pipelined update
+    (12_003, 67, 16),     # plain local-array update
+    (12_001, 130, 260),   # sorted update
+])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_kmeans_update_by_changes(mr, n, d, k, precision):
+    """Rounds in which few points change cluster update the sums by those
+    points alone.  Ten rounds in one call equal ten calls of one round (each a
+    full update), byte for byte: the sums are exact integers."""
+    if precision and (d > 64 or k > 256):
+        pytest.skip("shape outside the BF16 path")
+    x, _, _ = synth.kmeans_points(n, d, 8, seed=n + d, sigma=4.0)
+    dx = _dev(x)
+    cur = synth.kmeans_init(x, k, seed=n)
+    c10, a10, _ = mr.kmeans(dx, _dev(cur), 10, precision)
+    moved, last = [], None
+    for _ in range(10):
+        cur, a, _ = mr.kmeans(dx, _dev(cur), 1, precision)
+        moved.append(n if last is None else int((a != last).sum()))
+        last = a
+    assert np.array_equal(a10, last)
+    assert np.array_equal(c10, cur)
+    assert min(moved) <= n // 32 < max(moved)  # both kinds of update ran
