@@ -27,8 +27,7 @@
 //    per run instead of one per coordinate.
 #include <cmath>
 
-#include "dev_pipe.cuh"
-#include "mr_internal.h"
+#include "dev_tc.cuh"
 
 namespace mrgb {
 namespace {
@@ -149,7 +148,7 @@ template <bool KEYS>
 __global__ void __launch_bounds__(KM_THREADS, 2)
 km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, uint32_t k,
                       const float* __restrict__ cn, const unsigned int* cmax_bits, uint32_t* __restrict__ assign,
-                      uint32_t* nchg, uint32_t* flagged, uint32_t* nflag, uint2* __restrict__ pairs, uint32_t* npairs) {
+                      uint32_t* nchg, uint32_t* flagged, uint32_t* nflag, KmFew* __restrict__ pairs, uint32_t* npairs) {
   extern __shared__ float km_sm[];
   const int dc = d < DC_MAX ? (int)d : DC_MAX;
   const int kc = k < KC_MAX ? (int)k : KC_MAX;
@@ -331,7 +330,7 @@ km_assign_fp32_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const
       base = __shfl_sync(0xffffffffu, base, 0);
       if (pair) {
         const uint32_t p = pi;
-        pairs[base + __popc(pm & ((1u << lane) - 1))] = make_uint2(p, (uint32_t)mt.k1 | ((uint32_t)mt.k2 << 16));
+        pairs[base + __popc(pm & ((1u << lane) - 1))] = km_few(p, (uint32_t)mt.k1 | ((uint32_t)mt.k2 << 12), 2);
       }
     }
     const unsigned fm = __ballot_sync(0xffffffffu, flag);
@@ -368,8 +367,8 @@ __device__ __forceinline__ int fx_shift_of(float m, uint32_t n) {
 // ------------------------------------------------- settling the near ties
 // One kernel settles what the distance pass left open.
 //
-// Points with two candidates (pairs, eight lanes each): FP32 direct
-// differences to both centroids.  Their relative error is at most g =
+// Points with a few candidates (eight lanes each): FP32 direct differences to
+// those centroids.  Their relative error is at most g =
 // gamma_{D+3} for any summation order (Higham, eq. 3.5 on a sum of squares),
 // so a ratio beyond widen decides the exact order.
 //
@@ -502,13 +501,57 @@ __device__ void settle_fp64(const float* __restrict__ x, uint32_t d, const float
   }
 }
 
+__device__ __forceinline__ uint32_t few_cand(const KmFew& e, uint32_t i) {
+  return (uint32_t)(((uint64_t)e.lo | ((uint64_t)e.hi << 32)) >> (12 * i)) & 0xFFFu;
+}
+// FP32 squared distances of an entry's first M candidates, by eight lanes
+// (lane sl of them): every candidate's row and the point's are read together,
+// 16 bytes a lane where rows allow (vec).  All 32 lanes call this.
+template <int M>
+__device__ __forceinline__ void few_dists(const float* __restrict__ x, const float* __restrict__ c, uint32_t d,
+                                          const KmFew& e, uint32_t nc, uint32_t sl, bool vec,
+                                          float (&f)[KM_CAND_MAX]) {
+  const float* xp = x + (uint64_t)e.p * d;
+  const float* cp[M];
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    cp[i] = c + (uint64_t)few_cand(e, (uint32_t)i < nc ? i : 0) * d;
+    f[i] = 0.f;
+  }
+  if (nc == 0) {
+  } else if (vec) {
+    for (uint32_t j = 4 * sl; j < d; j += 32) {
+      const float4 xv = __ldg(reinterpret_cast<const float4*>(xp + j));
+#pragma unroll
+      for (int i = 0; i < M; ++i) {
+        const float4 cv = __ldg(reinterpret_cast<const float4*>(cp[i] + j));
+        const float t0 = xv.x - cv.x, t1 = xv.y - cv.y, t2 = xv.z - cv.z, t3 = xv.w - cv.w;
+        f[i] = fmaf(t0, t0, fmaf(t1, t1, fmaf(t2, t2, fmaf(t3, t3, f[i]))));
+      }
+    }
+  } else {
+    for (uint32_t j = sl; j < d; j += 8) {
+      const float xv = __ldg(xp + j);
+#pragma unroll
+      for (int i = 0; i < M; ++i) {
+        const float t = xv - __ldg(cp[i] + j);
+        f[i] = fmaf(t, t, f[i]);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < M; ++i)
+#pragma unroll
+    for (int o = 4; o; o >>= 1) f[i] += __shfl_xor_sync(0xffffffffu, f[i], o);
+}
+
 // MULTI: more centroids than threads, so each thread keeps a running top-2.
 // With maxabs not null (the first iteration, whose distance pass or a pass
 // before it found max |x|) one thread also sets the update's exponent.
 template <bool MULTI>
 __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
     const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, const float* __restrict__ ct,
-    uint32_t k, const uint2* __restrict__ pairs, const uint32_t* npairs, const uint32_t* __restrict__ list,
+    uint32_t k, const KmFew* __restrict__ pairs, const uint32_t* npairs, const uint32_t* __restrict__ list,
     const uint32_t* nlist, uint32_t* assign, uint32_t* nchg, unsigned long long* stat, const unsigned int* maxabs, int* shift,
     unsigned int* cmax_next) {
   pdl_wait();
@@ -529,7 +572,8 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
     if (np + nf) atomicAdd(stat, (unsigned long long)np + nf);
   }
   const float widen = rel_bound_widen(d);
-  const uint32_t ppb = blockDim.x >> 3;  // pairs per batch
+  const uint32_t ppb = blockDim.x >> 3;  // few-candidate points per batch
+  const bool vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   const uint64_t rb = ((uint64_t)nf + SET_RP - 1) / SET_RP, nb = rb + ((uint64_t)np + ppb - 1) / ppb;
   unsigned long long settled = 0;  // thread 0: points settled in FP64
   for (uint64_t b = blockIdx.x; b < nb; b += gridDim.x) {
@@ -610,28 +654,22 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
       const uint64_t f = (b - rb) * ppb + (threadIdx.x >> 3);
       const uint32_t sl = threadIdx.x & 7;
       const bool live = f < np;
-      const uint2 e = live ? pairs[f] : make_uint2(0u, 0u);
-      const uint32_t k1 = e.y & 0xffffu, k2 = e.y >> 16;
-      const float* xp = x + (uint64_t)e.x * d;
-      const float* c1 = c + (uint64_t)k1 * d;
-      const float* c2 = c + (uint64_t)k2 * d;
-      float f1 = 0.f, f2 = 0.f;
-      if (live)
-        for (uint32_t j = sl; j < d; j += 8) {
-          const float xv = xp[j];
-          const float t1 = xv - c1[j], t2 = xv - c2[j];
-          f1 = fmaf(t1, t1, f1);
-          f2 = fmaf(t2, t2, f2);
-        }
+      const KmFew e = live ? pairs[f] : KmFew{0, 0, 0};
+      const uint32_t nc = live ? e.hi >> 28 : 0;
+      float fd[KM_CAND_MAX];
+      if (__any_sync(0xffffffffu, nc > 2)) few_dists<KM_CAND_MAX>(x, c, d, e, nc, sl, vec, fd);
+      else few_dists<2>(x, c, d, e, nc, sl, vec, fd);
+      float m1 = INFINITY, m2 = INFINITY;
+      uint32_t k1 = 0;
 #pragma unroll
-      for (int o = 4; o; o >>= 1) {
-        f1 += __shfl_xor_sync(0xffffffffu, f1, o);
-        f2 += __shfl_xor_sync(0xffffffffu, f2, o);
-      }
+      for (uint32_t i = 0; i < KM_CAND_MAX; ++i)
+        if (i < nc) {
+          if (fd[i] < m1) m2 = m1, m1 = fd[i], k1 = few_cand(e, i);
+          else if (!(fd[i] >= m2)) m2 = fd[i];  // (a NaN makes m2 NaN: the point is left to FP64)
+        }
       if (live && sl == 0) {
-        if (f2 > f1 * widen) settle_put(assign, e.x, k1, nchg, S);
-        else if (f1 > f2 * widen) settle_put(assign, e.x, k2, nchg, S);
-        else S.open[atomicAdd(&S.nopen, 1u)] = e.x;
+        if (m2 > m1 * widen) settle_put(assign, e.p, k1, nchg, S);
+        else S.open[atomicAdd(&S.nopen, 1u)] = e.p;
       }
     }
     __syncthreads();
@@ -1392,7 +1430,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) km_window_sum_kernel(const floa
 // (sum_k * 2^-s) / count_k in FP64, rounded to FP32 (an empty cluster keeps
 // c_k), and what the next distance pass and re-check need of them: the shifted
 // norm cn[k] = ||c_k - center||^2 (FP32 FMAs; center null: no shift), the
-// largest norm, the transposed copy ct and cleared counters.  first: only the
+// largest norm, the transposed copy ct, the wide pass's operands bop (null:
+// none) and cleared counters.  first: only the
 // latter, for the initial centroids.
 constexpr int RF_THREADS = 256;
 __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long* __restrict__ part, uint32_t g,
@@ -1403,8 +1442,8 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
                                                                  const int* shift,
                                                                  const float* __restrict__ center,
                                                                  float* __restrict__ cn, unsigned int* cmax,
-                                                                 float* __restrict__ ct, uint32_t* nflag,
-                                                                 uint32_t first) {
+                                                                 float* __restrict__ ct, uint8_t* bop,
+                                                                 uint32_t* nflag, uint32_t first) {
   pdl_wait();
   __shared__ long long red[RF_THREADS / 32][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1441,6 +1480,7 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
       ct[(uint64_t)j * k + kk] = v;
       const float t = center ? __fsub_rn(v, center[j]) : v;
       nrm = fmaf(t, t, nrm);
+      if (bop) tc::put_operand(bop, d, (uint32_t)kk, j, t);
     }
   }
   if (w == 0) {
@@ -1489,7 +1529,7 @@ inline uint64_t a256(uint64_t x) { return (x + 255) & ~255ull; }
 
 }  // namespace
 
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k) {
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide) {
   uint64_t b = 0;
   b += a256((uint64_t)k * d * 4);      // cent
   b += a256((uint64_t)n * 4 + 16);     // assign (+16: the update copies ids in 16-byte units)
@@ -1497,16 +1537,17 @@ size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k) {
   b += a256((uint64_t)k * 8 * 2);      // counts, counts of a full update
   b += 256;                            // stats, counters (nflag, maxabs, cmax, pairs), shift
   b += a256((uint64_t)n * 4);          // points to re-check; the sorted update's permutation
-  b += a256((uint64_t)n * 8);          // pair list
+  b += a256((uint64_t)n * sizeof(KmFew));  // points with a few candidates
   b += a256((uint64_t)k * 4);          // ||c||^2
   b += a256((uint64_t)d * 4);          // center
   b += a256((uint64_t)k * d * 4);      // transposed centroids
   b += a256((uint64_t)k * 4);          // per-cluster write cursor
   if (local_sums_fit(d, k)) b += a256((uint64_t)LS_MAX_CTAS * k * d * 8);  // per-CTA partial sums
+  if (wide) b += a256(km_wide_operand_bytes(d, k));
   return (size_t)b;
 }
 
-cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes) {
+cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide) {
   const uint64_t n = b.n, d = b.d, k = b.k;
   uint8_t* q = p;
   auto take = [&](uint64_t sz) { uint8_t* r = q; q += a256(sz); return r; };
@@ -1520,12 +1561,13 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes) {
   b.maxabs = reinterpret_cast<unsigned int*>(b.nflag + 2);
   b.shift = reinterpret_cast<int*>(ctl + 128);
   b.flagged = reinterpret_cast<uint32_t*>(take(n * 4));
-  b.pairs = reinterpret_cast<uint2*>(take(n * 8));
+  b.pairs = reinterpret_cast<KmFew*>(take(n * sizeof(KmFew)));
   b.cnorm = reinterpret_cast<float*>(take(k * 4));
   b.center = reinterpret_cast<float*>(take(d * 4));
   b.ct = reinterpret_cast<float*>(take(k * d * 4));
   b.kcursor = reinterpret_cast<uint32_t*>(take(k * 4));
   b.part = local_sums_fit(d, k) ? reinterpret_cast<long long*>(take((uint64_t)LS_MAX_CTAS * k * d * 8)) : nullptr;
+  b.bop = wide ? take(km_wide_operand_bytes((uint32_t)d, (uint32_t)k)) : nullptr;
   if ((uint64_t)(q - p) > bytes) return cudaErrorInvalidValue;
   return cudaSuccess;
 }
@@ -1535,6 +1577,10 @@ bool km_tc_supported(uint32_t d, uint32_t k);
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                     KmBuffers& b, const unsigned int* cmax, uint32_t* nchg, const DevInfo& di,
                                     cudaStream_t s, uint64_t* nk, bool maxabs);
+
+cudaError_t launch_kmeans_wide_assign(const float* x, uint32_t n, uint32_t d, uint32_t k, KmBuffers& b,
+                                      const unsigned int* cmax, uint32_t* nchg, const DevInfo& di, cudaStream_t s,
+                                      uint64_t* nk, bool maxabs);
 
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,
                           cudaStream_t s, float* out_c, int32_t* out_a, unsigned long long* out_s, uint64_t* nk) {
@@ -1549,7 +1595,9 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   // and the whole ten-round call 0.91 ms instead of 2.11.  A context that has set a wait limit or stops
   // the copies (diagnostics of the pipelined passes) keeps FP32 jobs on the
   // SIMT pass, which waits on nothing.
-  const bool tc = b.precision != MR_KM_FP32 || (km_tc_supported(d, k) && b.polls < 0 && b.stop_copies == 0);
+  const bool plain = b.polls < 0 && b.stop_copies == 0;
+  const bool tc = b.precision != MR_KM_FP32 || (km_tc_supported(d, k) && plain);
+  const bool wide = !tc && b.bop && plain;
   const int asm_bytes = (DC_MAX * CS_LD + DC_MAX * XS_LD) * 4;
   if ((e = cudaFuncSetAttribute(km_assign_fp32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 asm_bytes)) != cudaSuccess ||
@@ -1616,11 +1664,13 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   ++*nk;
   // the fixed-point scale needs max |x|: a pass of its own for the SIMT
   // path; the tensor-core pass finds it while converting the first iteration
-  if (!tc) {
+  if (!tc && !wide) {
     km_maxabs_kernel<<<di.sms * 4, 256, 0, s>>>(x, (uint64_t)n * d, b.maxabs);
     ++*nk;
   }
-  const float* center = tc ? b.center : nullptr;
+  // rows and dimensions past K and D stay zero
+  if (wide && (e = cudaMemsetAsync(b.bop, 0, km_wide_operand_bytes(d, k), s)) != cudaSuccess) return e;
+  const float* center = tc || wide ? b.center : nullptr;
   const uint32_t lim = n / (local ? KM_DELTA_LOCAL : KM_DELTA_SORTED);  // points moved, at most, in an update by changes
   auto chg_of = [&](uint32_t it) { return b.nflag + ((it & 1) ? 5 : 0); };  // points that changed cluster in the round
   auto finalize = [&](uint32_t it, bool first) {
@@ -1629,7 +1679,8 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
                       local ? (const long long*)b.part : (const long long*)nullptr, ls_grid, b.sums, b.cent, k, d,
                       b.counts, b.counts + k, it > 1 ? (const uint32_t*)chg_of(it - 1) : (const uint32_t*)nullptr, lim,
                       chg_of(it),
-                      (const int*)shift, center, b.cnorm, cmax_of(it), b.ct, b.nflag, first ? 1u : 0u);
+                      (const int*)shift, center, b.cnorm, cmax_of(it), b.ct, wide ? b.bop : (uint8_t*)nullptr, b.nflag,
+                      first ? 1u : 0u);
   };
   if ((e = finalize(0, true)) != cudaSuccess) return e;
   unsigned long long* cnew = b.counts + k;
@@ -1640,6 +1691,9 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
     if (tc) {
       if ((e = launch_kmeans_tc_assign(x, n, d, b.cent, k, b, cmax_of(it), chg, di, s, nk, it == 0)) != cudaSuccess)
         return e;
+    } else if (wide) {
+      if ((e = launch_kmeans_wide_assign(x, n, d, k, b, cmax_of(it), chg, di, s, nk, it == 0)) != cudaSuccess)
+        return e;
     } else {
       if ((e = kt_begin(b.kt, s)) != cudaSuccess) return e;
       (k <= 256 ? km_assign_fp32_kernel<true> : km_assign_fp32_kernel<false>)<<<agrid, KM_THREADS, asm_bytes, s>>>(
@@ -1648,7 +1702,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
       ++*nk;
     }
     if ((e = launch_pdl(set_kernel, dim3(di.sms * (2048 / set_t < 8 ? 2048 / set_t : 8)), dim3(set_t), set_bytes, s, x,
-                        n, d, (const float*)b.cent, (const float*)b.ct, k, (const uint2*)b.pairs,
+                        n, d, (const float*)b.cent, (const float*)b.ct, k, (const KmFew*)b.pairs,
                         (const uint32_t*)(b.nflag + 4), (const uint32_t*)b.flagged, (const uint32_t*)(b.nflag + 1),
                         b.assign, chg, b.stats, it == 0 ? (const unsigned int*)b.maxabs : (const unsigned int*)nullptr,
                         shift, cmax_of(it + 1))) != cudaSuccess)

@@ -46,26 +46,22 @@
 // most twice that times (||x'|| + ||c'||): (D + 12) in place of (D + 8)
 // covers it, and x, c stand for x', c' in all of the bounds here.  The keys hold d~ truncated to 16 mantissa bits (t <= d~ <
 // t (1 + 2^-15)), so with G = 2E + 2^-14 t_1: if t_2 - t_1 > max(1e-3 t_1, G)
-// the tensor-core winner is the exact winner.  Otherwise, if b_3 - t_1 > G,
-// where b_3 is a lower bound of every key but the top two, every other
-// centroid has exact distance above t_1 (1 + 2^-15) + E >= d(k_1), so the
-// point only needs an exact FP64 choice between those two (pair list); every
-// other point goes to the FP32 pass (and from there, if still close, to
-// FP64), so assignments equal the FP64 argmin.
-#include <cuda_bf16.h>
-
-#include "dev_pipe.cuh"
-#include "mr_internal.h"
+// the tensor-core winner is the exact winner.  Otherwise, if b > t_1 + G for a
+// lower bound b of every key but each column quarter's two smallest, every
+// centroid not among those with a key up to t_1 + max(1e-3 t_1, G) has exact
+// distance above t_1 (1 + 2^-15) + E >= d(k_1); with at most KM_CAND_MAX of
+// them the point needs an exact choice between those few alone, else it is
+// listed and compared with every centroid (km_settle_kernel either way), so
+// assignments equal the FP64 argmin.
+#include "dev_tc.cuh"
 
 namespace mrgb {
 namespace {
 
-constexpr int TM = 128;          // points per tile = MMA M = TMEM lanes
-constexpr int KD = 64;           // padded dimension: one 128-byte row of BF16
-constexpr int NMAX = 256;        // centroids: MMA N
+using namespace tc;
+
 constexpr int EPI_WARPS = 16;     // four per TMEM lane quadrant, each on a quarter of the columns
-constexpr int QUARTERS = EPI_WARPS / 4;
-constexpr int EPI_COLS = NMAX / QUARTERS;  // 64 columns per epilogue warp
+static_assert(EPI_WARPS == 4 * QUARTERS, "one warp per TMEM lane quadrant and column quarter");
 constexpr int MMA_WARP = EPI_WARPS;
 constexpr int CVT_WARP0 = MMA_WARP + 1;
 constexpr int CVT_WARPS = 8;      // each converts TM / CVT_WARPS rows of a tile
@@ -80,9 +76,6 @@ constexpr int STAGES = 2;         // operand stages
 constexpr int XST = 2;            // FP32 staging buffers filled by the bulk copy engine
 constexpr int ACCS = 2;           // TMEM accumulators
 constexpr uint32_t TMEM_COLS = 512;  // two 256-column FP32 accumulators
-constexpr int NSET = 4;           // independent running top-2s per epilogue thread
-constexpr int CHUNK = 32;         // TMEM columns per tcgen05.ld in the epilogue
-
 struct __align__(1024) TcSmem {
   uint8_t b_hi[NMAX * 128];
   uint8_t b_lo[NMAX * 128];
@@ -105,123 +98,11 @@ struct __align__(1024) TcSmem {
 
 static_assert(sizeof(TcSmem) + 1024 <= 232448, "shared memory of one CTA");
 
-using namespace pipe;
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
-// 1024 bytes apart (stride byte offset), descriptor version 1.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-
-// Instruction descriptor, kind::f16: BF16 A and B (K-major), FP32 D, M = 128.
-__host__ __device__ constexpr uint32_t mma_idesc(uint32_t n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit(unsigned long long* b) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(b))
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[32]) { tmem_ld32(taddr, v); }
-
-// Sortable key of a distance: its FP32 bit pattern with the low 8 mantissa
-// bits replaced by the centroid column, compared as a signed integer.  For
-// non-negative floats the pattern is monotonic, so keys order by distance
-// truncated to 16 mantissa bits (an under-statement of less than 2^-15 of
-// it), then by column; a negative distance (only rounding of a point lying on
-// a centroid produces one) orders below every non-negative one, and a point
-// whose smallest key is negative is always re-checked.
-__device__ __forceinline__ int dist_key(float dist, uint32_t col) {
-  return (int)((__float_as_uint(dist) & 0xFFFFFF00u) | col);
-}
-__device__ __forceinline__ float key_dist(int key) { return __uint_as_float((uint32_t)key & 0xFFFFFF00u); }
-
-// Key of a column that holds no centroid: above every finite distance's key,
-// and it decodes to +inf.
-constexpr int KEY_NONE = 0x7F8000FF;
-
-// Insert key into the sorted pair (t1 <= t2): three min/max.
-__device__ __forceinline__ void top2_insert(int& t1, int& t2, int key) {
-  const int h = max(t1, key);
-  t1 = min(t1, key);
-  t2 = min(t2, h);
-}
-
-// Smallest two of two sorted pairs.
-__device__ __forceinline__ void top2_merge(int& a1, int& a2, int b1, int b2) {
-  const int c2 = min(max(a1, b1), min(a2, b2));
-  a1 = min(a1, b1);
-  a2 = c2;
-}
-
-// Distances of CHUNK columns (ch .. ch + CHUNK - 1) of one point into its
-// NSET running top-2s (column j goes to set j mod NSET).  MASK: some columns
-// are >= k (their TMEM words are not written by the MMA and may hold
-// anything), so those keys are forced to KEY_NONE.
-template <bool MASK>
-__device__ __forceinline__ void top2_keys(const uint32_t (&acc)[CHUNK], uint32_t ch, float nxv, const float* cn,
-                                          uint32_t k, int (&t1)[NSET], int (&t2)[NSET], float* dbg_row) {
-#pragma unroll
-  for (int j = 0; j < CHUNK; j += 4) {
-    const float4 c4 = *reinterpret_cast<const float4*>(cn + ch + j);
-    const float cv[4] = {c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint32_t kk = ch + (uint32_t)(j + e);
-      const float dist = fmaf(-2.f, __uint_as_float(acc[j + e]), nxv) + cv[e];
-      int key = dist_key(dist, kk);
-      if (MASK) {
-        if (kk >= k) key = KEY_NONE;
-        else if (dbg_row) dbg_row[kk] = dist;
-      }
-      top2_insert(t1[(j + e) % NSET], t2[(j + e) % NSET], key);
-    }
-  }
-}
-
-// BF16 hi/lo split of two values, packed little-endian (element 0 low half).
-// (one paired round-to-nearest conversion for each of hi and lo)
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  const float2 hf = __bfloat1622float2(h);
-  const __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  lo = *reinterpret_cast<const uint32_t*>(&l);
-}
-
-// Byte offset of 16-byte chunk c of row r in a 128-byte-swizzled tile whose
-// base is 1024-byte aligned (chunk index XOR row mod 8).
-__device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
-
 template <int TERMS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, uint32_t k,
                     const float* __restrict__ center, const float* __restrict__ cnorm, const unsigned int* cmax_bits, uint32_t* __restrict__ assign, uint32_t* nchg,
-                    uint32_t* __restrict__ list, uint32_t* nlist, uint2* __restrict__ pairs, uint32_t* npairs,
+                    uint32_t* __restrict__ list, uint32_t* nlist, KmFew* __restrict__ pairs, uint32_t* npairs,
                     unsigned long long* timeouts, float* dbg, long long polls, uint32_t stop_copies,
                     unsigned int* maxabs) {
   extern __shared__ uint8_t tc_raw[];
@@ -444,8 +325,7 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
     // ------------------------------------------------------------ finalizers
     // Warp f takes the points of TMEM lane quadrants FIN_QUADS f .. (rows
     // 32 q + lane of each): it merges the four column quarters' top-2 keys
-    // into the row's exact top-2 (g1, g2) and a lower bound g3 of every other
-    // key, then applies the margin tests.
+    // into the row's exact top-2 (g1, g2), then applies the margin tests.
     const int fw = warp - FIN_WARP0;
     const float eps_sum = TERMS == 3 ? (3.05f * 1.52587890625e-05f + (float)(3 * KD + 8) * 4.76837158203125e-07f)
                                      : (2.f * 3.90625e-03f + 1.52587890625e-05f + (float)(KD + 8) * 4.76837158203125e-07f);
@@ -481,52 +361,50 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
       if (lane == 0) mbar_arrive(&S.xfree[b]);
 #pragma unroll
       for (int h = 0; h < FIN_QUADS; ++h) {
-        int g1 = o1[h][0], g2 = o2[h][0], g3 = ol[h][0];
+        int g1 = o1[h][0], g2 = o2[h][0];
 #pragma unroll
         for (int u = 1; u < QUARTERS; ++u) top2_merge(g1, g2, o1[h][u], o2[h][u]);
-        // every key other than g1, g2 is >= g3: the quarters' bounds, and the
-        // quarters' top-2 keys that did not make the row's top-2
-#pragma unroll
-        for (int u = 0; u < QUARTERS; ++u) {
-          g3 = min(g3, ol[h][u]);
-          g3 = (o1[h][u] != g1 && o1[h][u] != g2) ? min(g3, o1[h][u]) : g3;
-          g3 = (o2[h][u] != g1 && o2[h][u] != g2) ? min(g3, o2[h][u]) : g3;
-        }
         const uint32_t p = tile * TM + (uint32_t)((fw * FIN_QUADS + h) * 32 + lane);
-        bool flag = false, pair = false;
+        bool flag = false, few = false;
+        uint64_t cand = 0;
+        uint32_t ncand = 0;
         if (p < n) {
-          const float d1 = key_dist(g1), d2 = key_dist(g2), d3 = key_dist(g3);
+          const float d1 = key_dist(g1), d2 = key_dist(g2);
           const float xn = sqrtf(nxv[h]);
           // (1e-36: the products of tiny values may be flushed to zero)
           const float e = 2.f * eps_sum * xn * cmax + eps32 * (xn + cmax) * (xn + cmax) + 1e-36f;
           // keys under-state a distance by less than 2^-15 of it (2^-14 allowed)
           const float gap = 2.f * e + 6.103515625e-05f * d1;
-          if (g1 < 0) flag = true;  // a negative smallest distance: re-check
-          else if (d2 - d1 > fmaxf(1e-3f * d1, gap)) {
+          const float lim = fmaxf(1e-3f * d1, gap);
+          if (g1 < 0) {
+            flag = true;  // a negative smallest distance: re-check
+          } else if (d2 - d1 > lim) {
             const uint32_t now = (uint32_t)g1 & 0xFFu;
             const uint32_t old = nchg ? was[h] : now;
             assign[p] = km_word(now, old);
             moved += now != old;
+          } else {
+            // candidates: the quarters' top-2 keys within the margin, if every
+            // other key is beyond it
+            bool rest = false;
+#pragma unroll
+            for (int u = 0; u < QUARTERS; ++u) {
+              rest |= !(key_dist(ol[h][u]) - d1 > gap);
+#pragma unroll
+              for (int t = 0; t < 2; ++t) {
+                const int key = t ? o2[h][u] : o1[h][u];
+                if (key_dist(key) - d1 <= lim) {
+                  cand = (cand << 12) | ((uint32_t)key & 0xFFu);
+                  ++ncand;
+                }
+              }
+            }
+            few = !rest && ncand >= 2 && ncand <= KM_CAND_MAX;
+            flag = !few;
           }
-          else if (d3 - d1 > gap) pair = true;  // only the top two can be the exact minimum
-          else flag = true;
         }
-        const unsigned pm = __ballot_sync(0xffffffffu, pair);
-        if (pm) {
-          uint32_t base = 0;
-          if (lane == 0) base = atomicAdd(npairs, (uint32_t)__popc(pm));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (pair)
-            pairs[base + __popc(pm & ((1u << lane) - 1))] =
-                make_uint2(p, ((uint32_t)g1 & 0xFFu) | (((uint32_t)g2 & 0xFFu) << 16));
-        }
-        const unsigned fm = __ballot_sync(0xffffffffu, flag);
-        if (fm) {
-          uint32_t base = 0;
-          if (lane == 0) base = atomicAdd(nlist, (uint32_t)__popc(fm));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (flag) list[base + __popc(fm & ((1u << lane) - 1))] = p;
-        }
+        warp_append(few, npairs, lane, [&](uint32_t at) { pairs[at] = km_few(p, cand, ncand); });
+        warp_append(flag, nlist, lane, [&](uint32_t at) { list[at] = p; });
       }
     }
     moved = __reduce_add_sync(0xffffffffu, moved);
@@ -574,12 +452,8 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.empty_acc[b]);
-      int w1 = t1[0], w2 = t2[0];
-#pragma unroll
-      for (int a = 1; a < NSET; ++a) top2_merge(w1, w2, t1[a], t2[a]);
-      int lb = KEY_NONE;
-#pragma unroll
-      for (int a = 0; a < NSET; ++a) lb = min(lb, (t1[a] == w1 || t1[a] == w2) ? t2[a] : t1[a]);
+      int w1, w2, lb;
+      top2_sets(t1, t2, w1, w2, lb);
       if (i >= ACCS) {
         const bool okf = mbar_wait(&S.xfree[b], (v + 1) & 1, err, polls);
         if (!__all_sync(0xffffffffu, okf)) break;
@@ -612,7 +486,7 @@ size_t km_tc_smem_bytes() { return sizeof(TcSmem) + 1024; }
 // two-candidate points; maxabs (when not null) receives the bits of max |x|.
 cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                 const float* center, const float* cnorm, const unsigned int* cmax_bits,
-                                uint32_t* assign, uint32_t* nchg, uint32_t* list, uint32_t* nlist, uint2* pairs, uint32_t* npairs, unsigned long long* timeouts,
+                                uint32_t* assign, uint32_t* nchg, uint32_t* list, uint32_t* nlist, KmFew* pairs, uint32_t* npairs, unsigned long long* timeouts,
                                 float* dbg, int grid, cudaStream_t s, long long polls, uint32_t stop_copies,
                                 unsigned int* maxabs) {
   const int smem = (int)km_tc_smem_bytes();

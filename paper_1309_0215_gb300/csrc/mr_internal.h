@@ -136,7 +136,16 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
+// A point with 2 to KM_CAND_MAX candidate centroids, 12 bits each (K <= 4096),
+// and their number in the top bits.
+constexpr uint32_t KM_CAND_MAX = 5;
+struct KmFew {
+  uint32_t p, lo, hi;
+};
 #ifdef __CUDACC__
+__device__ __forceinline__ KmFew km_few(uint32_t p, uint64_t cand, uint32_t ncand) {
+  return KmFew{p, (uint32_t)cand, ((uint32_t)(cand >> 32) & 0x0FFFFFFFu) | (ncand << 28)};
+}
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // An assignment word holds the point's cluster (low half) and the cluster it
@@ -157,12 +166,13 @@ struct KmBuffers {
   uint32_t* flagged = nullptr;  // [n] points to re-check; later the sorted update's permutation
   uint32_t* nflag = nullptr;    // [8] counters: [1] points to re-check, [2] max|x| bits, [4] pairs; of even and odd
                                 //     rounds: [0], [5] points that changed cluster, [6], [7] max||c|| bits
-  uint2* pairs = nullptr;       // [n] {point, k1 | k2 << 16}: exact choice between two centroids
+  KmFew* pairs = nullptr;       // [n] points with a few candidate centroids
   float* cnorm = nullptr;       // [k] ||c||^2 (of the shifted centroids on the tensor-core path)
   float* center = nullptr;      // [d] the shift
   float* ct = nullptr;          // [d][k] transposed centroids
   unsigned int* maxabs = nullptr;  // [1] bits of max |x|
   int* shift = nullptr;         // [1] fixed-point scale exponent
+  uint8_t* bop = nullptr;       // centroid operands of the wide tensor-core pass (nullptr: not taken)
   uint32_t* kcursor = nullptr;  // [k] counting-sort write cursors
   long long* part = nullptr;    // [CTAs][k][d] partial sums of the local-array update (nullptr: sort path)
   KTimer* kt = nullptr;         // times the distance pass of each iteration
@@ -174,12 +184,15 @@ struct KmBuffers {
   uint32_t grid_cap = 0;
   uint32_t stop_copies = 0;
 };
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k);
-cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes);
+// wide: with the wide tensor-core pass's operands
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide);
+cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes, bool wide);
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,
                           cudaStream_t s, float* out_cent, int32_t* out_assign, unsigned long long* out_stats,
                           uint64_t* nk);
 bool km_tc_supported(uint32_t d, uint32_t k);
+bool km_wide_supported(uint32_t d, uint32_t k);
+size_t km_wide_operand_bytes(uint32_t d, uint32_t k);
 
 // --------------------------------------------------------- batched launch
 struct BatchJob {

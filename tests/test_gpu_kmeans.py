@@ -348,3 +348,32 @@ def test_kmeans_update_by_changes(mr, n, d, k, precision):
     assert np.array_equal(a10, last)
     assert np.array_equal(c10, cur)
     assert min(moved) <= n // 32 < max(moved)  # both kinds of update ran
+
+
+@pytest.mark.parametrize("n,d,k,cap", [
+    (1_999, 65, 3, 0),      # one value in the second dimension chunk
+    (1_281, 128, 257, 0),   # one centroid in the second centroid chunk
+    (20_001, 96, 300, 3),   # many tiles per CTA: two point buffers, two ring stages
+    (12_003, 130, 520, 3),  # three dimension chunks (one point buffer), three centroid chunks, rows not 16-byte
+    (5_003, 256, 256, 3),   # the widest rows
+    (9_001, 5, 777, 3),     # few dimensions, many centroids: four ring stages
+    (2_001, 3, 4_096, 0),   # the most centroids
+    (130, 200, 100, 0),     # a last tile of two points
+])
+@pytest.mark.parametrize("offset", [0.0, 5e4])
+def test_kmeans_wide_tensor_core_pass(mr, n, d, k, cap, offset):
+    """FP32 jobs beyond 64 dimensions or 256 centroids: two rounds, each from
+    the oracle's centroids, give the oracle's assignments and centroids."""
+    x, _, _ = synth.kmeans_points(n, d, 16, seed=n + d)
+    x = x + np.float32(offset)
+    ctx = mr.Context()
+    ctx.set_option(mr.OPT_KM_GRID_CAP, cap)
+    dx, cur = _dev(x), synth.kmeans_init(x, min(k, n), seed=n)
+    for _ in range(2):
+        c_ref, a_ref = oracle.kmeans(x, cur, 1)
+        c, a, st = _run_ctx(mr, ctx, dx, cur, 1, 0)
+        assert np.array_equal(a, a_ref)
+        assert _rel_err(c, c_ref) <= TOL
+        assert int(st[3]) == 0
+        cur = c_ref
+    ctx.close()
