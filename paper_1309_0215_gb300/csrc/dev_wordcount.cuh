@@ -65,6 +65,7 @@ struct JobDev {
   uint32_t* state;           // [0] overflow flag; [2..7] filled by the post phase
   uint8_t* out;
   uint64_t blk0;             // first compaction block of this job
+  uint64_t* host;            // host memory for {flags, records, key bytes}, written by the last kernel; or null
 };
 
 __device__ __forceinline__ bool is_ws(uint32_t c) { return c == 32u || (c - 9u) < 5u; }

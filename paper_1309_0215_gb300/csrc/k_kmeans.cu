@@ -1500,7 +1500,7 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
 
 __global__ void km_finish_kernel(const float* c, uint64_t kd, float* out_c, const uint32_t* assign, uint32_t n,
                                  int32_t* out_a, const unsigned long long* stats, unsigned long long* out_s,
-                                 uint32_t iters) {
+                                 uint32_t iters, volatile uint64_t* host) {
   pdl_wait();
   const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
@@ -1522,6 +1522,7 @@ __global__ void km_finish_kernel(const float* c, uint64_t kd, float* out_c, cons
     out_s[1] = stats[1];
     out_s[2] = iters;
     out_s[3] = stats[3];
+    if (host) *host = stats[3];
   }
 }
 
@@ -1743,7 +1744,8 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
     if ((e = cudaGetLastError()) != cudaSuccess || (e = finalize(it + 1, false)) != cudaSuccess) return e;
   }
   if ((e = launch_pdl(km_finish_kernel, dim3(di.sms * 4), dim3(256), 0, s, (const float*)b.cent, (uint64_t)k * d,
-                      out_c, (const uint32_t*)b.assign, n, out_a, (const unsigned long long*)b.stats, out_s, iters)) !=
+                      out_c, (const uint32_t*)b.assign, n, out_a, (const unsigned long long*)b.stats, out_s, iters,
+                      (volatile uint64_t*)b.host)) !=
       cudaSuccess)
     return e;
   ++*nk;

@@ -787,6 +787,16 @@ __device__ __forceinline__ void emit_record(const JobDev& J, const Post& P, cons
     for (uint32_t q = 0; q < r.len; ++q) keys[q] = s[q];
   }
 }
+// The job's flags and the size of its result into host memory: the host reads
+// them once the job's event has completed, with no copy of its own (three
+// small device-to-host copies took 30 us per word count).
+__device__ __forceinline__ void put_status(const JobDev& J, uint64_t nrec, uint64_t kbytes) {
+  if (!J.host) return;
+  volatile uint64_t* h = J.host;
+  h[0] = J.state[0];
+  h[1] = nrec;
+  h[2] = kbytes;
+}
 __device__ __forceinline__ void gather_one(const JobDev* jobs, const JobDev& single, const Post& P,
                                            const SortRec* recs, uint64_t i) {
   const SortRec r = recs[i];
@@ -796,8 +806,13 @@ __device__ __forceinline__ void gather_one(const JobDev* jobs, const JobDev& sin
   const uint64_t first = st[1], scan0 = st[2], end = st[3], scan1 = st[4];
   emit_record(J, P, r, i - first, end - first, P.excl[i] - scan0, scan1 - scan0);
 }
-__global__ void __launch_bounds__(256) wc_gather_kernel(const JobDev* jobs, JobDev single, Post P) {
+__global__ void __launch_bounds__(256) wc_gather_kernel(const JobDev* jobs, uint32_t njobs, JobDev single, Post P) {
   pdl_wait();
+  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < njobs; j += gridDim.x * blockDim.x) {
+    const JobDev J = job_at(jobs, single, j);
+    const unsigned long long* st = reinterpret_cast<const unsigned long long*>(J.state);
+    put_status(J, st[3] - st[1], st[4] - st[2]);
+  }
   const SortRec* recs = P.r1;
   const uint64_t m = *P.glob;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x)
@@ -812,6 +827,7 @@ __global__ void __launch_bounds__(CB) wc_gather1_kernel(JobDev J, Post P) {
   __shared__ unsigned long long wsum[32];
   const SortRec* recs = P.r1;
   const uint64_t m = P.glob[0], kbytes = P.glob[9];
+  if (blockIdx.x == 0 && threadIdx.x == 0) put_status(J, m, kbytes);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (uint64_t blk = blockIdx.x; blk * CB < m; blk += gridDim.x) {
     const uint64_t i = blk * CB + threadIdx.x;
@@ -2055,6 +2071,7 @@ wc::JobDev wc_job_dev(const uint8_t* in, uint64_t n, const WcBuffers& b, uint64_
   J.state = b.state;
   J.out = b.out;
   J.blk0 = blk0;
+  J.host = b.host;
   return J;
 }
 
@@ -2179,7 +2196,7 @@ cudaError_t launch_wordcount_post_multi(const wc::JobDev* jobs, const wc::JobDev
   }
   if (jobs) {
     if ((e = launch_pdl(wc_bounds_kernel, dim3(gpcb), dim3(CB), 0, s, jobs, single, P)) != cudaSuccess ||
-        (e = launch_pdl(wc_gather_kernel, dim3(gp256), dim3(256), 0, s, jobs, single, P)) != cudaSuccess)
+        (e = launch_pdl(wc_gather_kernel, dim3(gp256), dim3(256), 0, s, jobs, njobs, single, P)) != cudaSuccess)
       return e;
   } else {  // one job: bounds known, scan and gather in one pass
     if ((e = launch_pdl(wc_gather1_kernel, dim3(gpcb), dim3(CB), 0, s, single, P)) != cudaSuccess) return e;

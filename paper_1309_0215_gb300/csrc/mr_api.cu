@@ -73,6 +73,7 @@ struct Job {
   void* hk_counters = nullptr;
   // k-means
   KmBuffers km;
+  uint64_t* host = nullptr;      // pinned status words (word count, k-means)
   float* km_init_dev = nullptr;
   void* km_init_owned = nullptr;
 };
@@ -143,6 +144,11 @@ struct mr_ctx {
   // later jobs so that adding a job creates none in the steady state
   std::vector<cudaEvent_t> ev_done, ev_timing;
   std::vector<KTimer*> kt_pool;
+  // pinned host memory: status words that a job's last kernel writes (32 bytes
+  // a job, reused), and a staging buffer for small results
+  std::vector<void*> status_slabs;
+  std::vector<uint64_t*> status_free;
+  void* staging = nullptr;
   // diagnostics (mr_set_option), applied to jobs when they are launched
   long long opt_polls = -1;       // bounded device waits: polls (< 0: default)
   uint32_t opt_km_grid_cap = 0;   // k-means persistent kernels: CTA cap (0: none)
@@ -159,6 +165,29 @@ cudaError_t pooled_event(mr_ctx* c, bool timing, cudaEvent_t* e) {
     return cudaSuccess;
   }
   return timing ? cudaEventCreate(e) : cudaEventCreateWithFlags(e, cudaEventDisableTiming);
+}
+
+constexpr size_t STATUS_WORDS = 4, STATUS_PER_SLAB = 256;
+constexpr size_t STAGING_BYTES = 256 * 1024;
+
+cudaError_t status_grow(mr_ctx* c) {
+  void* p = nullptr;
+  const cudaError_t e = cudaHostAlloc(&p, STATUS_WORDS * STATUS_PER_SLAB * 8, cudaHostAllocMapped);
+  if (e != cudaSuccess) return e;
+  c->status_slabs.push_back(p);
+  for (size_t i = 0; i < STATUS_PER_SLAB; ++i)
+    c->status_free.push_back(static_cast<uint64_t*>(p) + i * STATUS_WORDS);
+  return cudaSuccess;
+}
+
+cudaError_t status_get(mr_ctx* c, uint64_t** out) {
+  if (c->status_free.empty()) {
+    const cudaError_t e = status_grow(c);
+    if (e != cudaSuccess) return e;
+  }
+  *out = c->status_free.back();
+  c->status_free.pop_back();
+  return cudaSuccess;
 }
 
 struct DeviceGuard {
@@ -427,6 +456,7 @@ void free_job(mr_ctx* c, Job* j) {
   if (j->t0) c->ev_timing.push_back(j->t0);
   if (j->t1) c->ev_timing.push_back(j->t1);
   if (j->kt) c->kt_pool.push_back(j->kt);
+  if (j->host) c->status_free.push_back(j->host);
   dev_free(c, j->slab, j->slab_bytes);
   dev_free(c, j->in_owned, j->in_owned_bytes);
   delete j;
@@ -907,25 +937,14 @@ mr_status wait_job(mr_ctx* c, Job* j, uint64_t* wc_result_bytes = nullptr) {
   }
   if (j->state == JOB_PENDING) return MR_ENOTREADY;
   MR_CUDA_TRY(cudaEventSynchronize(j->done));
-  if (j->desc.kind == MR_KMEANS_F32) {
-    // stats[3] counts device waits that gave up (bounded mbarrier waits)
-    unsigned long long to = 0;
-    const uint64_t so = km_stats_offset(j->km.k, j->km.d, j->km.n) + 24;
-    MR_CUDA_TRY(cudaMemcpyAsync(&to, static_cast<uint8_t*>(j->result) + so, 8, cudaMemcpyDeviceToHost, c->stream));
-    MR_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    return to ? MR_ETIMEOUT : MR_OK;
-  }
+  // the status words the job's last kernel wrote
+  const volatile uint64_t* h = j->host;
+  if (j->desc.kind == MR_KMEANS_F32) return h[0] ? MR_ETIMEOUT : MR_OK;  // device waits that gave up
   if (j->desc.kind != MR_WORDCOUNT) return MR_OK;
   for (;;) {
-    // the flag words and the result header, read with one synchronisation
-    uint32_t st[4];
-    uint64_t hdr[2];
-    MR_CUDA_TRY(cudaMemcpyAsync(st, j->wc.state, 16, cudaMemcpyDeviceToHost, c->stream));
-    MR_CUDA_TRY(cudaMemcpyAsync(hdr, j->wc.out, 16, cudaMemcpyDeviceToHost, c->stream));
-    MR_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    if (st[0] & 2u) return MR_ETIMEOUT;  // a pipelined map pass whose reducer stalled
-    if (!(st[0] & 1u)) {
-      if (wc_result_bytes) *wc_result_bytes = 16 + 24 * hdr[0] + hdr[1];
+    if (h[0] & 2u) return MR_ETIMEOUT;  // a pipelined map pass whose reducer stalled
+    if (!(h[0] & 1u)) {
+      if (wc_result_bytes) *wc_result_bytes = 16 + 24 * h[1] + h[2];
       return MR_OK;
     }
     if (!j->wc_auto) return MR_EOVERFLOW;
@@ -948,18 +967,6 @@ mr_status wait_job(mr_ctx* c, Job* j, uint64_t* wc_result_bytes = nullptr) {
   }
 }
 
-mr_status result_size(mr_ctx* c, Job* j, uint64_t* bytes) {
-  if (j->desc.kind == MR_WORDCOUNT) {
-    uint64_t hdr[2];
-    MR_CUDA_TRY(cudaMemcpyAsync(hdr, j->wc.out, 16, cudaMemcpyDeviceToHost, c->stream));
-    MR_CUDA_TRY(cudaStreamSynchronize(c->stream));
-    *bytes = 16 + 24 * hdr[0] + hdr[1];
-  } else {
-    *bytes = j->result_bytes;
-  }
-  return MR_OK;
-}
-
 mr_status add_job_impl(mr_ctx* c, const mr_job_desc* desc, uint64_t* job_id) {
   if (!c || !job_id) return MR_EINVAL;
   mr_status st = validate(c, desc);
@@ -979,11 +986,13 @@ mr_status add_job_impl(mr_ctx* c, const mr_job_desc* desc, uint64_t* job_id) {
       e = cudaErrorMemoryAllocation;
     }
   }
+  if (e == cudaSuccess && (desc->kind == MR_WORDCOUNT || desc->kind == MR_KMEANS_F32)) e = status_get(c, &j->host);
   if (e != cudaSuccess) {
-    set_last_error("cudaEventCreate", e);
+    set_last_error("job events and status", e);
     free_job(c, j);
     return MR_ECUDA;
   }
+  j->wc.host = j->km.host = j->host;
   if (desc->input_on_device || desc->input_bytes == 0) {
     j->in = static_cast<const uint8_t*>(desc->input);
   } else {
@@ -1081,8 +1090,12 @@ mr_status mr_create(const mr_config* cfg, mr_ctx** out) {
       e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
   }
+  // the first status words and the staging buffer, so that no job waits for their pinning
+  if (e == cudaSuccess) e = cudaHostAlloc(&c->staging, STAGING_BYTES, cudaHostAllocDefault);
+  if (e == cudaSuccess) e = status_grow(c);
   if (e != cudaSuccess) {
     set_last_error("mr_create", e);
+    if (c->staging) cudaFreeHost(c->staging);
     if (c->pool) cudaMemPoolDestroy(c->pool);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -1133,6 +1146,8 @@ void mr_destroy(mr_ctx* c) {
   for (cudaEvent_t e : c->ev_timing) cudaEventDestroy(e);
   for (KTimer* t : c->kt_pool) kt_destroy(t);
   cudaStreamSynchronize(c->stream);
+  for (void* p : c->status_slabs) cudaFreeHost(p);
+  if (c->staging) cudaFreeHost(c->staging);
   // memory still held (none, normally) is released once it is freed
   if (c->pool) cudaMemPoolDestroy(c->pool);
   if (c->own_stream) cudaStreamDestroy(c->stream);
@@ -1178,13 +1193,20 @@ mr_status mr_fetch(mr_ctx* c, uint64_t job_id, void* buf, uint64_t buf_bytes, ui
   DeviceGuard g(c->device);
   Job* j = find_job(c, job_id);
   if (!j) return MR_ENOJOB;
-  uint64_t bytes = 0;
+  uint64_t bytes = j->result_bytes;
   mr_status st = wait_job(c, j, &bytes);
   if (st) return st;
-  if (j->desc.kind != MR_WORDCOUNT && (st = result_size(c, j, &bytes)) != MR_OK) return st;
   if (needed) *needed = bytes;
   if (!buf) return MR_OK;
   if (buf_bytes < bytes) return MR_EINVAL;
+  if (bytes <= STAGING_BYTES) {
+    // through pinned memory: one copy by the engine and one by this thread,
+    // instead of the driver's own staging of pageable memory
+    MR_CUDA_TRY(cudaMemcpyAsync(c->staging, j->result, bytes, cudaMemcpyDeviceToHost, c->stream));
+    MR_CUDA_TRY(cudaStreamSynchronize(c->stream));
+    memcpy(buf, c->staging, bytes);
+    return MR_OK;
+  }
   MR_CUDA_TRY(cudaMemcpyAsync(buf, j->result, bytes, cudaMemcpyDeviceToHost, c->stream));
   MR_CUDA_TRY(cudaStreamSynchronize(c->stream));
   return MR_OK;
@@ -1195,10 +1217,10 @@ mr_status mr_result_device(mr_ctx* c, uint64_t job_id, const void** dptr, uint64
   DeviceGuard g(c->device);
   Job* j = find_job(c, job_id);
   if (!j) return MR_ENOJOB;
-  mr_status st = wait_job(c, j);
+  uint64_t n = j->result_bytes;
+  mr_status st = wait_job(c, j, &n);
   if (st) return st;
-  st = result_size(c, j, bytes);
-  if (st) return st;
+  *bytes = n;
   *dptr = j->result;
   return MR_OK;
 }

@@ -90,6 +90,7 @@ struct WcBuffers {
   uint64_t* cnt = nullptr;     // [cap] combined counts (contiguous after key)
   uint32_t* state = nullptr;   // 64 bytes: word 0 overflow flag, 64-bit fields 1..4 post-phase bounds
   uint8_t* sortbuf = nullptr;  // post-phase scratch for cap records
+  uint64_t* host = nullptr;    // pinned host words {flags, records, key bytes}, written by the last kernel (or null)
   uint8_t* out = nullptr;      // result: header + records + key bytes
   uint64_t out_cap = 0;
 };
@@ -172,6 +173,7 @@ struct KmBuffers {
   float* ct = nullptr;          // [d][k] transposed centroids
   unsigned int* maxabs = nullptr;  // [1] bits of max |x|
   int* shift = nullptr;         // [1] fixed-point scale exponent
+  uint64_t* host = nullptr;     // pinned host word for the count of timed-out waits, written by the last kernel (or null)
   uint8_t* bop = nullptr;       // centroid operands of the wide tensor-core pass (nullptr: not taken)
   uint32_t* kcursor = nullptr;  // [k] counting-sort write cursors
   long long* part = nullptr;    // [CTAs][k][d] partial sums of the local-array update (nullptr: sort path)
