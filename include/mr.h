@@ -77,7 +77,10 @@ typedef enum {
    * keys, Sec. IV data sets; array container without local arrays,
    * Sec. III-E).  Input: uint32 keys (input_bytes a multiple of 4, a device
    * input 4-byte aligned); key k < hist_bins emits (k, 1), any other key
-   * (hist_bins, 1).  Output: uint64 bins[hist_bins + 1]. */
+   * (hist_bins, 1).  Output: uint64 bins[hist_bins + 1].  With many keys over
+   * many bins MR_C_AUTO groups the keys by ranges of bins first, through 2
+   * bytes of device scratch per key (at most 512 MiB); a context with an HBM
+   * budget, or without memory for it, counts in the global array instead. */
   MR_HIST_U32 = 4,
   /* Bloom-filter build (the paper's Bloom Filter application: k-mers of a
    * chromosome, 30M elements into 300M entries, Sec. IV data sets; array

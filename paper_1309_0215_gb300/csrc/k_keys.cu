@@ -222,6 +222,315 @@ __global__ void hk_widen_kernel(const uint32_t* __restrict__ c32, uint64_t nb, u
     out[i] = c32[i];
 }
 
+// ------------------------------------------------------ partitioned counting
+// Bins that do not fit one CTA's shared memory, many keys.  The global-array
+// kernel is bound by the L2's atomic rate (about 190G/s: 1.40 ms for 256M
+// uniform keys over 16M bins, 12% of the HBM rate), while adds in shared
+// memory run several times faster, so the keys are first grouped by ranges of
+// 2^PS bins ("ranges"), each of which does fit one CTA:
+//   1. hk_part_kernel: a CTA takes chunks of PCHUNK consecutive keys, counts
+//      them by bucket (up to 1,024 buckets of 2^F bins, whatever the number of
+//      ranges, so that few ranges do not mean few counters and many conflicts)
+//      in shared memory, scans the counts into cursors, reads the keys again
+//      (they are still in L2; holding them in registers halves the warps an SM
+//      runs), places every key at its bucket's cursor and writes the chunk,
+//      grouped, as 16-bit offsets within the range.  Where each range starts
+//      in the chunk goes into a table [range][chunk].  Bound by the shared
+//      memory pipe: three random accesses a key, 3.4 wavefronts per warp each.
+//   2. hk_plan_kernel cuts the ranges into units: one, or several over equal
+//      parts of the chunks for a range that holds much more than its share
+//      (skewed keys, or few ranges).
+//   3. hk_count_kernel: one CTA per unit adds its range's pieces of all chunks
+//      into shared memory and stores the counts (u64, no clearing, no widening)
+//      or, for a range of several units, adds the non-zero ones.
+// HBM traffic: 4 + 2 + 2 bytes a key instead of 4, but no atomics beyond the
+// SM: 256M keys over 16M bins take 0.87 ms instead of 1.51 in
+// all, skewed ones (rank density 1 / (rank + 1)) 0.87 instead of 8.2.
+// A warp whose 128 keys of a load share a bucket (sorted input) moves the cursor
+// once.
+constexpr int PT = 1024;                // threads of the partition kernel (two CTAs per SM)
+constexpr int PV = 8;                   // 16-byte loads per thread and chunk
+constexpr int PAHEAD = 2;               // of them in flight
+constexpr uint32_t PCHUNK = PT * PV * 4;  // 32,768 keys
+constexpr uint32_t PGROUP = 8;          // chunks per 16-byte table write
+constexpr uint32_t PS = 15;             // log2 of a range's bins (128 KiB of u32 counters)
+constexpr uint32_t PNF = 1024;          // buckets, at most
+constexpr uint32_t PRANGES = 1024;      // ranges, at most
+constexpr int PCT = 1024;               // threads of the counting kernel
+constexpr uint32_t PUNIT_MIN = 1u << 18;  // keys worth a unit of their own (8 per bin)
+constexpr uint32_t PUNITS = 256;        // units of an even split
+
+struct PartArgs {
+  uint16_t* item;      // [chunks][PCHUNK] grouped offsets within the range
+  uint16_t* start;     // [ranges + 1][chunks] first item of each range in each chunk
+  uint32_t* total;     // [ranges] keys of each range; then [0] the counting kernel's cursor, [1] number of units
+  uint4* unit;         // {range, first chunk, end chunk, several}
+  uint32_t chunks;     // a multiple of PGROUP
+  uint32_t ranges, nf, fshift;
+  uint32_t split;      // log2 of the parts a chunk's piece is counted in
+};
+
+// Exclusive scan in place of nf <= T counters by T threads (entry nf: the total).
+template <int T>
+__device__ __forceinline__ void block_scan(uint32_t* cnt, uint32_t nf, uint32_t* wsum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t a = threadIdx.x < nf ? cnt[threadIdx.x] : 0;
+  uint32_t incl = a;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t w = lane < T / 32 ? wsum[lane] : 0, wi = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, wi, o);
+      if (lane >= o) wi += v;
+    }
+    wsum[lane] = wi - w;
+    if (lane == 31) cnt[nf] = wi;
+  }
+  __syncthreads();
+  if (threadIdx.x < nf) cnt[threadIdx.x] = wsum[warp] + incl - a;
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n,
+                                                        uint32_t nbins, PartArgs P) {
+  extern __shared__ __align__(16) unsigned char hp_sm[];
+  uint16_t* buf = reinterpret_cast<uint16_t*>(hp_sm);                 // [PCHUNK]
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(buf + PCHUNK);          // [PNF + 1]
+  uint32_t* tot = cnt + PNF + 4;                                      // [PRANGES]
+  uint16_t* stage = reinterpret_cast<uint16_t*>(tot + PRANGES);       // [ranges + 1][PGROUP]
+  __shared__ uint32_t wsum[32];
+  const int lane = threadIdx.x & 31;
+  const uint64_t end = n + off;  // items in group space: item i of the stream is key i - off
+  const uint32_t step = PS - P.fshift, fs = P.fshift;
+  for (uint32_t i = threadIdx.x; i < P.ranges; i += PT) tot[i] = 0;
+  const uint32_t per = (P.chunks + gridDim.x - 1) / gridDim.x;
+  const uint32_t c0 = blockIdx.x * per, c1 = min(c0 + per, P.chunks);
+  for (uint32_t c = c0; c < c1; ++c) {
+    const uint64_t i0 = (uint64_t)c * PCHUNK;
+    for (uint32_t i = threadIdx.x; i < P.nf; i += PT) cnt[i] = 0;
+    __syncthreads();
+    const bool whole = i0 >= off && i0 + PCHUNK <= end;  // every item is a key
+    const uint4* src = base + i0 / 4 + threadIdx.x;
+    if (whole) {
+#pragma unroll 1
+      for (int q = 0; q < PV; q += PAHEAD) {
+        uint4 v[PAHEAD];
+#pragma unroll
+        for (int t = 0; t < PAHEAD; ++t) v[t] = __ldg(src + (q + t) * PT);
+#pragma unroll
+        for (int t = 0; t < PAHEAD; ++t)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) atomicAdd(cnt + (min(key_at(v[t], e), nbins) >> fs), 1u);
+      }
+    } else {
+      for (int q = 0; q < PV; ++q) {
+        const uint64_t e0 = i0 + 4 * ((uint64_t)q * PT + threadIdx.x);
+        if (e0 >= end) continue;
+        const uint4 v = __ldg(src + q * PT);
+        for (int e = 0; e < 4; ++e)
+          if (e0 + e >= off && e0 + e < end) atomicAdd(cnt + (min(key_at(v, e), nbins) >> fs), 1u);
+      }
+    }
+    __syncthreads();
+    block_scan<PT>(cnt, P.nf, wsum);
+    for (uint32_t b = threadIdx.x; b <= P.ranges; b += PT) {
+      const uint32_t at = cnt[min(b << step, P.nf)];
+      stage[b * PGROUP + c % PGROUP] = (uint16_t)at;
+      if (b < P.ranges) tot[b] += cnt[min((b + 1) << step, P.nf)] - at;
+    }
+    __syncthreads();  // the starts are read; the counters become cursors
+    if (whole) {
+#pragma unroll 1
+      for (int q = 0; q < PV; q += PAHEAD) {
+        uint4 v[PAHEAD];
+#pragma unroll
+        for (int t = 0; t < PAHEAD; ++t) v[t] = __ldg(src + (q + t) * PT);
+#pragma unroll
+        for (int t = 0; t < PAHEAD; ++t) {
+          uint32_t k[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) k[e] = min(key_at(v[t], e), nbins);
+          const uint32_t fw = __shfl_sync(0xffffffffu, k[0] >> fs, 0);
+          const uint32_t other = ((k[0] >> fs) ^ fw) | ((k[1] >> fs) ^ fw) | ((k[2] >> fs) ^ fw) | ((k[3] >> fs) ^ fw);
+          uint32_t r[4];
+          if (__all_sync(0xffffffffu, other == 0)) {
+            uint32_t r0 = 0;
+            if (lane == 0) r0 = atomicAdd(cnt + fw, 128u);
+            r0 = __shfl_sync(0xffffffffu, r0, 0) + 4 * lane;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r[e] = r0 + e;
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r[e] = atomicAdd(cnt + (k[e] >> fs), 1u);
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) buf[r[e]] = (uint16_t)(k[e] & ((1u << PS) - 1));
+        }
+      }
+    } else {
+      for (int q = 0; q < PV; ++q) {
+        const uint64_t e0 = i0 + 4 * ((uint64_t)q * PT + threadIdx.x);
+        if (e0 >= end) continue;
+        const uint4 v = __ldg(src + q * PT);
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t k = min(key_at(v, e), nbins);
+          if (e0 + e >= off && e0 + e < end) buf[atomicAdd(cnt + (k >> fs), 1u)] = (uint16_t)(k & ((1u << PS) - 1));
+        }
+      }
+    }
+    __syncthreads();
+    uint4* out = reinterpret_cast<uint4*>(P.item + i0);
+    const uint4* in = reinterpret_cast<const uint4*>(buf);
+#pragma unroll
+    for (uint32_t i = 0; i < PCHUNK * 2 / 16 / PT; ++i) out[i * PT + threadIdx.x] = in[i * PT + threadIdx.x];
+    // the starts of the chunks since the last table write
+    const uint32_t g0 = c / PGROUP * PGROUP;
+    if (c % PGROUP == PGROUP - 1 || c + 1 == c1) {
+      for (uint32_t b = threadIdx.x; b <= P.ranges; b += PT) {
+        uint16_t* t = P.start + (uint64_t)b * P.chunks + g0;
+        if (g0 >= c0 && c % PGROUP == PGROUP - 1)
+          *reinterpret_cast<uint4*>(t) = *reinterpret_cast<const uint4*>(stage + b * PGROUP);
+        else
+          for (uint32_t q = g0 < c0 ? c0 - g0 : 0; q <= c % PGROUP; ++q) t[q] = stage[b * PGROUP + q];
+      }
+    }
+  }
+  __syncthreads();
+  for (uint32_t b = threadIdx.x; b < P.ranges; b += PT)
+    if (tot[b]) atomicAdd(P.total + b, tot[b]);
+}
+
+// Units of every range (one CTA per range; every CTA scans all ranges' unit
+// counts).  A range of several units starts from zeroed bins (unless the
+// counts add to those of an earlier round).
+__global__ void __launch_bounds__(256) hk_plan_kernel(PartArgs P, uint32_t nbins, uint32_t unit_keys, uint32_t add,
+                                                      unsigned long long* __restrict__ out) {
+  pdl_wait();
+  __shared__ uint32_t s_before[8], s_all[8], s_mine;
+  const uint32_t b = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t before = 0, all = 0, mine = 0;
+  for (uint32_t r = threadIdx.x; r < P.ranges; r += 256) {
+    const uint32_t u = max(1u, (P.total[r] + unit_keys - 1) / unit_keys);
+    all += u;
+    before += r < b ? u : 0;
+    if (r == b) mine = u;
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  all = __reduce_add_sync(0xffffffffu, all);
+  if (lane == 0) s_before[warp] = before, s_all[warp] = all;
+  if ((b & 255) == threadIdx.x) s_mine = mine;  // this thread met r == b
+  __syncthreads();
+  before = all = 0;
+  for (int w = 0; w < 8; ++w) before += s_before[w], all += s_all[w];
+  const uint32_t parts = s_mine;
+  const uint32_t per = ((P.chunks + parts - 1) / parts + 31) & ~31u;
+  for (uint32_t i = threadIdx.x; i < parts; i += 256)
+    P.unit[before + i] = make_uint4(b, min(i * per, P.chunks), min((i + 1) * per, P.chunks), parts > 1 ? 1u : 0u);
+  if (b == 0 && threadIdx.x == 0) {
+    P.total[P.ranges] = 0;
+    P.total[P.ranges + 1] = all;
+  }
+  if (parts > 1 && !add)
+    for (uint64_t i = ((uint64_t)b << PS) + threadIdx.x; i < ((uint64_t)(b + 1) << PS) && i <= nbins; i += 256)
+      out[i] = 0;
+}
+
+// A chunk's piece of the range is cut into 2^split parts, so that a unit of few
+// chunks (few ranges, long pieces) has work for every warp.  A warp takes 32
+// parts at a time; they, in quads of four
+// offsets (8 aligned bytes), are laid end to end and shared out evenly: quad f
+// belongs to the part whose scanned quad count brackets it (a binary search
+// over the lanes).  CAHEAD quads per lane are in flight (the pieces lie in
+// DRAM).
+constexpr int CAHEAD = 4;
+__global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint32_t nbins, uint32_t add,
+                                                          unsigned long long* __restrict__ out) {
+  pdl_wait();
+  extern __shared__ __align__(16) uint32_t hc_bins[];  // [1 << PS]
+  __shared__ uint32_t s_unit;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t nunits = P.total[P.ranges + 1];
+  for (;;) {
+    __syncthreads();  // the previous unit's counts have been stored
+    if (threadIdx.x == 0) s_unit = atomicAdd(P.total + P.ranges, 1u);
+    for (uint32_t i = threadIdx.x; i < (1u << PS) / 4; i += PCT)
+      reinterpret_cast<uint4*>(hc_bins)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    if (s_unit >= nunits) return;
+    const uint4 u = P.unit[s_unit];
+    const uint16_t* s0 = P.start + (uint64_t)u.x * P.chunks;
+    const uint16_t* s1 = s0 + P.chunks;
+    const uint32_t nl = (u.z - u.y) << P.split;
+    for (uint32_t l0 = 32 * warp; l0 < nl; l0 += PCT) {
+      // this lane's piece: part `sub` of the quads of chunk c's
+      const uint32_t l = l0 + lane, c = u.y + (l >> P.split), sub = l & ((1u << P.split) - 1);
+      uint32_t piece = 0, nq = 0;  // first and end offset, quads
+      if (l < nl) {
+        const uint32_t a = s0[c], e = s1[c];
+        const uint32_t qa = a >> 2, n4 = e > a ? ((e + 3) >> 2) - qa : 0;
+        const uint32_t q0 = (n4 * sub) >> P.split, q1 = (n4 * (sub + 1)) >> P.split;
+        nq = q1 - q0;
+        if (nq) piece = max(a, 4 * (qa + q0)) | (min(e, 4 * (qa + q1)) << 16);
+      }
+      uint32_t ex = nq;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, ex, o);
+        if (lane >= o) ex += v;
+      }
+      const uint32_t all = __shfl_sync(0xffffffffu, ex, 31);
+      ex -= nq;
+      for (uint32_t f0 = 0; f0 < all; f0 += 32 * CAHEAD) {
+        uint2 w[CAHEAD];
+        uint32_t r[CAHEAD], len[CAHEAD];  // the quad's first offset relative to its piece, and the piece's length
+#pragma unroll
+        for (int t = 0; t < CAHEAD; ++t) {
+          const uint32_t f = f0 + 32 * t + lane;
+          int p = 0;
+#pragma unroll
+          for (int o = 16; o; o >>= 1)
+            if (__shfl_sync(0xffffffffu, ex, p + o) <= f) p += o;
+          const uint32_t pc = __shfl_sync(0xffffffffu, piece, p);
+          const uint32_t i = 4 * (f - __shfl_sync(0xffffffffu, ex, p)) + (pc & 0xfffcu);
+          r[t] = i - (pc & 0xffffu);
+          len[t] = 0;
+          if (f < all) {
+            len[t] = (pc >> 16) - (pc & 0xffffu);
+            const uint32_t cp = u.y + ((l0 + p) >> P.split);
+            w[t] = __ldg(reinterpret_cast<const uint2*>(P.item + (uint64_t)cp * PCHUNK + i));
+          }
+        }
+#pragma unroll
+        for (int t = 0; t < CAHEAD; ++t) {
+          if (r[t] < len[t]) atomicAdd(hc_bins + (w[t].x & 0xffffu), 1u);
+          if (r[t] + 1 < len[t]) atomicAdd(hc_bins + (w[t].x >> 16), 1u);
+          if (r[t] + 2 < len[t]) atomicAdd(hc_bins + (w[t].y & 0xffffu), 1u);
+          if (r[t] + 3 < len[t]) atomicAdd(hc_bins + (w[t].y >> 16), 1u);
+        }
+      }
+    }
+    __syncthreads();
+    const uint64_t b0 = (uint64_t)u.x << PS;
+    const uint32_t nb = (uint32_t)min((uint64_t)(1u << PS), (uint64_t)nbins + 1 - b0);
+    for (uint32_t i = threadIdx.x; i < nb; i += PCT) {
+      const uint32_t v = hc_bins[i];
+      if (u.w) {
+        if (v) atomicAdd(out + b0 + i, (unsigned long long)v);
+      } else {
+        out[b0 + i] = add ? out[b0 + i] + v : v;
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------ Bloom filter
 constexpr int BF_THREADS = 256;
 constexpr int BF_TILE = 8192;                     // windows per CTA tile
@@ -348,6 +657,78 @@ static cudaError_t launch_hk_cluster(const uint4* base, uint32_t off, uint64_t n
   if (want > (uint64_t)clusters) want = (uint64_t)clusters;
   cfg.gridDim = dim3((unsigned)(want * HKC), 1, 1);
   return cudaLaunchKernelEx(&cfg, hk_cluster_kernel<C>, base, off, n, nbins, slice, slice_mul, cnt);
+}
+
+// Partitioned counting: chosen for MR_C_AUTO jobs whose bins do not fit one
+// CTA, up to 2^25 bins (1,024 ranges), with at least a key per bin, from 2^24
+// keys on, and from 2^22 when there are enough ranges for the counting kernel's
+// CTAs (keys x ranges >= 2^26).  Measured, uniform / skewed keys, partitioned
+// against the global array, us a call: 2^24 keys over 60,000 bins 143 / 146
+// against 151 / 391; 2^23 over 60,000 124 / 124 against 91 / 211 (left to the
+// array); 2^22 over 2^20 59 / 77 against 67 / 121; 2^24 over 2^24 123 / 366
+// against 196 / 454; 2^28 over 30M 921 / 937 against 3,047 / 12,646.
+constexpr uint64_t PART_ROUND = 1ull << 28;  // keys grouped at a time (2 bytes each of scratch)
+bool hk_partitioned(uint64_t n, uint32_t nbins) {
+  const uint64_t ranges = ((uint64_t)nbins >> PS) + 1;
+  return ranges <= PRANGES && n >= nbins && (n >= 1ull << 24 || (n >= 1ull << 22 && n * ranges >= 1ull << 26));
+}
+static PartArgs hk_part_args(uint64_t n, uint32_t nbins, uint8_t* p, size_t* bytes) {
+  PartArgs P{};
+  const uint64_t m = n < PART_ROUND ? n : PART_ROUND;
+  const uint64_t chunks = (m + 3 + PCHUNK - 1) / PCHUNK;  // + 3: keys may start inside a 16-byte group
+  P.chunks = (uint32_t)((chunks + PGROUP - 1) / PGROUP * PGROUP);
+  P.ranges = (nbins >> PS) + 1;
+  while (((nbins >> P.fshift) + 1) > PNF) ++P.fshift;
+  P.nf = (nbins >> P.fshift) + 1;
+  while ((P.ranges << P.split) < 512) ++P.split;  // parts of 64 keys or so
+  size_t at = 0;
+  auto take = [&](size_t sz) {
+    uint8_t* r = p + at;
+    at += (sz + 255) & ~(size_t)255;
+    return r;
+  };
+  P.item = reinterpret_cast<uint16_t*>(take((size_t)P.chunks * PCHUNK * 2));
+  P.start = reinterpret_cast<uint16_t*>(take((size_t)(P.ranges + 1) * P.chunks * 2));
+  P.total = reinterpret_cast<uint32_t*>(take((size_t)(P.ranges + 2) * 4));
+  P.unit = reinterpret_cast<uint4*>(take((size_t)(2 * P.ranges + PUNITS) * 16));
+  *bytes = at;
+  return P;
+}
+size_t hk_part_bytes(uint64_t n, uint32_t nbins) {
+  size_t b = 0;
+  hk_part_args(n, nbins, nullptr, &b);
+  return b;
+}
+cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbins, uint8_t* scratch,
+                                  unsigned long long* out, const DevInfo& di, cudaStream_t s, uint64_t* nk,
+                                  KTimer* kt) {
+  size_t bytes = 0;
+  const PartArgs P = hk_part_args(n, nbins, scratch, &bytes);
+  const int psm = (int)(PCHUNK * 2 + (PNF + 4 + PRANGES) * 4 + (P.ranges + 1) * PGROUP * 2);
+  const int csm = (1 << PS) * 4;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(hk_part_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, psm)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(hk_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, csm)) != cudaSuccess)
+    return e;
+  if ((e = kt_begin(kt, s)) != cudaSuccess) return e;
+  for (uint64_t k0 = 0; k0 < n; k0 += PART_ROUND) {
+    const uint64_t m = n - k0 < PART_ROUND ? n - k0 : PART_ROUND;
+    const uintptr_t addr = reinterpret_cast<uintptr_t>(keys + k0);
+    const uint4* base = reinterpret_cast<const uint4*>(addr & ~uintptr_t(15));
+    const uint32_t off = (uint32_t)((addr & 15) / 4);
+    const uint32_t pg = (uint32_t)di.sms * 2;
+    const uint64_t uk = m / PUNITS > PUNIT_MIN ? m / PUNITS : PUNIT_MIN;
+    const uint32_t add = k0 ? 1u : 0u;
+    if ((e = cudaMemsetAsync(P.total, 0, (P.ranges + 2) * 4, s)) != cudaSuccess) return e;
+    hk_part_kernel<<<P.chunks < pg ? P.chunks : pg, PT, psm, s>>>(base, off, m, nbins, P);
+    if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = launch_pdl(hk_plan_kernel, dim3(P.ranges), dim3(256), 0, s, P, nbins, (uint32_t)uk, add, out)) !=
+            cudaSuccess ||
+        (e = launch_pdl(hk_count_kernel, dim3(di.sms), dim3(PCT), (size_t)csm, s, P, nbins, add, out)) != cudaSuccess)
+      return e;
+    *nk += 3;
+  }
+  return kt_end(kt, s);
 }
 
 cudaError_t launch_hist_keys(const uint32_t* keys, uint64_t n, uint32_t nbins, int container, void* counters,

@@ -71,6 +71,7 @@ struct Job {
   bool wc_auto = true;
   // large-key histogram: u32 counters (null: count straight into the u64 result)
   void* hk_counters = nullptr;
+  uint8_t* hk_part = nullptr;  // scratch of partitioned counting (null: not taken)
   // k-means
   KmBuffers km;
   uint64_t* host = nullptr;      // pinned status words (word count, k-means)
@@ -386,9 +387,24 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
     case MR_HIST_U32: {
       const uint64_t nb = (uint64_t)d.hist_bins + 1;
       const uint64_t res = align256(nb * 8);
-      // u32 counters while no bin can reach 2^32
-      const bool wide = d.input_bytes / 4 >= (1ull << 32);
-      const uint64_t cnt = wide ? 0 : align256(nb * 4);
+      // u32 counters while no bin can reach 2^32; local arrays are few enough
+      // to be added straight into the result
+      const bool wide = d.input_bytes / 4 >= (1ull << 32) || j->container == MR_C_SMEM_ARRAY;
+      uint64_t cnt = wide ? 0 : align256(nb * 4);
+      // partitioned counting, if the library chooses the container and there
+      // is memory for its scratch (a context with a budget keeps it for jobs);
+      // else counters of the global array
+      if (d.container == MR_C_AUTO && j->container == MR_C_GLOBAL_ARRAY && c->budget == 0 &&
+          hk_partitioned(d.input_bytes / 4, d.hist_bins)) {
+        const uint64_t scr = align256(hk_part_bytes(d.input_bytes / 4, d.hist_bins));
+        if (dev_alloc(c, res + scr, &j->slab) == MR_OK) {
+          j->slab_bytes = res + scr;
+          j->result = j->slab;
+          j->result_bytes = nb * 8;
+          j->hk_part = static_cast<uint8_t*>(j->slab) + res;
+          return MR_OK;
+        }
+      }
       mr_status st = dev_alloc(c, res + cnt, &j->slab);
       if (st) return st;
       j->slab_bytes = res + cnt;
@@ -511,6 +527,12 @@ mr_status enqueue_plain_on(mr_ctx* c, Job* j, cudaStream_t st) {
                                    c->opt_polls));
       break;
     case MR_HIST_U32:
+      if (j->hk_part) {
+        MR_CUDA_TRY(launch_hist_keys_part(reinterpret_cast<const uint32_t*>(j->in), n / 4, j->desc.hist_bins,
+                                          j->hk_part, static_cast<unsigned long long*>(j->result), c->di, st,
+                                          &c->launches, j->kt));
+        break;
+      }
       MR_CUDA_TRY(launch_hist_keys(reinterpret_cast<const uint32_t*>(j->in), n / 4, j->desc.hist_bins,
                                    (int)j->container, j->hk_counters, j->hk_counters == nullptr,
                                    static_cast<unsigned long long*>(j->result), c->di, st, &c->launches, j->kt));

@@ -79,6 +79,13 @@ int hk_cluster_max_bins(const DevInfo& di);
 cudaError_t launch_hist_keys(const uint32_t* keys, uint64_t n, uint32_t nbins, int container, void* counters,
                              bool wide, unsigned long long* out, const DevInfo& di, cudaStream_t s, uint64_t* nk,
                              KTimer* kt = nullptr);
+// The same for many keys over bins beyond one CTA's shared memory
+// (hk_partitioned), through hk_part_bytes of scratch; every bin is written.
+bool hk_partitioned(uint64_t n, uint32_t nbins);
+size_t hk_part_bytes(uint64_t n, uint32_t nbins);
+cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbins, uint8_t* scratch,
+                                  unsigned long long* out, const DevInfo& di, cudaStream_t s, uint64_t* nk,
+                                  KTimer* kt = nullptr);
 // Bloom-filter build over n bases into ceil(m / 32) u32 words (zeroed here).
 cudaError_t launch_bloom(const uint8_t* seq, uint64_t n, uint32_t L, uint64_t m, uint32_t h, uint32_t* bits,
                          const DevInfo& di, cudaStream_t s, uint64_t* nk, KTimer* kt = nullptr);

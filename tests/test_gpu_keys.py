@@ -140,3 +140,55 @@ def test_bloom_full_size(mr):
     seq = synth.dna(30_000_000 + L - 1)
     got = mr.bloom_dna(_dev(seq), L, 300_000_000, 7)
     assert np.array_equal(got, oracle.bloom_dna(seq, L, 300_000_000, 7))
+
+
+def _part_keys(kind, n, nbins, seed):
+    rng = np.random.default_rng(seed)
+    if kind == "skewed":
+        return synth.keys_u32(n, nbins, seed=seed, skewed=True)
+    if kind == "one":
+        return np.full(n, nbins // 3, dtype=np.uint32)
+    keys = rng.integers(0, nbins + nbins // 8 + 2, n, dtype=np.uint32)  # about one key in nine out of range
+    if kind == "sorted":
+        keys.sort()
+    if kind == "outside":
+        keys[rng.random(n) < 0.7] = 0xFFFFFFFF
+    return keys
+
+
+@pytest.mark.parametrize("n,nbins", [
+    (1 << 24, 58_112),            # two ranges of bins
+    ((1 << 24) + 4_099, 65_535),  # the last bin and the out-of-range bin share a range
+    ((1 << 24) + 5, 65_536),      # the out-of-range bin has a range of its own
+    (1 << 22, 1 << 20),           # the fewest keys; 33 ranges, buckets smaller than a range
+    (20_000_003, 5_000_000),
+])
+@pytest.mark.parametrize("kind", ["uniform", "skewed", "one", "sorted", "outside"])
+@pytest.mark.parametrize("offset", [0, 12])
+def test_hist_u32_partitioned(mr, n, nbins, kind, offset):
+    """Jobs large enough for partitioned counting: the oracle's counts, and the
+    same bytes as the global array's atomics (which a pinned container keeps)."""
+    keys = _part_keys(kind, n, nbins, seed=n % 1000 + nbins)
+    dev = _dev(keys, offset)
+    got = mr.hist_u32(dev, nbins)
+    assert np.array_equal(got, oracle.hist_u32(keys, nbins))
+    assert np.array_equal(got, mr.hist_u32(dev, nbins, container=mr.C_GLOBAL_ARRAY))
+
+
+def test_hist_u32_partitioned_rounds_and_budget(mr):
+    """More keys than one round groups (the second round's counts add to the
+    first's), and a context with an HBM budget, which keeps the global array."""
+    import torch
+    n, nbins = (1 << 28) + 70_001, 1_000_000
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    keys = torch.randint(0, nbins + 10, (n,), device="cuda", generator=g, dtype=torch.int32)
+    torch.cuda.synchronize()
+    want = torch.bincount(keys.clamp(max=nbins), minlength=nbins + 1).cpu().numpy().astype(np.uint64)
+    assert np.array_equal(mr.hist_u32(keys, nbins), want)
+    ctx = mr.Context(hbm_budget=64 << 20)
+    j = ctx.add_job(mr.HIST_U32, keys, hist_bins=nbins)
+    assert ctx.bytes_in_use < 16 << 20
+    ctx.run()
+    assert np.array_equal(np.frombuffer(ctx.fetch(j), dtype=np.uint64), want)
+    ctx.close()
