@@ -90,7 +90,10 @@ typedef enum {
    * significant).  With mix = the SplitMix64 output function, a = mix(code)
    * mod m and b = 1 + mix(code ^ 0x9E3779B97F4A7C15) mod (m - 1), the element
    * sets bits (a + i*b) mod m for i < bloom_hashes (m = bloom_bits).  Output:
-   * ceil(m / 8) bytes, bit j = bit (j mod 8) of byte j / 8. */
+   * ceil(m / 8) bytes, bit j = bit (j mod 8) of byte j / 8.  With many positions
+   * MR_C_AUTO groups them by ranges of bits first, through 4 bytes of device
+   * scratch per position (at most 2 GiB), under the same conditions as the
+   * large-key histogram. */
   MR_BLOOM_DNA = 5
 } mr_kind;
 

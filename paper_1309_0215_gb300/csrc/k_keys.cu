@@ -261,12 +261,13 @@ constexpr uint32_t PUNIT_MIN = 1u << 18;  // keys worth a unit of their own (8 p
 constexpr uint32_t PUNITS = 256;        // units of an even split
 
 struct PartArgs {
-  uint16_t* item;      // [chunks][PCHUNK] grouped offsets within the range
+  void* item;          // [chunks][items of a chunk] grouped offsets within the range
   uint16_t* start;     // [ranges + 1][chunks] first item of each range in each chunk
   uint32_t* total;     // [ranges] keys of each range; then [0] the counting kernel's cursor, [1] number of units
   uint4* unit;         // {range, first chunk, end chunk, several}
   uint32_t chunks;     // a multiple of PGROUP
   uint32_t ranges, nf, fshift;
+  uint32_t step;       // log2 of the buckets per range
   uint32_t split;      // log2 of the parts a chunk's piece is counted in
 };
 
@@ -298,6 +299,30 @@ __device__ __forceinline__ void block_scan(uint32_t* cnt, uint32_t nf, uint32_t*
   __syncthreads();
 }
 
+// Chunk c of this CTA's chunks c0 .. c1 - 1 is done: write the starts of the
+// chunks since the last write, a whole group at a time where it is this CTA's.
+__device__ __forceinline__ void write_starts(const PartArgs& P, const uint16_t* stage, uint32_t c, uint32_t c0,
+                                             uint32_t c1) {
+  if (c % PGROUP != PGROUP - 1 && c + 1 != c1) return;
+  const uint32_t g0 = c / PGROUP * PGROUP;
+  for (uint32_t b = threadIdx.x; b <= P.ranges; b += blockDim.x) {
+    uint16_t* t = P.start + (uint64_t)b * P.chunks + g0;
+    if (g0 >= c0 && c % PGROUP == PGROUP - 1)
+      *reinterpret_cast<uint4*>(t) = *reinterpret_cast<const uint4*>(stage + b * PGROUP);
+    else
+      for (uint32_t q = g0 < c0 ? c0 - g0 : 0; q <= c % PGROUP; ++q) t[q] = stage[b * PGROUP + q];
+  }
+}
+// The scanned bucket counts of chunk c: where its ranges start, and their totals.
+__device__ __forceinline__ void stage_starts(const PartArgs& P, const uint32_t* cnt, uint16_t* stage, uint32_t* tot,
+                                             uint32_t c) {
+  for (uint32_t b = threadIdx.x; b <= P.ranges; b += blockDim.x) {
+    const uint32_t at = cnt[min(b << P.step, P.nf)];
+    stage[b * PGROUP + c % PGROUP] = (uint16_t)at;
+    if (b < P.ranges) tot[b] += cnt[min((b + 1) << P.step, P.nf)] - at;
+  }
+}
+
 __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n,
                                                         uint32_t nbins, PartArgs P) {
   extern __shared__ __align__(16) unsigned char hp_sm[];
@@ -308,7 +333,7 @@ __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict_
   __shared__ uint32_t wsum[32];
   const int lane = threadIdx.x & 31;
   const uint64_t end = n + off;  // items in group space: item i of the stream is key i - off
-  const uint32_t step = PS - P.fshift, fs = P.fshift;
+  const uint32_t fs = P.fshift;
   for (uint32_t i = threadIdx.x; i < P.ranges; i += PT) tot[i] = 0;
   const uint32_t per = (P.chunks + gridDim.x - 1) / gridDim.x;
   const uint32_t c0 = blockIdx.x * per, c1 = min(c0 + per, P.chunks);
@@ -340,11 +365,7 @@ __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict_
     }
     __syncthreads();
     block_scan<PT>(cnt, P.nf, wsum);
-    for (uint32_t b = threadIdx.x; b <= P.ranges; b += PT) {
-      const uint32_t at = cnt[min(b << step, P.nf)];
-      stage[b * PGROUP + c % PGROUP] = (uint16_t)at;
-      if (b < P.ranges) tot[b] += cnt[min((b + 1) << step, P.nf)] - at;
-    }
+    stage_starts(P, cnt, stage, tot, c);
     __syncthreads();  // the starts are read; the counters become cursors
     if (whole) {
 #pragma unroll 1
@@ -386,21 +407,11 @@ __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict_
       }
     }
     __syncthreads();
-    uint4* out = reinterpret_cast<uint4*>(P.item + i0);
+    uint4* out = reinterpret_cast<uint4*>(static_cast<uint16_t*>(P.item) + i0);
     const uint4* in = reinterpret_cast<const uint4*>(buf);
 #pragma unroll
     for (uint32_t i = 0; i < PCHUNK * 2 / 16 / PT; ++i) out[i * PT + threadIdx.x] = in[i * PT + threadIdx.x];
-    // the starts of the chunks since the last table write
-    const uint32_t g0 = c / PGROUP * PGROUP;
-    if (c % PGROUP == PGROUP - 1 || c + 1 == c1) {
-      for (uint32_t b = threadIdx.x; b <= P.ranges; b += PT) {
-        uint16_t* t = P.start + (uint64_t)b * P.chunks + g0;
-        if (g0 >= c0 && c % PGROUP == PGROUP - 1)
-          *reinterpret_cast<uint4*>(t) = *reinterpret_cast<const uint4*>(stage + b * PGROUP);
-        else
-          for (uint32_t q = g0 < c0 ? c0 - g0 : 0; q <= c % PGROUP; ++q) t[q] = stage[b * PGROUP + q];
-      }
-    }
+    write_starts(P, stage, c, c0, c1);
   }
   __syncthreads();
   for (uint32_t b = threadIdx.x; b < P.ranges; b += PT)
@@ -410,8 +421,10 @@ __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict_
 // Units of every range (one CTA per range; every CTA scans all ranges' unit
 // counts).  A range of several units starts from zeroed bins (unless the
 // counts add to those of an earlier round).
-__global__ void __launch_bounds__(256) hk_plan_kernel(PartArgs P, uint32_t nbins, uint32_t unit_keys, uint32_t add,
-                                                      unsigned long long* __restrict__ out) {
+// (A range is 2^PS words of the result, words in all.)
+template <typename W>
+__global__ void __launch_bounds__(256) hk_plan_kernel(PartArgs P, uint64_t words, uint32_t unit_keys, uint32_t add,
+                                                      W* __restrict__ out) {
   pdl_wait();
   __shared__ uint32_t s_before[8], s_all[8], s_mine;
   const uint32_t b = blockIdx.x;
@@ -439,7 +452,7 @@ __global__ void __launch_bounds__(256) hk_plan_kernel(PartArgs P, uint32_t nbins
     P.total[P.ranges + 1] = all;
   }
   if (parts > 1 && !add)
-    for (uint64_t i = ((uint64_t)b << PS) + threadIdx.x; i < ((uint64_t)(b + 1) << PS) && i <= nbins; i += 256)
+    for (uint64_t i = ((uint64_t)b << PS) + threadIdx.x; i < ((uint64_t)(b + 1) << PS) && i < words; i += 256)
       out[i] = 0;
 }
 
@@ -451,9 +464,25 @@ __global__ void __launch_bounds__(256) hk_plan_kernel(PartArgs P, uint32_t nbins
 // over the lanes).  CAHEAD quads per lane are in flight (the pieces lie in
 // DRAM).
 constexpr int CAHEAD = 4;
-__global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint32_t nbins, uint32_t add,
-                                                          unsigned long long* __restrict__ out) {
+// What is grouped, and what a range's words are: keys (16-bit bin numbers, u32
+// counts, u64 results) or bit positions (32 bits, u32 words of a bit array).
+struct KeyItems {
+  using Item = uint16_t;
+  using Quad = uint2;
+  using Word = unsigned long long;
+  static constexpr uint32_t CHUNK = PCHUNK;
+  static __device__ __forceinline__ void put(uint32_t* w, uint32_t x) { atomicAdd(w + x, 1u); }
+  static __device__ __forceinline__ uint32_t item(const Quad& q, int i) {
+    return (i & 1) ? (i < 2 ? q.x : q.y) >> 16 : (i < 2 ? q.x : q.y) & 0xffffu;
+  }
+  static __device__ __forceinline__ void add(Word* o, uint32_t v) { atomicAdd(o, (Word)v); }
+  static __device__ __forceinline__ Word merged(Word o, uint32_t v) { return o + v; }
+};
+template <class T>
+__global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint64_t words, uint32_t add,
+                                                          typename T::Word* __restrict__ out) {
   pdl_wait();
+  const typename T::Item* items = static_cast<const typename T::Item*>(P.item);
   extern __shared__ __align__(16) uint32_t hc_bins[];  // [1 << PS]
   __shared__ uint32_t s_unit;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -489,7 +518,7 @@ __global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint32_t n
       const uint32_t all = __shfl_sync(0xffffffffu, ex, 31);
       ex -= nq;
       for (uint32_t f0 = 0; f0 < all; f0 += 32 * CAHEAD) {
-        uint2 w[CAHEAD];
+        typename T::Quad w[CAHEAD];
         uint32_t r[CAHEAD], len[CAHEAD];  // the quad's first offset relative to its piece, and the piece's length
 #pragma unroll
         for (int t = 0; t < CAHEAD; ++t) {
@@ -505,27 +534,26 @@ __global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint32_t n
           if (f < all) {
             len[t] = (pc >> 16) - (pc & 0xffffu);
             const uint32_t cp = u.y + ((l0 + p) >> P.split);
-            w[t] = __ldg(reinterpret_cast<const uint2*>(P.item + (uint64_t)cp * PCHUNK + i));
+            w[t] = __ldg(reinterpret_cast<const typename T::Quad*>(items + (uint64_t)cp * T::CHUNK + i));
           }
         }
 #pragma unroll
         for (int t = 0; t < CAHEAD; ++t) {
-          if (r[t] < len[t]) atomicAdd(hc_bins + (w[t].x & 0xffffu), 1u);
-          if (r[t] + 1 < len[t]) atomicAdd(hc_bins + (w[t].x >> 16), 1u);
-          if (r[t] + 2 < len[t]) atomicAdd(hc_bins + (w[t].y & 0xffffu), 1u);
-          if (r[t] + 3 < len[t]) atomicAdd(hc_bins + (w[t].y >> 16), 1u);
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (r[t] + e < len[t]) T::put(hc_bins, T::item(w[t], e));
         }
       }
     }
     __syncthreads();
     const uint64_t b0 = (uint64_t)u.x << PS;
-    const uint32_t nb = (uint32_t)min((uint64_t)(1u << PS), (uint64_t)nbins + 1 - b0);
+    const uint32_t nb = (uint32_t)min((uint64_t)(1u << PS), words - b0);
     for (uint32_t i = threadIdx.x; i < nb; i += PCT) {
       const uint32_t v = hc_bins[i];
       if (u.w) {
-        if (v) atomicAdd(out + b0 + i, (unsigned long long)v);
+        if (v) T::add(out + b0 + i, v);
       } else {
-        out[b0 + i] = add ? out[b0 + i] + v : v;
+        out[b0 + i] = add ? T::merged(out[b0 + i], v) : v;
       }
     }
   }
@@ -550,6 +578,14 @@ __device__ __forceinline__ uint64_t mod_barrett(uint64_t x, uint64_t m, uint64_t
   if (rem >= m) rem -= m;
   if (rem >= m) rem -= m;
   return rem;
+}
+
+// The same for m < 2^30: the remainder before the corrections is below 3 m, so
+// its low 32 bits are all of it.
+__device__ __forceinline__ uint32_t mod_barrett32(uint64_t x, uint32_t m, uint64_t r) {
+  uint32_t rem = (uint32_t)x - (uint32_t)__umul64hi(x, r) * m;
+  rem = min(rem, rem - m);  // (rem - m wraps to a large number when rem < m)
+  return min(rem, rem - m);
 }
 
 // 2-bit code and invalid flag of 4 bases packed little-endian in w (first
@@ -619,6 +655,132 @@ bloom_kernel(const uint8_t* __restrict__ seq, uint64_t n, uint32_t L, uint64_t m
   }
 }
 
+// ----------------------------------------------------- partitioned filter
+// The filter's atomicOrs are bound by the L2's atomic rate (210G bit-sets a
+// second: 1.00 ms for 30M windows, 7 hashes), so, as for the large-key
+// histogram, the positions of a job with many of them are grouped by ranges
+// of 2^20 bits and each range is set in one CTA's shared memory and stored
+// once.  A chunk is as many windows as have at most BCHUNK positions: they are
+// computed once into shared memory (counting them by bucket), then grouped.
+// 4 bytes a position are written and read again; 30M windows into 3e8 bits take
+// 0.85 ms instead of 1.04 in all (grouping 546 us, bound by issue and the
+// shared-memory pipe; setting 255 us), into 1e6 bits 0.83 instead of 2.16.
+constexpr int BT = 1024;                 // threads of the grouping kernel (two CTAs per SM)
+constexpr uint32_t BCHUNK = 16384;       // positions
+constexpr uint32_t BNF = 512;            // buckets, at most
+constexpr uint32_t BRANGES = 512;        // ranges, at most
+constexpr uint32_t BS = PS + 5;          // log2 of a range's bits
+constexpr uint32_t BNONE = 0xFFFFFFFFu;  // no position (m <= 2^29)
+// windows per chunk: whole rounds of the CTA's threads, or of a warp's
+__host__ __device__ constexpr uint32_t bloom_windows(uint32_t h) {
+  return BCHUNK / h >= (uint32_t)BT ? BCHUNK / h / BT * BT : BCHUNK / h / 32 * 32;
+}
+static_assert(bloom_windows(32) >= 32, "a chunk holds windows for every number of hashes");
+struct BitItems {
+  using Item = uint32_t;
+  using Quad = uint4;
+  using Word = uint32_t;
+  static constexpr uint32_t CHUNK = BCHUNK;
+  static __device__ __forceinline__ void put(uint32_t* w, uint32_t x) { atomicOr(w + (x >> 5), 1u << (x & 31)); }
+  static __device__ __forceinline__ uint32_t item(const Quad& q, int i) { return key_at(q, i); }
+  static __device__ __forceinline__ void add(Word* o, uint32_t v) { atomicOr(o, v); }
+  static __device__ __forceinline__ Word merged(Word o, uint32_t v) { return o | v; }
+};
+
+// Four bases at pos (little-endian, beyond n: 0): two aligned words where both
+// hold bases of the input, single bytes at its ends.
+__device__ __forceinline__ uint32_t bases4(const uint8_t* __restrict__ seq, uint64_t n, uint64_t pos) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(seq + pos);
+  const uint32_t sh = (uint32_t)(a & 3) * 8;
+  if (pos + 8 <= n && pos >= 4) {
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(a & ~uintptr_t(3));
+    return __funnelshift_r(__ldg(w), __ldg(w + 1), sh);
+  }
+  uint32_t v = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v |= (pos + j < n ? (uint32_t)seq[pos + j] : 0u) << (8 * j);
+  return v;
+}
+
+// Windows w0 .. w0 + nwin - 1 of the sequence, wt per chunk.
+__global__ void __launch_bounds__(BT, 2) bloom_part_kernel(const uint8_t* __restrict__ seq, uint64_t n, uint64_t w0,
+                                                           uint64_t nwin, uint32_t wt, uint32_t L, uint32_t m,
+                                                           uint64_t rm, uint64_t rm1, uint32_t h, PartArgs P) {
+  extern __shared__ __align__(16) unsigned char bp_sm[];
+  uint32_t* pos = reinterpret_cast<uint32_t*>(bp_sm);             // [BCHUNK] in the order of the windows, then grouped
+  uint32_t* cnt = pos + BCHUNK;                                   // [BNF + 1]
+  uint32_t* tot = cnt + BNF + 4;                                  // [BRANGES]
+  uint16_t* stage = reinterpret_cast<uint16_t*>(tot + BRANGES);   // [ranges + 1][PGROUP]
+  __shared__ unsigned long long sc[BCHUNK / 32 + 2];  // 32 bases per word, first base in the top bits
+  __shared__ uint32_t sb[BCHUNK / 32 + 2];            // 1 = not A/C/G/T, same order
+  __shared__ uint32_t wsum[32];
+  const uint32_t fs = P.fshift;
+  for (uint32_t i = threadIdx.x; i < P.ranges; i += BT) tot[i] = 0;
+  const uint32_t per = (P.chunks + gridDim.x - 1) / gridDim.x;
+  const uint32_t c0 = blockIdx.x * per, c1 = min(c0 + per, P.chunks);
+  for (uint32_t c = c0; c < c1; ++c) {
+    const uint64_t first = (uint64_t)c * wt;
+    const uint32_t count = first < nwin ? (uint32_t)min((uint64_t)wt, nwin - first) : 0;
+    const uint64_t p0 = w0 + first;
+    for (uint32_t i = threadIdx.x; i < P.nf; i += BT) cnt[i] = 0;
+    // pack 8 bases per thread
+    const uint32_t nw = count ? (count + L - 1 + 31) / 32 + 1 : 0;  // words, one of them past the last base
+    for (uint32_t t = threadIdx.x; t < 4 * nw; t += BT) {
+      uint32_t ca, ba, cb, bb;
+      pack4(bases4(seq, n, p0 + 8 * t), ca, ba);
+      pack4(bases4(seq, n, p0 + 8 * t + 4), cb, bb);
+      const uint32_t wi = t >> 2, q = t & 3;
+      reinterpret_cast<uint16_t*>(sc + wi)[3 - q] = (uint16_t)((ca << 8) | cb);
+      reinterpret_cast<uint8_t*>(sb + wi)[3 - q] = (uint8_t)((ba << 4) | bb);
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < count; i += BT) {
+      const uint32_t wi = i >> 5, o = i & 31;
+      const uint64_t bm = (((uint64_t)sb[wi] << 32) | sb[wi + 1]) << o;
+      if (bm >> (64 - L)) {  // a base of the window is not A/C/G/T
+        for (uint32_t q = 0; q < h; ++q) pos[q * count + i] = BNONE;
+        continue;
+      }
+      const uint64_t hi = sc[wi], lo = sc[wi + 1];
+      const uint64_t cat = o ? (hi << (2 * o)) | (lo >> (64 - 2 * o)) : hi;
+      const uint64_t code = cat >> (64 - 2 * L);
+      uint32_t x = mod_barrett32(mix64(code), m, rm);
+      const uint32_t step = 1 + mod_barrett32(mix64(code ^ 0x9E3779B97F4A7C15ull), m - 1, rm1);
+      uint32_t* at = pos + i;
+#pragma unroll 4
+      for (uint32_t q = 0; q < h; ++q, at += count) {
+        *at = x;
+        atomicAdd(cnt + (x >> fs), 1u);
+        x += step;  // below 2^30
+        x = min(x, x - m);
+      }
+    }
+    __syncthreads();
+    block_scan<BT>(cnt, P.nf, wsum);
+    stage_starts(P, cnt, stage, tot, c);
+    const uint32_t all = cnt[P.nf], np = count * h;
+    // grouped in place, from registers
+    uint32_t x[BCHUNK / BT];
+#pragma unroll
+    for (int q = 0; q < (int)(BCHUNK / BT); ++q) {
+      const uint32_t i = q * BT + threadIdx.x;
+      x[q] = i < np ? pos[i] : BNONE;
+    }
+    __syncthreads();  // the starts and positions are read; the counters become cursors
+#pragma unroll
+    for (int q = 0; q < (int)(BCHUNK / BT); ++q)
+      if (x[q] != BNONE) pos[atomicAdd(cnt + (x[q] >> fs), 1u)] = x[q] & ((1u << BS) - 1);
+    __syncthreads();
+    uint4* out = reinterpret_cast<uint4*>(static_cast<uint32_t*>(P.item) + (uint64_t)c * BCHUNK);
+    for (uint32_t i = threadIdx.x; i < (all + 3) / 4; i += BT) out[i] = reinterpret_cast<const uint4*>(pos)[i];
+    __syncthreads();  // (the next chunk's positions go where these were)
+    write_starts(P, stage, c, c0, c1);
+  }
+  __syncthreads();
+  for (uint32_t b = threadIdx.x; b < P.ranges; b += BT)
+    if (tot[b]) atomicAdd(P.total + b, tot[b]);
+}
+
 }  // namespace
 
 int hk_smem_max_bins(const DevInfo& di) { return di.smem_optin / 4 - 1; }
@@ -672,26 +834,33 @@ bool hk_partitioned(uint64_t n, uint32_t nbins) {
   const uint64_t ranges = ((uint64_t)nbins >> PS) + 1;
   return ranges <= PRANGES && n >= nbins && (n >= 1ull << 24 || (n >= 1ull << 22 && n * ranges >= 1ull << 26));
 }
-static PartArgs hk_part_args(uint64_t n, uint32_t nbins, uint8_t* p, size_t* bytes) {
+// Scratch for `chunks` chunks, the result's words in ranges.
+static PartArgs part_args(uint64_t chunks, uint32_t chunk_items, size_t item_bytes, uint32_t ranges, uint8_t* p,
+                          size_t* bytes) {
   PartArgs P{};
-  const uint64_t m = n < PART_ROUND ? n : PART_ROUND;
-  const uint64_t chunks = (m + 3 + PCHUNK - 1) / PCHUNK;  // + 3: keys may start inside a 16-byte group
   P.chunks = (uint32_t)((chunks + PGROUP - 1) / PGROUP * PGROUP);
-  P.ranges = (nbins >> PS) + 1;
-  while (((nbins >> P.fshift) + 1) > PNF) ++P.fshift;
-  P.nf = (nbins >> P.fshift) + 1;
-  while ((P.ranges << P.split) < 512) ++P.split;  // parts of 64 keys or so
+  P.ranges = ranges;
+  while ((chunk_items / ranges) >> (P.split + 1) >= 64) ++P.split;  // parts of at least 64 items
   size_t at = 0;
   auto take = [&](size_t sz) {
     uint8_t* r = p + at;
     at += (sz + 255) & ~(size_t)255;
     return r;
   };
-  P.item = reinterpret_cast<uint16_t*>(take((size_t)P.chunks * PCHUNK * 2));
+  P.item = take((size_t)P.chunks * chunk_items * item_bytes);
   P.start = reinterpret_cast<uint16_t*>(take((size_t)(P.ranges + 1) * P.chunks * 2));
   P.total = reinterpret_cast<uint32_t*>(take((size_t)(P.ranges + 2) * 4));
   P.unit = reinterpret_cast<uint4*>(take((size_t)(2 * P.ranges + PUNITS) * 16));
   *bytes = at;
+  return P;
+}
+static PartArgs hk_part_args(uint64_t n, uint32_t nbins, uint8_t* p, size_t* bytes) {
+  const uint64_t m = n < PART_ROUND ? n : PART_ROUND;
+  // + 3: keys may start inside a 16-byte group
+  PartArgs P = part_args((m + 3 + PCHUNK - 1) / PCHUNK, PCHUNK, 2, (nbins >> PS) + 1, p, bytes);
+  while (((nbins >> P.fshift) + 1) > PNF) ++P.fshift;
+  P.nf = (nbins >> P.fshift) + 1;
+  P.step = PS - P.fshift;
   return P;
 }
 size_t hk_part_bytes(uint64_t n, uint32_t nbins) {
@@ -708,7 +877,7 @@ cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbi
   const int csm = (1 << PS) * 4;
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(hk_part_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, psm)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(hk_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, csm)) != cudaSuccess)
+      (e = cudaFuncSetAttribute(hk_count_kernel<KeyItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm)) != cudaSuccess)
     return e;
   if ((e = kt_begin(kt, s)) != cudaSuccess) return e;
   for (uint64_t k0 = 0; k0 < n; k0 += PART_ROUND) {
@@ -722,9 +891,11 @@ cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbi
     if ((e = cudaMemsetAsync(P.total, 0, (P.ranges + 2) * 4, s)) != cudaSuccess) return e;
     hk_part_kernel<<<P.chunks < pg ? P.chunks : pg, PT, psm, s>>>(base, off, m, nbins, P);
     if ((e = cudaGetLastError()) != cudaSuccess ||
-        (e = launch_pdl(hk_plan_kernel, dim3(P.ranges), dim3(256), 0, s, P, nbins, (uint32_t)uk, add, out)) !=
+        (e = launch_pdl(hk_plan_kernel<unsigned long long>, dim3(P.ranges), dim3(256), 0, s, P, (uint64_t)nbins + 1,
+                        (uint32_t)uk, add, out)) !=
             cudaSuccess ||
-        (e = launch_pdl(hk_count_kernel, dim3(di.sms), dim3(PCT), (size_t)csm, s, P, nbins, add, out)) != cudaSuccess)
+        (e = launch_pdl(hk_count_kernel<KeyItems>, dim3(di.sms), dim3(PCT), (size_t)csm, s, P, (uint64_t)nbins + 1, add,
+                        out)) != cudaSuccess)
       return e;
     *nk += 3;
   }
@@ -801,6 +972,63 @@ cudaError_t launch_bloom(const uint8_t* seq, uint64_t n, uint32_t L, uint64_t m,
   if ((e = cudaGetLastError()) != cudaSuccess || (e = kt_end(kt, s)) != cudaSuccess) return e;
   ++*nk;
   return cudaSuccess;
+}
+
+// Partitioned filter: up to 2^29 bits (512 ranges), from 2^24 positions on, with
+// at least 5 hashes (the two 64-bit mixes of a window are paid once) or few
+// ranges, whose words the L2's atomics contend for.  Measured, partitioned
+// against atomicOr on the global array, us a call: 30M windows x 7 into 2.4e8
+// bits 949 / 1,032, x 3 500 / 465 (left to the array), x 3 into 1e6 472 / 944;
+// 3M x 7 into 2.4e7 124 / 144; 5.6M x 3 into 1e6 155 / 203.
+constexpr uint64_t BLOOM_ROUND = 1ull << 29;  // positions grouped at a time (4 bytes each of scratch)
+bool bloom_partitioned(uint64_t n, uint32_t L, uint64_t m, uint32_t h) {
+  return n >= L && m <= (uint64_t)BRANGES << BS && (n - L + 1) * h >= 1ull << 24 && (h >= 5 || m <= 1ull << 24);
+}
+static uint64_t bloom_round(uint32_t h) { return BLOOM_ROUND / BCHUNK * bloom_windows(h); }  // windows grouped at a time
+static PartArgs bloom_part_args(uint64_t n, uint32_t L, uint64_t m, uint32_t h, uint8_t* p, size_t* bytes) {
+  const uint64_t nwin = n - L + 1, w = nwin < bloom_round(h) ? nwin : bloom_round(h);
+  const uint32_t wt = bloom_windows(h);
+  PartArgs P = part_args((w + wt - 1) / wt, BCHUNK, 4, (uint32_t)((m - 1) >> BS) + 1, p, bytes);
+  while (((m - 1) >> P.fshift) + 1 > BNF) ++P.fshift;
+  P.nf = (uint32_t)((m - 1) >> P.fshift) + 1;
+  P.step = BS - P.fshift;
+  return P;
+}
+size_t bloom_part_bytes(uint64_t n, uint32_t L, uint64_t m, uint32_t h) {
+  size_t b = 0;
+  bloom_part_args(n, L, m, h, nullptr, &b);
+  return b;
+}
+cudaError_t launch_bloom_part(const uint8_t* seq, uint64_t n, uint32_t L, uint64_t m, uint32_t h, uint8_t* scratch,
+                              uint32_t* bits, const DevInfo& di, cudaStream_t s, uint64_t* nk, KTimer* kt) {
+  size_t bytes = 0;
+  const PartArgs P = bloom_part_args(n, L, m, h, scratch, &bytes);
+  const int psm = (int)((BCHUNK + BNF + 4 + BRANGES) * 4 + (P.ranges + 1) * PGROUP * 2);
+  const int csm = (1 << PS) * 4;
+  const uint64_t words = (m + 31) / 32, nwin = n - L + 1, rm = ~0ull / m, rm1 = ~0ull / (m - 1);
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(bloom_part_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, psm)) !=
+          cudaSuccess ||
+      (e = cudaFuncSetAttribute(hk_count_kernel<BitItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm)) !=
+          cudaSuccess)
+    return e;
+  if ((e = kt_begin(kt, s)) != cudaSuccess) return e;
+  for (uint64_t w0 = 0; w0 < nwin; w0 += bloom_round(h)) {
+    const uint64_t w = nwin - w0 < bloom_round(h) ? nwin - w0 : bloom_round(h);
+    const uint64_t uk = w * h / PUNITS > PUNIT_MIN ? w * h / PUNITS : PUNIT_MIN;
+    const uint32_t add = w0 ? 1u : 0u, pg = (uint32_t)di.sms * 2;
+    if ((e = cudaMemsetAsync(P.total, 0, (P.ranges + 2) * 4, s)) != cudaSuccess) return e;
+    bloom_part_kernel<<<P.chunks < pg ? P.chunks : pg, BT, psm, s>>>(seq, n, w0, w, bloom_windows(h), L, (uint32_t)m, rm,
+                                                                     rm1, h, P);
+    if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = launch_pdl(hk_plan_kernel<uint32_t>, dim3(P.ranges), dim3(256), 0, s, P, words, (uint32_t)uk, add,
+                        bits)) != cudaSuccess ||
+        (e = launch_pdl(hk_count_kernel<BitItems>, dim3(di.sms), dim3(PCT), (size_t)csm, s, P, words, add, bits)) !=
+            cudaSuccess)
+      return e;
+    *nk += 3;
+  }
+  return kt_end(kt, s);
 }
 
 }  // namespace mrgb

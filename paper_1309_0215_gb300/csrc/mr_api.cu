@@ -71,7 +71,7 @@ struct Job {
   bool wc_auto = true;
   // large-key histogram: u32 counters (null: count straight into the u64 result)
   void* hk_counters = nullptr;
-  uint8_t* hk_part = nullptr;  // scratch of partitioned counting (null: not taken)
+  uint8_t* part = nullptr;  // scratch of partitioned counting, large-key histogram and Bloom filter (null: not taken)
   // k-means
   KmBuffers km;
   uint64_t* host = nullptr;      // pinned status words (word count, k-means)
@@ -401,7 +401,7 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
           j->slab_bytes = res + scr;
           j->result = j->slab;
           j->result_bytes = nb * 8;
-          j->hk_part = static_cast<uint8_t*>(j->slab) + res;
+          j->part = static_cast<uint8_t*>(j->slab) + res;
           return MR_OK;
         }
       }
@@ -415,6 +415,18 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
     }
     case MR_BLOOM_DNA: {
       const uint64_t bytes = align256((d.bloom_bits + 31) / 32 * 4);
+      j->result_bytes = (d.bloom_bits + 7) / 8;
+      // as for the large-key histogram
+      if (d.container == MR_C_AUTO && c->budget == 0 &&
+          bloom_partitioned(d.input_bytes, d.bloom_kmer, d.bloom_bits, d.bloom_hashes)) {
+        const uint64_t scr = align256(bloom_part_bytes(d.input_bytes, d.bloom_kmer, d.bloom_bits, d.bloom_hashes));
+        if (dev_alloc(c, bytes + scr, &j->slab) == MR_OK) {
+          j->slab_bytes = bytes + scr;
+          j->result = j->slab;
+          j->part = static_cast<uint8_t*>(j->slab) + bytes;
+          return MR_OK;
+        }
+      }
       mr_status st = dev_alloc(c, bytes, &j->slab);
       if (st) return st;
       j->slab_bytes = bytes;
@@ -527,9 +539,9 @@ mr_status enqueue_plain_on(mr_ctx* c, Job* j, cudaStream_t st) {
                                    c->opt_polls));
       break;
     case MR_HIST_U32:
-      if (j->hk_part) {
+      if (j->part) {
         MR_CUDA_TRY(launch_hist_keys_part(reinterpret_cast<const uint32_t*>(j->in), n / 4, j->desc.hist_bins,
-                                          j->hk_part, static_cast<unsigned long long*>(j->result), c->di, st,
+                                          j->part, static_cast<unsigned long long*>(j->result), c->di, st,
                                           &c->launches, j->kt));
         break;
       }
@@ -538,6 +550,11 @@ mr_status enqueue_plain_on(mr_ctx* c, Job* j, cudaStream_t st) {
                                    static_cast<unsigned long long*>(j->result), c->di, st, &c->launches, j->kt));
       break;
     case MR_BLOOM_DNA:
+      if (j->part) {
+        MR_CUDA_TRY(launch_bloom_part(j->in, n, j->desc.bloom_kmer, j->desc.bloom_bits, j->desc.bloom_hashes, j->part,
+                                      static_cast<uint32_t*>(j->result), c->di, st, &c->launches, j->kt));
+        break;
+      }
       MR_CUDA_TRY(launch_bloom(j->in, n, j->desc.bloom_kmer, j->desc.bloom_bits, j->desc.bloom_hashes,
                                static_cast<uint32_t*>(j->result), c->di, st, &c->launches, j->kt));
       break;

@@ -90,6 +90,13 @@ cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbi
 cudaError_t launch_bloom(const uint8_t* seq, uint64_t n, uint32_t L, uint64_t m, uint32_t h, uint32_t* bits,
                          const DevInfo& di, cudaStream_t s, uint64_t* nk, KTimer* kt = nullptr);
 
+// The same for many positions (bloom_partitioned), through bloom_part_bytes of
+// scratch; every word is written.
+bool bloom_partitioned(uint64_t n, uint32_t L, uint64_t m, uint32_t h);
+size_t bloom_part_bytes(uint64_t n, uint32_t L, uint64_t m, uint32_t h);
+cudaError_t launch_bloom_part(const uint8_t* seq, uint64_t n, uint32_t L, uint64_t m, uint32_t h, uint8_t* scratch,
+                              uint32_t* bits, const DevInfo& di, cudaStream_t s, uint64_t* nk, KTimer* kt = nullptr);
+
 // --------------------------------------------------------- word count job
 struct WcBuffers {
   uint64_t cap = 0;            // global hash-table slots (power of two)

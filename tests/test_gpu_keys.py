@@ -192,3 +192,33 @@ def test_hist_u32_partitioned_rounds_and_budget(mr):
     ctx.run()
     assert np.array_equal(np.frombuffer(ctx.fetch(j), dtype=np.uint64), want)
     ctx.close()
+
+
+@pytest.mark.parametrize("n,L,m,h", [
+    (2_396_776, 32, 20_000_003, 7),     # 2^24 positions and a few
+    (16_777_217, 2, 97, 1),             # one range of four words, 8,192 windows a chunk
+    (2_400_001, 15, (1 << 20) + 1, 7),  # a second range of one bit
+    (530_001, 20, 1 << 22, 32),         # the most hashes
+    (3_400_007, 31, 1 << 29, 5),        # the most ranges
+])
+@pytest.mark.parametrize("offset", [0, 1, 3])
+def test_bloom_partitioned(mr, n, L, m, h, offset):
+    """Filters with enough positions to be grouped by ranges of bits: the
+    oracle's bytes (runs of N, a sequence that starts at any byte)."""
+    seq = synth.dna(n, seed=n + L, n_runs=50, max_run=3000)
+    assert np.array_equal(mr.bloom_dna(_dev(seq, offset), L, m, h), oracle.bloom_dna(seq, L, m, h))
+
+
+def test_bloom_partitioned_rounds_and_budget(mr):
+    """More positions than one round groups, against a context with an HBM
+    budget, which sets every bit with an atomicOr on the global array."""
+    n, L, m, h = 17_000_031, 21, 400_000_007, 32
+    seq = _dev(synth.dna(n, seed=9, n_runs=300, max_run=1000))
+    import torch
+    torch.cuda.synchronize()
+    ctx = mr.Context(hbm_budget=1 << 30)
+    j = ctx.add_job(mr.BLOOM_DNA, seq, bloom_kmer=L, bloom_bits=m, bloom_hashes=h)
+    ctx.run()
+    want = np.frombuffer(ctx.fetch(j), dtype=np.uint8)
+    ctx.close()
+    assert np.array_equal(mr.bloom_dna(seq, L, m, h), want)
