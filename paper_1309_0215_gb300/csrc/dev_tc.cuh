@@ -157,6 +157,10 @@ __device__ __forceinline__ void top2_sets(const int (&t1)[NSET], const int (&t2)
   for (int a = 0; a < NSET; ++a) lb = min(lb, (t1[a] == w1 || t1[a] == w2) ? t2[a] : t1[a]);
 }
 
+// Whether the distance pass takes the filter's list (its rows are gathered) or
+// all points (whole tiles in one copy): the line is the list's extra cost.
+__device__ __forceinline__ bool km_use_list(uint32_t nact, uint32_t n) { return nact < n - n / 8; }
+
 // Append one entry per lane with `on` to a list, the warp's entries together;
 // put(slot) writes it.  All 32 lanes call this.
 template <class F>

@@ -132,7 +132,8 @@ __global__ void __launch_bounds__(SETUP_THREADS) km_setup_kernel(const float* __
   }
   if (blockIdx.x == 0)
     for (uint32_t i = threadIdx.x; i < k; i += SETUP_THREADS) cnew[i] = 0;
-  if (blockIdx.x == 0 && threadIdx.x < 8) nflag[threadIdx.x] = 0;
+  // counters, and the words behind the exponent (largest drift, sum of them)
+  if (blockIdx.x == 0 && threadIdx.x < 24) nflag[threadIdx.x] = 0;
   if (blockIdx.x == 0 && threadIdx.x < 4) stats[threadIdx.x] = 0;
 }
 
@@ -381,7 +382,8 @@ __device__ __forceinline__ int fx_shift_of(float m, uint32_t n) {
 // the second is beyond widen times the first, the first is the FP64 winner.
 //
 // A point that FP32 cannot decide is settled by the definition in FP64 on the
-// spot, by its whole CTA: the candidates are the centroids whose FP32
+// spot: one with a few candidates by its eight lanes, a candidate each; a
+// listed one by its whole CTA: the candidates are the centroids whose FP32
 // distance is within the bound of the smallest; the products (x_j - c_j)^2,
 // separately rounded, for all dimensions of a chunk of candidates at once
 // (the FP64 pipe is narrow on this GPU), and one thread per candidate adding
@@ -421,7 +423,7 @@ __device__ __forceinline__ void sqdiff2(unsigned long long& a, unsigned long lon
 
 struct SettleShared {
   uint32_t m1[SET_T_MAX / 32][SET_RP], k1[SET_T_MAX / 32][SET_RP], m2[SET_T_MAX / 32][SET_RP];
-  uint32_t open[SET_T_MAX / 8 > SET_RP ? SET_T_MAX / 8 : SET_RP];  // points of the batch left to FP64
+  uint32_t open[SET_RP];  // points of the batch left to FP64
   uint32_t nopen, ncand, moved;
   float red_f[SET_T_MAX / 32];
   double red_d[SET_T_MAX / 32];
@@ -545,6 +547,10 @@ __device__ __forceinline__ void few_dists(const float* __restrict__ x, const flo
     for (int o = 4; o; o >>= 1) f[i] += __shfl_xor_sync(0xffffffffu, f[i], o);
 }
 
+__device__ __forceinline__ KmFew load_few(const KmFew* __restrict__ few, uint32_t n, uint64_t i) {
+  return i < n ? few[i] : KmFew{0, 0, 0};
+}
+
 // MULTI: more centroids than threads, so each thread keeps a running top-2.
 // With maxabs not null (the first iteration, whose distance pass or a pass
 // before it found max |x|) one thread also sets the update's exponent.
@@ -553,7 +559,7 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
     const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, const float* __restrict__ ct,
     uint32_t k, const KmFew* __restrict__ pairs, const uint32_t* npairs, const uint32_t* __restrict__ list,
     const uint32_t* nlist, uint32_t* assign, uint32_t* nchg, unsigned long long* stat, const unsigned int* maxabs, int* shift,
-    unsigned int* cmax_next) {
+    unsigned int* cmax_next, KmBounds B) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char set_sm[];
   __shared__ SettleShared S;
@@ -566,20 +572,80 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const uint32_t np = *npairs, nf = *nlist;
   if (threadIdx.x == 0) S.moved = 0;
+  __syncthreads();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     if (maxabs) *shift = fx_shift_of(__uint_as_float(*maxabs), n);
     *cmax_next = 0;  // the next iteration's max ||c||
     if (np + nf) atomicAdd(stat, (unsigned long long)np + nf);
   }
   const float widen = rel_bound_widen(d);
-  const uint32_t ppb = blockDim.x >> 3;  // few-candidate points per batch
   const bool vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-  const uint64_t rb = ((uint64_t)nf + SET_RP - 1) / SET_RP, nb = rb + ((uint64_t)np + ppb - 1) / ppb;
-  unsigned long long settled = 0;  // thread 0: points settled in FP64
-  for (uint64_t b = blockIdx.x; b < nb; b += gridDim.x) {
+  const uint64_t rb = ((uint64_t)nf + SET_RP - 1) / SET_RP;
+  unsigned long long settled = 0;  // points settled in FP64
+  // the few-candidate points: warps on their own, four points at a time (the
+  // last CTAs first: the listed points' batches start with the first ones)
+  {
+    const uint32_t sl = lane & 7;
+    const uint64_t w0 = (uint64_t)(gridDim.x - 1 - blockIdx.x) * nw + warp;
+    KmFew next = load_few(pairs, np, 4 * w0 + (lane >> 3));
+    for (uint64_t f0 = 4 * w0; f0 < np; f0 += 4 * (uint64_t)gridDim.x * nw) {
+      const KmFew e = next;
+      next = load_few(pairs, np, f0 + 4 * (uint64_t)gridDim.x * nw + (lane >> 3));
+      const uint32_t nc = e.hi >> 28;
+      float fd[KM_CAND_MAX];
+      if (__any_sync(0xffffffffu, nc > 2)) few_dists<KM_CAND_MAX>(x, c, d, e, nc, sl, vec, fd);
+      else few_dists<2>(x, c, d, e, nc, sl, vec, fd);
+      float m1 = INFINITY, m2 = INFINITY;
+      uint32_t k1 = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < KM_CAND_MAX; ++i)
+        if (i < nc) {
+          if (fd[i] < m1) m2 = m1, m1 = fd[i], k1 = few_cand(e, i);
+          else if (!(fd[i] >= m2)) m2 = fd[i];  // (a NaN makes m2 NaN: the point is left to FP64)
+        }
+      const bool clear = nc == 0 || m2 > m1 * widen;
+      if (!__all_sync(0xffffffffu, clear)) {
+        // the definition, one candidate per lane, dimensions in order
+        double best = INFINITY;
+        uint32_t bk = 0xffffffffu;
+        if (!clear && sl < nc) {
+          bk = few_cand(e, sl);
+          const float* xp = x + (uint64_t)e.p * d;
+          const float* cp = c + (uint64_t)bk * d;
+          double s64 = 0.0;
+          for (uint32_t j = 0; j < d; ++j) {
+            const double t = __dsub_rn((double)__ldg(xp + j), (double)__ldg(cp + j));
+            s64 = __dadd_rn(s64, __dmul_rn(t, t));
+          }
+          best = s64;
+          if (best != best) best = INFINITY, bk = 0xffffffffu;  // NaN never wins
+        }
+#pragma unroll
+        for (int o = 4; o; o >>= 1) {
+          const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+          const uint32_t ok = __shfl_xor_sync(0xffffffffu, bk, o);
+          if (ob < best || (ob == best && ok < bk)) best = ob, bk = ok;
+        }
+        if (!clear && sl == 0) {
+          settle_put(assign, e.p, bk == 0xffffffffu ? 0u : bk, nchg, S);
+          if (B.ub) B.ub[e.p] = INFINITY;  // no bounds: the next round computes it again
+          ++settled;
+        }
+      }
+      if (clear && nc && sl == 0) {
+        settle_put(assign, e.p, k1, nchg, S);
+        if (B.ub) {  // the distance pass left the bound of the other centroids
+          const float l = B.lb[e.p];
+          km_put_bounds(B, e.p, B.drift[k1], *B.far, m1 * widen + 1e-36f,
+                        fminf(m2 * (2.f - widen) - 1e-36f, l * l * 0.999999f));
+        }
+      }
+    }
+  }
+  for (uint64_t b = blockIdx.x; b < rb; b += gridDim.x) {
     __syncthreads();  // the previous batch's shared arrays are no longer read
     if (threadIdx.x == 0) S.nopen = 0;
-    if (b < rb) {
+    {
       const uint32_t f0 = (uint32_t)b * SET_RP;
       const uint32_t cnt = nf - f0 < (uint32_t)SET_RP ? nf - f0 : (uint32_t)SET_RP;
       for (uint32_t r = warp; r < (uint32_t)SET_RP; r += nw) {
@@ -646,39 +712,22 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
           else m2 = min(m2, o1);
         }
         const uint32_t p = list[f0 + r];
-        if (__uint_as_float(m2) > __uint_as_float(m1) * widen) settle_put(assign, p, k1, nchg, S);
-        else S.open[atomicAdd(&S.nopen, 1u)] = p;
-      }
-    } else {
-      __syncthreads();
-      const uint64_t f = (b - rb) * ppb + (threadIdx.x >> 3);
-      const uint32_t sl = threadIdx.x & 7;
-      const bool live = f < np;
-      const KmFew e = live ? pairs[f] : KmFew{0, 0, 0};
-      const uint32_t nc = live ? e.hi >> 28 : 0;
-      float fd[KM_CAND_MAX];
-      if (__any_sync(0xffffffffu, nc > 2)) few_dists<KM_CAND_MAX>(x, c, d, e, nc, sl, vec, fd);
-      else few_dists<2>(x, c, d, e, nc, sl, vec, fd);
-      float m1 = INFINITY, m2 = INFINITY;
-      uint32_t k1 = 0;
-#pragma unroll
-      for (uint32_t i = 0; i < KM_CAND_MAX; ++i)
-        if (i < nc) {
-          if (fd[i] < m1) m2 = m1, m1 = fd[i], k1 = few_cand(e, i);
-          else if (!(fd[i] >= m2)) m2 = fd[i];  // (a NaN makes m2 NaN: the point is left to FP64)
+        if (__uint_as_float(m2) > __uint_as_float(m1) * widen) {
+          settle_put(assign, p, k1, nchg, S);
+          if (B.ub) km_put_bounds(B, p, B.drift[k1], *B.far, __uint_as_float(m1) * widen + 1e-36f, __uint_as_float(m2) * (2.f - widen) - 1e-36f);
+        } else {
+          S.open[atomicAdd(&S.nopen, 1u)] = p;
         }
-      if (live && sl == 0) {
-        if (m2 > m1 * widen) settle_put(assign, e.p, k1, nchg, S);
-        else S.open[atomicAdd(&S.nopen, 1u)] = e.p;
       }
     }
     __syncthreads();
     const uint32_t no = S.nopen;
+    if (B.ub && threadIdx.x < no) B.ub[S.open[threadIdx.x]] = INFINITY;  // no bounds: the next round computes it again
     for (uint32_t i = 0; i < no; ++i) settle_fp64(x, d, c, ct, k, S.open[i], assign, nchg, prod, xs, dist, cand, S);
-    settled += no;
+    if (threadIdx.x == 0) settled += no;
   }
+  if (settled) atomicAdd(stat + 1, settled);
   __syncthreads();
-  if (threadIdx.x == 0 && settled) atomicAdd(stat + 1, settled);
   if (threadIdx.x == 0 && S.moved) atomicAdd(nchg, S.moved);
 }
 
@@ -1431,7 +1480,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) km_window_sum_kernel(const floa
 // c_k), and what the next distance pass and re-check need of them: the shifted
 // norm cn[k] = ||c_k - center||^2 (FP32 FMAs; center null: no shift), the
 // largest norm, the transposed copy ct, the wide pass's operands bop (null:
-// none) and cleared counters.  first: only the
+// none), each centroid's drift so far and the largest of the round (drift null:
+// not kept) and cleared counters.  first: only the
 // latter, for the initial centroids.
 constexpr int RF_THREADS = 256;
 __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long* __restrict__ part, uint32_t g,
@@ -1443,6 +1493,7 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
                                                                  const float* __restrict__ center,
                                                                  float* __restrict__ cn, unsigned int* cmax,
                                                                  float* __restrict__ ct, uint8_t* bop,
+                                                                 float* drift, unsigned int* maxdrift,
                                                                  uint32_t* nflag, uint32_t first) {
   pdl_wait();
   __shared__ long long red[RF_THREADS / 32][32];
@@ -1451,7 +1502,7 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
   const bool full = !km_by_changes(chg, lim);
   const unsigned long long cnt = first ? 0 : full ? cnew[kk] : counts[kk];
   const double inv = cnt ? ldexp(1.0, -*shift) : 0.0;
-  float nrm = 0.f;
+  float nrm = 0.f, moved2 = 0.f;
   __syncthreads();  // every thread has read the count that is cleared below
   for (uint32_t j0 = 0; j0 < d; j0 += 32) {
     const uint32_t j = j0 + lane;
@@ -1475,8 +1526,10 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
       } else if (cnt) {
         a = sums[row + j];
       }
-      const float v = cnt ? (float)(((double)a * inv) / (double)cnt) : c[row + j];
+      const float was = c[row + j];
+      const float v = cnt ? (float)(((double)a * inv) / (double)cnt) : was;
       if (cnt) c[row + j] = v;
+      moved2 = fmaf(v - was, v - was, moved2) + (v != was ? 1e-36f : 0.f);  // (tiny squares are flushed)
       ct[(uint64_t)j * k + kk] = v;
       const float t = center ? __fsub_rn(v, center[j]) : v;
       nrm = fmaf(t, t, nrm);
@@ -1484,9 +1537,17 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
     }
   }
   if (w == 0) {
-    for (int o = 16; o; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+    for (int o = 16; o; o >>= 1) {
+      nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+      moved2 += __shfl_xor_sync(0xffffffffu, moved2, o);
+    }
     if (lane == 0) {
       cn[kk] = nrm;
+      if (drift) {
+        const float dr = __fmul_ru(__fsqrt_ru(moved2), 1.0001f);  // (the sum's relative error is below 1e-5 at D <= 64)
+        drift[kk] = first ? 0.f : __fadd_ru(drift[kk], dr);
+        if (!first) atomicMax(maxdrift, __float_as_uint(dr));
+      }
       atomicMax(cmax, __float_as_uint(sqrtf(nrm)));
       if (full) counts[kk] = cnt;
       cnew[kk] = 0;
@@ -1495,6 +1556,124 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
         *chg_next = 0;
       }
     }
+  }
+}
+
+// ------------------------------------------------------------- the filter
+// After the first rounds most points cannot change cluster (on a mixture of
+// 256 Gaussians in 64 dimensions, K = 256: 82, 75, 40, 25, 15, 14, 13, 11, 12%
+// of the points could in rounds 2 to 10), and the triangle inequality tells
+// which without computing a distance (Hamerly, "Making k-means even faster",
+// 2010): with ub >= the distance to the own centroid a and lb <= the distance
+// to every other one, both moved along by the centroids' drifts, the point
+// keeps a if ub < lb, or if ub < half the distance from a to the nearest other
+// centroid.  Bounds come from the distance and settle passes with their error
+// bounds added, are stored relative to the drifts so far (so a skipped point
+// writes nothing) and are compared with more slack than all roundings, so a
+// skipped point's assignment is the FP64 definition's, by a relative margin of
+// 1e-5.  The listed points go through the distance pass by index.
+//
+// km_half_kernel: half[k], one CTA per centroid, one thread per other centroid;
+// and the largest drift of the round added to the sum of them.
+constexpr int HALF_THREADS = 256;
+__global__ void __launch_bounds__(HALF_THREADS) km_half_kernel(const float* __restrict__ c,
+                                                               const float* __restrict__ ct, uint32_t k, uint32_t d,
+                                                               float* __restrict__ half, unsigned int* maxdrift,
+                                                               float* far, uint32_t* nact) {
+  pdl_wait();
+  __shared__ float own[64], red[HALF_THREADS / 32];
+  const uint32_t i = blockIdx.x;
+  if (i == 0 && threadIdx.x == 0) {
+    *far = __fadd_ru(*far, __uint_as_float(*maxdrift));
+    *maxdrift = 0;
+    *nact = 0;
+  }
+  for (uint32_t t = threadIdx.x; t < d; t += HALF_THREADS) own[t] = c[(uint64_t)i * d + t];
+  __syncthreads();
+  float best = INFINITY;
+  for (uint32_t j = threadIdx.x; j < k; j += HALF_THREADS) {
+    float s = 0.f;
+#pragma unroll 16
+    for (uint32_t t = 0; t < d; ++t) {
+      const float v = __ldg(ct + (uint64_t)t * k + j) - own[t];
+      s = fmaf(v, v, s);
+    }
+    if (j != i) best = s != s ? 0.f : fminf(best, s);  // (NaN: no bound; no thread has two centroids at K <= 256)
+  }
+  for (int o = 16; o; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < HALF_THREADS / 32; ++w) best = fminf(best, red[w]);
+    half[i] = 0.5f * __fsqrt_rd(best) * 0.9999f;
+  }
+}
+// Bound by the 12 bytes a point it reads (4M points: 14 us).
+constexpr int FI_THREADS = 1024;
+__global__ void __launch_bounds__(FI_THREADS) km_filter_kernel(const uint32_t* __restrict__ assign, uint32_t n,
+                                                               uint32_t k, KmBounds B, const float* __restrict__ half,
+                                                               uint32_t* __restrict__ act, uint32_t* nact) {
+  pdl_wait();
+  __shared__ float s_drift[256], s_half[256];
+  __shared__ uint32_t wcnt[FI_THREADS / 32], s_base;
+  for (uint32_t i = threadIdx.x; i < k; i += FI_THREADS) s_drift[i] = B.drift[i], s_half[i] = half[i];
+  const float far = *B.far;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (uint64_t b = (uint64_t)blockIdx.x * FI_THREADS * 4; b < n; b += (uint64_t)gridDim.x * FI_THREADS * 4) {
+    const uint64_t i0 = b + 4 * threadIdx.x;  // four consecutive points per thread
+    uint32_t w[4];
+    float u[4], l[4];
+    if (i0 + 4 <= n) {
+      const uint4 v = *reinterpret_cast<const uint4*>(assign + i0);
+      const float4 uv = *reinterpret_cast<const float4*>(B.ub + i0), lv = *reinterpret_cast<const float4*>(B.lb + i0);
+      w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+      u[0] = uv.x, u[1] = uv.y, u[2] = uv.z, u[3] = uv.w;
+      l[0] = lv.x, l[1] = lv.y, l[2] = lv.z, l[3] = lv.w;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const bool in = i0 + q < n;
+        w[q] = in ? assign[i0 + q] : 0u;
+        u[q] = in ? B.ub[i0 + q] : 0.f;
+        l[q] = in ? B.lb[i0 + q] : 0.f;
+      }
+    }
+    __syncthreads();  // the drifts are loaded; the previous batch's counts have been read
+    uint32_t on = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t a = km_now(w[q], k);
+      const float dr = s_drift[a];
+      // 2.4e-7: two roundings of each sum
+      const float ub = u[q] + dr + 2.4e-7f * (fabsf(u[q]) + dr);
+      const float lb = l[q] - far - 2.4e-7f * (fabsf(l[q]) + far);
+      if (i0 + q < n && !(ub * 1.00001f < fmaxf(lb, s_half[a]))) on |= 1u << q;
+    }
+    const uint32_t c = __popc(on);
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) wcnt[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+      const uint32_t t = wcnt[lane];
+      uint32_t ti = t;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, ti, o);
+        if (lane >= o) ti += v;
+      }
+      wcnt[lane] = ti - t;
+      if (lane == 31) s_base = ti ? atomicAdd(nact, ti) : 0u;
+    }
+    __syncthreads();
+    uint32_t at = s_base + wcnt[warp] + incl - c;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (on >> q & 1) act[at++] = (uint32_t)(i0 + q);
   }
 }
 
@@ -1530,7 +1709,7 @@ inline uint64_t a256(uint64_t x) { return (x + 255) & ~255ull; }
 
 }  // namespace
 
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide) {
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool bounds) {
   uint64_t b = 0;
   b += a256((uint64_t)k * d * 4);      // cent
   b += a256((uint64_t)n * 4 + 16);     // assign (+16: the update copies ids in 16-byte units)
@@ -1545,10 +1724,11 @@ size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide) {
   b += a256((uint64_t)k * 4);          // per-cluster write cursor
   if (local_sums_fit(d, k)) b += a256((uint64_t)LS_MAX_CTAS * k * d * 8);  // per-CTA partial sums
   if (wide) b += a256(km_wide_operand_bytes(d, k));
+  if (bounds) b += 3 * a256((uint64_t)n * 4) + 2 * a256((uint64_t)k * 4);
   return (size_t)b;
 }
 
-cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide) {
+cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide, bool bounds) {
   const uint64_t n = b.n, d = b.d, k = b.k;
   uint8_t* q = p;
   auto take = [&](uint64_t sz) { uint8_t* r = q; q += a256(sz); return r; };
@@ -1558,7 +1738,7 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide) {
   b.counts = reinterpret_cast<unsigned long long*>(take(k * 8 * 2));
   uint8_t* ctl = take(256);
   b.stats = reinterpret_cast<unsigned long long*>(ctl);
-  b.nflag = reinterpret_cast<uint32_t*>(ctl + 64);
+  b.nflag = reinterpret_cast<uint32_t*>(ctl + 64);  // 24 words are cleared: to ctl + 160
   b.maxabs = reinterpret_cast<unsigned int*>(b.nflag + 2);
   b.shift = reinterpret_cast<int*>(ctl + 128);
   b.flagged = reinterpret_cast<uint32_t*>(take(n * 4));
@@ -1569,15 +1749,30 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide) {
   b.kcursor = reinterpret_cast<uint32_t*>(take(k * 4));
   b.part = local_sums_fit(d, k) ? reinterpret_cast<long long*>(take((uint64_t)LS_MAX_CTAS * k * d * 8)) : nullptr;
   b.bop = wide ? take(km_wide_operand_bytes((uint32_t)d, (uint32_t)k)) : nullptr;
+  if (bounds) {
+    b.bounds.ub = reinterpret_cast<float*>(take(n * 4));
+    b.bounds.lb = reinterpret_cast<float*>(take(n * 4));
+    b.act = reinterpret_cast<uint32_t*>(take(n * 4));
+    b.bounds.drift = reinterpret_cast<float*>(take(k * 4));
+    b.half = reinterpret_cast<float*>(take(k * 4));
+    b.bounds.far = reinterpret_cast<float*>(ctl + 136);
+  }
   if ((uint64_t)(q - p) > bytes) return cudaErrorInvalidValue;
   return cudaSuccess;
 }
 
-bool km_tc_supported(uint32_t d, uint32_t k);
+// The filter pays for its two kernels (15 us a round at 4M points) and its
+// memory where the distance pass takes well over that: from 2^27 distances
+// (60 us) on, and when there are rounds to skip points in.
+bool km_bounds_pay(uint32_t n, uint32_t d, uint32_t k, uint32_t iters) {
+  (void)d;
+  return (uint64_t)n * ((k + 15) & ~15u) >= 1ull << 27 && iters >= 3;
+}
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                     KmBuffers& b, const unsigned int* cmax, uint32_t* nchg, const DevInfo& di,
-                                    cudaStream_t s, uint64_t* nk, bool maxabs);
+                                    cudaStream_t s, uint64_t* nk, bool maxabs, const uint32_t* act,
+                                    const uint32_t* nact);
 
 cudaError_t launch_kmeans_wide_assign(const float* x, uint32_t n, uint32_t d, uint32_t k, KmBuffers& b,
                                       const unsigned int* cmax, uint32_t* nchg, const DevInfo& di, cudaStream_t s,
@@ -1671,6 +1866,12 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   }
   // rows and dimensions past K and D stay zero
   if (wide && (e = cudaMemsetAsync(b.bop, 0, km_wide_operand_bytes(d, k), s)) != cudaSuccess) return e;
+  const bool filter = tc && b.bounds.ub;
+  float* drift = filter ? const_cast<float*>(b.bounds.drift) : nullptr;
+  unsigned int* maxdrift = reinterpret_cast<unsigned int*>(shift) + 1;
+  float* far = reinterpret_cast<float*>(shift) + 2;
+  uint32_t* nact = b.nflag + 8;
+  const KmBounds bounds = filter ? b.bounds : KmBounds{};
   const float* center = tc || wide ? b.center : nullptr;
   const uint32_t lim = n / (local ? KM_DELTA_LOCAL : KM_DELTA_SORTED);  // points moved, at most, in an update by changes
   auto chg_of = [&](uint32_t it) { return b.nflag + ((it & 1) ? 5 : 0); };  // points that changed cluster in the round
@@ -1680,8 +1881,8 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
                       local ? (const long long*)b.part : (const long long*)nullptr, ls_grid, b.sums, b.cent, k, d,
                       b.counts, b.counts + k, it > 1 ? (const uint32_t*)chg_of(it - 1) : (const uint32_t*)nullptr, lim,
                       chg_of(it),
-                      (const int*)shift, center, b.cnorm, cmax_of(it), b.ct, wide ? b.bop : (uint8_t*)nullptr, b.nflag,
-                      first ? 1u : 0u);
+                      (const int*)shift, center, b.cnorm, cmax_of(it), b.ct, wide ? b.bop : (uint8_t*)nullptr, drift,
+                      maxdrift, b.nflag, first ? 1u : 0u);
   };
   if ((e = finalize(0, true)) != cudaSuccess) return e;
   unsigned long long* cnew = b.counts + k;
@@ -1690,7 +1891,19 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
     // kernels that follow another kernel of this job on the stream start
     // while it drains (programmatic dependent launch; each waits first)
     if (tc) {
-      if ((e = launch_kmeans_tc_assign(x, n, d, b.cent, k, b, cmax_of(it), chg, di, s, nk, it == 0)) != cudaSuccess)
+      const bool skip = filter && it > 0;
+      if (skip) {
+        const uint64_t fb = ((uint64_t)n + FI_THREADS * 4 - 1) / (FI_THREADS * 4);
+        if ((e = launch_pdl(km_half_kernel, dim3(k), dim3(HALF_THREADS), 0, s, (const float*)b.cent,
+                            (const float*)b.ct, k, d, b.half, maxdrift, far, nact)) != cudaSuccess ||
+            (e = launch_pdl(km_filter_kernel, dim3((unsigned)(fb < 2ull * di.sms ? fb : 2ull * di.sms)),
+                            dim3(FI_THREADS), 0, s, (const uint32_t*)b.assign, n, k, bounds, (const float*)b.half,
+                            b.act, nact)) != cudaSuccess)
+          return e;
+        *nk += 2;
+      }
+      if ((e = launch_kmeans_tc_assign(x, n, d, b.cent, k, b, cmax_of(it), chg, di, s, nk, it == 0,
+                                       skip ? b.act : nullptr, nact)) != cudaSuccess)
         return e;
     } else if (wide) {
       if ((e = launch_kmeans_wide_assign(x, n, d, k, b, cmax_of(it), chg, di, s, nk, it == 0)) != cudaSuccess)
@@ -1706,7 +1919,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
                         n, d, (const float*)b.cent, (const float*)b.ct, k, (const KmFew*)b.pairs,
                         (const uint32_t*)(b.nflag + 4), (const uint32_t*)b.flagged, (const uint32_t*)(b.nflag + 1),
                         b.assign, chg, b.stats, it == 0 ? (const unsigned int*)b.maxabs : (const unsigned int*)nullptr,
-                        shift, cmax_of(it + 1))) != cudaSuccess)
+                        shift, cmax_of(it + 1), bounds)) != cudaSuccess)
       return e;
     ++*nk;
     if (local) {  // update with local arrays

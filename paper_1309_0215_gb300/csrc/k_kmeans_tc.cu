@@ -23,9 +23,12 @@
 //     with its column into one sortable 32-bit key and keep the two smallest
 //     keys with signed min/max (four independent top-2s per thread) plus
 //     a lower bound of all other keys, and hand them to
-//   * 2 finalizer warps (two lane quadrants each), which merge the four
+//   * 4 finalizer warps (one lane quadrant each), which merge the four
 //     column quarters of each point and apply the margin tests below, so
 //     that no epilogue warp carries the per-point tail on its own path.
+//     (Per tile a finalizer waits for one list reservation and writes scattered
+//     words and bounds; with two warps, two quadrants each, they set the pace:
+//     the pass over 3.3M of 4M listed points took 977 us, with four 515.)
 // Copies, converters, MMA issue, epilogue and finalizers overlap through the
 // staging ring, two operand stages, two TMEM accumulators and two hand-off
 // buffers.  Every mbarrier wait is bounded; on timeout the
@@ -67,13 +70,15 @@ constexpr int CVT_WARP0 = MMA_WARP + 1;
 constexpr int CVT_WARPS = 8;      // each converts TM / CVT_WARPS rows of a tile
 constexpr int CVT_ROWS = TM / CVT_WARPS;
 constexpr int FIN_WARP0 = CVT_WARP0 + CVT_WARPS;
-constexpr int FIN_WARPS = 2;      // each finalizes 4 / FIN_WARPS TMEM lane quadrants (32 points each)
+constexpr int FIN_WARPS = 4;      // each finalizes 4 / FIN_WARPS TMEM lane quadrants (32 points each)
 constexpr int FIN_QUADS = 4 / FIN_WARPS;
-constexpr int TMA_WARP = FIN_WARP0 + FIN_WARPS;  // 27
-constexpr int TC_THREADS = (EPI_WARPS + 1 + CVT_WARPS + FIN_WARPS + 1) * 32;  // 896
+constexpr int TMA_WARP = FIN_WARP0 + FIN_WARPS;  // 29
+constexpr int TC_THREADS = (EPI_WARPS + 1 + CVT_WARPS + FIN_WARPS + 1) * 32;  // 960
 static_assert(CVT_ROWS % 16 == 0 && 4 % FIN_WARPS == 0, "converter rows and finalizer quadrants");
 constexpr int STAGES = 2;         // operand stages
 constexpr int XST = 2;            // FP32 staging buffers filled by the bulk copy engine
+constexpr uint32_t BEYOND = 0xFFFFFFFFu;  // no point (n < 2^31)
+constexpr uint32_t LISTED = 0xFFu;        // (number of candidates) too many: every centroid
 constexpr int ACCS = 2;           // TMEM accumulators
 constexpr uint32_t TMEM_COLS = 512;  // two 256-column FP32 accumulators
 struct __align__(1024) TcSmem {
@@ -84,6 +89,7 @@ struct __align__(1024) TcSmem {
   float xs[XST][TM * KD];             // FP32 point tiles (D == 64 path)
   float nx[STAGES][TM];
   float cn[NMAX];
+  float drift[NMAX];                  // (bounds) the centroids' drifts so far
   // per column quarter and row: top-2 keys and the lower bound of the
   // other keys; and the row's ||x||^2 (epilogue -> finalizers)
   uint32_t xw1[ACCS][QUARTERS][TM], xw2[ACCS][QUARTERS][TM], xlb[ACCS][QUARTERS][TM];
@@ -100,16 +106,15 @@ static_assert(sizeof(TcSmem) + 1024 <= 232448, "shared memory of one CTA");
 
 template <int TERMS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const float* __restrict__ c, uint32_t k,
+km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, const float* __restrict__ c, uint32_t k,
                     const float* __restrict__ center, const float* __restrict__ cnorm, const unsigned int* cmax_bits, uint32_t* __restrict__ assign, uint32_t* nchg,
                     uint32_t* __restrict__ list, uint32_t* nlist, KmFew* __restrict__ pairs, uint32_t* npairs,
                     unsigned long long* timeouts, float* dbg, long long polls, uint32_t stop_copies,
-                    unsigned int* maxabs) {
+                    unsigned int* maxabs, const uint32_t* __restrict__ act, const uint32_t* nact, KmBounds B) {
   extern __shared__ uint8_t tc_raw[];
   TcSmem& S = *reinterpret_cast<TcSmem*>((reinterpret_cast<uintptr_t>(tc_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t npad = (k + 15) & ~15u;
-  const uint32_t ntiles = (n + TM - 1) / TM;
   volatile int* err = &S.err;
 
   if (threadIdx.x == 0) {
@@ -125,12 +130,8 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
       mbar_init(&S.xfull[b], EPI_WARPS);
       mbar_init(&S.xfree[b], FIN_WARPS);
     }
-    for (int q = 0; q < XST; ++q) {
-      mbar_init(&S.tfull[q], 1);
-      mbar_init(&S.tempty[q], CVT_WARPS);
-    }
+    for (int q = 0; q < XST; ++q) mbar_init(&S.tempty[q], CVT_WARPS);
     mbar_init(&S.drained, 1);
-    fence_mbar_init();
   }
   if (warp == MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&S.tmem_base)),
@@ -140,6 +141,15 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
   }
   // everything read from here on was written by earlier kernels of the job
   pdl_wait();
+  // the points: all of them, or those the filter listed (unless that is nearly all)
+  const uint32_t* idx = act && km_use_list(*nact, n_all) ? act : nullptr;
+  const uint32_t n = idx ? *nact : n_all;
+  const uint32_t ntiles = (n + TM - 1) / TM;
+  if (threadIdx.x == 0) {
+    // a tile's copy arrives once, a listed tile's rows once per lane of the copying warp
+    for (int q = 0; q < XST; ++q) mbar_init(&S.tfull[q], idx ? 32 : 1);
+    fence_mbar_init();
+  }
   // centroid operands (rows >= k and dims >= d are zero) and norms
   for (uint32_t t = threadIdx.x; t < npad * (KD / 2); t += blockDim.x) {
     const uint32_t row = t / (KD / 2), pr = t % (KD / 2);
@@ -156,7 +166,10 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
     *reinterpret_cast<uint32_t*>(S.b_lo + off) = lo;
   }
   // padded centroid columns get an infinite norm, so they never win
-  for (uint32_t t = threadIdx.x; t < NMAX; t += blockDim.x) S.cn[t] = t < k ? cnorm[t] : INFINITY;
+  for (uint32_t t = threadIdx.x; t < NMAX; t += blockDim.x) {
+    S.cn[t] = t < k ? cnorm[t] : INFINITY;
+    S.drift[t] = B.ub && t < k ? B.drift[t] : 0.f;
+  }
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
@@ -205,7 +218,7 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
           for (int q = 0; q < 8; ++q) {
             const uint32_t p = tile * TM + r0 + 2 * q + rsub;
             const uint32_t d0 = 4 * col;
-            const float* row = x + (uint64_t)p * d;
+            const float* row = x + (uint64_t)(idx && p < n ? idx[p] : p) * d;
             v[q].x = (p < n && d0 < d) ? row[d0] : 0.f;
             v[q].y = (p < n && d0 + 1 < d) ? row[d0 + 1] : 0.f;
             v[q].z = (p < n && d0 + 2 < d) ? row[d0 + 2] : 0.f;
@@ -260,25 +273,55 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
     }
   } else if (warp == TMA_WARP) {
     // ------------------------------------------------- bulk-copy producer
-    if (lane == 0 && d == KD && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
+    // One bulk copy per tile; listed rows by 16-byte asynchronous copies, two
+    // rows per warp instruction (one bulk copy per row took 75 cycles of the
+    // copy engine each: 817 us for
+    // 3.3M listed points when the finalizers were not yet the limit).
+    if (d == KD && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
       uint32_t issued = 0;
       for (uint32_t i = 0;; ++i) {
         const uint32_t tile = blockIdx.x + i * gridDim.x;
         if (tile >= ntiles || (stop_copies && i >= stop_copies)) break;
         const int q2 = (int)(i % XST);
-        if (i >= XST && !mbar_wait(&S.tempty[q2], ((i / XST) + 1) & 1, err, polls)) break;
         const uint32_t rows = (n - tile * TM) < (uint32_t)TM ? (n - tile * TM) : (uint32_t)TM;
-        const uint32_t bytes = rows * KD * 4;
-        mbar_expect_tx(&S.tfull[q2], bytes);
-        bulk_g2s(S.xs[q2], x + (uint64_t)tile * TM * KD, bytes, &S.tfull[q2]);
+        uint32_t row[TM / 32];
+        if (idx) {
+#pragma unroll
+          for (int q = 0; q < TM / 32; ++q) row[q] = q * 32 + lane < (int)rows ? idx[tile * TM + q * 32 + lane] : 0;
+        }
+        bool ok = true;
+        if (lane == 0) {
+          ok = i < XST || mbar_wait(&S.tempty[q2], ((i / XST) + 1) & 1, err, polls);
+          if (ok && !idx) {
+            mbar_expect_tx(&S.tfull[q2], rows * KD * 4);
+            bulk_g2s(S.xs[q2], x + (uint64_t)tile * TM * KD, rows * KD * 4, &S.tfull[q2]);
+          }
+        }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (idx) {
+          const uint32_t half = (uint32_t)lane >> 4, part = (uint32_t)lane & 15;
+#pragma unroll
+          for (int q = 0; q < TM / 32; ++q)
+#pragma unroll 4
+            for (int t = 0; t < 16; ++t) {
+              const uint32_t rr = q * 32 + 2 * t + half;
+              const uint32_t r = __shfl_sync(0xffffffffu, row[q], 2 * t + half);
+              if (rr < rows) cp_async16(S.xs[q2] + rr * KD + 4 * part, x + (uint64_t)r * KD + 4 * part);
+            }
+          cp_async_arrive(&S.tfull[q2]);
+        }
         ++issued;
       }
       // No copy may still be landing in shared memory when the CTA exits.
       // Copy i was issued only after the converters released copy i - XST
       // (which they do after its completion), so only the last XST copies
       // can be in flight; wait for them even when a wait gave up elsewhere.
-      for (uint32_t i = issued > (uint32_t)XST ? issued - XST : 0; i < issued; ++i)
-        mbar_drain(&S.tfull[i % XST], (i / XST) & 1);
+      if (idx) cp_async_wait_all();
+      __syncwarp();
+      if (lane == 0 && !idx)
+        for (uint32_t i = issued > (uint32_t)XST ? issued - XST : 0; i < issued; ++i)
+          mbar_drain(&S.tfull[i % XST], (i / XST) & 1);
     }
     __syncwarp();
   } else if (warp == MMA_WARP) {
@@ -316,9 +359,10 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
       // operand buffers go away with the CTA): the commit arrives once every
       // MMA issued above has completed, and that is waited for even when a
       // wait gave up elsewhere.
-      mma_commit(&S.drained);
-      mbar_drain(&S.drained, 0);
-      (void)issued;
+      if (issued) {
+        mma_commit(&S.drained);
+        mbar_drain(&S.drained, 0);
+      }
     }
     __syncwarp();
   } else if (warp >= FIN_WARP0 && warp < FIN_WARP0 + FIN_WARPS) {
@@ -331,17 +375,29 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
                                      : (2.f * 3.90625e-03f + 1.52587890625e-05f + (float)(KD + 8) * 4.76837158203125e-07f);
     const float eps32 = 1.01f * (float)(d + 12) * 5.9604644775390625e-08f;
     uint32_t moved = 0;  // this lane's points that changed cluster
+    const float far = B.ub ? *B.far : 0.f;
+    // the points of the next two tiles and the words of the next one, so that no
+    // load waits for another
+    uint32_t p[FIN_QUADS], word[FIN_QUADS], p1[FIN_QUADS], word1[FIN_QUADS], p2[FIN_QUADS];
+    auto load_points = [&](uint32_t tile, uint32_t (&to)[FIN_QUADS]) {
+#pragma unroll
+      for (int h = 0; h < FIN_QUADS; ++h) {
+        const uint32_t r = tile * TM + (uint32_t)((fw * FIN_QUADS + h) * 32 + lane);
+        to[h] = tile >= ntiles || r >= n ? BEYOND : idx ? idx[r] : r;
+      }
+    };
+    auto load_words = [&](const uint32_t (&of)[FIN_QUADS], uint32_t (&to)[FIN_QUADS]) {
+#pragma unroll
+      for (int h = 0; h < FIN_QUADS; ++h) to[h] = nchg && of[h] != BEYOND ? assign[of[h]] : 0u;
+    };
+    load_points(blockIdx.x, p1);
+    load_points(blockIdx.x + gridDim.x, p2);
+    load_words(p1, word1);
     for (uint32_t i = 0;; ++i) {
       const uint32_t tile = blockIdx.x + i * gridDim.x;
       if (tile >= ntiles) break;
       const int b = (int)(i & 1);
       const uint32_t v = i >> 1;
-      uint32_t was[FIN_QUADS];  // the points' words, loaded while the tile is in the pipeline
-#pragma unroll
-      for (int h = 0; h < FIN_QUADS; ++h) {
-        const uint32_t p = tile * TM + (uint32_t)((fw * FIN_QUADS + h) * 32 + lane);
-        was[h] = nchg && p < n ? assign[p] & 0xffffu : 0u;
-      }
       const bool okx = mbar_wait(&S.xfull[b], v & 1, err, polls);
       if (!__all_sync(0xffffffffu, okx)) break;
       int o1[FIN_QUADS][QUARTERS], o2[FIN_QUADS][QUARTERS], ol[FIN_QUADS][QUARTERS];
@@ -359,52 +415,83 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, const f
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.xfree[b]);
+      uint32_t ncand[FIN_QUADS];
+      uint64_t cand[FIN_QUADS];
+#pragma unroll
+      for (int h = 0; h < FIN_QUADS; ++h) p[h] = p1[h], word[h] = word1[h], p1[h] = p2[h];
+      load_words(p1, word1);
+      load_points(tile + 2 * gridDim.x, p2);
 #pragma unroll
       for (int h = 0; h < FIN_QUADS; ++h) {
         int g1 = o1[h][0], g2 = o2[h][0];
 #pragma unroll
         for (int u = 1; u < QUARTERS; ++u) top2_merge(g1, g2, o1[h][u], o2[h][u]);
-        const uint32_t p = tile * TM + (uint32_t)((fw * FIN_QUADS + h) * 32 + lane);
-        bool flag = false, few = false;
-        uint64_t cand = 0;
-        uint32_t ncand = 0;
-        if (p < n) {
+        cand[h] = 0;
+        ncand[h] = 0;  // 0: decided; 2 .. KM_CAND_MAX: few; LISTED
+        if (p[h] != BEYOND) {
           const float d1 = key_dist(g1), d2 = key_dist(g2);
-          const float xn = sqrtf(nxv[h]);
+          const float xn = km_sqrt(nxv[h]) * 1.000001f;
           // (1e-36: the products of tiny values may be flushed to zero)
           const float e = 2.f * eps_sum * xn * cmax + eps32 * (xn + cmax) * (xn + cmax) + 1e-36f;
           // keys under-state a distance by less than 2^-15 of it (2^-14 allowed)
           const float gap = 2.f * e + 6.103515625e-05f * d1;
           const float lim = fmaxf(1e-3f * d1, gap);
           if (g1 < 0) {
-            flag = true;  // a negative smallest distance: re-check
+            ncand[h] = LISTED;  // a negative smallest distance: re-check
           } else if (d2 - d1 > lim) {
-            const uint32_t now = (uint32_t)g1 & 0xFFu;
-            const uint32_t old = nchg ? was[h] : now;
-            assign[p] = km_word(now, old);
-            moved += now != old;
+            const uint32_t now = (uint32_t)g1 & 0xFFu, o = nchg ? word[h] & 0xffffu : now;
+            assign[p[h]] = km_word(now, o);
+            moved += now != o;
+            if (B.ub) km_put_bounds(B, p[h], S.drift[now], far, fmaf(d1, 1.00006103515625f, e), d2 - e);
           } else {
             // candidates: the quarters' top-2 keys within the margin, if every
             // other key is beyond it
-            bool rest = false;
+            int rest = KEY_NONE;
+            uint32_t nc = 0;
 #pragma unroll
             for (int u = 0; u < QUARTERS; ++u) {
-              rest |= !(key_dist(ol[h][u]) - d1 > gap);
+              rest = min(rest, ol[h][u]);
 #pragma unroll
               for (int t = 0; t < 2; ++t) {
                 const int key = t ? o2[h][u] : o1[h][u];
                 if (key_dist(key) - d1 <= lim) {
-                  cand = (cand << 12) | ((uint32_t)key & 0xFFu);
-                  ++ncand;
+                  cand[h] = (cand[h] << 12) | ((uint32_t)key & 0xFFu);
+                  ++nc;
+                } else {
+                  rest = min(rest, key);
                 }
               }
             }
-            few = !rest && ncand >= 2 && ncand <= KM_CAND_MAX;
-            flag = !few;
+            const bool few = key_dist(rest) - d1 > gap && nc >= 2 && nc <= KM_CAND_MAX;
+            ncand[h] = few ? nc : LISTED;
+            // (the settle pass lowers it by the candidates' distances)
+            if (B.ub && few) B.lb[p[h]] = km_sqrt(fmaxf(key_dist(rest) - e, 0.f)) * 0.999999f;
           }
         }
-        warp_append(few, npairs, lane, [&](uint32_t at) { pairs[at] = km_few(p, cand, ncand); });
-        warp_append(flag, nlist, lane, [&](uint32_t at) { list[at] = p; });
+      }
+      // one reservation in each list for all of the warp's points, both at once
+      unsigned mf[FIN_QUADS], ml[FIN_QUADS];
+      uint32_t tf = 0, tl = 0;
+#pragma unroll
+      for (int h = 0; h < FIN_QUADS; ++h) {
+        mf[h] = __ballot_sync(0xffffffffu, ncand[h] != 0 && ncand[h] != LISTED);
+        ml[h] = __ballot_sync(0xffffffffu, ncand[h] == LISTED);
+        tf += __popc(mf[h]);
+        tl += __popc(ml[h]);
+      }
+      if (tf + tl) {
+        uint32_t base = 0;
+        if (lane == 0 && tf) base = atomicAdd(npairs, tf);
+        if (lane == 1 && tl) base = atomicAdd(nlist, tl);
+        uint32_t bf = __shfl_sync(0xffffffffu, base, 0), bl = __shfl_sync(0xffffffffu, base, 1);
+        const uint32_t below = (1u << lane) - 1;
+#pragma unroll
+        for (int h = 0; h < FIN_QUADS; ++h) {
+          if (mf[h] >> lane & 1) pairs[bf + __popc(mf[h] & below)] = km_few(p[h], cand[h], ncand[h]);
+          if (ml[h] >> lane & 1) list[bl + __popc(ml[h] & below)] = p[h];
+          bf += __popc(mf[h]);
+          bl += __popc(ml[h]);
+        }
       }
     }
     moved = __reduce_add_sync(0xffffffffu, moved);
@@ -483,12 +570,13 @@ size_t km_tc_smem_bytes() { return sizeof(TcSmem) + 1024; }
 
 // Raw launch: nchg (null in a job's first round, whose words hold nothing yet)
 // counts the points that changed cluster; list/nlist receive the points to re-check, pairs/npairs the
-// two-candidate points; maxabs (when not null) receives the bits of max |x|.
+// few-candidate points; act/nact (or null) name the points to take; maxabs (when not null) receives the bits of max |x|.
 cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                 const float* center, const float* cnorm, const unsigned int* cmax_bits,
                                 uint32_t* assign, uint32_t* nchg, uint32_t* list, uint32_t* nlist, KmFew* pairs, uint32_t* npairs, unsigned long long* timeouts,
                                 float* dbg, int grid, cudaStream_t s, long long polls, uint32_t stop_copies,
-                                unsigned int* maxabs) {
+                                unsigned int* maxabs, const uint32_t* act, const uint32_t* nact,
+                                const KmBounds& B) {
   const int smem = (int)km_tc_smem_bytes();
   cudaError_t e;
   if (terms == 3) {
@@ -497,20 +585,21 @@ cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t 
       return e;
     return launch_pdl(km_tc_assign_kernel<3>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
                       cnorm, cmax_bits, assign, nchg, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
-                      maxabs);
+                      maxabs, act, nact, B);
   } else {
     if ((e = cudaFuncSetAttribute(km_tc_assign_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
         cudaSuccess)
       return e;
     return launch_pdl(km_tc_assign_kernel<1>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
                       cnorm, cmax_bits, assign, nchg, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
-                      maxabs);
+                      maxabs, act, nact, B);
   }
 }
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                     KmBuffers& b, const unsigned int* cmax, uint32_t* nchg, const DevInfo& di,
-                                    cudaStream_t s, uint64_t* nk, bool maxabs) {
+                                    cudaStream_t s, uint64_t* nk, bool maxabs, const uint32_t* act,
+                                    const uint32_t* nact) {
   const uint32_t ntiles = (n + TM - 1) / TM;
   uint32_t grid = ntiles < (uint32_t)di.sms ? ntiles : (uint32_t)di.sms;
   if (b.grid_cap && grid > b.grid_cap) grid = b.grid_cap;
@@ -519,7 +608,7 @@ cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, cons
   if (e != cudaSuccess) return e;
   e = launch_km_tc_kernel(terms, x, n, d, c, k, b.center, b.cnorm, cmax, b.assign, nchg, b.flagged, b.nflag + 1,
                           b.pairs, b.nflag + 4, b.stats + 3, nullptr, (int)grid, s, b.polls < 0 ? SPIN_LIMIT : b.polls,
-                          b.stop_copies, maxabs ? b.maxabs : nullptr);
+                          b.stop_copies, maxabs ? b.maxabs : nullptr, act, nact, b.bounds);
   if (e != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;
   ++*nk;
   // the caller re-checks the pairs and the listed near ties

@@ -440,15 +440,16 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
       // result: centroids [K*D] f32 | assignments [N] i32 | pad to 8 | stats [4] u64
       const uint64_t res_bytes = km_stats_offset(K, D, N) + 32;
       const uint64_t res = align256(res_bytes);
-      // the wide tensor-core pass keeps its centroid operands in scratch; a
-      // budget that does not hold them leaves the job on the SIMT pass
+      // the wide tensor-core pass keeps its centroid operands in scratch, the
+      // filter its bounds; a context without room for them runs without
       bool wide = d.km_precision == MR_KM_FP32 && !km_tc_supported(D, K) && km_wide_supported(D, K);
-      uint64_t scr = align256(km_scratch_bytes(N, D, K, wide));
+      bool bounds = !c->budget && !wide && km_tc_supported(D, K) && km_bounds_pay(N, D, K, d.km_iters);
+      uint64_t scr = align256(km_scratch_bytes(N, D, K, wide, bounds));
       const uint64_t init_bytes = d.input_on_device ? 0 : align256((uint64_t)K * D * 4);
       mr_status st = dev_alloc(c, res + scr + init_bytes, &j->slab);
-      if (st == MR_EBUDGET && wide) {
-        wide = false;
-        scr = align256(km_scratch_bytes(N, D, K, false));
+      if ((st == MR_EBUDGET && wide) || (st == MR_ENOMEM && bounds)) {
+        wide = bounds = false;
+        scr = align256(km_scratch_bytes(N, D, K, false, false));
         st = dev_alloc(c, res + scr + init_bytes, &j->slab);
       }
       if (st) return st;
@@ -460,7 +461,7 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
       j->km.d = D;
       j->km.k = K;
       j->km.precision = (int)d.km_precision;
-      cudaError_t e = km_carve(j->km, p + res, scr, wide);
+      cudaError_t e = km_carve(j->km, p + res, scr, wide, bounds);
       if (e != cudaSuccess) {
         set_last_error("km_carve", e);
         return MR_EINVAL;

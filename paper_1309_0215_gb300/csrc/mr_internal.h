@@ -151,6 +151,14 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
+// Distance bounds that let later rounds skip points (see km_filter_kernel).
+struct KmBounds {
+  float* ub = nullptr;           // [n] upper bound on the distance to the own centroid, less that centroid's drift so far
+  float* lb = nullptr;           // [n] lower bound on the distance to any other, plus the largest drifts so far
+  const float* drift = nullptr;  // [k] each centroid's drift so far
+  const float* far = nullptr;    // [1] the sum of the rounds' largest drifts
+};
+
 // A point with 2 to KM_CAND_MAX candidate centroids, 12 bits each (K <= 4096),
 // and their number in the top bits.
 constexpr uint32_t KM_CAND_MAX = 5;
@@ -168,6 +176,19 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ uint32_t km_word(uint32_t now, uint32_t summed) { return now | (summed << 16); }
 // Both, for indexing: a word that a timed-out pass left unwritten counts as cluster 0.
 __device__ __forceinline__ uint32_t km_now(uint32_t w, uint32_t k) { return (w & 0xffffu) < k ? w & 0xffffu : 0u; }
+// Bounds of point p from squared distances: at most u2 to its centroid, whose
+// drift so far is given, at least l2 to every other (sqrt.approx and the sums
+// below are good to a few units in the last place, 1e-6 is eight).
+__device__ __forceinline__ float km_sqrt(float v) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ void km_put_bounds(const KmBounds& B, uint32_t p, float drift, float far, float u2,
+                                              float l2) {
+  B.ub[p] = fmaf(km_sqrt(u2), 1.000001f, -drift);
+  B.lb[p] = fmaf(km_sqrt(fmaxf(l2, 0.f)), 0.999999f, far);
+}
 __device__ __forceinline__ uint32_t km_summed(uint32_t w, uint32_t k) { return (w >> 16) < k ? w >> 16 : 0u; }
 #endif
 
@@ -187,6 +208,9 @@ struct KmBuffers {
   float* ct = nullptr;          // [d][k] transposed centroids
   unsigned int* maxabs = nullptr;  // [1] bits of max |x|
   int* shift = nullptr;         // [1] fixed-point scale exponent
+  KmBounds bounds;              // ub nullptr: not kept
+  float* half = nullptr;        // [k] half the distance to the nearest other centroid
+  uint32_t* act = nullptr;      // [n] points whose distances the round computes
   uint64_t* host = nullptr;     // pinned host word for the count of timed-out waits, written by the last kernel (or null)
   uint8_t* bop = nullptr;       // centroid operands of the wide tensor-core pass (nullptr: not taken)
   uint32_t* kcursor = nullptr;  // [k] counting-sort write cursors
@@ -200,9 +224,10 @@ struct KmBuffers {
   uint32_t grid_cap = 0;
   uint32_t stop_copies = 0;
 };
-// wide: with the wide tensor-core pass's operands
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide);
-cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes, bool wide);
+// wide: with the wide tensor-core pass's operands; bounds: with the points' bounds
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool bounds);
+bool km_bounds_pay(uint32_t n, uint32_t d, uint32_t k, uint32_t iters);
+cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes, bool wide, bool bounds);
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,
                           cudaStream_t s, float* out_cent, int32_t* out_assign, unsigned long long* out_stats,
                           uint64_t* nk);

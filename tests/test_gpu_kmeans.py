@@ -377,3 +377,23 @@ def test_kmeans_wide_tensor_core_pass(mr, n, d, k, cap, offset):
         assert int(st[3]) == 0
         cur = c_ref
     ctx.close()
+
+
+@pytest.mark.parametrize("n,d,k,comps,sigma", [
+    (600_011, 64, 256, 256, 1.0),    # listed rows copied by the bulk copy engine; most points skipped
+    (600_011, 64, 256, 8, 4.0),      # overlapping clusters: few points skipped
+    (2_000_003, 21, 67, 40, 2.0),    # listed rows loaded by the converters
+    (1_100_001, 2, 130, 256, 1.0),   # many small clusters in the plane
+])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_kmeans_skipped_points(mr, n, d, k, comps, sigma, precision):
+    """Jobs large enough for the filter: nine rounds in one call equal nine
+    calls of one round (which compute every distance), byte for byte."""
+    x, _, _ = synth.kmeans_points(n, d, comps, seed=n + d, sigma=sigma)
+    dx = _dev(x)
+    cur = synth.kmeans_init(x, k, seed=n)
+    c9, a9, _ = mr.kmeans(dx, _dev(cur), 9, precision)
+    for _ in range(9):
+        cur, a, _ = mr.kmeans(dx, _dev(cur), 1, precision)
+    assert np.array_equal(a9, a)
+    assert np.array_equal(c9, cur)
