@@ -38,7 +38,7 @@
 // split leaves |x.c - (hi.hi + hi.lo + lo.hi)| <= 3.05 * 2^-16 ||x|| ||c||
 // (one value: |x - hi - lo| <= u_b^2 |x|; sums by Cauchy-Schwarz); a single
 // BF16 product leaves (2 u_b + u_b^2) ||x|| ||c||.  The tensor-core sum of the
-// exact BF16 products is charged (products + 8) * 2^-21 ||x|| ||c|| (four
+// exact BF16 products is charged (products + 8) * 2^-22 ||x|| ||c|| (four
 // times the round-to-nearest bound, allowing truncating adders), and the FP32
 // norms and the final fma/add (D + 8) * 2^-24 (||x|| + ||c||)^2 (Higham,
 // eq. 3.5).  Points and centroids are first shifted by the mean m of the
@@ -371,8 +371,8 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
     // 32 q + lane of each): it merges the four column quarters' top-2 keys
     // into the row's exact top-2 (g1, g2), then applies the margin tests.
     const int fw = warp - FIN_WARP0;
-    const float eps_sum = TERMS == 3 ? (3.05f * 1.52587890625e-05f + (float)(3 * KD + 8) * 4.76837158203125e-07f)
-                                     : (2.f * 3.90625e-03f + 1.52587890625e-05f + (float)(KD + 8) * 4.76837158203125e-07f);
+    const float eps_sum = TERMS == 3 ? (3.05f * 1.52587890625e-05f + (float)(3 * KD + 8) * 2.384185791015625e-07f)
+                                     : (2.f * 3.90625e-03f + 1.52587890625e-05f + (float)(KD + 8) * 2.384185791015625e-07f);
     const float eps32 = 1.01f * (float)(d + 12) * 5.9604644775390625e-08f;
     uint32_t moved = 0;  // this lane's points that changed cluster
     const float far = B.ub ? *B.far : 0.f;

@@ -302,7 +302,7 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
   } else if (warp >= FIN_WARP0 && warp < FIN_WARP0 + FIN_WARPS) {
     // ------------------------------------------------------------ finalizers
     const int fw = warp - FIN_WARP0;
-    const float eps_sum = 3.05f * 1.52587890625e-05f + (float)(3 * KD * dc + 8) * 4.76837158203125e-07f;
+    const float eps_sum = 3.05f * 1.52587890625e-05f + (float)(3 * KD * dc + 8) * 2.384185791015625e-07f;
     const float eps32 = 1.01f * (float)(d + 12) * 5.9604644775390625e-08f;
     uint32_t moved = 0;  // this lane's points that changed cluster
     uint32_t cc = 0;
