@@ -134,6 +134,387 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) wc_map_cta_kernel(JobDev J) {
 }
 
 
+// ------------------------------------------------------------- small texts
+// A text of up to 64 KiB is counted, ordered and written by one CTA in one
+// launch.  Through the passes for larger texts a 48 KB text took twelve
+// launches whose kernels, a few microseconds each, wait for one another
+// (65 us of GPU time, 26 us of launching); nothing of such a text needs more
+// than one SM's shared memory:
+//   * the whole text and its whitespace bitmap are staged (each thread 64 bytes);
+//   * the token starts are listed and threads take them in turn (a thread that
+//     took those of its own 64 bytes met the other lanes' bank on every access:
+//     24 us): length from the bitmap, hash over 4-byte words, then a
+//     shared-memory table of 4,096 slots.  A slot is one word, 15 bits of hash and the token's offset + 1:
+//     one 32-bit CAS claims it for good, and the key itself is the staged text,
+//     so that no key is copied and long tokens are like short ones;
+//   * the occupied slots become records; a 64-bit key (count, first four key
+//     bytes, record) is sorted by a bitonic network in registers, exchanging by
+//     shuffles within a warp and through shared memory beyond; runs that tie on
+//     count and four bytes are put in order by a thread each.  A long run sends
+//     the records {~count, first 8 bytes, offset} through a network with the full
+//     comparison instead;
+//   * records and keys are written by a thread per record.
+// Too many distinct words for the table (4,096, or a cluster that long probes
+// do not pass) raise the overflow flag, as the global table does, and the job
+// is run again with a larger table.  48 KB, 2,000 words:
+// 44 us of GPU time in one launch (tokens 15, sort 15).
+constexpr uint32_t TINY_MAX = 65536;   // bytes of text
+constexpr uint32_t TINY_SLOTS = 4096;
+constexpr uint32_t TINY_RUN = 32;      // ties one thread puts in order
+constexpr uint32_t TINY_PROBES = 512;  // then the table counts as full
+constexpr int TINY_T = 1024;
+struct TinySmem {
+  union {
+    uint16_t starts[TINY_MAX / 2];     // offsets of the tokens, then
+    ulonglong2 rec[TINY_SLOTS];        // {~count, bytes 0..3 | bytes 4..7, offset}, bytes big-endian
+  };
+  uint32_t text[TINY_MAX / 4 + 8];     // then spaces
+  uint32_t wsb[TINY_MAX / 32 + 4];     // bit j of word q: byte 32 q + j is whitespace
+  uint32_t slot[TINY_SLOTS];           // hash tag << 17 | offset + 1; 0: empty
+  uint32_t cnt[TINY_SLOTS];
+  unsigned long long key[TINY_SLOTS];  // (count, bytes 0..3, record) to sort; then the order
+  uint32_t wsum[TINY_T / 32];
+  uint32_t m, overflow, longrun;
+};
+static_assert(sizeof(TinySmem) <= 232448, "shared memory of one CTA");
+static_assert(TINY_MAX == (uint32_t)TINY_T * 64, "64 bytes per thread");
+
+// Four bytes of the staged text at any offset.
+__device__ __forceinline__ uint32_t tiny_word(const uint32_t* text, uint32_t p) {
+  return __funnelshift_r(text[p >> 2], text[(p >> 2) + 1], (p & 3) * 8);
+}
+// Length of the token at p (the bytes past the text are whitespace).
+__device__ __forceinline__ uint32_t tiny_len(const uint32_t* wsb, uint32_t p) {
+  uint32_t q = p + 1, w = wsb[q >> 5] >> (q & 31);
+  if (w) return q + __ffs(w) - 1 - p;
+  for (q = (q | 31) + 1; !(w = wsb[q >> 5]); q += 32) {
+  }
+  return q + __ffs(w) - 1 - p;
+}
+// Its first 16 bytes (and what follows a shorter one).
+__device__ __forceinline__ void tiny_words(const uint32_t* text, uint32_t p, uint32_t (&w)[4]) {
+  const uint32_t a = p >> 2, sh = (p & 3) * 8;
+  const uint32_t x0 = text[a], x1 = text[a + 1], x2 = text[a + 2], x3 = text[a + 3], x4 = text[a + 4];
+  w[0] = __funnelshift_r(x0, x1, sh);
+  w[1] = __funnelshift_r(x1, x2, sh);
+  w[2] = __funnelshift_r(x2, x3, sh);
+  w[3] = __funnelshift_r(x3, x4, sh);
+}
+// The token at a (length len) and the one at b, whose first 16 bytes (of len)
+// agree, are the same.
+__device__ __forceinline__ bool tiny_equal(const TinySmem& S, uint32_t a, uint32_t b, uint32_t len) {
+  if (a == b) return true;
+  if (b + len > TINY_MAX) return false;
+  if (!(S.wsb[(b + len) >> 5] >> ((b + len) & 31) & 1u)) return false;
+  if (len <= 16) return true;
+  uint32_t j = 16;
+  for (; j + 4 <= len; j += 4)
+    if (tiny_word(S.text, a + j) != tiny_word(S.text, b + j)) return false;
+  return j == len || ((tiny_word(S.text, a + j) ^ tiny_word(S.text, b + j)) << (8 * (4 - (len - j)))) == 0;
+}
+// Record a before record b: the records' words, then the tokens' bytes from the ninth on.
+__device__ __forceinline__ bool tiny_before(const TinySmem& S, const ulonglong2& a, const ulonglong2& b) {
+  if (a.x != b.x) return a.x < b.x;
+  if ((a.y ^ b.y) >> 32) return a.y < b.y;
+  const uint32_t pa = (uint32_t)a.y, pb = (uint32_t)b.y;
+  if (pa == 0xFFFFFFFFu || pb == 0xFFFFFFFFu) return pa < pb;  // padding last
+  const uint32_t la = tiny_len(S.wsb, pa), lb = tiny_len(S.wsb, pb), m = la < lb ? la : lb;
+  const uint8_t* t = reinterpret_cast<const uint8_t*>(S.text);
+  for (uint32_t j = 8; j < m; ++j)
+    if (t[pa + j] != t[pb + j]) return t[pa + j] < t[pb + j];
+  return la < lb;
+}
+
+// Exclusive scan over the CTA, and the total.
+__device__ __forceinline__ uint32_t tiny_scan(uint32_t v, uint32_t* wsum, uint32_t& total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  __syncthreads();  // (wsum's previous use is over)
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  const uint32_t w = wsum[lane];
+  uint32_t wi = w;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, wi, o);
+    if (lane >= o) wi += t;
+  }
+  total = __shfl_sync(0xffffffffu, wi, 31);
+  return __shfl_sync(0xffffffffu, wi - w, warp) + incl - v;
+}
+
+// Bitonic sort of E * TINY_T keys, element e * TINY_T + thread in v[e].
+template <int E>
+__device__ __forceinline__ void tiny_sort(unsigned long long* sh, uint32_t n) {
+  const uint32_t tid = threadIdx.x;
+  unsigned long long v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) v[e] = sh[e * TINY_T + tid];
+  for (uint32_t k = 2; k <= n; k <<= 1) {
+    for (uint32_t j = k >> 1; j; j >>= 1) {
+      if (j >= (uint32_t)TINY_T) {  // within the thread
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int f = e ^ (int)(j / TINY_T);
+          if (f > e && f < E) {
+            const bool up = ((uint32_t)(e * TINY_T) & k) == 0;
+            if ((v[e] > v[f]) == up) {
+              const unsigned long long t = v[e];
+              v[e] = v[f];
+              v[f] = t;
+            }
+          }
+        }
+        continue;
+      }
+      unsigned long long o[E];
+      if (j >= 32) {
+        __syncthreads();  // (the previous exchange has been read)
+#pragma unroll
+        for (int e = 0; e < E; ++e) sh[e * TINY_T + tid] = v[e];
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) o[e] = sh[e * TINY_T + (tid ^ j)];
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) o[e] = __shfl_xor_sync(0xffffffffu, v[e], j);
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const uint32_t i = e * TINY_T + tid;
+        const bool low = ((i & k) == 0) == ((i & j) == 0);  // this element keeps the smaller
+        v[e] = (o[e] < v[e]) == low ? o[e] : v[e];
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < E; ++e) sh[e * TINY_T + tid] = v[e];
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(TINY_T, 1) wc_tiny_kernel(const uint8_t* __restrict__ in, uint32_t n,
+                                                            uint8_t* __restrict__ out, uint32_t* state,
+                                                            volatile uint64_t* host) {
+  extern __shared__ __align__(16) unsigned char tiny_raw[];
+  TinySmem& S = *reinterpret_cast<TinySmem*>(tiny_raw);
+  const uint32_t tid = threadIdx.x;
+  const int lane = tid & 31;
+  // stage the text: thread t words t, t + 1024, ..; whole words where the input
+  // holds them, whatever its alignment
+  const uintptr_t ia = reinterpret_cast<uintptr_t>(in);
+  const uint32_t sh = (uint32_t)(ia & 3) * 8;
+  const uint32_t* wi = reinterpret_cast<const uint32_t*>(ia & ~uintptr_t(3));
+  // whole 16-byte groups first (n16 words of the text), the rest word by word
+  const uint32_t words = (n + 3) / 4, n16 = n >= 32 ? (n - 16) / 16 * 4 : 0;
+  const uintptr_t ga = ia & ~uintptr_t(15);
+  const uint32_t gs = (uint32_t)(ia & 15);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint32_t i = q * TINY_T + tid;
+    if (4 * i < n16) {
+      const uint4* g = reinterpret_cast<const uint4*>(ga) + i;
+      const uint4 a = __ldg(g);
+      reinterpret_cast<uint4*>(S.text)[i] = gs ? wc::shift_window(a, __ldg(g + 1), gs) : a;
+    }
+  }
+  for (uint32_t i = n16 + tid; i < words; i += TINY_T) {
+    uint32_t w;
+    // (both aligned words hold bytes of the input unless the word is the last)
+    if (4 * i + 8 <= n) {
+      w = sh ? __funnelshift_r(__ldg(wi + i), __ldg(wi + i + 1), sh) : __ldg(wi + i);
+    } else {
+      w = 0;
+      for (uint32_t j = 0; j < 4; ++j) w |= (4 * i + j < n ? (uint32_t)in[4 * i + j] : 32u) << (8 * j);
+    }
+    S.text[i] = w;
+  }
+  for (uint32_t i = words + tid; i < TINY_MAX / 4 + 8; i += TINY_T) S.text[i] = 0x20202020u;
+  reinterpret_cast<uint4*>(S.slot)[tid] = make_uint4(0, 0, 0, 0);
+  reinterpret_cast<uint4*>(S.cnt)[tid] = make_uint4(0, 0, 0, 0);
+  if (tid < 4) S.wsb[TINY_MAX / 32 + tid] = 0xFFFFFFFFu;
+  if (tid == 0) S.m = S.overflow = S.longrun = 0;
+  __syncthreads();
+  // whitespace of this thread's 64 bytes; a rotated order of the words keeps the banks apart
+  uint64_t ws = 0;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const uint32_t i = (q + lane) & 15;
+    ws |= (uint64_t)wc::byte_bits(wc::ws_bytes(S.text[16 * tid + i])) << (4 * i);
+  }
+  S.wsb[2 * tid] = (uint32_t)ws;
+  S.wsb[2 * tid + 1] = (uint32_t)(ws >> 32);
+  __syncthreads();
+  const uint64_t before = tid ? S.wsb[2 * tid - 1] >> 31 : 1u;
+  uint64_t starts = ~ws & ((ws << 1) | before);
+  const uint32_t mine = (uint32_t)__popcll(starts);
+  uint32_t ntok;
+  uint32_t at = tiny_scan(mine, S.wsum, ntok);
+  for (; starts; starts &= starts - 1) S.starts[at++] = (uint16_t)(64 * tid + (uint32_t)__ffsll((long long)starts) - 1);
+  __syncthreads();
+  for (uint32_t tok = tid; tok < ntok; tok += TINY_T) {
+    const uint32_t p = S.starts[tok];
+    const uint32_t len = tiny_len(S.wsb, p);
+    // the first 16 bytes, in registers for the hash and the comparisons
+    uint32_t w[4], mask[4], h = len * 0x9E3779B1u;
+    tiny_words(S.text, p, w);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      mask[j] = len >= 4u * j + 4 ? ~0u : len <= 4u * j ? 0u : (1u << (8 * (len - 4 * j))) - 1;
+      h = (h ^ (w[j] & mask[j])) * 0x85EBCA77u;
+      h ^= h >> 15;
+    }
+    for (uint32_t j = 16; j < len; j += 4) {
+      uint32_t v = tiny_word(S.text, p + j);
+      if (len - j < 4) v &= (1u << (8 * (len - j))) - 1;
+      h = (h ^ v) * 0x85EBCA77u;
+      h ^= h >> 15;
+    }
+    h *= 0x2C1B3C6Du;
+    h ^= h >> 16;
+    const uint32_t tag = h >> 17, mine = (tag << 17) | (p + 1);
+    uint32_t s = h & (TINY_SLOTS - 1), probe = 0;
+    bool done = false;
+    while (!done && probe < TINY_PROBES) {
+      // on to an empty slot or one with this tag, before the lanes compare together
+      uint32_t cur = *reinterpret_cast<volatile uint32_t*>(&S.slot[s]);
+      while (cur != 0 && cur >> 17 != tag && probe < TINY_PROBES) {
+        s = (s + 1) & (TINY_SLOTS - 1);
+        ++probe;
+        cur = *reinterpret_cast<volatile uint32_t*>(&S.slot[s]);
+      }
+      if (cur == 0) {
+        cur = atomicCAS(&S.slot[s], 0u, mine);
+        done = cur == 0;
+      }
+      if (!done && cur >> 17 == tag) {
+        const uint32_t q = (cur & 0x1FFFFu) - 1;
+        uint32_t v[4];
+        tiny_words(S.text, q, v);
+        const uint32_t diff = ((v[0] ^ w[0]) & mask[0]) | ((v[1] ^ w[1]) & mask[1]) | ((v[2] ^ w[2]) & mask[2]) |
+                              ((v[3] ^ w[3]) & mask[3]);
+        done = diff == 0 && tiny_equal(S, p, q, len);
+      }
+      if (done) {
+        atomicAdd(&S.cnt[s], 1u);
+      } else if (cur >> 17 == tag || cur != 0) {
+        s = (s + 1) & (TINY_SLOTS - 1);
+        ++probe;
+      }
+    }
+    if (!done) S.overflow = 1;
+    if (*reinterpret_cast<volatile uint32_t*>(&S.overflow)) break;
+  }
+  __syncthreads();
+  if (S.overflow) {
+    if (tid == 0) {
+      state[0] = 1;
+      if (host) host[0] = 1;
+    }
+    return;
+  }
+  // occupied slots -> records
+  for (uint32_t s = tid; s < TINY_SLOTS; s += TINY_T) {
+    const uint32_t v = S.slot[s];
+    if (v) {
+      const uint32_t p = (v & 0x1FFFFu) - 1, len = tiny_len(S.wsb, p);
+      uint32_t w0 = tiny_word(S.text, p), w1 = tiny_word(S.text, p + 4);
+      if (len < 4) w0 &= (1u << (8 * len)) - 1;
+      if (len < 8) w1 = len > 4 ? w1 & ((1u << (8 * (len - 4))) - 1) : 0;
+      const uint32_t i = atomicAdd(&S.m, 1u), b0 = __byte_perm(w0, 0, 0x0123), c = S.cnt[s];
+      S.rec[i] = make_ulonglong2(((uint64_t)~c << 32) | b0, ((uint64_t)__byte_perm(w1, 0, 0x0123) << 32) | p);
+      S.key[i] = ((uint64_t)(TINY_MAX - c) << 44) | ((uint64_t)b0 << 12) | i;  // count < 2^16
+    }
+  }
+  __syncthreads();
+  const uint32_t m = S.m;
+  const uint32_t N = m <= (uint32_t)TINY_T ? TINY_T : m <= 2u * TINY_T ? 2 * TINY_T : 4 * TINY_T;
+  for (uint32_t i = m + tid; i < N; i += TINY_T) S.key[i] = ~0ull;
+  __syncthreads();
+  if (N == TINY_T) tiny_sort<1>(S.key, N);
+  else if (N == 2 * TINY_T) tiny_sort<2>(S.key, N);
+  else tiny_sort<4>(S.key, N);
+  // runs that tie on count and four bytes: their records in the full order,
+  // by the thread of the first one (insertion)
+  for (uint32_t i = tid; i < m; i += TINY_T) {
+    const unsigned long long t = S.key[i] >> 12;
+    if ((i && S.key[i - 1] >> 12 == t) || i + 1 >= m || S.key[i + 1] >> 12 != t) continue;
+    uint32_t e = i + 2;
+    while (e < m && e - i <= TINY_RUN && S.key[e] >> 12 == t) ++e;
+    if (e - i > TINY_RUN) {
+      S.longrun = 1;
+      continue;
+    }
+    for (uint32_t a = i + 1; a < e; ++a) {
+      const unsigned long long v = S.key[a];
+      const ulonglong2 rv = S.rec[v & 0xFFFu];
+      uint32_t b = a;
+      for (; b > i && tiny_before(S, rv, S.rec[S.key[b - 1] & 0xFFFu]); --b) S.key[b] = S.key[b - 1];
+      S.key[b] = v;
+    }
+  }
+  __syncthreads();
+  const bool direct = S.longrun;  // the records themselves are sorted
+  if (direct) {
+    for (uint32_t i = m + tid; i < N; i += TINY_T) S.rec[i] = make_ulonglong2(~0ull, ~0ull);
+    __syncthreads();
+    // bitonic network; with strides up to 32 a warp's 32 pairs lie in 64
+    // consecutive records of its own
+    for (uint32_t k = 2; k <= N; k <<= 1) {
+      for (uint32_t j = k >> 1; j; j >>= 1) {
+        for (uint32_t i = tid; i < N / 2; i += TINY_T) {
+          const uint32_t a = 2 * i - (i & (j - 1)), b = a + j;
+          const ulonglong2 ra = S.rec[a], rb = S.rec[b];
+          if (tiny_before(S, rb, ra) == ((a & k) == 0)) S.rec[a] = rb, S.rec[b] = ra;
+        }
+        if (j > 32 || (j == 1 && k >= 64)) __syncthreads();
+        else __syncwarp();
+      }
+    }
+    __syncthreads();
+  }
+  // records and keys, 1,024 at a time
+  unsigned long long* head = reinterpret_cast<unsigned long long*>(out);
+  const uint8_t* text = reinterpret_cast<const uint8_t*>(S.text);
+  uint8_t* keys = out + 16 + 24 * (uint64_t)m;
+  uint32_t base = 0;
+  for (uint32_t i0 = 0; i0 < m; i0 += TINY_T) {
+    const uint32_t i = i0 + tid;
+    ulonglong2 r = make_ulonglong2(0, 0);
+    uint32_t len = 0;
+    if (i < m) {
+      r = S.rec[direct ? i : (uint32_t)(S.key[i] & 0xFFFu)];
+      len = tiny_len(S.wsb, (uint32_t)r.y);
+    }
+    uint32_t all;
+    const uint32_t off = base + tiny_scan(len, S.wsum, all);
+    base += all;
+    if (i < m) {
+      unsigned long long* o = head + 2 + 3 * (uint64_t)i;
+      o[0] = ~(uint32_t)(r.x >> 32);
+      o[1] = off;
+      o[2] = len;
+      const uint32_t p = (uint32_t)r.y;
+      for (uint32_t j = 0; j < len; ++j) keys[off + j] = text[p + j];
+    }
+  }
+  if (tid == 0) {
+    head[0] = m;
+    head[1] = base;
+    state[0] = 0;
+    if (host) {
+      host[0] = 0;
+      host[1] = m;
+      host[2] = base;
+    }
+  }
+}
+
 // ------------------------------------------------- pipelined map / reduce
 // Sec. III-D pipelines the map and reduce phases on the hyper-threads of a
 // core: map threads combine into a bounded local table and hand what it
@@ -2210,6 +2591,16 @@ cudaError_t launch_wordcount_post_multi(const wc::JobDev* jobs, const wc::JobDev
 cudaError_t launch_wordcount(const uint8_t* in, uint64_t n, const WcBuffers& b, const DevInfo& di, cudaStream_t s,
                              uint64_t* nk, bool pipelined, KTimer* kt, long long pipe_polls) {
   cudaError_t e;
+  if (n <= TINY_MAX && b.one_cta && b.cap == TINY_SLOTS && !pipelined) {
+    const int smem = (int)sizeof(TinySmem);
+    if ((e = cudaFuncSetAttribute(wc_tiny_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
+        (e = kt_begin(kt, s)) != cudaSuccess)
+      return e;
+    wc_tiny_kernel<<<1, TINY_T, smem, s>>>(in, (uint32_t)n, b.out, b.state, b.host);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = kt_end(kt, s)) != cudaSuccess) return e;
+    ++*nk;
+    return cudaSuccess;
+  }
   // table (keys then counts) and state words start at zero
   if ((e = cudaMemsetAsync(b.key, 0, wc_table_bytes(b.cap), s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(b.state, 0, wc_state_bytes(), s)) != cudaSuccess) return e;

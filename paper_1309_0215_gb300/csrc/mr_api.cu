@@ -358,7 +358,7 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
   switch (d.kind) {
     case MR_WORDCOUNT: {
       uint64_t cap = d.wc_slots;
-      j->wc_auto = cap == 0;
+      j->wc_auto = j->wc.one_cta = cap == 0;
       if (!cap) {
         // estimate: at most one distinct key per 16 input bytes, capped at
         // 2^17 slots; a table that overflows is regrown 4x and the job re-run

@@ -105,6 +105,7 @@ struct WcBuffers {
   uint32_t* state = nullptr;   // 64 bytes: word 0 overflow flag, 64-bit fields 1..4 post-phase bounds
   uint8_t* sortbuf = nullptr;  // post-phase scratch for cap records
   uint64_t* host = nullptr;    // pinned host words {flags, records, key bytes}, written by the last kernel (or null)
+  bool one_cta = false;        // a small text may take the one-CTA kernel (automatic tables)
   uint8_t* out = nullptr;      // result: header + records + key bytes
   uint64_t out_cap = 0;
 };

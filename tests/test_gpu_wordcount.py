@@ -197,3 +197,40 @@ def test_contexts_release_their_memory(mr, torch_alloc):
     torch.cuda.synchronize()
     free1, _ = torch.cuda.mem_get_info()
     assert free1 >= free0 - (64 << 20), (free0, free1)
+
+
+def _tiny_texts():
+    rng = np.random.default_rng(77)
+    letters = np.frombuffer(b"abcdefghijklmnopqrstuvwxyz\xc3\xa9\x00", dtype=np.uint8)
+
+    def words(n, lo, hi):
+        return [bytes(rng.choice(letters, rng.integers(lo, hi + 1))) for _ in range(n)]
+    zipf, _, _ = synth.wc_text(65536, nwords=3000, seed=5)
+    yield "most bytes", bytes(zipf)
+    yield "one byte more", bytes(zipf) + b"x"
+    yield "few bytes", b"a"
+    yield "no token", b" \t\n\v\f\r" * 100
+    yield "one token", b"q" * 65536
+    yield "long tokens", b" ".join(w * 7 for w in words(300, 3, 9))[:65536]
+    shared = b"prefixes"  # ties on count and on the first eight bytes
+    yield "ties", b"\n".join(shared + w for w in words(3000, 0, 12))[:65536]
+    yield "prefixes of one another", b" ".join((b"ab" * 40)[: 1 + i % 70] for i in range(1200))[:65536]
+    yield "table full", b" ".join(b"%05x" % (i * 7919 % 1048576) for i in range(4096))
+    yield "table overflows", b" ".join(b"%05x" % (i * 7919 % 1048576) for i in range(9000))
+    for n in (63, 64, 65, 127, 128, 4095, 4096, 40001):
+        yield "cut at %d" % n, bytes(zipf[:n])
+
+
+@pytest.mark.parametrize("name,text", list(_tiny_texts()), ids=lambda v: v if isinstance(v, str) else "")
+def test_wc_small_texts_one_cta(mr, name, text):
+    """Texts of up to 64 KiB (one CTA, one launch), at every alignment of their
+    first byte, and against a pinned table, which takes the larger passes."""
+    import torch
+    want = oracle.wordcount(np.frombuffer(text, dtype=np.uint8))
+    for off in range(5):
+        buf = torch.full((len(text) + off + 9,), ord("z"), dtype=torch.uint8, device="cuda")
+        buf[off: off + len(text)] = torch.from_numpy(np.frombuffer(text, dtype=np.uint8).copy()).cuda()
+        torch.cuda.synchronize()
+        view = buf[off: off + len(text)]
+        assert mr.wordcount(view) == want, off
+    assert mr.wordcount(view, wc_slots=1 << 14) == want
