@@ -430,9 +430,11 @@ struct SettleShared {
   int red_k[SET_T_MAX / 32];
 };
 
-// The settled cluster of point p; has: its word holds the cluster of the round before.
-__device__ __forceinline__ void settle_put(uint32_t* assign, uint32_t p, uint32_t now, bool has, SettleShared& S) {
-  const uint32_t old = has ? assign[p] & 0xffffu : now;
+// The settled cluster of point p; has: its word holds the cluster of the round
+// before (not in a job's first round).
+__device__ __forceinline__ void settle_put(uint32_t* assign, uint32_t p, uint32_t now, bool has, uint32_t word,
+                                           SettleShared& S) {
+  const uint32_t old = has ? word & 0xffffu : now;
   assign[p] = km_word(now, old);
   if (now != old) atomicAdd(&S.moved, 1u);
 }
@@ -452,6 +454,7 @@ __device__ void settle_fp64(const float* __restrict__ x, uint32_t d, const float
   float m = INFINITY;
   for (uint32_t kk = threadIdx.x; kk < k; kk += blockDim.x) {
     float s32 = 0.f;
+#pragma unroll 16
     for (uint32_t j = 0; j < d; ++j) {
       const float t = xs[j] - __ldg(ct + (uint64_t)j * k + kk);
       s32 = fmaf(t, t, s32);
@@ -483,6 +486,7 @@ __device__ void settle_fp64(const float* __restrict__ x, uint32_t d, const float
     __syncthreads();
     if (threadIdx.x < cn) {
       double s64 = 0.0;
+#pragma unroll 8
       for (uint32_t j = 0; j < d; ++j) s64 = __dadd_rn(s64, prod[threadIdx.x * d + j]);
       const int kk = (int)cand[c0 + threadIdx.x];
       if (s64 < best || (s64 == best && kk < bk)) best = s64, bk = kk;
@@ -499,7 +503,7 @@ __device__ void settle_fp64(const float* __restrict__ x, uint32_t d, const float
   if (threadIdx.x == 0) {
     for (int w = 1; w < nw; ++w)
       if (S.red_d[w] < best || (S.red_d[w] == best && S.red_k[w] < bk)) best = S.red_d[w], bk = S.red_k[w];
-    settle_put(assign, p, bk == 0x7fffffff ? 0u : (uint32_t)bk, has, S);
+    settle_put(assign, p, bk == 0x7fffffff ? 0u : (uint32_t)bk, has, has ? assign[p] : 0u, S);
   }
 }
 
@@ -582,15 +586,20 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
   const bool vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   const uint64_t rb = ((uint64_t)nf + SET_RP - 1) / SET_RP;
   unsigned long long settled = 0;  // points settled in FP64
-  // the few-candidate points: warps on their own, four points at a time (the
-  // last CTAs first: the listed points' batches start with the first ones)
-  {
+  // the few-candidate points: warps on their own, four points at a time.  The
+  // CTAs that have a batch of listed points leave them to the others (up to
+  // half of the CTAs), so that no CTA's chain of loads holds both.
+  const uint32_t lead = (uint32_t)(rb < gridDim.x / 2 ? rb : gridDim.x / 2);
+  if (blockIdx.x >= lead) {
     const uint32_t sl = lane & 7;
-    const uint64_t w0 = (uint64_t)(gridDim.x - 1 - blockIdx.x) * nw + warp;
+    const uint64_t w0 = (uint64_t)(blockIdx.x - lead) * nw + warp, ws = (uint64_t)(gridDim.x - lead) * nw;
     KmFew next = load_few(pairs, np, 4 * w0 + (lane >> 3));
-    for (uint64_t f0 = 4 * w0; f0 < np; f0 += 4 * (uint64_t)gridDim.x * nw) {
+    for (uint64_t f0 = 4 * w0; f0 < np; f0 += 4 * ws) {
       const KmFew e = next;
-      next = load_few(pairs, np, f0 + 4 * (uint64_t)gridDim.x * nw + (lane >> 3));
+      next = load_few(pairs, np, f0 + 4 * ws + (lane >> 3));
+      // (loaded with the rows, not after them)
+      const uint32_t word = nchg ? assign[e.p] : 0u;
+      const float l = B.ub ? B.lb[e.p] : 0.f;
       const uint32_t nc = e.hi >> 28;
       float fd[KM_CAND_MAX];
       if (__any_sync(0xffffffffu, nc > 2)) few_dists<KM_CAND_MAX>(x, c, d, e, nc, sl, vec, fd);
@@ -613,6 +622,7 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
           const float* xp = x + (uint64_t)e.p * d;
           const float* cp = c + (uint64_t)bk * d;
           double s64 = 0.0;
+#pragma unroll 8
           for (uint32_t j = 0; j < d; ++j) {
             const double t = __dsub_rn((double)__ldg(xp + j), (double)__ldg(cp + j));
             s64 = __dadd_rn(s64, __dmul_rn(t, t));
@@ -627,15 +637,14 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
           if (ob < best || (ob == best && ok < bk)) best = ob, bk = ok;
         }
         if (!clear && sl == 0) {
-          settle_put(assign, e.p, bk == 0xffffffffu ? 0u : bk, nchg, S);
+          settle_put(assign, e.p, bk == 0xffffffffu ? 0u : bk, nchg, word, S);
           if (B.ub) B.ub[e.p] = INFINITY;  // no bounds: the next round computes it again
           ++settled;
         }
       }
       if (clear && nc && sl == 0) {
-        settle_put(assign, e.p, k1, nchg, S);
+        settle_put(assign, e.p, k1, nchg, word, S);
         if (B.ub) {  // the distance pass left the bound of the other centroids
-          const float l = B.lb[e.p];
           km_put_bounds(B, e.p, B.drift[k1], *B.far, m1 * widen + 1e-36f,
                         fminf(m2 * (2.f - widen) - 1e-36f, l * l * 0.999999f));
         }
@@ -663,7 +672,7 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
 #pragma unroll
         for (int q = 0; q < SET_RP / 2; ++q) acc[q] = 0ull;
         if (kk < k) {
-#pragma unroll 2
+#pragma unroll 8
           for (uint32_t j = 0; j < d; ++j) {
             const float cv = -__ldg(ct + (uint64_t)j * k + kk);
             const unsigned long long nc = pack2(cv, cv);
@@ -713,7 +722,7 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
         }
         const uint32_t p = list[f0 + r];
         if (__uint_as_float(m2) > __uint_as_float(m1) * widen) {
-          settle_put(assign, p, k1, nchg, S);
+          settle_put(assign, p, k1, nchg, nchg ? assign[p] : 0u, S);
           if (B.ub) km_put_bounds(B, p, B.drift[k1], *B.far, __uint_as_float(m1) * widen + 1e-36f, __uint_as_float(m2) * (2.f - widen) - 1e-36f);
         } else {
           S.open[atomicAdd(&S.nopen, 1u)] = p;
@@ -1761,13 +1770,13 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide, bool bou
   return cudaSuccess;
 }
 
-// The filter pays for its two kernels (15 us a round at 4M points) and its
-// memory where the distance pass takes well over that: from 2^27 distances
-// (60 us) on, and when there are rounds to skip points in.
-bool km_bounds_pay(uint32_t n, uint32_t d, uint32_t k, uint32_t iters) {
-  (void)d;
-  return (uint64_t)n * ((k + 15) & ~15u) >= 1ull << 27 && iters >= 3;
-}
+// The filter pays for its two kernels (10 - 24 us a round) and the bounds the
+// first rounds write for nothing where the distance pass is long enough (its
+// time goes by the points, about 130 us per million whatever D and K) and
+// enough rounds follow.  Ten rounds with / without, us: 200,000 x 37, K = 100
+// 484 / 522, 200,000 x 8 559 / 547, 400,000 x 37 689 / 808, 400,000 x 50 907 /
+// 920, 1.6M x 8 2,169 / 2,528; three rounds at 400,000 x 37 350 / 318.
+bool km_bounds_pay(uint32_t n, uint32_t iters) { return n >= 3u << 17 && iters >= 5; }
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                     KmBuffers& b, const unsigned int* cmax, uint32_t* nchg, const DevInfo& di,

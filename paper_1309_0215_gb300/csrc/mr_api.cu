@@ -169,13 +169,18 @@ cudaError_t pooled_event(mr_ctx* c, bool timing, cudaEvent_t* e) {
 }
 
 constexpr size_t STATUS_WORDS = 4, STATUS_PER_SLAB = 256;
-constexpr size_t STAGING_BYTES = 256 * 1024;
+constexpr size_t STAGING_BYTES = 64 * 1024;
 
+// One more slab of status words; the context's first one holds the staging
+// buffer too (one allocation: pinning costs tens of microseconds each time).
 cudaError_t status_grow(mr_ctx* c) {
   void* p = nullptr;
-  const cudaError_t e = cudaHostAlloc(&p, STATUS_WORDS * STATUS_PER_SLAB * 8, cudaHostAllocMapped);
+  const bool first = c->status_slabs.empty();
+  const size_t words = STATUS_WORDS * STATUS_PER_SLAB * 8;
+  const cudaError_t e = cudaHostAlloc(&p, words + (first ? STAGING_BYTES : 0), cudaHostAllocMapped);
   if (e != cudaSuccess) return e;
   c->status_slabs.push_back(p);
+  if (first) c->staging = static_cast<uint8_t*>(p) + words;
   for (size_t i = 0; i < STATUS_PER_SLAB; ++i)
     c->status_free.push_back(static_cast<uint64_t*>(p) + i * STATUS_WORDS);
   return cudaSuccess;
@@ -443,7 +448,7 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
       // the wide tensor-core pass keeps its centroid operands in scratch, the
       // filter its bounds; a context without room for them runs without
       bool wide = d.km_precision == MR_KM_FP32 && !km_tc_supported(D, K) && km_wide_supported(D, K);
-      bool bounds = !c->budget && !wide && km_tc_supported(D, K) && km_bounds_pay(N, D, K, d.km_iters);
+      bool bounds = !c->budget && !wide && km_tc_supported(D, K) && km_bounds_pay(N, d.km_iters);
       uint64_t scr = align256(km_scratch_bytes(N, D, K, wide, bounds));
       const uint64_t init_bytes = d.input_on_device ? 0 : align256((uint64_t)K * D * 4);
       mr_status st = dev_alloc(c, res + scr + init_bytes, &j->slab);
@@ -1131,11 +1136,9 @@ mr_status mr_create(const mr_config* cfg, mr_ctx** out) {
     }
   }
   // the first status words and the staging buffer, so that no job waits for their pinning
-  if (e == cudaSuccess) e = cudaHostAlloc(&c->staging, STAGING_BYTES, cudaHostAllocDefault);
   if (e == cudaSuccess) e = status_grow(c);
   if (e != cudaSuccess) {
     set_last_error("mr_create", e);
-    if (c->staging) cudaFreeHost(c->staging);
     if (c->pool) cudaMemPoolDestroy(c->pool);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -1187,7 +1190,6 @@ void mr_destroy(mr_ctx* c) {
   for (KTimer* t : c->kt_pool) kt_destroy(t);
   cudaStreamSynchronize(c->stream);
   for (void* p : c->status_slabs) cudaFreeHost(p);
-  if (c->staging) cudaFreeHost(c->staging);
   // memory still held (none, normally) is released once it is freed
   if (c->pool) cudaMemPoolDestroy(c->pool);
   if (c->own_stream) cudaStreamDestroy(c->stream);

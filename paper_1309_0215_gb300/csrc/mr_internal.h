@@ -227,7 +227,7 @@ struct KmBuffers {
 };
 // wide: with the wide tensor-core pass's operands; bounds: with the points' bounds
 size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool bounds);
-bool km_bounds_pay(uint32_t n, uint32_t d, uint32_t k, uint32_t iters);
+bool km_bounds_pay(uint32_t n, uint32_t iters);
 cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes, bool wide, bool bounds);
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,
                           cudaStream_t s, float* out_cent, int32_t* out_assign, unsigned long long* out_stats,
