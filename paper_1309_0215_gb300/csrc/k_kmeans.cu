@@ -394,9 +394,11 @@ __device__ __forceinline__ int fx_shift_of(float m, uint32_t n) {
 // and by latency for short ones.  As three launches (pairs, a re-check with the
 // centroids staged in each CTA's shared memory and one warp per point, a
 // kernel for the FP64 points) this took 15 + 56 + 20 us at 4M x 64, K = 256
-// (181K pairs, 22K listed points, 100 FP64 points); now 43 us.  For K x D
+// (181K pairs, 22K listed points, 100 FP64 points); now 36 us.  For K x D
 // beyond shared memory the re-check went warp by warp over the centroids: 531
-// of 576 us at 250,000 x 128, K = 512; now 55 us.
+// of 576 us at 250,000 x 128, K = 512; now 55 us (85 before the loads of a
+// point's rows, word and bound, and of eight dimensions' centroids, went out
+// together, and the CTAs with listed points left the others alone).
 // stat[0] counts the points re-checked, stat[1] those settled in FP64.
 constexpr int SET_RP = 16;        // listed points per batch
 constexpr int SET_LD = SET_RP + 4;  // row stride of the staged points (16-byte rows)
@@ -777,12 +779,14 @@ __device__ __forceinline__ uint32_t cluster_of(const uint32_t* assign, uint64_t 
 // kernel of the update alike, from the count the distance and settle passes
 // left (chg null: the first round).
 //
-// The line: n / 32 beside the local-array updates, which stream the points near
-// the HBM rate (4M x 64, K = 256: all points 186 us; 1.9% moved 124 us, most of
-// it adds to the few clusters that exchange points; 0.8% 30 us, 0.2% 16 us),
-// n / 8 beside the sorted update (250,000 x 128, K = 512: all points 107 us,
-// 4.1% moved 27 us, 1.6% 20 us).
-constexpr uint32_t KM_DELTA_LOCAL = 32, KM_DELTA_SORTED = 8;
+// The line: n / 4 beside the window-sorted update, whose CTAs collect the
+// changes in their shared-memory sums, unless at most n / 256 points moved
+// (4M x 64, K = 256: all points 186 us; 21% moved 183 us (the ten rounds 30 us
+// shorter than with n / 8), 1.8% 49 us and 124
+// straight to the global sums, 0.6% 32 us; 0.2% 17 us straight); n / 32 beside
+// the other local-array updates; n / 8 beside the sorted update (250,000 x 128,
+// K = 512: all points 107 us, 4.1% moved 27 us, 2.3% 20 us).
+constexpr uint32_t KM_DELTA_WINDOW = 4, KM_DELTA_DIRECT = 256, KM_DELTA_LOCAL = 32, KM_DELTA_SORTED = 8;
 __device__ __forceinline__ bool km_by_changes(const uint32_t* chg, uint32_t lim) { return chg && *chg <= lim; }
 
 __device__ __forceinline__ void lq_split(float v, int& hi, int& lo);
@@ -791,8 +795,9 @@ __device__ __forceinline__ void lq_split(float v, int& hi, int& lo);
 // takes 128 consecutive words, 16 bytes a lane, and up to KM_DELTA_ROWS moved
 // points' rows at a time.
 constexpr int KM_DELTA_ROWS = 4;
-__device__ void km_apply_changes(const float* __restrict__ x, uint32_t n, uint32_t d, uint32_t k, uint32_t* assign,
-                                 const int* shift, long long* sums, unsigned long long* counts) {
+__device__ __forceinline__ void km_apply_changes(const float* __restrict__ x, uint32_t n, uint32_t d, uint32_t k,
+                                                 uint32_t* assign, const int* shift, long long* sums,
+                                                 unsigned long long* counts) {
   const int lane = threadIdx.x & 31;
   const float scale = ldexpf(1.f, *shift);
   const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1365,12 +1370,26 @@ __global__ void __launch_bounds__(WS_THREADS, 1) km_window_sum_kernel(const floa
   const uint32_t d = MODE == WS_D64 ? 64u : d_arg;  // a constant on the 64-wide path
   constexpr bool TWO = MODE != WS_D32;            // two dimensions per lane
   pdl_wait();
-  if (km_by_changes(chg, lim)) {
-    km_apply_changes(x, n, d, k, assign, shift, sums, counts);
-    return;
-  }
   extern __shared__ __align__(16) unsigned char ws_sm[];
   long long* S = reinterpret_cast<long long*>(ws_sm);
+  if (km_by_changes(chg, lim)) {
+    if (*chg <= n / KM_DELTA_DIRECT) {
+      km_apply_changes(x, n, d, k, assign, shift, sums, counts);
+      return;
+    }
+    // many: the clusters that exchange points are few, and the adds to their
+    // sums would queue in L2; collected per CTA first
+    unsigned long long* dc = reinterpret_cast<unsigned long long*>(S + (uint64_t)k * d);  // [k] count changes
+    for (uint64_t i = threadIdx.x; i < (uint64_t)k * (d + 1); i += WS_THREADS) S[i] = 0;
+    __syncthreads();
+    km_apply_changes(x, n, d, k, assign, shift, S, dc);
+    __syncthreads();
+    for (uint64_t i = threadIdx.x; i < (uint64_t)k * d; i += WS_THREADS)
+      if (S[i]) atomicAdd(reinterpret_cast<unsigned long long*>(sums) + i, (unsigned long long)S[i]);
+    for (uint32_t i = threadIdx.x; i < k; i += WS_THREADS)
+      if (dc[i]) atomicAdd(counts + i, dc[i]);
+    return;
+  }
   uint32_t* hc = reinterpret_cast<uint32_t*>(S + (uint64_t)k * d);
   uint32_t* off = hc + k;
   uint32_t* C = off + k;
@@ -1882,7 +1901,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   uint32_t* nact = b.nflag + 8;
   const KmBounds bounds = filter ? b.bounds : KmBounds{};
   const float* center = tc || wide ? b.center : nullptr;
-  const uint32_t lim = n / (local ? KM_DELTA_LOCAL : KM_DELTA_SORTED);  // points moved, at most, in an update by changes
+  const uint32_t lim = n / (wsum ? KM_DELTA_WINDOW : local ? KM_DELTA_LOCAL : KM_DELTA_SORTED);  // points moved, at most, in an update by changes
   auto chg_of = [&](uint32_t it) { return b.nflag + ((it & 1) ? 5 : 0); };  // points that changed cluster in the round
   auto finalize = [&](uint32_t it, bool first) {
     ++*nk;

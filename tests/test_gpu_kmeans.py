@@ -350,6 +350,27 @@ def test_kmeans_update_by_changes(mr, n, d, k, precision):
     assert min(moved) <= n // 32 < max(moved)  # both kinds of update ran
 
 
+@pytest.mark.parametrize("n,d", [(30_001, 64), (30_001, 21), (20_003, 33)])
+def test_kmeans_changes_collected_or_direct(mr, n, d):
+    """The window-sorted update collects the changes per CTA (up to n / 4 moved
+    points) or adds them straight (up to n / 256): the rounds reach both, and
+    equal single rounds (each a full update) byte for byte."""
+    x, _, _ = synth.kmeans_points(n, d, 8, seed=n + d, sigma=2.0)
+    cur = synth.kmeans_init(x, 8, seed=n)
+    dx = _dev(x)
+    c14, a14, _ = mr.kmeans(dx, _dev(cur), 14, 0)
+    moved, last = [], None
+    for _ in range(14):
+        cur, a, _ = mr.kmeans(dx, _dev(cur), 1, 0)
+        if last is not None:
+            moved.append(int((a != last).sum()))
+        last = a
+    assert np.array_equal(a14, last)
+    assert np.array_equal(c14, cur)
+    assert any(0 < m <= n // 256 for m in moved)
+    assert any(n // 256 < m <= n // 4 for m in moved)
+
+
 @pytest.mark.parametrize("n,d,k,cap", [
     (1_999, 65, 3, 0),      # one value in the second dimension chunk
     (1_281, 128, 257, 0),   # one centroid in the second centroid chunk
