@@ -34,9 +34,8 @@
 namespace mrgb {
 namespace wc {
 
-constexpr int SEG = 512;                // bytes per warp step (16 per lane)
-constexpr int HALO = 64;                // staged bytes after the segment
-constexpr int BUF = SEG + HALO;
+constexpr int SEG = 512;                // bytes per warp step (16 per lane), but for MapWarp
+constexpr int HALO = 32;                // staged bytes after the segment (a token's first 16 and word loads)
 constexpr int LT = 128;                 // hot-key cache entries per warp
 constexpr int CACHE_EPOCH = 64;         // segments between cache merges
 constexpr int MAX_PROBES = 4096;
@@ -44,13 +43,13 @@ constexpr uint64_t LONG_TAG = 0xFFull << 56;
 constexpr uint64_t LEN_MASK = (1ull << 56) - 1;
 
 struct WarpLocal {
+  static constexpr int LANE = 16;  // bytes of the segment per lane
   unsigned long long w0[LT];
   unsigned long long w1[LT];
   uint32_t h[LT];
   uint32_t cnt[LT];
-  uint8_t buf[BUF];
-  uint32_t wsb[BUF / 32 + 2];  // whitespace bitmap of buf: bit j of word q = byte 32q + j
-  uint16_t starts[SEG / 2];
+  uint8_t buf[SEG + HALO];
+  uint16_t starts[SEG / 2];    // the tokens: first byte | length << 12 (0: 16 bytes or more)
 };
 static_assert(sizeof(WarpLocal) % 16 == 0, "WarpLocal must keep 16-byte alignment");
 
@@ -82,8 +81,21 @@ __device__ __forceinline__ uint32_t ws_bytes(uint32_t u) {
   const uint32_t rg = (h + 0x77777777u) & ~(h + 0x72727272u) & ~u;
   return (sp | rg) & 0x80808080u;
 }
-// compress a 0xFF-per-byte mask to 4 bits (byte i -> bit i)
-__device__ __forceinline__ uint32_t byte_bits(uint32_t m) { return ((m & 0x80808080u) * 0x00204081u) >> 28; }
+// compress ws_bytes' mask to 4 bits (byte i -> bit i)
+__device__ __forceinline__ uint32_t byte_bits(uint32_t m) { return (m * 0x00204081u) >> 28; }
+// The 16 whitespace bits of 16 bytes: four dot products of the byte masks with
+// powers of two (each sum is 128 times eight bits).
+__device__ __forceinline__ uint32_t ws_bits(const uint4& v) {
+  const uint32_t lo = __dp4a(ws_bytes(v.y), 0x80402010u, __dp4a(ws_bytes(v.x), 0x08040201u, 0u));
+  const uint32_t hi = __dp4a(ws_bytes(v.w), 0x80402010u, __dp4a(ws_bytes(v.z), 0x08040201u, 0u));
+  return (lo >> 7) | (hi << 1);
+}
+// the low n bits of v (n <= 0: none; n >= 32: all)
+__device__ __forceinline__ uint32_t low_bits(uint32_t v, int n) {
+  uint32_t r;
+  asm("szext.clamp.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"((uint32_t)(n > 0 ? n : 0)));
+  return r;
+}
 
 __device__ __forceinline__ uint64_t fmix64(uint64_t k) {
   k ^= k >> 33;
@@ -94,13 +106,11 @@ __device__ __forceinline__ uint64_t fmix64(uint64_t k) {
   return k;
 }
 
-// 32-bit multiply-xorshift mix of the four 32-bit words of a short key
-// (the key is compared exactly; the hash only spreads slots).
-__device__ __forceinline__ uint32_t hash_short(uint64_t w0, uint64_t w1) {
-  uint32_t h = (uint32_t)w0 * 0x9E3779B1u;
-  h ^= __funnelshift_l((uint32_t)(w0 >> 32) * 0x85EBCA77u, (uint32_t)(w0 >> 32) * 0x85EBCA77u, 13);
-  h ^= __funnelshift_l((uint32_t)w1 * 0xC2B2AE3Du, (uint32_t)w1 * 0xC2B2AE3Du, 7);
-  h ^= (uint32_t)(w1 >> 32) * 0x27D4EB2Fu;
+// 32-bit mix of the four 32-bit words of a short key: a sum of products (four
+// multiply-adds), whose high bits are folded down (the key is compared exactly;
+// the hash only spreads slots).
+__device__ __forceinline__ uint32_t hash_short(uint32_t u0, uint32_t u1, uint32_t u2, uint32_t u3) {
+  uint32_t h = u0 * 0x9E3779B1u + u1 * 0x85EBCA77u + u2 * 0xC2B2AE3Du + u3 * 0x27D4EB2Fu;
   h ^= h >> 15;
   h *= 0x2C1B3C6Du;
   h ^= h >> 12;
@@ -120,42 +130,34 @@ __device__ inline bool long_equal(const uint8_t* __restrict__ in, uint64_t a, ui
   return true;
 }
 
-// The token starting at segment-relative byte r (its first 16 bytes are
-// always inside the staged buffer; bytes past the input end were staged as
-// spaces).  Its length comes from the segment's whitespace bitmap.
+// The token of list entry e (stage_tokens): it starts at segment-relative byte
+// r, its first 16 bytes are inside the staged buffer (bytes past the input end
+// were staged as spaces), and its length, if below 16, comes with the entry.
+// An inactive lane passes entry 0 and gets an empty short token: the warp takes
+// one path unless a token is long.
 template <class B>
 __device__ __forceinline__ Tok read_token(const uint8_t* __restrict__ in, uint64_t n, uint64_t base, const B& W,
-                                          uint32_t r) {
+                                          uint32_t e, bool active) {
   const uint32_t* wb = reinterpret_cast<const uint32_t*>(W.buf);
-  // m bit i: byte r + 1 + i is whitespace
-  const uint32_t p = r + 1, wi = p >> 5, bs = p & 31;
-  const uint32_t m = __funnelshift_r(W.wsb[wi], W.wsb[wi + 1], bs);
+  const uint32_t r = e & 0xFFFu, L = e >> 12;
+  const uint32_t a = r >> 2, sh = r * 8;  // the shift counts modulo 32
+  const uint32_t x0 = wb[a], x1 = wb[a + 1], x2 = wb[a + 2], x3 = wb[a + 3], x4 = wb[a + 4];
+  const int bits = 8 * (int)L;
+  const uint32_t u0 = low_bits(__funnelshift_r(x0, x1, sh), bits);
+  const uint32_t u1 = low_bits(__funnelshift_r(x1, x2, sh), bits - 32);
+  const uint32_t u2 = low_bits(__funnelshift_r(x2, x3, sh), bits - 64);
+  const uint32_t u3 = low_bits(__funnelshift_r(x3, x4, sh), bits - 96) | (L << 24);
   Tok t;
-  if (m & 0x7FFFu) {
-    const uint32_t a = r >> 2, sh = (r & 3) * 8;
-    const uint32_t x0 = wb[a], x1 = wb[a + 1], x2 = wb[a + 2], x3 = wb[a + 3], x4 = wb[a + 4];
-    const uint32_t u0 = __funnelshift_r(x0, x1, sh), u1 = __funnelshift_r(x1, x2, sh);
-    const uint32_t u2 = __funnelshift_r(x2, x3, sh), u3 = __funnelshift_r(x3, x4, sh);
-    const uint32_t L = __ffs(m);  // 1..15 (byte 0 is a token byte)
-    uint64_t k0 = (uint64_t)u0 | ((uint64_t)u1 << 32);
-    uint64_t k1 = (uint64_t)u2 | ((uint64_t)u3 << 32);
-    if (L < 8) {
-      k0 &= (1ull << (8 * L)) - 1;
-      k1 = 0;
-    } else {
-      k1 &= (1ull << (8 * (L - 8))) - 1;
-    }
-    t.w0 = k0;
-    t.w1 = k1 | ((uint64_t)L << 56);
-    t.h = hash_short(t.w0, t.w1);
-    return t;
-  }
+  t.w0 = (uint64_t)u0 | ((uint64_t)u1 << 32);
+  t.w1 = (uint64_t)u2 | ((uint64_t)u3 << 32);
+  t.h = hash_short(u0, u1, u2, u3);
+  if (L || !active) return t;
   // long token: FNV-1a 64 over its bytes, then the length is mixed in
   const uint64_t off = base + r;
   uint64_t h = 0xcbf29ce484222325ull, len = 0;
   for (uint64_t i = off; i < n; ++i) {
     const uint32_t rel = (uint32_t)(i - base);
-    const uint32_t c = (i - base) < (uint64_t)BUF ? W.buf[rel] : in[i];
+    const uint32_t c = (i - base) < sizeof(W.buf) ? W.buf[rel] : in[i];
     if (is_ws(c)) break;
     h = (h ^ c) * 0x100000001b3ull;
     ++len;
@@ -166,10 +168,14 @@ __device__ __forceinline__ Tok read_token(const uint8_t* __restrict__ in, uint64
   return t;
 }
 
-__device__ __forceinline__ void ld_slot(const unsigned long long* p, uint64_t& a, uint64_t& b) {
-  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+// an even slot and the one after it (tables are 256-byte aligned)
+__device__ __forceinline__ void ld_pair(const unsigned long long* p, uint64_t& a0, uint64_t& a1, uint64_t& b0,
+                                        uint64_t& b1) {
+  asm volatile("ld.volatile.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(a0), "=l"(a1), "=l"(b0), "=l"(b1)
+               : "l"(p)
+               : "memory");
 }
-
 __device__ __forceinline__ void cas_slot(unsigned long long* p, uint64_t n0, uint64_t n1, uint64_t& o0, uint64_t& o1) {
   asm volatile(
       "{\n\t.reg .b128 d, c, v;\n\t"
@@ -186,12 +192,13 @@ __device__ __forceinline__ uint64_t global_slot(uint32_t h, uint32_t log2cap) {
   return log2cap ? (uint64_t)((h * 0x9E3779B1u) >> (32 - log2cap)) : 0;
 }
 
-// Combine (key, c) into the job's global container.  Linear probing, two
-// slots per step: both slots are loaded before either is examined, so a
-// key that is not in its first slot costs no second round trip to L2, and
-// the lanes of a warp, which probe different keys, finish in fewer steps.
-// A slot loaded before a CAS on the slot before it may be stale, which is
-// harmless: a slot only ever changes from empty to a key.
+// Combine (key, c) into the job's global container.  Linear probing from the
+// first slot of the key's pair, a pair per step with one 32-byte load (as two
+// 16-byte loads the lanes' separate lines took the L1 twice as long: 4 us of 414
+// for 256 MB of 50,000 words).
+// Both slots are loaded before either is examined; a slot loaded before a CAS
+// on the slot before it may be stale, which is harmless: a slot only ever
+// changes from empty to a key.
 __device__ __forceinline__ bool slot_take(const JobDev& J, uint64_t s, uint64_t r0, uint64_t r1, uint64_t w0,
                                           uint64_t w1, bool is_long, uint64_t c) {
   unsigned long long* sp = J.key + 2 * s;
@@ -209,27 +216,16 @@ __device__ __forceinline__ bool slot_take(const JobDev& J, uint64_t s, uint64_t 
   return false;
 }
 
-// WIDTH = 2 loads two slots per step; WIDTH = 1 is plain linear probing,
-// kept for the persistent batch kernel, whose registers are tight.
-template <int WIDTH = 2>
 __device__ inline void global_insert(const JobDev& J, uint64_t w0, uint64_t w1, uint32_t h, uint64_t c) {
-  uint64_t slot = global_slot(h, J.log2cap);
+  uint64_t slot = global_slot(h, J.log2cap) & ~1ull;
   const bool is_long = (w1 >> 56) == 0xFF;
   const uint64_t mask = J.cap - 1;
-  for (int p = 0; p < MAX_PROBES; p += WIDTH) {
-    if (WIDTH == 2) {
-      const uint64_t sb = (slot + 1) & mask;
-      uint64_t a0, a1, b0, b1;
-      ld_slot(J.key + 2 * slot, a0, a1);
-      ld_slot(J.key + 2 * sb, b0, b1);
-      if (slot_take(J, slot, a0, a1, w0, w1, is_long, c)) return;
-      if (slot_take(J, sb, b0, b1, w0, w1, is_long, c)) return;
-    } else {
-      uint64_t a0, a1;
-      ld_slot(J.key + 2 * slot, a0, a1);
-      if (slot_take(J, slot, a0, a1, w0, w1, is_long, c)) return;
-    }
-    slot = (slot + WIDTH) & mask;
+  for (int p = 0; p < MAX_PROBES; p += 2) {
+    uint64_t a0, a1, b0, b1;
+    ld_pair(J.key + 2 * slot, a0, a1, b0, b1);
+    if (slot_take(J, slot, a0, a1, w0, w1, is_long, c)) return;
+    if (slot_take(J, slot + 1, b0, b1, w0, w1, is_long, c)) return;
+    slot = (slot + 2) & mask;
   }
   atomicOr(J.state, 1u);
 }
@@ -285,12 +281,11 @@ __device__ inline void local_clear(WarpLocal& L) {
 }
 
 // Merge the warp's cache into the global container and empty it.
-template <int WIDTH = 2>
 __device__ inline void local_flush(WarpLocal& L, int& occ, const JobDev& J) {
   __syncwarp();
   for (int s = threadIdx.x & 31; s < LT; s += 32) {
     if (L.w1[s] != 0) {
-      global_insert<WIDTH>(J, L.w0[s], L.w1[s], L.h[s], L.cnt[s]);
+      global_insert(J, L.w0[s], L.w1[s], L.h[s], L.cnt[s]);
       L.w1[s] = 0;
     }
   }
@@ -319,75 +314,82 @@ __device__ __forceinline__ uint4 shift_window(const uint4& a, const uint4& b, ui
                     __funnelshift_r(t3, t4, r));
 }
 
-// Stage segment seg of the job (and its 64-byte halo) in the warp's buffer
-// W (members buf, wsb, starts), build the whitespace bitmap and the list of
-// token starts (segment-relative offsets of the tokens whose first byte lies
-// in the segment) and return how many there are.  All 32 lanes call this.
-// pre: when not null, the caller already loaded this lane's 16 bytes of the
-// segment (pre[0]) and, for lanes 0..3, of the halo (pre[1]) from a
-// 16-byte-aligned segment with at least BUF bytes left (seg_prefetchable).
+// Stage the segment that starts at byte base (32 * B::LANE bytes, and a halo)
+// in the warp's buffer W (members buf, starts), and list the tokens whose first
+// byte lies in it: first byte (segment-relative) | length << 12.  A token's
+// length comes from the whitespace bits of its lane and of the next one, so the
+// round that reads the token needs no bitmap (eight instructions and two
+// shared-memory loads less per token).  Returns how many there are.  All 32
+// lanes call this.
+// end: tokens that start there or beyond are left to another caller.
+// The loads are not issued a segment ahead: the 24 to 32 warps of an SM hide
+// them, and with the next segment's data held in registers the kernels were
+// slower (256 MB 419 against 414 us, a batch of 60 jobs 640 against 621).
 template <class B>
-__device__ inline int stage_tokens(const JobDev& J, uint64_t seg, B& L, const uint4* pre = nullptr) {
+__device__ inline int stage_tokens(const JobDev& J, uint64_t base, B& L, uint64_t end = ~0ull) {
+  constexpr int NCH = B::LANE / 16;  // 16-byte chunks per lane: chunk 32 c + lane
+  constexpr uint32_t SB = 32 * B::LANE, BUF = SB + HALO;
+  static_assert((NCH == 1 || NCH == 2) && HALO == 32 && sizeof(L.buf) == BUF, "segment layout");
   const int lane = threadIdx.x & 31;
-  const uint64_t base = seg * SEG;
   const uint8_t* __restrict__ in = J.in;
-  const uint64_t n = J.n;
-  const uint64_t rem = n - base;
+  const uint64_t rem = J.n - base;
   // stage the segment and its halo; bytes past the input end read as spaces
   const uintptr_t sa = reinterpret_cast<uintptr_t>(in + base);
-  uint4 mine;
-  if (pre) {
-    mine = pre[0];
-    reinterpret_cast<uint4*>(L.buf)[lane] = mine;
-    if (lane < HALO / 16) reinterpret_cast<uint4*>(L.buf)[32 + lane] = pre[1];
-  } else if (rem >= (uint64_t)BUF && (sa & 15) == 0) {
+  uint4* buf = reinterpret_cast<uint4*>(L.buf);
+  uint4 ch[NCH];
+  uint32_t before = ' ';  // the byte before the segment (lane 0)
+  if (lane == 0 && base) before = in[base - 1];
+  if (rem >= BUF && (sa & 15) == 0) {
     const uint4* src = reinterpret_cast<const uint4*>(sa);
-    mine = __ldg(src + lane);
-    reinterpret_cast<uint4*>(L.buf)[lane] = mine;
-    if (lane < HALO / 16) reinterpret_cast<uint4*>(L.buf)[32 + lane] = __ldg(src + 32 + lane);
-  } else if (rem >= (uint64_t)BUF) {
-    // unaligned input: the 37 aligned words covering the 576 staged bytes
-    // (each holds at least one input byte, so no load leaves the input's
-    // 16-byte blocks), shifted into place; lane l needs words l and l + 1,
-    // lanes 0..3 also words 32 + l and 33 + l for the halo
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) buf[32 * c + lane] = ch[c] = __ldg(src + 32 * c + lane);
+    if (lane < HALO / 16) buf[32 * NCH + lane] = __ldg(src + 32 * NCH + lane);
+  } else if (rem >= BUF) {
+    // unaligned input: the aligned words covering the staged bytes (each
+    // holds at least one input byte, so no load leaves the input's 16-byte
+    // blocks), shifted into place; chunk q needs words q and q + 1
     const uint32_t sh = (uint32_t)(sa & 15);
     const uint4* src = reinterpret_cast<const uint4*>(sa - sh);
-    const uint4 a = __ldg(src + lane);
-    const uint4 e = lane <= HALO / 16 ? __ldg(src + 32 + lane) : make_uint4(0u, 0u, 0u, 0u);
-    uint4 b = shfl_down_u4(a, 1), en = shfl_down_u4(e, 1);
-    const uint4 w32 = shfl_u4(e, 0);
-    if (lane == 31) b = w32;
-    mine = shift_window(a, b, sh);
-    reinterpret_cast<uint4*>(L.buf)[lane] = mine;
-    if (lane < HALO / 16) reinterpret_cast<uint4*>(L.buf)[32 + lane] = shift_window(e, en, sh);
-  } else {
-    for (uint32_t r = lane; r < (uint32_t)BUF; r += 32) L.buf[r] = r < rem ? in[base + r] : (uint8_t)' ';
-    __syncwarp();
-    mine = reinterpret_cast<const uint4*>(L.buf)[lane];
-  }
-  // token starts among this lane's 16 bytes (staged bytes past the input
-  // end are spaces, so the input end needs no test of its own)
-  const uint32_t wsm = byte_bits(ws_bytes(mine.x)) | (byte_bits(ws_bytes(mine.y)) << 4) |
-                       (byte_bits(ws_bytes(mine.z)) << 8) | (byte_bits(ws_bytes(mine.w)) << 12);
-  {
-    // whitespace bitmap of the staged bytes: the segment from the lanes'
-    // masks; the halo by lane l testing its bytes l and 32 + l, one ballot
-    // per 32 bytes
-    static_assert(HALO == 64, "the halo is two bitmap words");
-    __syncwarp();  // lanes 0..3 staged the halo
-    const uint32_t h0 = __ballot_sync(0xffffffffu, is_ws(L.buf[SEG + lane]));
-    const uint32_t h1 = __ballot_sync(0xffffffffu, is_ws(L.buf[SEG + 32 + lane]));
-    const uint32_t up = __shfl_down_sync(0xffffffffu, wsm, 1);
-    if ((lane & 1) == 0) L.wsb[lane >> 1] = (wsm & 0xFFFFu) | (up << 16);
-    if (lane == 0) {
-      L.wsb[SEG / 32] = h0;
-      L.wsb[SEG / 32 + 1] = h1;
-      L.wsb[BUF / 32] = 0xFFFFFFFFu;  // past the halo
+    uint4 a[NCH + 1];
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) a[c] = __ldg(src + 32 * c + lane);
+    a[NCH] = lane <= HALO / 16 ? __ldg(src + 32 * NCH + lane) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+      uint4 b = shfl_down_u4(a[c], 1);
+      const uint4 nx = shfl_u4(a[c + 1], 0);
+      if (lane == 31) b = nx;
+      buf[32 * c + lane] = ch[c] = shift_window(a[c], b, sh);
     }
+    const uint4 en = shfl_down_u4(a[NCH], 1);
+    if (lane < HALO / 16) buf[32 * NCH + lane] = shift_window(a[NCH], en, sh);
+  } else {
+    for (uint32_t r = lane; r < BUF; r += 32) L.buf[r] = r < rem ? in[base + r] : (uint8_t)' ';
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) ch[c] = buf[32 * c + lane];
   }
-  uint32_t prev = __shfl_up_sync(0xffffffffu, wsm >> 15, 1) & 1u;
-  if (lane == 0) prev = (base == 0) ? 1u : (uint32_t)is_ws(in[base - 1]);
-  const uint32_t start = ~wsm & ((wsm << 1) | prev) & 0xFFFFu;
+  // whitespace bits of this lane's B::LANE consecutive bytes (ws) and of the
+  // bytes after them (next)
+  uint32_t ws = ws_bits(ch[0]), next;
+  if (NCH == 2) {
+    const uint32_t p = ws | (ws_bits(ch[NCH - 1]) << 16);
+    const uint32_t p0 = __shfl_sync(0xffffffffu, p, 2 * lane), p1 = __shfl_sync(0xffffffffu, p, 2 * lane + 1);
+    ws = __byte_perm(p0, p1, lane < 16 ? 0x5410 : 0x7632);
+  }
+  __syncwarp();  // lanes 0 and 1 staged the halo
+  const uint32_t halo = __ballot_sync(0xffffffffu, is_ws(L.buf[SB + lane]));
+  next = __shfl_down_sync(0xffffffffu, ws, 1);
+  if (lane == 31) next = halo;
+  const uint32_t last = __ballot_sync(0xffffffffu, ws >> (B::LANE - 1));
+  const uint32_t first = __shfl_sync(0xffffffffu, (uint32_t)is_ws(before), 0);
+  const uint32_t prev = (((last << 1) | first) >> lane) & 1u;
+  uint32_t start = ~ws & ((ws << 1) | prev);
+  if (NCH == 1) {
+    start &= 0xFFFFu;
+    ws |= next << 16;
+  }
+  if (base + SB > end) start = low_bits(start, (int)(end - base) - lane * B::LANE);
   const int c = __popc(start);
   int incl = c;
 #pragma unroll
@@ -397,11 +399,13 @@ __device__ inline int stage_tokens(const JobDev& J, uint64_t seg, B& L, const ui
   }
   const int total = __shfl_sync(0xffffffffu, incl, 31);
   {
-    int o = incl - c;
+    uint16_t* o = L.starts + (incl - c);
     uint32_t m = start;
     while (m) {
-      const int j = __ffs(m) - 1;
-      L.starts[o++] = (uint16_t)(lane * 16 + j);
+      const uint32_t j = __ffs(m) - 1;
+      // the whitespace after byte j, 15 bytes of it
+      const uint32_t after = NCH == 1 ? ws >> (j + 1) : __funnelshift_rc(ws, next, j + 1);
+      *o++ = (uint16_t)((lane * B::LANE + j) | (__ffs(after & 0x7FFFu) << 12));
       m &= m - 1;
     }
   }
@@ -409,144 +413,169 @@ __device__ inline int stage_tokens(const JobDev& J, uint64_t seg, B& L, const ui
   return total;
 }
 
-// Whether segment seg can be staged from registers loaded ahead of time
-// (16-byte aligned, a full buffer of input left), and that load.
-__device__ __forceinline__ bool seg_prefetchable(const JobDev& J, uint64_t seg) {
-  return seg * SEG + BUF <= J.n && (reinterpret_cast<uintptr_t>(J.in + seg * SEG) & 15) == 0;
-}
-__device__ __forceinline__ void seg_prefetch(const JobDev& J, uint64_t seg, uint4 (&pre)[2]) {
-  const int lane = threadIdx.x & 31;
-  const uint4* src = reinterpret_cast<const uint4*>(J.in + seg * SEG);
-  pre[0] = __ldg(src + lane);
-  if (lane < HALO / 16) pre[1] = __ldg(src + 32 + lane);
-}
-
 // One warp maps and combines the tokens whose first byte lies in segment seg.
 // miss(lane_has_miss, token) is called by all 32 lanes after each round of
 // up to 32 tokens and disposes of the tokens the cache did not take.
-template <int WIDTH = 2, class Miss>
+template <class Miss>
 __device__ inline void warp_segment_t(const JobDev& J, uint64_t seg, WarpLocal& L, int& occ, Miss&& miss) {
   const int lane = threadIdx.x & 31;
   const uint64_t base = seg * SEG;
-  const int total = stage_tokens(J, seg, L);
+  const int total = stage_tokens(J, base, L);
   for (int r0 = 0; r0 < total; r0 += 32) {
     const int i = r0 + lane;
     const bool active = i < total;
     Tok t;
-    if (active) t = read_token(J.in, J.n, base, L, L.starts[i]);
-    else t.w0 = 0, t.w1 = 0, t.h = 0;
+    t = read_token(J.in, J.n, base, L, active ? L.starts[i] : 0u, active);
     const bool m = combine_local(L, active, t);
     miss(m, t);
     __syncwarp();
   }
   // occ counts segments since the last cache merge
-  if (++occ >= CACHE_EPOCH) local_flush<WIDTH>(L, occ, J);
+  if (++occ >= CACHE_EPOCH) local_flush(L, occ, J);
 }
 
 // ---------------------------------------------------------------------------
 // Local container of the plain map kernel for large inputs: one table per CTA
 // in shared memory, shared by its warps (the paper's bounded local table,
-// Sec. III-D, here per thread block).  Open addressing with two candidate
-// slots per key; a slot is claimed once and never changes key, so once a
-// CTA has seen a couple of thousand distinct keys the table is read-only
-// apart from its counts, and it holds the keys that were frequent early on
-// (for a Zipf-like stream, the hot ones).  A slot is {w0, w1} read with one
-// 128-bit load.  A claim CASes w1 from 0 to CT_BUSY, writes w0, hash and
-// count, fences and then stores w1.  Both words start at zero and keys whose
-// w0 is 0 (tokens of NUL bytes) never enter the table, so a read that meets
-// a claim half done (w1 already stored, w0 not yet seen) does not match and
-// the token goes on as a miss.  A key may end up in two slots (two lanes
-// claiming it at once); both counts reach the global container, which
-// merges them.
-constexpr unsigned long long CT_BUSY = 1ull;  // no key has w1 == 1 (its length byte is >= 1)
+// Sec. III-D, here per thread block).  Buckets of four slots; a slot is claimed
+// once and never changes key, so once a CTA has seen a few thousand distinct
+// keys the table is read-only apart from its counts, and it holds the keys that
+// were frequent early on (for a Zipf-like stream, the hot ones).
+//
+// A bucket's word of four 8-bit tags (of the hash; 0: empty) says which slot to
+// compare, so a token costs one 4-byte load and, if a tag matches, one 16-byte
+// load of that slot's key; most misses load no key at all.  (Two slots' keys in
+// turn, without tags, took 128 of the 360 us the map kernel spends on 256 MB of
+// 50,000 words; with tags a fifth less.)  A claim CASes the tag into the word and then
+// stores the key with one 16-byte store.  Keys start at zero and keys whose w0
+// is 0 (tokens of NUL bytes) never enter the table, so a read that meets a
+// claim half done does not match; that token, like one whose tag matches
+// another key's, goes on as a miss.  A key may end up in two slots (two lanes
+// claiming it at once) or also in the global container, which merges them.
 template <int NS>
 struct CtaTableT {
-  static constexpr int SLOTS = NS;  // a power of two
+  static constexpr int SLOTS = NS;  // a multiple of 4
   ulonglong2 key[NS];  // {w0, w1}
-  uint32_t h[NS];
   uint32_t cnt[NS];
+  uint32_t tag[NS / 4];
+  // all threads of the CTA
+  __device__ void clear() {
+    for (int i = threadIdx.x; i < NS; i += blockDim.x) {
+      key[i] = make_ulonglong2(0ull, 0ull);
+      cnt[i] = 0;
+      if (i < NS / 4) tag[i] = 0;
+    }
+  }
 };
 // the table of the large-input map kernel and the batch kernel (one CTA of
 // 32 warps per SM)
 using CtaTableBig = CtaTableT<4096>;
 
-// Per-warp state of the plain map kernel: the staged segment, its
-// whitespace bitmap and token list, and a queue of the tokens the table did
-// not take, which go to the global container 32 at a time (full warps, so
-// the global probing runs once per 32 misses instead of once per round).
+// Per-warp state beside such a table: the staged segment, its token list, and a
+// queue of the tokens the table did not take, which go to the global container
+// 32 at a time (full warps, so the global probing runs once per 32 misses
+// instead of once per round).  With 32 bytes a lane the segment's fixed work
+// (halo, scan) serves twice the tokens of 16, and the last round of up to 32
+// tokens is one in four or five instead of one in two or three (256 MB of
+// 50,000 words: 434 against 470 us).
 constexpr int MQ = 64;
 struct MapWarp {
-  uint8_t buf[BUF];
-  uint32_t wsb[BUF / 32 + 2];
-  uint16_t starts[SEG / 2];
+  static constexpr int LANE = 32;  // bytes of the segment per lane
+  uint8_t buf[32 * LANE + HALO];
+  uint16_t starts[16 * LANE];
   unsigned long long qw0[MQ], qw1[MQ];
   uint32_t qh[MQ];
 };
 static_assert(sizeof(CtaTableBig) % 16 == 0 && sizeof(MapWarp) % 16 == 0, "staging buffers must stay 16-byte aligned");
 
-// Count one short token in the CTA table; false if neither of its two
-// slots holds it or could be claimed for it (and for every long token).
+// The hash of a key of the table, all of which are short.
+__device__ __forceinline__ uint32_t cta_hash(const ulonglong2& k) {
+  return hash_short((uint32_t)k.x, (uint32_t)(k.x >> 32), (uint32_t)k.y, (uint32_t)(k.y >> 32));
+}
+
+// 0x80 in the zero bytes of v: exact up to and including the lowest one
+__device__ __forceinline__ uint32_t zero_bytes(uint32_t v) { return (v - 0x01010101u) & ~v & 0x80808080u; }
+
+// Count one token in the CTA table; false if it is long, or its bucket neither
+// holds it nor has a slot that could be claimed for it.
 template <class TT>
 __device__ __forceinline__ bool cta_add(TT& T, const Tok& t) {
-  if ((t.w1 >> 56) == 0xFF || t.w0 == 0) return false;
-  const uint32_t s0 = t.h & (TT::SLOTS - 1);
-#pragma unroll
-  for (int p = 0; p < 2; ++p) {
-    const uint32_t s = (s0 + p) & (TT::SLOTS - 1);
+  const bool able = (t.w1 >> 56) != 0xFF && t.w0 != 0;
+  const uint32_t b = __umulhi(t.h, TT::SLOTS / 4);
+  const uint32_t tag = max(t.h & 0xFFu, 1u);
+  const uint32_t tw = *reinterpret_cast<volatile uint32_t*>(&T.tag[b]);
+  const uint32_t z = able ? zero_bytes(tw ^ (tag * 0x01010101u)) : 0u;
+  bool hit = false;
+  if (z) {
+    const uint32_t s = 4 * b + (31 - __clz(z & -z)) / 8;
     unsigned long long k0, k1;
     asm volatile("ld.volatile.shared::cta.v2.u64 {%0, %1}, [%2];"
                  : "=l"(k0), "=l"(k1)
                  : "r"((uint32_t)__cvta_generic_to_shared(&T.key[s]))
                  : "memory");
-    if (k1 == t.w1 && k0 == t.w0) {
-      atomicAdd(&T.cnt[s], 1u);
-      return true;
-    }
-    if (k1 == 0 && atomicCAS(&T.key[s].y, 0ull, CT_BUSY) == 0ull) {
-      T.key[s].x = t.w0;
-      T.h[s] = t.h;
-      T.cnt[s] = 1u;
-      __threadfence_block();
-      *reinterpret_cast<volatile unsigned long long*>(&T.key[s].y) = t.w1;
-      return true;
+    hit = k1 == t.w1 && k0 == t.w0;
+    if (hit) atomicAdd(&T.cnt[s], 1u);
+  }
+  if (able && z == 0) {
+    const uint32_t e = zero_bytes(tw);
+    if (e) {
+      const uint32_t q = (31 - __clz(e & -e)) / 8, s = 4 * b + q;
+      hit = atomicCAS(&T.tag[b], tw, tw | (tag << (8 * q))) == tw;
+      if (hit) {
+        asm volatile("st.volatile.shared::cta.v2.u64 [%0], {%1, %2};" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(&T.key[s])),
+                     "l"(t.w0), "l"(t.w1)
+                     : "memory");
+        atomicAdd(&T.cnt[s], 1u);
+      }
     }
   }
-  return false;
+  return hit;
 }
 
-// Queue the round's misses (m: this lane has one); once 32 are queued, the
-// warp inserts the oldest 32 into the global container (WIDTH table slots
-// loaded per probe step; the batch kernel, whose many small jobs keep the
-// global tables in L2, is faster with one).  qn / qhd: queued entries and
-// queue head, warp-uniform.
-template <int WIDTH = 2>
-__device__ __forceinline__ void mq_push(const JobDev& J, MapWarp& W, bool m, const Tok& t, uint32_t& qn,
-                                        uint32_t& qhd) {
-  const int lane = threadIdx.x & 31;
-  const unsigned mm = __ballot_sync(0xffffffffu, m);
-  if (!mm) return;
-  if (m) {
-    const uint32_t pos = (qhd + qn + (uint32_t)__popc(mm & ((1u << lane) - 1u))) & (MQ - 1);
-    W.qw0[pos] = t.w0;
-    W.qw1[pos] = t.w1;
-    W.qh[pos] = t.h;
+// A warp's queue of misses: once 32 are queued, the warp inserts the oldest 32
+// into the global container (loading their slots a round ahead took longer: 434
+// against 417 us for 256 MB, 50,000 words).  Warp-uniform.
+struct MissQueue {
+  uint32_t n = 0, head = 0;  // queued entries, the oldest
+
+  // m: this lane has a miss
+  __device__ __forceinline__ void push(const JobDev& J, MapWarp& W, bool m, const Tok& t) {
+    const int lane = threadIdx.x & 31;
+    const unsigned mm = __ballot_sync(0xffffffffu, m);
+    if (!mm) return;
+    if (m) {
+      const uint32_t pos = (head + n + (uint32_t)__popc(mm & ((1u << lane) - 1u))) & (MQ - 1);
+      W.qw0[pos] = t.w0;
+      W.qw1[pos] = t.w1;
+      W.qh[pos] = t.h;
+    }
+    n += (uint32_t)__popc(mm);
+    if (n >= 32) {
+      __syncwarp();
+      const uint32_t e = (head + (uint32_t)lane) & (MQ - 1);
+      global_insert(J, W.qw0[e], W.qw1[e], W.qh[e], 1);
+      head = (head + 32) & (MQ - 1);
+      n -= 32;
+    }
   }
-  qn += (uint32_t)__popc(mm);
-  if (qn >= 32) {
+  __device__ __forceinline__ void drain(const JobDev& J, MapWarp& W) {
+    const uint32_t lane = threadIdx.x & 31;
     __syncwarp();
-    const uint32_t q = (qhd + (uint32_t)lane) & (MQ - 1);
-    global_insert<WIDTH>(J, W.qw0[q], W.qw1[q], W.qh[q], 1);
-    qhd = (qhd + 32) & (MQ - 1);
-    qn -= 32;
+    if (lane < n) {
+      const uint32_t e = (head + lane) & (MQ - 1);
+      global_insert(J, W.qw0[e], W.qw1[e], W.qh[e], 1);
+    }
+    n = head = 0;
+    __syncwarp();
   }
-}
+};
 
 // The direct form: a token the cache did not take goes straight to the
 // global container.
-template <int WIDTH = 2>
 __device__ inline void warp_segment(const JobDev& J, uint64_t seg, WarpLocal& L, int& occ) {
-  warp_segment_t<WIDTH>(J, seg, L, occ, [&](bool m, const Tok& t) {
-    if (m) global_insert<WIDTH>(J, t.w0, t.w1, t.h, 1);
+  warp_segment_t(J, seg, L, occ, [&](bool m, const Tok& t) {
+    if (m) global_insert(J, t.w0, t.w1, t.h, 1);
   });
 }
 

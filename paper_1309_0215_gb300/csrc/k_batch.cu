@@ -187,7 +187,7 @@ batch_kernel(const BatchJob* __restrict__ jobs, uint32_t njobs, uint64_t total_t
   const int lane = threadIdx.x & 31;
   int64_t cur = -1;
   uint32_t kind = 0, cont = 0;
-  uint32_t qn = 0, qhd = 0;  // this warp's queued misses (word count)
+  wc::MissQueue mq;  // this warp's misses (word count)
 
   auto flush = [&](const BatchJob& J) {
     if (kind == MR_HIST_RGB8 && cont != MR_C_GLOBAL_ARRAY) {
@@ -203,16 +203,11 @@ batch_kernel(const BatchJob* __restrict__ jobs, uint32_t njobs, uint64_t total_t
     } else if (kind == MR_WORDCOUNT) {
       // every warp's queued misses, then the CTA's table, into the job's
       // global container
-      __syncwarp();
-      if ((uint32_t)lane < qn) {
-        const uint32_t q = (qhd + (uint32_t)lane) & (wc::MQ - 1);
-        wc::global_insert(s_jd, W.qw0[q], W.qw1[q], W.qh[q], 1);
-      }
-      qn = qhd = 0;
+      mq.drain(s_jd, W);
       __syncthreads();
       for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += BT) {
         const ulonglong2 k = T.key[i];
-        if (k.y != 0) wc::global_insert(s_jd, k.x, k.y, T.h[i], T.cnt[i]);
+        if (k.y != 0) wc::global_insert(s_jd, k.x, k.y, wc::cta_hash(k), T.cnt[i]);
       }
       __syncthreads();
     }
@@ -225,8 +220,7 @@ batch_kernel(const BatchJob* __restrict__ jobs, uint32_t njobs, uint64_t total_t
       __syncthreads();
     } else if (kind == MR_WORDCOUNT) {
       if (threadIdx.x == 0) s_jd = J.wc;
-      for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += BT) T.key[i] = make_ulonglong2(0ull, 0ull);
-      qn = qhd = 0;
+      T.clear();
       __syncthreads();
     }
   };
@@ -250,33 +244,20 @@ batch_kernel(const BatchJob* __restrict__ jobs, uint32_t njobs, uint64_t total_t
     }
     const uint64_t local = t - J.tile_begin;
     if (J.kind == MR_WORDCOUNT) {
-      const uint64_t s0 = local * (wc_tile / wc::SEG);
-      uint64_t s1 = s0 + wc_tile / wc::SEG;
-      const uint64_t nseg = (J.n + wc::SEG - 1) / wc::SEG;
-      if (s1 > nseg) s1 = nseg;
+      uint64_t end = (local + 1) * wc_tile;
+      if (end > J.n) end = J.n;
       // the job's descriptor from shared memory (copied at the job switch):
       // through a reference to global memory every use in the hot loop would
       // be a global reload, and a register copy would not fit
-      const uint64_t w0 = s0 + (threadIdx.x >> 5);
-      uint4 pre[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-      bool have = w0 < s1 && wc::seg_prefetchable(s_jd, w0);
-      if (have) wc::seg_prefetch(s_jd, w0, pre);
-      for (uint64_t sg = w0; sg < s1; sg += BWARPS) {
-        const uint64_t base = sg * wc::SEG;
-        uint4 cp[2] = {pre[0], pre[1]};
-        const bool cp_ok = have;
-        have = sg + BWARPS < s1 && wc::seg_prefetchable(s_jd, sg + BWARPS);
-        if (have) wc::seg_prefetch(s_jd, sg + BWARPS, pre);
-        const int total = wc::stage_tokens(s_jd, sg, W, cp_ok ? cp : nullptr);
+      constexpr uint64_t SB = 32 * wc::MapWarp::LANE, step = BWARPS * SB;
+      for (uint64_t base = local * wc_tile + (threadIdx.x >> 5) * SB; base < end; base += step) {
+        const int total = wc::stage_tokens(s_jd, base, W, end);
         for (int r0 = 0; r0 < total; r0 += 32) {
           const int i = r0 + lane;
-          bool m = false;
-          wc::Tok tk{0, 0, 0};
-          if (i < total) {
-            tk = wc::read_token(s_jd.in, s_jd.n, base, W, W.starts[i]);
-            m = !wc::cta_add(T, tk);
-          }
-          wc::mq_push<1>(s_jd, W, m, tk, qn, qhd);
+          const bool active = i < total;
+          const wc::Tok tk = wc::read_token(s_jd.in, s_jd.n, base, W, active ? W.starts[i] : 0u, active);
+          const bool hit = wc::cta_add(T, tk);
+          mq.push(s_jd, W, active && !hit, tk);
           __syncwarp();
         }
       }

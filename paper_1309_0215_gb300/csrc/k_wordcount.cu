@@ -53,12 +53,15 @@ constexpr int MAP_WARPS = 8;                 // per-warp-cache map kernel: 5 CTA
 constexpr int MAP_THREADS = MAP_WARPS * 32;
 constexpr int CTA_WARPS = 32;               // CTA-table map kernel: 1 CTA per SM
 constexpr int CTA_THREADS = CTA_WARPS * 32;
-// From this input size on the plain map pass uses the CTA-table kernel for a
-// 16-byte-aligned input (whose next segment each warp loads ahead): each CTA
-// then sees enough tokens (tens of thousands) that its table pays for its
-// final merge of up to 4,096 keys into the global container (at 16 MiB the
-// two kernels take the same time, at 48 MiB this one 6% less).
-constexpr uint64_t CTA_MAP_MIN_BYTES = 32ull << 20;
+constexpr int MAP_CTA_SEG = 32 * wc::MapWarp::LANE;
+// From this input size on the plain map pass uses the CTA-table kernel: each
+// CTA then sees enough tokens (thousands) that its table pays for its final
+// merge of up to 4,096 keys into the global container.  Whole calls, per-warp
+// caches against CTA tables: 256 KiB of 5,000 words 92 and 99 us, 1 MiB of
+// 20,000 words 102 and 106, 4 MiB of 1,000 words 92.7 and 89.8, of 50,000 words
+// 121 and 121, 8 MiB of 50,000 longer words 182 and 167, 16 MiB of 90,000 words
+// 168 and 173, of 1,000 words 111 and 104.
+constexpr uint64_t CTA_MAP_MIN_BYTES = 4ull << 20;
 constexpr int CB = 1024;            // records per compaction / sort / scan block
 constexpr uint64_t CNT_MAX = (1ull << 40) - 1;
 
@@ -78,58 +81,44 @@ __global__ void __launch_bounds__(MAP_THREADS, 5) wc_map_kernel(JobDev J) {
   const uint64_t nseg = (J.n + wc::SEG - 1) / wc::SEG;
   const uint64_t gw = (uint64_t)blockIdx.x * MAP_WARPS + (threadIdx.x >> 5);
   const uint64_t nw = (uint64_t)gridDim.x * MAP_WARPS;
-  for (uint64_t seg = gw; seg < nseg; seg += nw) wc::warp_segment<1>(J, seg, L, occ);
-  wc::local_flush<1>(L, occ, J);
+  for (uint64_t seg = gw; seg < nseg; seg += nw) wc::warp_segment(J, seg, L, occ);
+  wc::local_flush(L, occ, J);
 }
 
 // Plain map + combine pass for large inputs: one CTA of CTA_WARPS warps per
 // SM, sharing one local table (wc::CtaTableBig, 4,096 slots); a warp's
 // misses are queued and sent to the global container 32 at a time; at the
 // end every warp empties its queue and the CTA merges its table into the
-// global container.
+// global container.  Bounded by instruction issue and shared-memory bandwidth
+// (72% and 65% of their peaks; 0.83 TB/s of text): 256 MB, 50,000 words, 386 ->
+// 306 us, by 1,024-byte segments, lengths taken with the token list, tagged
+// buckets and pair loads in the global table.
 __global__ void __launch_bounds__(CTA_THREADS, 1) wc_map_cta_kernel(JobDev J) {
   extern __shared__ __align__(16) unsigned char wc_smem[];
   wc::CtaTableBig& T = *reinterpret_cast<wc::CtaTableBig*>(wc_smem);
   wc::MapWarp& W = reinterpret_cast<wc::MapWarp*>(wc_smem + sizeof(wc::CtaTableBig))[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += CTA_THREADS) T.key[i] = make_ulonglong2(0ull, 0ull);
+  T.clear();
   __syncthreads();
-  const uint64_t nseg = (J.n + wc::SEG - 1) / wc::SEG;
-  const uint64_t gw = (uint64_t)blockIdx.x * CTA_WARPS + (threadIdx.x >> 5);
-  const uint64_t nw = (uint64_t)gridDim.x * CTA_WARPS;
-  uint32_t qn = 0, qhd = 0;
-  // the warp's next segment is loaded while it works on the current one
-  uint4 pre[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-  bool have = gw < nseg && wc::seg_prefetchable(J, gw);
-  if (have) wc::seg_prefetch(J, gw, pre);
-  for (uint64_t seg = gw; seg < nseg; seg += nw) {
-    const uint64_t base = seg * wc::SEG;
-    uint4 cur[2] = {pre[0], pre[1]};
-    const bool cur_ok = have;
-    have = seg + nw < nseg && wc::seg_prefetchable(J, seg + nw);
-    if (have) wc::seg_prefetch(J, seg + nw, pre);
-    const int total = wc::stage_tokens(J, seg, W, cur_ok ? cur : nullptr);
+  constexpr uint64_t SB = MAP_CTA_SEG;
+  const uint64_t step = (uint64_t)gridDim.x * CTA_WARPS * SB;
+  wc::MissQueue mq;
+  for (uint64_t base = ((uint64_t)blockIdx.x * CTA_WARPS + (threadIdx.x >> 5)) * SB; base < J.n; base += step) {
+    const int total = wc::stage_tokens(J, base, W);
     for (int r0 = 0; r0 < total; r0 += 32) {
       const int i = r0 + lane;
-      bool m = false;
-      wc::Tok t{0, 0, 0};
-      if (i < total) {
-        t = wc::read_token(J.in, J.n, base, W, W.starts[i]);
-        m = !wc::cta_add(T, t);
-      }
-      wc::mq_push(J, W, m, t, qn, qhd);
+      const bool active = i < total;
+      const wc::Tok t = wc::read_token(J.in, J.n, base, W, active ? W.starts[i] : 0u, active);
+      const bool hit = wc::cta_add(T, t);
+      mq.push(J, W, active && !hit, t);
       __syncwarp();
     }
   }
-  __syncwarp();
-  if ((uint32_t)lane < qn) {
-    const uint32_t q = (qhd + (uint32_t)lane) & (wc::MQ - 1);
-    wc::global_insert(J, W.qw0[q], W.qw1[q], W.qh[q], 1);
-  }
+  mq.drain(J, W);
   __syncthreads();
   for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += CTA_THREADS) {
     const ulonglong2 k = T.key[i];
-    if (k.y != 0) wc::global_insert(J, k.x, k.y, T.h[i], T.cnt[i]);
+    if (k.y != 0) wc::global_insert(J, k.x, k.y, wc::cta_hash(k), T.cnt[i]);
   }
 }
 
@@ -2617,12 +2606,12 @@ cudaError_t launch_wordcount(const uint8_t* in, uint64_t n, const WcBuffers& b, 
     wc_pipe_kernel<<<(unsigned)grid, PIPE_THREADS, smem, s>>>(J, pipe_polls < 0 ? PIPE_SPIN_LIMIT : pipe_polls);
     if ((e = cudaGetLastError()) != cudaSuccess || (e = kt_end(kt, s)) != cudaSuccess) return e;
     ++*nk;
-  } else if (n >= CTA_MAP_MIN_BYTES && (reinterpret_cast<uintptr_t>(in) & 15) == 0) {
+  } else if (n >= CTA_MAP_MIN_BYTES) {
     const int smem = wc_map_cta_smem_bytes();
     if ((e = cudaFuncSetAttribute(wc_map_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
         cudaSuccess)
       return e;
-    const uint64_t nseg = (n + wc::SEG - 1) / wc::SEG;
+    const uint64_t nseg = (n + MAP_CTA_SEG - 1) / MAP_CTA_SEG;
     uint64_t grid = (nseg + CTA_WARPS - 1) / CTA_WARPS;
     const uint64_t gmax = (uint64_t)di.sms;
     if (grid > gmax) grid = gmax;

@@ -234,3 +234,22 @@ def test_wc_small_texts_one_cta(mr, name, text):
         view = buf[off: off + len(text)]
         assert mr.wordcount(view) == want, off
     assert mr.wordcount(view, wc_slots=1 << 14) == want
+
+
+@pytest.mark.parametrize("extra,off", [(0, 0), (1, 1), (1023, 7), (1025, 16), (40_000, 9)])
+def test_wc_cta_table_pass(mr, extra, off):
+    """Texts from 4 MiB on (one table per CTA, 1,024-byte segments), aligned and
+    not: words of 1 to 20 bytes (15 and 16 part short from long keys), NUL and
+    high bytes, runs of delimiters, more keys than a table holds, an open end."""
+    rng = np.random.default_rng(extra + off)
+    n = (4 << 20) + extra
+    lens = rng.integers(1, 21, 9_000)
+    vocab = [rng.integers(97, 123, ln).astype(np.uint8).tobytes() for ln in lens]
+    vocab += [b"\x00", b"\x00" * 9, b"\x00" * 16, b"\xff" * 15, b"\xa0", b"\x85b", b"x" * 15, b"x" * 16, b"y" * 400]
+    w = rng.zipf(1.3, 700_000) % len(vocab)
+    seps = (b" ", b"\n", b"  ", b"\t\r\n", b"\x0b\x0c")
+    pick = rng.integers(0, len(seps), len(w))
+    text = b"".join(vocab[i] + seps[j] for i, j in zip(w, pick))
+    text = (text * (n // len(text) + 1))[: n - 1] + b"q"
+    got = mr.wordcount(_dev(text, off))
+    assert got == oracle.wordcount(text)
