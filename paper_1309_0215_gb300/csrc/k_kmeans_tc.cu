@@ -8,8 +8,9 @@
 //   * for D = 64 one producer thread moves each FP32 tile (128 rows, 32 KB,
 //     contiguous) into a two-deep shared-memory ring with one bulk copy
 //     (cp.async.bulk, completion counted on an mbarrier), so loads stay in
-//     flight without registers; 8 converter warps read the tile (or load it
-//     themselves for other D), compute ||x||^2 in FP32, and write BF16
+//     flight without registers; 8 converter warps read the tile (rows
+//     of the filter's list they fetch themselves, by 16-byte asynchronous copies a
+//     tile ahead; for other D they load the values as they need them), compute ||x||^2 in FP32, and write BF16
 //     operands in the 128-byte-swizzled K-major layout the MMA reads.  With TERMS = 3 each value is split as
 //     x = hi + lo (hi = bf16(x), lo = bf16(x - hi)) and the MMA accumulates
 //     hi.hi + hi.lo + lo.hi, so the cross term is good to about 2^-15
@@ -56,6 +57,8 @@
 // them the point needs an exact choice between those few alone, else it is
 // listed and compared with every centroid (km_settle_kernel either way), so
 // assignments equal the FP64 argmin.
+#include <type_traits>
+
 #include "dev_tc.cuh"
 
 namespace mrgb {
@@ -104,6 +107,13 @@ struct __align__(1024) TcSmem {
 
 static_assert(sizeof(TcSmem) + 1024 <= 232448, "shared memory of one CTA");
 
+// a load that stays where it is written (its value is used a tile later)
+__device__ __forceinline__ uint32_t ld_now(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 template <int TERMS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, const float* __restrict__ c, uint32_t k,
@@ -146,10 +156,13 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
   const uint32_t n = idx ? *nact : n_all;
   const uint32_t ntiles = (n + TM - 1) / TM;
   if (threadIdx.x == 0) {
-    // a tile's copy arrives once, a listed tile's rows once per lane of the copying warp
-    for (int q = 0; q < XST; ++q) mbar_init(&S.tfull[q], idx ? 32 : 1);
+    for (int q = 0; q < XST; ++q) mbar_init(&S.tfull[q], 1);
     fence_mbar_init();
   }
+  // Points of KD aligned values are staged in shared memory: whole tiles by the
+  // copy engine, the rows of the filter's list by the converters.
+  const bool vec = d == KD && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
+  const bool gather = vec && idx, bulk = vec && !idx;
   // centroid operands (rows >= k and dims >= d are zero) and norms
   for (uint32_t t = threadIdx.x; t < npad * (KD / 2); t += blockDim.x) {
     const uint32_t row = t / (KD / 2), pr = t % (KD / 2);
@@ -186,142 +199,155 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
     // swizzled BF16 rows: no shared-memory bank conflicts.
     const int cw = warp - CVT_WARP0;
     const int col = lane & 15, rsub = lane >> 4;
-    const bool vec = d == KD && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
     float mv[4];  // the shift of this lane's four dimensions
 #pragma unroll
     for (int j = 0; j < 4; ++j) mv[j] = 4u * col + j < d ? center[4 * col + j] : 0.f;
-    unsigned int mabs = 0;  // bits of max |x| over the values this thread converts (non-negative floats order as ints)
-    for (uint32_t i = 0;; ++i) {
-      const uint32_t tile = blockIdx.x + i * gridDim.x;
-      if (tile >= ntiles) break;
-      const int s = (int)(i % STAGES);
-      const uint32_t u = i / STAGES;
-      const int q2 = (int)(i % XST);
-      if (vec) {
-        // the tile was staged by the bulk copy engine
-        const bool okt = mbar_wait(&S.tfull[q2], (i / XST) & 1, err, polls);
-        if (!__all_sync(0xffffffffu, okt)) break;
+    // Listed rows: each warp fetches its own rows of the next tile while it
+    // converts this one, 16 bytes a lane and two rows per instruction, the row
+    // numbers a tile ahead of that.  (By the copy warp, through the barriers of
+    // the staging ring, each tile waited for the row numbers, the copies and a
+    // hand-over in turn: 3.3M of 4M listed points 517 us, now 431; one bulk
+    // copy per row 817.)
+    const uint32_t r0w = CVT_ROWS * cw;
+    auto list_row = [&](uint32_t t) {
+      const uint32_t r = t * TM + r0w + lane;
+      return t < ntiles && lane < CVT_ROWS && r < n ? ld_now(idx + r) : BEYOND;
+    };
+    auto fetch = [&](uint32_t listed, uint32_t slot) {  // lane r: row r
+#pragma unroll
+      for (int t = 0; t < CVT_ROWS / 2; ++t) {
+        const uint32_t r = 2 * t + rsub, p = __shfl_sync(0xffffffffu, listed, r);
+        if (p != BEYOND) cp_async16(&S.xs[slot][(r0w + r) * KD + 4 * col], x + (uint64_t)p * KD + 4 * col);
       }
-      bool ok = true;
-      for (int hf = 0; hf < CVT_ROWS / 16; ++hf) {
-        const int r0 = CVT_ROWS * cw + 16 * hf;
-        float4 v[8];
-        if (vec) {
+      cp_async_commit();
+    };
+    static_assert(CVT_ROWS <= 32 && XST == 2, "a lane per row; two fetched tiles");
+    unsigned int mabs = 0;  // bits of max |x| over the values this thread converts (non-negative floats order as ints)
+    // (a loop of its own for listed rows: sharing one cost the other paths 5%)
+    auto convert = [&](auto gather_t) {
+      constexpr bool GATHER = decltype(gather_t)::value;
+      uint32_t listed = 0;  // the rows of the tile fetched next
+      if (GATHER) {
+        fetch(list_row(blockIdx.x), 0);
+        listed = list_row(blockIdx.x + gridDim.x);
+      }
+      for (uint32_t i = 0;; ++i) {
+        const uint32_t tile = blockIdx.x + i * gridDim.x;
+        if (tile >= ntiles) break;
+        const int s = (int)(i % STAGES);
+        const uint32_t u = i / STAGES;
+        const int q2 = (int)(i % XST);
+        if (!GATHER && vec) {
+          // the tile was staged by the bulk copy engine
+          const bool okt = mbar_wait(&S.tfull[q2], (i / XST) & 1, err, polls);
+          if (!__all_sync(0xffffffffu, okt)) break;
+        } else if (GATHER) {
+          fetch(listed, (i + 1) & 1);
+          listed = list_row(tile + 2 * gridDim.x);
+          cp_async_wait<1>();
+          __syncwarp();
+        }
+        bool ok = true;
+        for (int hf = 0; hf < CVT_ROWS / 16; ++hf) {
+          const int r0 = CVT_ROWS * cw + 16 * hf;
+          float4 v[8];
+          if (GATHER || vec) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const int rr = r0 + 2 * q + rsub;
+              v[q] = tile * TM + rr < n ? *reinterpret_cast<const float4*>(&S.xs[q2][rr * KD + 4 * col])
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const uint32_t p = tile * TM + r0 + 2 * q + rsub;
+              const uint32_t d0 = 4 * col;
+              const float* row = x + (uint64_t)(idx && p < n ? idx[p] : p) * d;
+              v[q].x = (p < n && d0 < d) ? row[d0] : 0.f;
+              v[q].y = (p < n && d0 + 1 < d) ? row[d0 + 1] : 0.f;
+              v[q].z = (p < n && d0 + 2 < d) ? row[d0 + 2] : 0.f;
+              v[q].w = (p < n && d0 + 3 < d) ? row[d0 + 3] : 0.f;
+            }
+          }
+          if (hf == 0 && i >= STAGES) {
+            ok = mbar_wait(&S.empty_a[s], (u + 1) & 1, err, polls);
+            ok = ok && mbar_wait(&S.nx_free[s], (u + 1) & 1, err, polls);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+          }
+          float ss[8];  // this lane's part of its eight rows' norms
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             const int rr = r0 + 2 * q + rsub;
-            v[q] = tile * TM + rr < n ? *reinterpret_cast<const float4*>(&S.xs[q2][rr * KD + 4 * col])
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (maxabs)
+              mabs = max(mabs, max(max(__float_as_uint(fabsf(v[q].x)), __float_as_uint(fabsf(v[q].y))),
+                                   max(__float_as_uint(fabsf(v[q].z)), __float_as_uint(fabsf(v[q].w)))));
+            v[q].x = __fsub_rn(v[q].x, mv[0]);
+            v[q].y = __fsub_rn(v[q].y, mv[1]);
+            v[q].z = __fsub_rn(v[q].z, mv[2]);
+            v[q].w = __fsub_rn(v[q].w, mv[3]);
+            ss[q] = fmaf(v[q].w, v[q].w, fmaf(v[q].z, v[q].z, fmaf(v[q].y, v[q].y, v[q].x * v[q].x)));
+            uint32_t hi0, lo0, hi1, lo1;
+            split2(v[q].x, v[q].y, hi0, lo0);
+            split2(v[q].z, v[q].w, hi1, lo1);
+            const uint32_t off = swz(rr, col >> 1) + (uint32_t)(col & 1) * 8u;
+            *reinterpret_cast<uint2*>(S.a_hi[s] + off) = make_uint2(hi0, hi1);
+            if (TERMS == 3) *reinterpret_cast<uint2*>(S.a_lo[s] + off) = make_uint2(lo0, lo1);
           }
-        } else {
+          // the 16 lanes' sums of eight rows at once: half of the rows stay at
+          // each exchange (8 shuffles in place of 32)
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const uint32_t p = tile * TM + r0 + 2 * q + rsub;
-            const uint32_t d0 = 4 * col;
-            const float* row = x + (uint64_t)(idx && p < n ? idx[p] : p) * d;
-            v[q].x = (p < n && d0 < d) ? row[d0] : 0.f;
-            v[q].y = (p < n && d0 + 1 < d) ? row[d0 + 1] : 0.f;
-            v[q].z = (p < n && d0 + 2 < d) ? row[d0 + 2] : 0.f;
-            v[q].w = (p < n && d0 + 3 < d) ? row[d0 + 3] : 0.f;
+          for (int w = 4; w; w >>= 1) {
+            const bool up = col & 2 * w;
+#pragma unroll
+            for (int q = 0; q < w; ++q)
+              ss[q] = (up ? ss[q + w] : ss[q]) + __shfl_xor_sync(0xffffffffu, up ? ss[q] : ss[q + w], 2 * w);
           }
+          ss[0] += __shfl_xor_sync(0xffffffffu, ss[0], 1);
+          if ((col & 1) == 0) S.nx[s][r0 + 2 * (col >> 1) + rsub] = ss[0];
         }
-        if (hf == 0 && i >= STAGES) {
-          ok = mbar_wait(&S.empty_a[s], (u + 1) & 1, err, polls);
-          ok = ok && mbar_wait(&S.nx_free[s], (u + 1) & 1, err, polls);
-          ok = __all_sync(0xffffffffu, ok);
-          if (!ok) break;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int rr = r0 + 2 * q + rsub;
-          if (maxabs)
-            mabs = max(mabs, max(max(__float_as_uint(fabsf(v[q].x)), __float_as_uint(fabsf(v[q].y))),
-                                 max(__float_as_uint(fabsf(v[q].z)), __float_as_uint(fabsf(v[q].w)))));
-          v[q].x = __fsub_rn(v[q].x, mv[0]);
-          v[q].y = __fsub_rn(v[q].y, mv[1]);
-          v[q].z = __fsub_rn(v[q].z, mv[2]);
-          v[q].w = __fsub_rn(v[q].w, mv[3]);
-          float ss = fmaf(v[q].w, v[q].w, fmaf(v[q].z, v[q].z, fmaf(v[q].y, v[q].y, v[q].x * v[q].x)));
-          ss += __shfl_xor_sync(0xffffffffu, ss, 8);
-          ss += __shfl_xor_sync(0xffffffffu, ss, 4);
-          ss += __shfl_xor_sync(0xffffffffu, ss, 2);
-          ss += __shfl_xor_sync(0xffffffffu, ss, 1);
-          if (col == 0) S.nx[s][rr] = ss;
-          uint32_t hi0, lo0, hi1, lo1;
-          split2(v[q].x, v[q].y, hi0, lo0);
-          split2(v[q].z, v[q].w, hi1, lo1);
-          const uint32_t off = swz(rr, col >> 1) + (uint32_t)(col & 1) * 8u;
-          *reinterpret_cast<uint2*>(S.a_hi[s] + off) = make_uint2(hi0, hi1);
-          if (TERMS == 3) *reinterpret_cast<uint2*>(S.a_lo[s] + off) = make_uint2(lo0, lo1);
+        if (!ok) break;
+        // The staging buffer is released only here: the bulk copy engine writes
+        // through the async proxy, so the shared loads above must be ordered
+        // before its next fill by this proxy fence (the stores that consumed
+        // them precede it), not just by the mbarrier arrive.
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&S.full_a[s]);
+          if (!GATHER && vec) mbar_arrive(&S.tempty[q2]);
         }
       }
-      if (!ok) break;
-      // The staging buffer is released only here: the bulk copy engine writes
-      // through the async proxy, so the shared loads above must be ordered
-      // before its next fill by this proxy fence (the stores that consumed
-      // them precede it), not just by the mbarrier arrive.
-      fence_proxy_async();
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&S.full_a[s]);
-        if (vec) mbar_arrive(&S.tempty[q2]);
-      }
-    }
+      if (GATHER) cp_async_wait<0>();
+    };
+    if (gather) convert(std::true_type{});
+    else convert(std::false_type{});
     if (maxabs) {
       for (int o = 16; o; o >>= 1) mabs = max(mabs, __shfl_xor_sync(0xffffffffu, mabs, o));
       if (lane == 0) atomicMax(maxabs, mabs);
     }
   } else if (warp == TMA_WARP) {
     // ------------------------------------------------- bulk-copy producer
-    // One bulk copy per tile; listed rows by 16-byte asynchronous copies, two
-    // rows per warp instruction (one bulk copy per row took 75 cycles of the
-    // copy engine each: 817 us for
-    // 3.3M listed points when the finalizers were not yet the limit).
-    if (d == KD && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
+    // one bulk copy per tile
+    if (bulk && lane == 0) {
       uint32_t issued = 0;
       for (uint32_t i = 0;; ++i) {
         const uint32_t tile = blockIdx.x + i * gridDim.x;
         if (tile >= ntiles || (stop_copies && i >= stop_copies)) break;
         const int q2 = (int)(i % XST);
         const uint32_t rows = (n - tile * TM) < (uint32_t)TM ? (n - tile * TM) : (uint32_t)TM;
-        uint32_t row[TM / 32];
-        if (idx) {
-#pragma unroll
-          for (int q = 0; q < TM / 32; ++q) row[q] = q * 32 + lane < (int)rows ? idx[tile * TM + q * 32 + lane] : 0;
-        }
-        bool ok = true;
-        if (lane == 0) {
-          ok = i < XST || mbar_wait(&S.tempty[q2], ((i / XST) + 1) & 1, err, polls);
-          if (ok && !idx) {
-            mbar_expect_tx(&S.tfull[q2], rows * KD * 4);
-            bulk_g2s(S.xs[q2], x + (uint64_t)tile * TM * KD, rows * KD * 4, &S.tfull[q2]);
-          }
-        }
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        if (idx) {
-          const uint32_t half = (uint32_t)lane >> 4, part = (uint32_t)lane & 15;
-#pragma unroll
-          for (int q = 0; q < TM / 32; ++q)
-#pragma unroll 4
-            for (int t = 0; t < 16; ++t) {
-              const uint32_t rr = q * 32 + 2 * t + half;
-              const uint32_t r = __shfl_sync(0xffffffffu, row[q], 2 * t + half);
-              if (rr < rows) cp_async16(S.xs[q2] + rr * KD + 4 * part, x + (uint64_t)r * KD + 4 * part);
-            }
-          cp_async_arrive(&S.tfull[q2]);
-        }
+        if (i >= XST && !mbar_wait(&S.tempty[q2], ((i / XST) + 1) & 1, err, polls)) break;
+        mbar_expect_tx(&S.tfull[q2], rows * KD * 4);
+        bulk_g2s(S.xs[q2], x + (uint64_t)tile * TM * KD, rows * KD * 4, &S.tfull[q2]);
         ++issued;
       }
       // No copy may still be landing in shared memory when the CTA exits.
       // Copy i was issued only after the converters released copy i - XST
       // (which they do after its completion), so only the last XST copies
       // can be in flight; wait for them even when a wait gave up elsewhere.
-      if (idx) cp_async_wait_all();
-      __syncwarp();
-      if (lane == 0 && !idx)
-        for (uint32_t i = issued > (uint32_t)XST ? issued - XST : 0; i < issued; ++i)
-          mbar_drain(&S.tfull[i % XST], (i / XST) & 1);
+      for (uint32_t i = issued > (uint32_t)XST ? issued - XST : 0; i < issued; ++i)
+        mbar_drain(&S.tfull[i % XST], (i / XST) & 1);
     }
     __syncwarp();
   } else if (warp == MMA_WARP) {
