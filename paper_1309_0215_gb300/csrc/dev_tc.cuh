@@ -15,9 +15,10 @@ constexpr int TM = 128;          // points per tile = MMA M = TMEM lanes
 constexpr int KD = 64;           // dimensions per operand tile: one 128-byte row of BF16
 constexpr int NMAX = 256;        // centroids per accumulator: MMA N
 constexpr int QUARTERS = 4;      // column quarters of an accumulator, one epilogue warp each per lane quadrant
-constexpr int EPI_COLS = NMAX / QUARTERS;  // 64 columns per epilogue warp
-constexpr int NSET = 4;           // independent running top-2s per epilogue thread
-constexpr int CHUNK = 32;         // TMEM columns per tcgen05.ld in the epilogue
+constexpr int EPI_COLS = NMAX / QUARTERS;  // at most 64 columns per epilogue warp
+constexpr int GRID = 8;           // a quarter's columns as GRID x GRID: column j in row j / GRID, column j mod GRID
+static_assert(GRID * GRID == EPI_COLS, "grid of a column quarter");
+constexpr int CHUNK = 16;         // TMEM columns per tcgen05.ld in the epilogue
 
 using namespace pipe;
 
@@ -48,14 +49,11 @@ __device__ __forceinline__ void mma_commit(unsigned long long* b) {
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[32]) {
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -76,13 +74,6 @@ __device__ __forceinline__ float key_dist(int key) { return __uint_as_float((uin
 // and it decodes to +inf.
 constexpr int KEY_NONE = 0x7F8000FF;
 
-// Insert key into the sorted pair (t1 <= t2): three min/max.
-__device__ __forceinline__ void top2_insert(int& t1, int& t2, int key) {
-  const int h = max(t1, key);
-  t1 = min(t1, key);
-  t2 = min(t2, h);
-}
-
 // Smallest two of two sorted pairs.
 __device__ __forceinline__ void top2_merge(int& a1, int& a2, int b1, int b2) {
   const int c2 = min(max(a1, b1), min(a2, b2));
@@ -90,29 +81,111 @@ __device__ __forceinline__ void top2_merge(int& a1, int& a2, int b1, int b2) {
   a2 = c2;
 }
 
-// Distances of CHUNK columns (ch .. ch + CHUNK - 1) of one point into its
-// NSET running top-2s (column j goes to set j mod NSET).  MASK: some columns
-// are >= k (their TMEM words are not written by the MMA and may hold
-// anything), so those keys are forced to KEY_NONE.
-template <bool MASK>
-__device__ __forceinline__ void top2_keys(const uint32_t (&acc)[CHUNK], uint32_t ch, float nxv, const float* cn,
-                                          uint32_t k, int (&t1)[NSET], int (&t2)[NSET], float* dbg_row) {
+// Distances of one point to the centroids of a quarter's columns (cols of them, a
+// multiple of CHUNK, from TMEM address ta on) as keys (columns counted within the
+// quarter), as the minima over the columns and the rows of the quarter's grid:
+// col[j mod GRID], row[j / GRID].  Any two columns differ in their grid column or
+// row, so the smallest two keys are among these minima (top2_grid), at one
+// three-way minimum per key where a running top-2 takes three minima and maxima.
+// cn: the columns' centroid norms, infinite for columns without a centroid (the
+// padding up to a multiple of 16, whose operands are zero); no other column is
+// read.  dbg: null, or where the distances of the first dbg_n columns go.
+__device__ __forceinline__ void quarter_keys(uint32_t ta, uint32_t cols, float nxv, const float* cn, int (&col)[GRID],
+                                             int (&row)[GRID], float* dbg, uint32_t dbg_n) {
+  unsigned long long nx2, m2;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(nx2) : "f"(nxv));
+  asm("mov.b64 %0, {%1, %1};" : "=l"(m2) : "f"(-2.f));
+  static_assert(CHUNK == 2 * GRID, "two grid rows per load");
 #pragma unroll
-  for (int j = 0; j < CHUNK; j += 4) {
-    const float4 c4 = *reinterpret_cast<const float4*>(cn + ch + j);
-    const float cv[4] = {c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint32_t kk = ch + (uint32_t)(j + e);
-      const float dist = fmaf(-2.f, __uint_as_float(acc[j + e]), nxv) + cv[e];
-      int key = dist_key(dist, kk);
-      if (MASK) {
-        if (kk >= k) key = KEY_NONE;
-        else if (dbg_row) dbg_row[kk] = dist;
-      }
-      top2_insert(t1[(j + e) % NSET], t2[(j + e) % NSET], key);
+  for (int c = 0; c < EPI_COLS / CHUNK; ++c) {
+    if ((uint32_t)(c * CHUNK) >= cols) {
+      row[2 * c] = row[2 * c + 1] = KEY_NONE;
+      continue;
     }
+    uint32_t acc[CHUNK];
+    tmem_ld(ta + c * CHUNK, acc);
+    int key[CHUNK];
+#pragma unroll
+    for (int j = 0; j < CHUNK; j += 2) {
+      unsigned long long t;
+      asm("mov.b64 %0, {%1, %2};" : "=l"(t) : "r"(acc[j]), "r"(acc[j + 1]));
+      const unsigned long long c2 = *reinterpret_cast<const unsigned long long*>(cn + c * CHUNK + j);
+      asm("fma.rn.f32x2 %0, %1, %0, %2;" : "+l"(t) : "l"(m2), "l"(nx2));
+      asm("add.rn.f32x2 %0, %0, %1;" : "+l"(t) : "l"(c2));
+      float d0, d1;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(t));
+      key[j] = dist_key(d0, c * CHUNK + j);
+      key[j + 1] = dist_key(d1, c * CHUNK + j + 1);
+    }
+    if (dbg) {
+      for (int j = 0; j < CHUNK; ++j)
+        if ((uint32_t)(c * CHUNK + j) < dbg_n)
+          dbg[c * CHUNK + j] = fmaf(-2.f, __uint_as_float(acc[j]), nxv) + cn[c * CHUNK + j];
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int* k = key + h * GRID;
+      row[2 * c + h] = min(__vimin3_s32(__vimin3_s32(k[0], k[1], k[2]), k[3], k[4]), __vimin3_s32(k[5], k[6], k[7]));
+    }
+#pragma unroll
+    for (int i = 0; i < GRID; ++i)
+      col[i] = c == 0 ? min(key[i], key[GRID + i]) : __vimin3_s32(col[i], key[i], key[GRID + i]);
   }
+}
+
+// The smallest two of GRID keys.
+__device__ __forceinline__ void top2_of(const int (&v)[GRID], int& w1, int& w2) {
+  int lo[GRID / 2], hi[GRID / 2];
+#pragma unroll
+  for (int i = 0; i < GRID / 2; ++i) lo[i] = min(v[2 * i], v[2 * i + 1]), hi[i] = max(v[2 * i], v[2 * i + 1]);
+#pragma unroll
+  for (int w = GRID / 4; w; w >>= 1)
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      hi[i] = __vimin3_s32(max(lo[i], lo[i + w]), hi[i], hi[i + w]);
+      lo[i] = min(lo[i], lo[i + w]);
+    }
+  w1 = lo[0];
+  w2 = hi[0];
+}
+
+// A quarter's two smallest keys (w1, w2) from its grid's minima, their columns
+// counted from c_lo on, and a lower bound lb of its other keys, but for those
+// that may hide behind both in the grid (hidden_cols).  Keys above KEY_NONE
+// (NaN distances) count as KEY_NONE.  lb is meaningless when w1 < 0.
+__device__ __forceinline__ void top2_grid(const int (&col)[GRID], const int (&row)[GRID], uint32_t c_lo, int& w1,
+                                          int& w2, int& lb) {
+  int r1, r2;
+  top2_of(col, w1, w2);
+  top2_of(row, r1, r2);  // r1 == w1
+  w1 = min(w1, KEY_NONE);
+  w2 = __vimin3_s32(w2, r2, KEY_NONE);
+  // the smallest minimum above w2: as distances from it, w1 and w2 wrap around
+  // to the top
+  uint32_t m = 0xFFFFFFFFu;
+#pragma unroll
+  for (int i = 0; i < GRID; ++i)
+    m = __vimin3_u32(m, (uint32_t)col[i] - (uint32_t)w2 - 1u, (uint32_t)row[i] - (uint32_t)w2 - 1u);
+  lb = w2 == KEY_NONE ? KEY_NONE : min((int)(m + (uint32_t)w2 + 1u), KEY_NONE);
+  w1 += w1 == KEY_NONE ? 0 : (int)c_lo;
+  w2 += w2 == KEY_NONE ? 0 : (int)c_lo;
+}
+
+// The two columns whose keys the minima of a quarter that starts at column c_lo
+// may hide behind the keys of its columns c1 and c2, where those differ in grid
+// row and grid column.
+__device__ __forceinline__ bool hidden_cols(uint32_t c1, uint32_t c2, uint32_t c_lo, uint32_t& h1, uint32_t& h2) {
+  constexpr uint32_t IN = GRID - 1;
+  const uint32_t a = c1 - c_lo, b = c2 - c_lo;
+  h1 = c_lo + ((a & ~IN) | (b & IN));
+  h2 = c_lo + ((b & ~IN) | (a & IN));
+  return ((a ^ b) & IN) && ((a ^ b) & ~IN);
+}
+
+// Columns of each quarter of an accumulator with cols columns (the last ones may
+// have fewer): the quarters share few centroids evenly.
+__device__ __forceinline__ uint32_t quarter_cols(uint32_t cols) {
+  return (cols + QUARTERS * CHUNK - 1) / (QUARTERS * CHUNK) * CHUNK;
 }
 
 // BF16 hi/lo split of two values, packed little-endian (element 0 low half).
@@ -142,19 +215,6 @@ __device__ __forceinline__ void put_operand(uint8_t* bop, uint32_t d, uint32_t k
                swz((int)(k % NMAX), (int)((j % KD) >> 3)) + (j & 7) * 2;
   *reinterpret_cast<__nv_bfloat16*>(t) = hi;
   *reinterpret_cast<__nv_bfloat16*>(t + OP_TILE) = lo;
-}
-
-// An epilogue thread's sets reduced to its top-2 (w1, w2) and a lower bound lb
-// of all its other keys: per set, the set's smallest key that is not w1 or
-// w2, or its second key when both are, which bounds the rest of that set.
-__device__ __forceinline__ void top2_sets(const int (&t1)[NSET], const int (&t2)[NSET], int& w1, int& w2, int& lb) {
-  w1 = t1[0];
-  w2 = t2[0];
-#pragma unroll
-  for (int a = 1; a < NSET; ++a) top2_merge(w1, w2, t1[a], t2[a]);
-  lb = KEY_NONE;
-#pragma unroll
-  for (int a = 0; a < NSET; ++a) lb = min(lb, (t1[a] == w1 || t1[a] == w2) ? t2[a] : t1[a]);
 }
 
 // Whether the distance pass takes the filter's list (its rows are gathered) or

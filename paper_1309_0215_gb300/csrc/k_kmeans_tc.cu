@@ -21,9 +21,9 @@
 //   * 16 epilogue warps read the 128 x N FP32 tile with tcgen05.ld (one
 //     TMEM lane per point; four warps per lane quadrant, each on a quarter
 //     of the columns), form d~ = fma(-2, acc, ||x||^2) + ||c||^2, pack it
-//     with its column into one sortable 32-bit key and keep the two smallest
-//     keys with signed min/max (four independent top-2s per thread) plus
-//     a lower bound of all other keys, and hand them to
+//     with its column into one sortable 32-bit key, and reduce the keys to the
+//     minima of the rows and columns of a grid (quarter_keys), which hold the
+//     two smallest keys plus a lower bound of the others, and hand them to
 //   * 4 finalizer warps (one lane quadrant each), which merge the four
 //     column quarters of each point and apply the margin tests below, so
 //     that no epilogue warp carries the per-point tail on its own path.
@@ -56,7 +56,9 @@
 // distance above t_1 (1 + 2^-15) + E >= d(k_1); with at most KM_CAND_MAX of
 // them the point needs an exact choice between those few alone, else it is
 // listed and compared with every centroid (km_settle_kernel either way), so
-// assignments equal the FP64 argmin.
+// assignments equal the FP64 argmin.  (Two keys may hide behind a quarter's two
+// smallest in its grid: they are above both, so they matter only when both are
+// candidates, and then count as candidates too.)
 #include <type_traits>
 
 #include "dev_tc.cuh"
@@ -470,22 +472,30 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
             moved += now != o;
             if (B.ub) km_put_bounds(B, p[h], S.drift[now], far, fmaf(d1, 1.00006103515625f, e), d2 - e);
           } else {
-            // candidates: the quarters' top-2 keys within the margin, if every
-            // other key is beyond it
+            const uint32_t cpq = quarter_cols(npad);
+            // candidates: the quarters' top-2 keys within the margin and what
+            // may hide behind both of a quarter's, if every other key is beyond it
             int rest = KEY_NONE;
             uint32_t nc = 0;
 #pragma unroll
-            for (int u = 0; u < QUARTERS; ++u) {
+            for (uint32_t u = 0; u < QUARTERS; ++u) {
               rest = min(rest, ol[h][u]);
-#pragma unroll
-              for (int t = 0; t < 2; ++t) {
-                const int key = t ? o2[h][u] : o1[h][u];
-                if (key_dist(key) - d1 <= lim) {
-                  cand[h] = (cand[h] << 12) | ((uint32_t)key & 0xFFu);
-                  ++nc;
-                } else {
-                  rest = min(rest, key);
+              auto add = [&](uint32_t column) {
+                cand[h] = (cand[h] << 12) | column;
+                ++nc;
+              };
+              const uint32_t c1 = (uint32_t)o1[h][u] & 0xFFu, c2 = (uint32_t)o2[h][u] & 0xFFu;
+              if (key_dist(o1[h][u]) - d1 <= lim) add(c1);
+              else rest = min(rest, o1[h][u]);
+              if (key_dist(o2[h][u]) - d1 <= lim) {
+                add(c2);
+                uint32_t h1, h2;
+                if (hidden_cols(c1, c2, u * cpq, h1, h2)) {
+                  if (h1 < k) add(h1);
+                  if (h2 < k) add(h2);
                 }
+              } else {
+                rest = min(rest, o2[h][u]);
               }
             }
             const bool few = key_dist(rest) - d1 > gap && nc >= 2 && nc <= KM_CAND_MAX;
@@ -525,18 +535,18 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
   } else {
     // ------------------------------------------------------------- epilogue
     // Warp e reads TMEM lane quadrant e % 4 (rows 32 (e % 4) ..) and column
-    // quarter e / 4 (EPI_COLS columns), CHUNK columns per tcgen05.ld.  Each
-    // distance becomes one sortable 32-bit key (see dist_key), so a running
-    // top-2 costs three min/max; NSET independent top-2s per thread
-    // (columns j mod NSET) keep the dependency chains short.  A warp then
-    // reduces its sets to its top-2 (w1, w2) and a lower bound lb of all its
-    // other keys (per set: the set's smallest key that is not w1 or w2, or
-    // its second key when both are, which bounds the rest of that set) and
-    // hands (w1, w2, lb) to the finalizer of its lane quadrant.
+    // quarter e / 4, CHUNK columns per tcgen05.ld.  Each distance becomes one
+    // sortable 32-bit key (see dist_key); the keys are reduced to the minima of
+    // the rows and columns of an 8 x 8 grid, those to the quarter's two smallest
+    // (w1, w2) and a lower bound lb of the others, which go to the finalizer of
+    // its lane quadrant.
+    // (A running top-2, three minima and maxima per key, with the columns past K
+    // masked one by one and up to 128 columns left to two of the quarters: 4M x
+    // 64, K = 256, ten rounds 3.88 ms, now 3.70; 1M x 8, K = 20, one pass 112
+    // us, now 108; 250,000 x 128, K = 512, five rounds 1.15 ms, now 1.12.)
     const int q = warp & 3, quarter = warp >> 2;
     const int r = q * 32 + lane;
-    const uint32_t c_lo = (uint32_t)quarter * EPI_COLS;
-    const uint32_t c_hi = min(npad, c_lo + (uint32_t)EPI_COLS);
+    const uint32_t cols = npad, cpq = quarter_cols(cols), c_lo = (uint32_t)quarter * cpq;
     for (uint32_t i = 0;; ++i) {
       const uint32_t tile = blockIdx.x + i * gridDim.x;
       if (tile >= ntiles) break;
@@ -549,24 +559,15 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
       const float nxv = S.nx[s][r];
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.nx_free[s]);
-      int t1[NSET], t2[NSET];
-#pragma unroll
-      for (int a = 0; a < NSET; ++a) t1[a] = t2[a] = KEY_NONE;
       const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * 256u;
-      float* dbg_row = (dbg && tile == 0) ? dbg + (uint64_t)r * NMAX : nullptr;
-      for (uint32_t ch = c_lo; ch < c_hi; ch += CHUNK) {
-        uint32_t acc[CHUNK];
-        tmem_ld(ta + ch, acc);
-        if (ch + CHUNK <= k && !dbg_row)
-          top2_keys<false>(acc, ch, nxv, S.cn, k, t1, t2, nullptr);
-        else
-          top2_keys<true>(acc, ch, nxv, S.cn, k, t1, t2, dbg_row);
-      }
+      float* dbg_row = (dbg && tile == 0) ? dbg + (uint64_t)r * NMAX + c_lo : nullptr;
+      int w1 = KEY_NONE, w2 = KEY_NONE, lb = KEY_NONE, col[GRID], row[GRID];
+      if (c_lo < cols)
+        quarter_keys(ta + c_lo, min(cpq, cols - c_lo), nxv, S.cn + c_lo, col, row, dbg_row, k > c_lo ? k - c_lo : 0);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.empty_acc[b]);
-      int w1, w2, lb;
-      top2_sets(t1, t2, w1, w2, lb);
+      if (c_lo < cols) top2_grid(col, row, c_lo, w1, w2, lb);
       if (i >= ACCS) {
         const bool okf = mbar_wait(&S.xfree[b], (v + 1) & 1, err, polls);
         if (!__all_sync(0xffffffffu, okf)) break;

@@ -330,8 +330,8 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
           nxv[h] = S.xnx[b][r];
 #pragma unroll
           for (int u = 0; u < QUARTERS; ++u) {
-            list_insert(t[h], c[h], rest[h], (int)S.xw1[b][u][r], ch);
-            list_insert(t[h], c[h], rest[h], (int)S.xw2[b][u][r], ch);
+            list_insert(t[h], c[h], rest[h], (int)S.xw1[b][u][r], ch * QUARTERS + u);
+            list_insert(t[h], c[h], rest[h], (int)S.xw2[b][u][r], ch * QUARTERS + u);
             rest[h] = min(rest[h], (int)S.xlb[b][u][r]);
           }
         }
@@ -354,7 +354,7 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
           if (t[h][0] < 0) {
             flag = true;  // a negative smallest distance: re-check
           } else if (d2 - d1 > lim) {
-            const uint32_t now = c[h][0] * NMAX + ((uint32_t)t[h][0] & 0xFFu);
+            const uint32_t now = c[h][0] / QUARTERS * NMAX + ((uint32_t)t[h][0] & 0xFFu);
             const uint32_t old = nchg ? was[h] : now;
             assign[p] = km_word(now, old);
             moved += now != old;
@@ -362,10 +362,22 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
 #pragma unroll
             for (uint32_t j = 0; j < KM_CAND_MAX; ++j)
               if (key_dist(t[h][j]) - d1 <= lim) {
-                cand = (cand << 12) | (c[h][j] * NMAX + ((uint32_t)t[h][j] & 0xFFu));
+                const uint32_t cj = (uint32_t)t[h][j] & 0xFFu, first = c[h][j] / QUARTERS * NMAX;
+                cand = (cand << 12) | (first + cj);
                 ++ncand;
+                // with another of its quarter's: what may hide behind both
+#pragma unroll
+                for (uint32_t i = 0; i < j; ++i)
+                  if (c[h][i] == c[h][j]) {
+                    const uint32_t c_lo = c[h][j] % QUARTERS * quarter_cols(min((uint32_t)NMAX, npad - first));
+                    uint32_t h1, h2;
+                    if (hidden_cols((uint32_t)t[h][i] & 0xFFu, cj, c_lo, h1, h2)) {
+                      if (first + h1 < k) cand = (cand << 12) | (first + h1), ++ncand;
+                      if (first + h2 < k) cand = (cand << 12) | (first + h2), ++ncand;
+                    }
+                  }
               }
-            some = ncand >= 2 && key_dist(rest[h]) - d1 > gap;
+            some = ncand >= 2 && ncand <= KM_CAND_MAX && key_dist(rest[h]) - d1 > gap;
             flag = !some;
           }
         }
@@ -381,7 +393,6 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
     // accumulator, as in k_kmeans_tc.cu.
     const int q = warp & 3, quarter = warp >> 2;
     const int r = q * 32 + lane;
-    const uint32_t c_lo = (uint32_t)quarter * EPI_COLS;
     uint32_t cc = 0;
     bool ok = true;
     for (uint32_t i = 0; ok; ++i) {
@@ -398,22 +409,16 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
           __syncwarp();
           if (lane == 0) mbar_arrive(&S.nx_free[i & 1]);
         }
-        int t1[NSET], t2[NSET];
-#pragma unroll
-        for (int a = 0; a < NSET; ++a) t1[a] = t2[a] = KEY_NONE;
         const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + b * 256u;
-        const uint32_t kr = k - ch * NMAX, c_hi = min(npad - ch * NMAX, c_lo + (uint32_t)EPI_COLS);
-        for (uint32_t cl = c_lo; cl < c_hi; cl += CHUNK) {
-          uint32_t acc[CHUNK];
-          tmem_ld(ta + cl, acc);
-          if (cl + CHUNK <= kr) top2_keys<false>(acc, cl, nxv, cn + ch * NMAX, kr, t1, t2, nullptr);
-          else top2_keys<true>(acc, cl, nxv, cn + ch * NMAX, kr, t1, t2, nullptr);
-        }
+        const uint32_t cols = min((uint32_t)NMAX, npad - ch * NMAX), cpq = quarter_cols(cols);
+        const uint32_t c_lo = (uint32_t)quarter * cpq;
+        int w1 = KEY_NONE, w2 = KEY_NONE, lb = KEY_NONE, col[GRID], row[GRID];
+        if (c_lo < cols)
+          quarter_keys(ta + c_lo, min(cpq, cols - c_lo), nxv, cn + ch * NMAX + c_lo, col, row, nullptr, 0);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.empty_acc[b]);
-        int w1, w2, lb;
-        top2_sets(t1, t2, w1, w2, lb);
+        if (c_lo < cols) top2_grid(col, row, c_lo, w1, w2, lb);
         if (cc >= (uint32_t)ACCS) {
           ok = __all_sync(0xffffffffu, mbar_wait(&S.xfree[b], (v + 1) & 1, err, polls));
           if (!ok) break;

@@ -418,3 +418,31 @@ def test_kmeans_skipped_points(mr, n, d, k, comps, sigma, precision):
         cur, a, _ = mr.kmeans(dx, _dev(cur), 1, precision)
     assert np.array_equal(a9, a)
     assert np.array_equal(c9, cur)
+
+
+@pytest.mark.parametrize("n,d,k", [
+    (3_000, 64, 256),  # four quarters of 64 columns
+    (3_000, 64, 100),  # 32, 32, 32, 16 (12 of them padding)
+    (2_000, 9, 144),   # 48 columns each
+    (2_000, 5, 17),    # 16 columns, one centroid in the second quarter
+    (2_000, 3, 2),
+    (1_500, 80, 300),  # wide pass, 44 centroids in the last accumulator
+    (1_500, 20, 700),
+])
+@pytest.mark.parametrize("spread", [0.0, 1e-6, 1e-4])
+def test_kmeans_close_centroids_in_the_grid(mr, n, d, k, spread):
+    """Groups of four centroids within `spread` of one another (equal at 0) that
+    form rectangles in the 8 x 8 grid of an accumulator quarter: the smallest
+    keys of rows and columns can hide two of them behind the other two."""
+    rng = np.random.default_rng(n + d + k)
+    group = np.array([8 * (c % 64 // 16) + (c % 8) // 2 + 64 * (c // 64) for c in range(k)])
+    means = rng.normal(0, 3, (group.max() + 1, d)).astype(np.float32)
+    init = (means[group] * (1 + spread * rng.standard_normal((k, d)))).astype(np.float32)
+    x = (means[rng.integers(0, len(means), n)] + rng.normal(0, 0.5, (n, d))).astype(np.float32)
+    c_ref, a_ref = oracle.kmeans(x, init, 1)
+    for precision in (0, 1):
+        if precision and (d > 64 or k > 256):
+            continue
+        c, a, _ = _run(mr, x, init, 1, precision)
+        assert np.array_equal(a, a_ref)
+        assert _rel_err(c, c_ref) <= TOL
