@@ -50,14 +50,6 @@ def _peaks():
         return 6800.0, 1900.0, 1700.0, "fallback"
 
 
-def _sm_max_mhz() -> float:
-    try:
-        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            return float(json.load(f)["sm_max_mhz"])
-    except Exception:
-        return 2070.0
-
-
 def source_sha(sources) -> str:
     h = hashlib.sha256()
     for src in sources:
@@ -204,7 +196,7 @@ def workload_config(workload: str, inp, pipelined: bool = False) -> dict:
         return {"workload": "large-key histogram: %d u32 keys (%d B) uniform over %d bins" % (
             inp["keys"].size, inp["keys"].nbytes, HK_BINS),
             "inputs": "synthetic, resident in HBM, larger than L2 (no flush needed)",
-            "containers": "global array (u32 counters, 64 MiB, L2-resident), no local arrays"}
+            "containers": "keys grouped by ranges of bins, counted in shared memory, added to the u64 result"}
     if workload == "bloom":
         return {"workload": "Bloom-filter build: %d-base windows of %d uniform ACGT bases (%d elements) into %d bits, "
                             "%d hashes" % (BF_KMER, inp["seq"].size, inp["seq"].size - BF_KMER + 1, BF_BITS, BF_HASHES),
@@ -261,10 +253,10 @@ def run_ours(args):
                             km_precision=args.precision)
             ctx.run()
             return [a]
-        kname = "km_tc_assign_kernel" if args.precision else "km_assign_fp32_kernel"
-        dominant = (kname, ["paper_1309_0215_gb300/csrc/k_kmeans_tc.cu" if args.precision else
-                            "paper_1309_0215_gb300/csrc/k_kmeans.cu", "paper_1309_0215_gb300/csrc/dev_pipe.cuh"],
-                    d_x.numel() * 4)
+        # (FP32 jobs of this shape take the tensor-core pass too, with split operands)
+        dominant = ("km_tc_assign_kernel", ["paper_1309_0215_gb300/csrc/k_kmeans_tc.cu",
+                                            "paper_1309_0215_gb300/csrc/dev_tc.cuh",
+                                            "paper_1309_0215_gb300/csrc/dev_pipe.cuh"], d_x.numel() * 4)
     elif args.workload == "histkeys":
         d_k = dinp["keys"]
         total_bytes = d_k.numel() * 4
@@ -273,7 +265,8 @@ def run_ours(args):
             a = ctx.add_job(mr.HIST_U32, d_k, hist_bins=HK_BINS)
             ctx.run()
             return [a]
-        dominant = ("hk_global_kernel", ["paper_1309_0215_gb300/csrc/k_keys.cu"], d_k.numel() * 4)
+        # (one launch pair per job: keys grouped by bin range, then counted)
+        dominant = ("hk_part_kernel + hk_count_kernel", ["paper_1309_0215_gb300/csrc/k_keys.cu"], d_k.numel() * 4)
     elif args.workload == "bloom":
         d_s = dinp["seq"]
         total_bytes = d_s.numel()
@@ -282,7 +275,7 @@ def run_ours(args):
             a = ctx.add_job(mr.BLOOM_DNA, d_s, bloom_kmer=BF_KMER, bloom_bits=BF_BITS, bloom_hashes=BF_HASHES)
             ctx.run()
             return [a]
-        dominant = ("bloom_kernel", ["paper_1309_0215_gb300/csrc/k_keys.cu"], d_s.numel())
+        dominant = ("bloom_part_kernel + hk_count_kernel", ["paper_1309_0215_gb300/csrc/k_keys.cu"], d_s.numel())
     else:
         d_t = dinp["text"]
         total_bytes = d_t.numel()
@@ -291,9 +284,9 @@ def run_ours(args):
             a = ctx.add_job(mr.WORDCOUNT, d_t, wc_pipelined=int(args.pipelined))
             ctx.run()
             return [a]
-        # the plain map pass runs the CTA-table kernel from 64 MiB on
+        # the plain map pass runs the CTA-table kernel from 4 MiB on
         mapk = "wc_pipe_kernel" if args.pipelined else (
-            "wc_map_cta_kernel" if d_t.numel() >= (64 << 20) else "wc_map_kernel")
+            "wc_map_cta_kernel" if d_t.numel() >= (4 << 20) else "wc_map_kernel")
         dominant = (mapk, ["paper_1309_0215_gb300/csrc/k_wordcount.cu",
                            "paper_1309_0215_gb300/csrc/dev_wordcount.cuh"], d_t.numel())
 
@@ -429,6 +422,21 @@ def run_ours(args):
             per_job_alone[name] = {"bytes": int(t.numel()), "launch_ms": round(ms, 5), "gbs": round(gbs, 1),
                                    "frac": round(gbs / hbm_peak, 4), "measured": "alone (RUN_PLAIN), 5 launches"}
 
+    # k-means: the distance pass over all points, from jobs of one round (the
+    # timed jobs' later rounds leave out points that cannot change cluster)
+    if args.workload == "kmeans":
+        ts = []
+        for i in range(8):
+            j = ctx.add_job(mr.KMEANS_F32, d_x, km_dims=dd, km_k=kk, km_iters=1, km_init=d_i,
+                            km_precision=args.precision)
+            ctx.run()
+            ctx.fetch(j)
+            if i >= 3:
+                kt, kc = ctx.kernel_ms(j)
+                ts.append(kt / max(1, kc))
+            ctx.release(j)
+        kern_ms = statistics.median(ts)
+
     cpu = None
     if rank == 0 and not args.no_cpu_baseline and args.workload != "kmeans":
         cpu = cpu_baseline(args.workload, inp)
@@ -452,24 +460,18 @@ def run_ours(args):
                             "launch gaps)")
         if args.workload == "kmeans":
             # a dense contraction: work is the distance GEMM, not bytes
-            if args.precision:
-                terms = 3 if args.precision == 1 else 1
-                flops = 2.0 * nn * kk * dd * terms
-                peak, bound, unit = _peaks()[1], "tensor", "TFLOP/s"
-                note = ("BF16 tcgen05 products (%d per distance: x*c split into hi/lo parts) x 2*N*K*D, "
-                        "per launch of the distance pass; peak = measured cuBLAS bf16 burst" % terms)
-            else:
-                flops = 2.0 * nn * kk * dd
-                props = torch.cuda.get_device_properties(dev)
-                peak = props.multi_processor_count * 128 * 2 * _sm_max_mhz() * 1e6 / 1e12
-                bound, unit = "alu", "TFLOP/s"
-                note = "FP32 FMA: 2*N*K*D per launch; peak = SMs x 128 FP32 lanes x 2 x max SM clock"
+            terms = 1 if args.precision == 2 else 3
+            flops = 2.0 * nn * kk * dd * terms
+            peak, bound, unit = _peaks()[1], "tensor", "TFLOP/s"
+            note = ("BF16 tcgen05 products (%d per distance: x*c split into hi/lo parts) x 2*N*K*D, one distance "
+                    "pass over all points (jobs of one round, after the timed region: later rounds of a job leave "
+                    "out points that cannot change cluster); peak = measured cuBLAS bf16 burst" % terms)
             ach = flops / (kern_ms / 1e3) / 1e12
             roof = {"bound": bound, "kernel": kname, "achieved": round(ach, 1), "peak": round(peak, 1),
-                    "peak_source": peak_src if args.precision else "derived", "unit": unit,
+                    "peak_source": peak_src, "unit": unit,
                     "frac": round(ach / peak, 4), "traffic": _traffic(kname, ksrc, kbytes),
                     "algorithmic_flops_per_launch": flops, "launch_ms": round(kern_ms, 5),
-                    "launches_timed": int(sum(c for _, (_, c) in job_stats)), "note": note}
+                    "launches_timed": 5, "note": note}
         line = {
             "metric": METRIC, "value": round(value, 3), "unit": "GB/s", "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": round(ms_per_step, 5), "higher_is_better": True,
@@ -1008,7 +1010,6 @@ def kmeans_eval(steps: int, warmup: int) -> dict:
         di = torch.from_numpy(init).cuda()
     stream.synchronize()
     hbm_peak, bf16_peak, _, _ = _peaks()
-    fp32_peak = torch.cuda.get_device_properties(0).multi_processor_count * 128 * 2 * _sm_max_mhz() * 1e6 / 1e12
     ctx = mr.Context(0, stream=stream, timing=True)
 
     def job(prec, iters, init_t):
@@ -1024,27 +1025,29 @@ def kmeans_eval(steps: int, warmup: int) -> dict:
             ctx.run()
             if i >= warmup:
                 el.append(ctx.elapsed_ms(j))
+            raw = ctx.fetch(j)
+            ctx.release(j)
+        for i in range(4):  # the distance pass over all points: jobs of one round
+            j = job(prec, 1, di)
+            ctx.run()
+            if i:
                 t, c = ctx.kernel_ms(j)
                 km[0] += t
                 km[1] += c
-            raw = ctx.fetch(j)
             ctx.release(j)
         c10, a10, st = mr.split_kmeans_result(raw, n, dd, kk)
         results[prec] = (c10, a10)
         it_ms = statistics.median(el) / KM_ITERS
         dk = km[0] / max(1, km[1])
-        terms = 3 if prec == 1 else 1
+        terms = 1 if prec == 2 else 3
         r = {"ms_per_iteration": round(it_ms, 4), "distance_kernel_ms": round(dk, 4),
              "method_tflops": round(2.0 * n * kk * dd / (dk / 1e3) / 1e12, 1),
              "points_gbs": round(x.nbytes / (dk / 1e3) / 1e9, 1),
              "points_frac_of_hbm": round(x.nbytes / (dk / 1e3) / 1e9 / hbm_peak, 4),
              "fp32_rechecks": int(st[0]), "fp64_rechecks": int(st[1]), "timeouts": int(st[3])}
-        if prec:
-            tt = 2.0 * n * kk * dd * terms / (dk / 1e3) / 1e12
-            r.update({"tensor_products_per_distance": terms, "tensor_tflops": round(tt, 1),
-                      "tensor_frac_of_bf16_peak": round(tt / bf16_peak, 4)})
-        else:
-            r.update({"fp32_frac_of_fma_peak": round(2.0 * n * kk * dd / (dk / 1e3) / 1e12 / fp32_peak, 4)})
+        tt = 2.0 * n * kk * dd * terms / (dk / 1e3) / 1e12
+        r.update({"tensor_products_per_distance": terms, "tensor_tflops": round(tt, 1),
+                  "tensor_frac_of_bf16_peak": round(tt / bf16_peak, 4)})
         out[name] = r
     # the three paths give identical results (each iteration's assignment is
     # the FP64 argmin, and the update's integer sums make it order-free)

@@ -1054,7 +1054,7 @@ __global__ void __launch_bounds__(256) km_sum_kernel(const float* __restrict__ x
 // hi * 2^32 + lo is the exact sum modulo 2^64 (which holds it: the scale
 // keeps |sum| below 2^62).  The CTA then stores its sums as one partial
 // (plain stores) and adds its counts to the global counts;
-// km_reduce_finalize_kernel adds the partials.  Integer sums make the result
+// km_finalize_kernel adds the partials.  Integer sums make the result
 // independent of the order.
 __device__ __forceinline__ void add64_split(uint32_t* lo, uint32_t* hi, long long q) {
   const uint32_t ql = (uint32_t)q;
