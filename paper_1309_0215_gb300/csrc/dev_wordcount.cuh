@@ -168,7 +168,7 @@ __device__ __forceinline__ Tok read_token(const uint8_t* __restrict__ in, uint64
   return t;
 }
 
-// an even slot and the one after it (tables are 256-byte aligned)
+// an even slot and the one after it (tables are 32-byte aligned)
 __device__ __forceinline__ void ld_pair(const unsigned long long* p, uint64_t& a0, uint64_t& a1, uint64_t& b0,
                                         uint64_t& b1) {
   asm volatile("ld.volatile.global.v4.u64 {%0, %1, %2, %3}, [%4];"

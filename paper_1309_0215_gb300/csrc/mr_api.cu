@@ -346,9 +346,12 @@ mr_status alloc_wc(mr_ctx* c, Job* j, uint64_t cap) {
   if (st) return st;
   uint8_t* p = static_cast<uint8_t*>(slab);
   b.cap = cap;
-  b.key = reinterpret_cast<uint64_t*>(p);
+  // the table's slots are read in pairs of 32 bytes: up to 31 bytes of the state's
+  // slack make up for a caller's allocator that aligns to less
+  const uint64_t shift = (0 - reinterpret_cast<uintptr_t>(p)) & 31;
+  b.key = reinterpret_cast<uint64_t*>(p + shift);
   b.cnt = b.key + 2 * cap;
-  b.state = reinterpret_cast<uint32_t*>(p + t_bytes);
+  b.state = reinterpret_cast<uint32_t*>(p + shift + t_bytes);
   b.sortbuf = p + t_bytes + s_bytes;
   b.out = p + t_bytes + s_bytes + sb_bytes;
   b.out_cap = wc_out_bytes(cap, n);

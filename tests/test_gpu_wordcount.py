@@ -253,3 +253,28 @@ def test_wc_cta_table_pass(mr, extra, off):
     text = (text * (n // len(text) + 1))[: n - 1] + b"q"
     got = mr.wordcount(_dev(text, off))
     assert got == oracle.wordcount(text)
+
+
+@pytest.mark.parametrize("nbytes", [100_000, (4 << 20) + 777])
+def test_wc_tables_on_odd_16_byte_boundaries(mr, nbytes):
+    """Tables in memory of a caller's allocator that is 16-byte but not 32-byte
+    aligned: plain runs and a batch."""
+    import torch
+    dev, stream = torch.cuda.current_device(), torch.cuda.current_stream().cuda_stream
+
+    def alloc(n):
+        return torch.cuda.caching_allocator_alloc(n + 16, dev, stream) + 16
+
+    text, _, _ = synth.wc_text(nbytes, nwords=9000, seed=3)
+    want = oracle.wordcount(text)
+    buf = _dev(bytes(text), 1)
+    torch.cuda.synchronize()
+    ctx = mr.Context(allocator=(alloc, lambda p: torch.cuda.caching_allocator_delete(p - 16)))
+    for flags in (mr.RUN_PLAIN, mr.RUN_BATCHED):
+        ids = [ctx.add_job(mr.WORDCOUNT, buf) for _ in range(2)]
+        ctx.run(flags)
+        ctx.sync()
+        for j in ids:
+            assert ctx.fetch(j) == want
+            ctx.release(j)
+    ctx.close()
