@@ -58,7 +58,9 @@
 // listed and compared with every centroid (km_settle_kernel either way), so
 // assignments equal the FP64 argmin.  (Two keys may hide behind a quarter's two
 // smallest in its grid: they are above both, so they matter only when both are
-// candidates, and then count as candidates too.)
+// candidates, and then count as candidates too.)  A centroid that is not finite,
+// or whose norm overflows, makes max ||c|| and with it E infinite or NaN: no
+// test then holds, and every point is listed.
 #include <type_traits>
 
 #include "dev_tc.cuh"
@@ -470,8 +472,8 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
           // keys under-state a distance by less than 2^-15 of it (2^-14 allowed)
           const float gap = 2.f * e + 6.103515625e-05f * d1;
           const float lim = fmaxf(1e-3f * d1, gap);
-          if (g1 < 0) {
-            ncand[h] = LISTED;  // a negative smallest distance: re-check
+          if (g1 < 0 || !(gap < INFINITY)) {
+            ncand[h] = LISTED;  // a negative smallest distance, or no bound at all: re-check
           } else if (d2 - d1 > lim) {
             const uint32_t now = (uint32_t)g1 & 0xFFu, o = nchg ? word[h] & 0xffffu : now;
             assign[p[h]] = km_word(now, o);

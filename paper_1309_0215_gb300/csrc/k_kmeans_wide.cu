@@ -351,8 +351,8 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
           const float e = 2.f * eps_sum * xn * cmax + eps32 * (xn + cmax) * (xn + cmax) + 1e-36f;
           const float gap = 2.f * e + 6.103515625e-05f * d1;
           const float lim = fmaxf(1e-3f * d1, gap);
-          if (t[h][0] < 0) {
-            flag = true;  // a negative smallest distance: re-check
+          if (t[h][0] < 0 || !(gap < INFINITY)) {
+            flag = true;  // a negative smallest distance, or no bound at all: re-check
           } else if (d2 - d1 > lim) {
             const uint32_t now = c[h][0] / QUARTERS * NMAX + ((uint32_t)t[h][0] & 0xFFu);
             const uint32_t old = nchg ? was[h] : now;

@@ -446,3 +446,32 @@ def test_kmeans_close_centroids_in_the_grid(mr, n, d, k, spread):
         c, a, _ = _run(mr, x, init, 1, precision)
         assert np.array_equal(a, a_ref)
         assert _rel_err(c, c_ref) <= TOL
+
+
+@pytest.mark.parametrize("n,d,k,iters", [
+    (20_000, 64, 64, 2),    # tensor-core pass, whole tiles in bulk copies
+    (6_001, 37, 50, 2),     # values loaded by the converters
+    (6_001, 100, 300, 2),   # wide tensor-core pass
+    (400_009, 16, 20, 5),   # with the filter's bounds
+    (3_000, 300, 20, 2),    # FP32 SIMT pass
+])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, 3e30])
+@pytest.mark.parametrize("offset", [0.0, 1000.0])
+def test_kmeans_centroids_not_finite(mr, n, d, k, iters, bad, offset):
+    """Initial centroids with NaN or infinite coordinates, or whose norm
+    overflows: the bound on the distances' error is then not finite, so it may
+    decide no point.  Such a centroid wins no point and stays."""
+    x, _, _ = synth.kmeans_points(n, d, 16, seed=n + d, sigma=4.0)
+    x = x + np.float32(offset)
+    init = synth.kmeans_init(x, k, seed=n)
+    init[3] = bad
+    init[k - 1, d // 2] = bad
+    c_ref, a_ref = oracle.kmeans(x, init, iters)
+    finite = np.isfinite(c_ref).all(axis=1)
+    for precision in (0, 1, 2):
+        if precision and (d > 64 or k > 256):
+            continue
+        c, a, _ = _run(mr, x, init, iters, precision)
+        assert np.array_equal(a, a_ref), precision
+        assert _rel_err(c[finite], c_ref[finite]) <= TOL
+        assert np.array_equal(c[~finite], c_ref[~finite], equal_nan=True)
