@@ -349,7 +349,8 @@ __global__ void __launch_bounds__(TINY_T, 1) wc_tiny_kernel(const uint8_t* __res
   for (uint32_t tok = tid; tok < ntok; tok += TINY_T) {
     const uint32_t p = S.starts[tok];
     const uint32_t len = tiny_len(S.wsb, p);
-    // the first 16 bytes, in registers for the hash and the comparisons
+    // the first 16 bytes, in registers for the hash (multiply and xorshift per
+    // word, with hash_short's multipliers) and the comparisons
     uint32_t w[4], mask[4], h = len * 0x9E3779B1u;
     tiny_words(S.text, p, w);
 #pragma unroll
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(TINY_T, 1) wc_tiny_kernel(const uint8_t* __res
       h = (h ^ v) * 0x85EBCA77u;
       h ^= h >> 15;
     }
-    h *= 0x2C1B3C6Du;
+    h *= 0x85EBCA6Bu;
     h ^= h >> 16;
     const uint32_t tag = h >> 17, mine = (tag << 17) | (p + 1);
     uint32_t s = h & (TINY_SLOTS - 1), probe = 0;

@@ -278,3 +278,17 @@ def test_wc_tables_on_odd_16_byte_boundaries(mr, nbytes):
             assert ctx.fetch(j) == want
             ctx.release(j)
     ctx.close()
+
+
+def test_wc_keys_that_differ_in_the_last_byte_of_each_word(mr):
+    """128^3 keys of 12 bytes that differ only in bytes 3, 7 and 11: their hashes
+    differ too, so a table of twice as many slots holds them within the longest
+    probe (with few hash values it would report an overflow)."""
+    text = np.full((128 ** 3, 13), ord("a"), dtype=np.uint8)
+    text[:, 12] = ord(" ")
+    i = np.random.default_rng(5).permutation(128 ** 3)
+    for p in (3, 7, 11):
+        text[:, p] = 128 + i % 128
+        i //= 128
+    text = text.ravel()
+    assert mr.wordcount(_dev(text.tobytes()), wc_slots=1 << 22) == oracle.wordcount(text)
