@@ -795,7 +795,7 @@ static cudaError_t launch_hk_cluster(const uint4* base, uint32_t off, uint64_t n
   const uint64_t sm64 = (1ull << 32) / slice;
   const uint32_t slice_mul = sm64 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)sm64;
   const int bytes = (int)(slice * 4);
-  cudaError_t e = cudaFuncSetAttribute(hk_cluster_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = allow_smem<hk_cluster_kernel<C>>(di);
   if (e != cudaSuccess) return e;
   const uint64_t groups = (n + off + 3) / 4;
   cudaLaunchConfig_t cfg = {};
@@ -876,8 +876,8 @@ cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbi
   const int psm = (int)(PCHUNK * 2 + (PNF + 4 + PRANGES) * 4 + (P.ranges + 1) * PGROUP * 2);
   const int csm = (1 << PS) * 4;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(hk_part_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, psm)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(hk_count_kernel<KeyItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm)) != cudaSuccess)
+  if ((e = allow_smem<hk_part_kernel>(di)) != cudaSuccess ||
+      (e = allow_smem<hk_count_kernel<KeyItems>>(di)) != cudaSuccess)
     return e;
   if ((e = kt_begin(kt, s)) != cudaSuccess) return e;
   for (uint64_t k0 = 0; k0 < n; k0 += PART_ROUND) {
@@ -922,14 +922,10 @@ cudaError_t launch_hist_keys(const uint32_t* keys, uint64_t n, uint32_t nbins, i
       g = g < 1 ? 1 : g;
       g = g > (uint64_t)di.sms * per_sm ? (uint64_t)di.sms * per_sm : g;
       if (wide) {
-        if ((e = cudaFuncSetAttribute(hk_smem_kernel<unsigned long long>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      bytes)) != cudaSuccess)
-          return e;
+        if ((e = allow_smem<hk_smem_kernel<unsigned long long>>(di)) != cudaSuccess) return e;
         hk_smem_kernel<unsigned long long><<<(int)g, HK_SMEM_THREADS, bytes, s>>>(base, off, n, nbins, out);
       } else {
-        if ((e = cudaFuncSetAttribute(hk_smem_kernel<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      bytes)) != cudaSuccess)
-          return e;
+        if ((e = allow_smem<hk_smem_kernel<uint32_t>>(di)) != cudaSuccess) return e;
         hk_smem_kernel<uint32_t><<<(int)g, HK_SMEM_THREADS, bytes, s>>>(base, off, n, nbins,
                                                                         static_cast<uint32_t*>(counters));
       }
@@ -1007,10 +1003,8 @@ cudaError_t launch_bloom_part(const uint8_t* seq, uint64_t n, uint32_t L, uint64
   const int csm = (1 << PS) * 4;
   const uint64_t words = (m + 31) / 32, nwin = n - L + 1, rm = ~0ull / m, rm1 = ~0ull / (m - 1);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(bloom_part_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, psm)) !=
-          cudaSuccess ||
-      (e = cudaFuncSetAttribute(hk_count_kernel<BitItems>, cudaFuncAttributeMaxDynamicSharedMemorySize, csm)) !=
-          cudaSuccess)
+  if ((e = allow_smem<bloom_part_kernel>(di)) != cudaSuccess ||
+      (e = allow_smem<hk_count_kernel<BitItems>>(di)) != cudaSuccess)
     return e;
   if ((e = kt_begin(kt, s)) != cudaSuccess) return e;
   for (uint64_t w0 = 0; w0 < nwin; w0 += bloom_round(h)) {

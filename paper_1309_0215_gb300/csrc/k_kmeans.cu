@@ -1823,22 +1823,13 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   const bool tc = b.precision != MR_KM_FP32 || (km_tc_supported(d, k) && plain);
   const bool wide = !tc && b.bop && plain;
   const int asm_bytes = (DC_MAX * CS_LD + DC_MAX * XS_LD) * 4;
-  if ((e = cudaFuncSetAttribute(km_assign_fp32_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                asm_bytes)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(km_assign_fp32_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                asm_bytes)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(km_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(k * 4))) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(km_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(k * 4))) !=
-      cudaSuccess)
+  if ((e = allow_smem<km_assign_fp32_kernel<true>>(di)) != cudaSuccess ||
+      (e = allow_smem<km_assign_fp32_kernel<false>>(di)) != cudaSuccess ||
+      (e = allow_smem<km_count_kernel>(di)) != cudaSuccess || (e = allow_smem<km_scatter_kernel>(di)) != cudaSuccess)
     return e;
   const int ls_bytes = (int)((uint64_t)k * d * 8 + (uint64_t)k * 4);
   const bool local = b.part != nullptr && ls_bytes <= di.smem_optin;
-  if (local && (e = cudaFuncSetAttribute(km_local_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         ls_bytes)) != cudaSuccess)
-    return e;
+  if (local && (e = allow_smem<km_local_sum_kernel>(di)) != cudaSuccess) return e;
   // pipelined update: rows of a multiple of 4 floats, 16-byte aligned points, and a ring of >= 4 rows a stage
   uint32_t lp_rows = 0;
   int lp_bytes = 0;
@@ -1851,10 +1842,8 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
     if (r >= 4) {
       lp_rows = (uint32_t)r;
       lp_bytes = (int)(fixed + LP_ST * r * ((uint64_t)d * 4 + 4));
-      if ((e = cudaFuncSetAttribute(km_local_sum_pipe_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    lp_bytes)) != cudaSuccess ||
-          (e = cudaFuncSetAttribute(km_local_sum_pipe_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    lp_bytes)) != cudaSuccess)
+      if ((e = allow_smem<km_local_sum_pipe_kernel<true>>(di)) != cudaSuccess ||
+          (e = allow_smem<km_local_sum_pipe_kernel<false>>(di)) != cudaSuccess)
         return e;
     }
   }
@@ -1866,8 +1855,9 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   auto ws_kernel = d == 64 && (reinterpret_cast<uintptr_t>(x) & 7) == 0 ? km_window_sum_kernel<WS_D64>
                    : d <= 32                                               ? km_window_sum_kernel<WS_D32>
                                                                            : km_window_sum_kernel<WS_DANY>;
-  if (wsum && (e = cudaFuncSetAttribute(ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)ws_smem_bytes(k, d, ws_win))) != cudaSuccess)
+  if (wsum && ((e = allow_smem<km_window_sum_kernel<WS_D64>>(di)) != cudaSuccess ||
+               (e = allow_smem<km_window_sum_kernel<WS_D32>>(di)) != cudaSuccess ||
+               (e = allow_smem<km_window_sum_kernel<WS_DANY>>(di)) != cudaSuccess))
     return e;
   uint32_t ls_grid = (uint32_t)di.sms < LS_MAX_CTAS ? (uint32_t)di.sms : LS_MAX_CTAS;
   if ((uint64_t)ls_grid * 1024 > n) ls_grid = (uint32_t)((n + 1023) / 1024);
@@ -1877,8 +1867,8 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   const int set_t = set_threads(k);
   const size_t set_bytes = set_smem(d, k);
   auto set_kernel = k > (uint32_t)set_t ? km_settle_kernel<true> : km_settle_kernel<false>;
-  if ((e = cudaFuncSetAttribute(set_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)set_bytes)) !=
-      cudaSuccess)
+  if ((e = allow_smem<km_settle_kernel<true>>(di)) != cudaSuccess ||
+      (e = allow_smem<km_settle_kernel<false>>(di)) != cudaSuccess)
     return e;
   const uint32_t ntiles = (n + TP - 1) / TP;
   uint32_t agrid = ntiles < (uint32_t)di.sms * 2 ? ntiles : (uint32_t)di.sms * 2;

@@ -456,8 +456,7 @@ cudaError_t launch_kmeans_wide_assign(const float* x, uint32_t n, uint32_t d, ui
   uint32_t grid = ntiles < (uint32_t)di.sms ? ntiles : (uint32_t)di.sms;
   if (b.grid_cap && grid > b.grid_cap) grid = b.grid_cap;
   const size_t smem = wide_smem(k);
-  cudaError_t e =
-      cudaFuncSetAttribute(km_wide_assign_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem<km_wide_assign_kernel>(di);
   if (e != cudaSuccess || (e = kt_begin(b.kt, s)) != cudaSuccess) return e;
   e = launch_pdl(km_wide_assign_kernel, dim3(grid), dim3(WD_THREADS), smem, s, x, n, d, k, (const uint8_t*)b.bop,
                  (const float*)b.center, (const float*)b.cnorm, cmax, b.assign, nchg, b.flagged, b.nflag + 1, b.pairs,

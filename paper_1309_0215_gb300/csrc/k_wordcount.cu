@@ -2462,8 +2462,9 @@ cudaError_t launch_wordcount_post_multi(const wc::JobDev* jobs, const wc::JobDev
     int n2 = 1;
     while ((uint64_t)n2 < G.smax) n2 <<= 1;
     const int sg_smem = n2 * (int)sizeof(KeyRec);
-    if ((e = cudaFuncSetAttribute(wc_seg_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sg_smem)) !=
-            cudaSuccess ||
+    // (limits for any job, not this one's size: another thread's launches see them too)
+    if ((e = cudaFuncSetAttribute(wc_seg_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  SEG_SMAX * (int)sizeof(KeyRec))) != cudaSuccess ||
         (e = cudaFuncSetAttribute(wc_seg_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   SEG_COUNT_SMEM)) != cudaSuccess)
       return e;

@@ -1,5 +1,6 @@
 // Internal declarations shared by the CUDA translation units of libmrgb.so.
 #pragma once
+#include <atomic>
 #include <utility>
 #include <cuda_runtime.h>
 #include <cstdint>
@@ -27,6 +28,26 @@ struct DevInfo {
   int smem_optin = 0;   // max dynamic shared memory per block (opt-in)
   int l2_bytes = 0;
 };
+
+#ifdef __CUDACC__
+// Lets KERN be launched with any dynamic shared memory a CTA of the device can
+// have.  The limit is an attribute of the function on the device, shared by all
+// contexts and threads, and nothing holds it between a launcher's setting it and
+// its launches: every launcher sets the same value, never its own job's size,
+// which another thread's larger job would then exceed.
+template <auto KERN>
+inline cudaError_t allow_smem(const DevInfo& di) {
+  static std::atomic<int> fixed{-1};  // the kernel's static shared memory
+  int f = fixed.load(std::memory_order_relaxed);
+  if (f < 0) {
+    cudaFuncAttributes a{};
+    const cudaError_t e = cudaFuncGetAttributes(&a, KERN);
+    if (e != cudaSuccess) return e;
+    fixed.store(f = (int)a.sharedSizeBytes, std::memory_order_relaxed);
+  }
+  return cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, di.smem_optin - f);
+}
+#endif
 
 // ------------------------------------------------------------ array jobs
 // RGB8 histogram, local arrays in shared memory ("lane-column" layout:
