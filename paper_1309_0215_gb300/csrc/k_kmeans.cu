@@ -107,7 +107,7 @@ __device__ __forceinline__ void top2lb_merge(uint32_t& a1, uint32_t& a2, uint32_
 // Start of a job: the current centroids are the initial ones, the counters
 // and statistics are zero, and center[j] is the mean of the initial centroids'
 // coordinate j (0 where that is not finite), the shift the tensor-core pass
-// applies to points and centroids alike.  One CTA per 32 dimensions.
+// applies to points and centroids alike (center null: not wanted).  One CTA per 32 dimensions.
 constexpr int SETUP_THREADS = 1024;
 __global__ void __launch_bounds__(SETUP_THREADS) km_setup_kernel(const float* __restrict__ init, uint32_t k,
                                                                  uint32_t d, float* __restrict__ c,
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(SETUP_THREADS) km_setup_kernel(const float* __
   if (w == 0 && j < d) {
     for (int i = 1; i < SETUP_THREADS / 32; ++i) s += red[i][lane];
     const float m = (float)(s / (double)k);
-    center[j] = isfinite(m) ? m : 0.f;
+    if (center) center[j] = isfinite(m) ? m : 0.f;
   }
   if (blockIdx.x == 0)
     for (uint32_t i = threadIdx.x; i < k; i += SETUP_THREADS) cnew[i] = 0;
@@ -1737,6 +1737,11 @@ inline uint64_t a256(uint64_t x) { return (x + 255) & ~255ull; }
 
 }  // namespace
 
+// A job needs no more memory than the form that kept lists of one purpose each
+// did, so a budget that held it holds it: the transposed centroids lie in the
+// result's place for the centroids, which the last kernel writes; the sorted
+// update's cursors and the norms share theirs (the distance pass has read the
+// norms by then, and the centroids' kernel makes the next ones after the sums).
 size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool bounds) {
   uint64_t b = 0;
   b += a256((uint64_t)k * d * 4);      // cent
@@ -1746,10 +1751,8 @@ size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool boun
   b += 256;                            // stats, counters (nflag, maxabs, cmax, pairs), shift
   b += a256((uint64_t)n * 4);          // points to re-check; the sorted update's permutation
   b += a256((uint64_t)n * sizeof(KmFew));  // points with a few candidates
-  b += a256((uint64_t)k * 4);          // ||c||^2
-  b += a256((uint64_t)d * 4);          // center
-  b += a256((uint64_t)k * d * 4);      // transposed centroids
-  b += a256((uint64_t)k * 4);          // per-cluster write cursor
+  b += a256((uint64_t)k * 4);          // ||c||^2; per-cluster write cursor
+  if (wide || km_tc_supported(d, k)) b += a256((uint64_t)d * 4);  // center
   if (local_sums_fit(d, k)) b += a256((uint64_t)LS_MAX_CTAS * k * d * 8);  // per-CTA partial sums
   if (wide) b += a256(km_wide_operand_bytes(d, k));
   if (bounds) b += 3 * a256((uint64_t)n * 4) + 2 * a256((uint64_t)k * 4);
@@ -1772,9 +1775,8 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide, bool bou
   b.flagged = reinterpret_cast<uint32_t*>(take(n * 4));
   b.pairs = reinterpret_cast<KmFew*>(take(n * sizeof(KmFew)));
   b.cnorm = reinterpret_cast<float*>(take(k * 4));
-  b.center = reinterpret_cast<float*>(take(d * 4));
-  b.ct = reinterpret_cast<float*>(take(k * d * 4));
-  b.kcursor = reinterpret_cast<uint32_t*>(take(k * 4));
+  b.kcursor = reinterpret_cast<uint32_t*>(b.cnorm);
+  b.center = wide || km_tc_supported(b.d, b.k) ? reinterpret_cast<float*>(take(d * 4)) : nullptr;
   b.part = local_sums_fit(d, k) ? reinterpret_cast<long long*>(take((uint64_t)LS_MAX_CTAS * k * d * 8)) : nullptr;
   b.bop = wide ? take(km_wide_operand_bytes((uint32_t)d, (uint32_t)k)) : nullptr;
   if (bounds) {
@@ -1811,6 +1813,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   cudaError_t e;
   const uint32_t n = b.n, d = b.d, k = b.k;
   int* shift = b.shift;
+  float* ct = out_c;  // [d][k] transposed centroids, until km_finish_kernel writes the result there
   auto cmax_of = [&](uint32_t it) { return b.nflag + 6 + (it & 1); };  // max ||c||, one word per parity of the round
     // The distance pass only has to settle the clear cases (every near tie is
   // re-checked), so an FP32 job takes the tensor-core pass on split operands
@@ -1899,7 +1902,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
                       local ? (const long long*)b.part : (const long long*)nullptr, ls_grid, b.sums, b.cent, k, d,
                       b.counts, b.counts + k, it > 1 ? (const uint32_t*)chg_of(it - 1) : (const uint32_t*)nullptr, lim,
                       chg_of(it),
-                      (const int*)shift, center, b.cnorm, cmax_of(it), b.ct, wide ? b.bop : (uint8_t*)nullptr, drift,
+                      (const int*)shift, center, b.cnorm, cmax_of(it), ct, wide ? b.bop : (uint8_t*)nullptr, drift,
                       maxdrift, b.nflag, first ? 1u : 0u);
   };
   if ((e = finalize(0, true)) != cudaSuccess) return e;
@@ -1913,7 +1916,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
       if (skip) {
         const uint64_t fb = ((uint64_t)n + FI_THREADS * 4 - 1) / (FI_THREADS * 4);
         if ((e = launch_pdl(km_half_kernel, dim3(k), dim3(HALF_THREADS), 0, s, (const float*)b.cent,
-                            (const float*)b.ct, k, d, b.half, maxdrift, far, nact)) != cudaSuccess ||
+                            (const float*)ct, k, d, b.half, maxdrift, far, nact)) != cudaSuccess ||
             (e = launch_pdl(km_filter_kernel, dim3((unsigned)(fb < 2ull * di.sms ? fb : 2ull * di.sms)),
                             dim3(FI_THREADS), 0, s, (const uint32_t*)b.assign, n, k, bounds, (const float*)b.half,
                             b.act, nact)) != cudaSuccess)
@@ -1934,7 +1937,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
       ++*nk;
     }
     if ((e = launch_pdl(set_kernel, dim3(di.sms * (2048 / set_t < 8 ? 2048 / set_t : 8)), dim3(set_t), set_bytes, s, x,
-                        n, d, (const float*)b.cent, (const float*)b.ct, k, (const KmFew*)b.pairs,
+                        n, d, (const float*)b.cent, (const float*)ct, k, (const KmFew*)b.pairs,
                         (const uint32_t*)(b.nflag + 4), (const uint32_t*)b.flagged, (const uint32_t*)(b.nflag + 1),
                         b.assign, chg, b.stats, it == 0 ? (const unsigned int*)b.maxabs : (const unsigned int*)nullptr,
                         shift, cmax_of(it + 1), bounds)) != cudaSuccess)

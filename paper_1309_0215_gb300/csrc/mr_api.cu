@@ -455,7 +455,7 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
       uint64_t scr = align256(km_scratch_bytes(N, D, K, wide, bounds));
       const uint64_t init_bytes = d.input_on_device ? 0 : align256((uint64_t)K * D * 4);
       mr_status st = dev_alloc(c, res + scr + init_bytes, &j->slab);
-      if ((st == MR_EBUDGET && wide) || (st == MR_ENOMEM && bounds)) {
+      if ((st == MR_EBUDGET || st == MR_ENOMEM) && (wide || bounds)) {
         wide = bounds = false;
         scr = align256(km_scratch_bytes(N, D, K, false, false));
         st = dev_alloc(c, res + scr + init_bytes, &j->slab);

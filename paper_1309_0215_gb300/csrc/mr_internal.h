@@ -226,8 +226,7 @@ struct KmBuffers {
                                 //     rounds: [0], [5] points that changed cluster, [6], [7] max||c|| bits
   KmFew* pairs = nullptr;       // [n] points with a few candidate centroids
   float* cnorm = nullptr;       // [k] ||c||^2 (of the shifted centroids on the tensor-core path)
-  float* center = nullptr;      // [d] the shift
-  float* ct = nullptr;          // [d][k] transposed centroids
+  float* center = nullptr;      // [d] the shift (nullptr where no tensor-core pass covers the shape)
   unsigned int* maxabs = nullptr;  // [1] bits of max |x|
   int* shift = nullptr;         // [1] fixed-point scale exponent
   KmBounds bounds;              // ub nullptr: not kept
@@ -235,7 +234,7 @@ struct KmBuffers {
   uint32_t* act = nullptr;      // [n] points whose distances the round computes
   uint64_t* host = nullptr;     // pinned host word for the count of timed-out waits, written by the last kernel (or null)
   uint8_t* bop = nullptr;       // centroid operands of the wide tensor-core pass (nullptr: not taken)
-  uint32_t* kcursor = nullptr;  // [k] counting-sort write cursors
+  uint32_t* kcursor = nullptr;  // [k] counting-sort write cursors, in the norms' place
   long long* part = nullptr;    // [CTAs][k][d] partial sums of the local-array update (nullptr: sort path)
   KTimer* kt = nullptr;         // times the distance pass of each iteration
   int precision = 0;

@@ -475,3 +475,51 @@ def test_kmeans_centroids_not_finite(mr, n, d, k, iters, bad, offset):
         assert np.array_equal(a, a_ref), precision
         assert _rel_err(c[finite], c_ref[finite]) <= TOL
         assert np.array_equal(c[~finite], c_ref[~finite], equal_nan=True)
+
+
+def _a256(v):
+    return (v + 255) // 256 * 256
+
+
+def _km_bytes(n, d, k, precision):
+    """Device bytes within which a job has always run: the result, and scratch of
+    the sizes the first form of the passes took."""
+    scratch = (_a256(4 * k * d) + _a256(4 * n + 16) + _a256(8 * k * d) + 2 * _a256(8 * k) + 3 * 256 +
+               2 * _a256(4 * n) + _a256(8 * n) + _a256(4 * k))
+    if precision:
+        scratch += _a256(4 * n) + _a256(4 * k * d)
+    if 8 * k * d + 4 * k <= 200 * 1024:
+        scratch += _a256(160 * 8 * k * d)
+    return _a256((4 * k * d + 4 * n + 7) // 8 * 8 + 32) + scratch
+
+
+@pytest.mark.parametrize("limit", ["budget", "allocator"])
+@pytest.mark.parametrize("n,d,k,precision", [
+    (3_000, 64, 256, 0), (3_000, 64, 256, 1), (500, 1, 1, 0), (40, 48, 17, 1), (7, 33, 250, 1),
+    (2_000, 100, 300, 0), (900, 256, 1_000, 0),    # the wide pass's shapes, without room for its operands
+    (600, 1_024, 64, 0), (50, 1_024, 4_096, 0), (700, 7, 4_096, 0), (2_100, 300, 200, 0),
+])
+def test_kmeans_runs_in_as_much_memory_as_ever(mr, n, d, k, precision, limit):
+    """A budget, or an allocator's largest piece, of what a job needs at least."""
+    import torch
+    x, _, _ = synth.kmeans_points(n, d, 4, seed=n)
+    init = x[np.random.default_rng(k).integers(0, n, k)].copy()
+    room = _km_bytes(n, d, k, precision)
+    if limit == "budget":
+        ctx = mr.Context(hbm_budget=room)
+    else:
+        dev, stream = torch.cuda.current_device(), torch.cuda.current_stream().cuda_stream
+        ctx = mr.Context(allocator=(
+            lambda b: torch.cuda.caching_allocator_alloc(b, dev, stream) if b <= room else 0,
+            torch.cuda.caching_allocator_delete))
+    c2, a2, _ = _run_ctx(mr, ctx, _dev(x), init, 2, precision)
+    ctx.close()
+    # (the initial centroids hold equal ones, whose ties follow the last bit of
+    # the first round's means: each round is compared from its own start)
+    for _ in range(2):
+        a_ref = oracle.kmeans_assign(x, init)
+        c_ref, _ = oracle.kmeans_update(x, a_ref, init)
+        init, a, _ = _run(mr, x, init, 1, precision)
+        assert np.array_equal(a, a_ref)
+        assert _rel_err(init, c_ref) <= TOL
+    assert np.array_equal(a2, a) and np.array_equal(c2, init)
