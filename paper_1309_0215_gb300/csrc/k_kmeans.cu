@@ -1742,7 +1742,7 @@ inline uint64_t a256(uint64_t x) { return (x + 255) & ~255ull; }
 // result's place for the centroids, which the last kernel writes; the sorted
 // update's cursors and the norms share theirs (the distance pass has read the
 // norms by then, and the centroids' kernel makes the next ones after the sums).
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool bounds) {
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide) {
   uint64_t b = 0;
   b += a256((uint64_t)k * d * 4);      // cent
   b += a256((uint64_t)n * 4 + 16);     // assign (+16: the update copies ids in 16-byte units)
@@ -1755,11 +1755,10 @@ size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool boun
   if (wide || km_tc_supported(d, k)) b += a256((uint64_t)d * 4);  // center
   if (local_sums_fit(d, k)) b += a256((uint64_t)LS_MAX_CTAS * k * d * 8);  // per-CTA partial sums
   if (wide) b += a256(km_wide_operand_bytes(d, k));
-  if (bounds) b += 3 * a256((uint64_t)n * 4) + 2 * a256((uint64_t)k * 4);
   return (size_t)b;
 }
 
-cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide, bool bounds) {
+cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide) {
   const uint64_t n = b.n, d = b.d, k = b.k;
   uint8_t* q = p;
   auto take = [&](uint64_t sz) { uint8_t* r = q; q += a256(sz); return r; };
@@ -1779,16 +1778,20 @@ cudaError_t km_carve(KmBuffers& b, uint8_t* p, size_t bytes, bool wide, bool bou
   b.center = wide || km_tc_supported(b.d, b.k) ? reinterpret_cast<float*>(take(d * 4)) : nullptr;
   b.part = local_sums_fit(d, k) ? reinterpret_cast<long long*>(take((uint64_t)LS_MAX_CTAS * k * d * 8)) : nullptr;
   b.bop = wide ? take(km_wide_operand_bytes((uint32_t)d, (uint32_t)k)) : nullptr;
-  if (bounds) {
-    b.bounds.ub = reinterpret_cast<float*>(take(n * 4));
-    b.bounds.lb = reinterpret_cast<float*>(take(n * 4));
-    b.act = reinterpret_cast<uint32_t*>(take(n * 4));
-    b.bounds.drift = reinterpret_cast<float*>(take(k * 4));
-    b.half = reinterpret_cast<float*>(take(k * 4));
-    b.bounds.far = reinterpret_cast<float*>(ctl + 136);
-  }
   if ((uint64_t)(q - p) > bytes) return cudaErrorInvalidValue;
   return cudaSuccess;
+}
+
+size_t km_bounds_bytes(uint32_t n, uint32_t k) { return 3 * a256((uint64_t)n * 4) + 2 * a256((uint64_t)k * 4); }
+
+void km_carve_bounds(KmBuffers& b, uint8_t* p) {
+  auto take = [&](uint64_t words) { uint8_t* r = p; p += a256(words * 4); return r; };
+  b.bounds.ub = reinterpret_cast<float*>(take(b.n));
+  b.bounds.lb = reinterpret_cast<float*>(take(b.n));
+  b.act = reinterpret_cast<uint32_t*>(take(b.n));
+  b.bounds.drift = reinterpret_cast<float*>(take(b.k));
+  b.half = reinterpret_cast<float*>(take(b.k));
+  b.bounds.far = reinterpret_cast<float*>(b.shift) + 2;
 }
 
 // The filter pays for its two kernels (10 - 24 us a round) and the bounds the

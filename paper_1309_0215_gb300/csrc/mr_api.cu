@@ -56,6 +56,7 @@ struct Job {
   mr_job_desc desc{};
   mr_container container = MR_C_AUTO;
   JobState state = JOB_PENDING;
+  bool launched = false;         // its kernels use its memory (or did, until a launch failed)
   const uint8_t* in = nullptr;   // device input
   void* in_owned = nullptr;      // device copy of a host input
   uint64_t in_owned_bytes = 0;
@@ -71,7 +72,11 @@ struct Job {
   bool wc_auto = true;
   // large-key histogram: u32 counters (null: count straight into the u64 result)
   void* hk_counters = nullptr;
-  uint8_t* part = nullptr;  // scratch of partitioned counting, large-key histogram and Bloom filter (null: not taken)
+  // scratch that a faster form of the job needs and the job does not: of
+  // partitioned counting (large-key histogram, Bloom filter), or the k-means
+  // filter's bounds (null: the job runs, or ran, without)
+  void* extra = nullptr;
+  uint64_t extra_bytes = 0;
   // k-means
   KmBuffers km;
   uint64_t* host = nullptr;      // pinned status words (word count, k-means)
@@ -208,7 +213,7 @@ struct DeviceGuard {
   }
 };
 
-mr_status dev_alloc(mr_ctx* c, uint64_t bytes, void** out) {
+mr_status dev_alloc_once(mr_ctx* c, uint64_t bytes, void** out) {
   *out = nullptr;
   if (bytes == 0) bytes = 256;
   if (c->budget && c->in_use + bytes > c->budget) return MR_EBUDGET;
@@ -237,7 +242,36 @@ void dev_free(mr_ctx* c, void* p, uint64_t bytes) {
   c->in_use -= bytes < c->in_use ? bytes : c->in_use;
 }
 
+// A job's extra scratch goes back; a job not launched yet then takes its other form.
+void free_extra(mr_ctx* c, Job* j) {
+  dev_free(c, j->extra, j->extra_bytes);
+  j->extra = nullptr;
+  j->km.bounds = KmBounds{};
+}
+
+// Device memory that a job or the context cannot do without: when there is none
+// left, the extra scratch of jobs that are not running makes room.
+mr_status dev_alloc(mr_ctx* c, uint64_t bytes, void** out) {
+  mr_status st = dev_alloc_once(c, bytes, out);
+  if (st != MR_ENOMEM) return st;
+  bool freed = false;
+  for (auto& it : c->jobs) {
+    Job* j = it.second;
+    if (!j->extra || (j->launched && (j->state != JOB_ENQUEUED || cudaEventQuery(j->done) != cudaSuccess))) continue;
+    free_extra(c, j);
+    freed = true;
+  }
+  return freed ? dev_alloc_once(c, bytes, out) : st;
+}
+
 inline uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
+
+bool alloc_extra(mr_ctx* c, Job* j, uint64_t bytes) {
+  bytes = align256(bytes);
+  if (dev_alloc_once(c, bytes, &j->extra) != MR_OK) return false;
+  j->extra_bytes = bytes;
+  return true;
+}
 
 inline uint64_t km_stats_offset(uint64_t K, uint64_t D, uint64_t N) { return (K * D * 4 + N * 4 + 7) & ~7ull; }
 
@@ -395,51 +429,39 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
     case MR_HIST_U32: {
       const uint64_t nb = (uint64_t)d.hist_bins + 1;
       const uint64_t res = align256(nb * 8);
-      // u32 counters while no bin can reach 2^32; local arrays are few enough
-      // to be added straight into the result
-      const bool wide = d.input_bytes / 4 >= (1ull << 32) || j->container == MR_C_SMEM_ARRAY;
-      uint64_t cnt = wide ? 0 : align256(nb * 4);
-      // partitioned counting, if the library chooses the container and there
-      // is memory for its scratch (a context with a budget keeps it for jobs);
-      // else counters of the global array
+      // partitioned counting, if the library chooses the container and there is
+      // memory for its scratch (a context with a budget keeps it for jobs)
       if (d.container == MR_C_AUTO && j->container == MR_C_GLOBAL_ARRAY && c->budget == 0 &&
-          hk_partitioned(d.input_bytes / 4, d.hist_bins)) {
-        const uint64_t scr = align256(hk_part_bytes(d.input_bytes / 4, d.hist_bins));
-        if (dev_alloc(c, res + scr, &j->slab) == MR_OK) {
-          j->slab_bytes = res + scr;
-          j->result = j->slab;
-          j->result_bytes = nb * 8;
-          j->part = static_cast<uint8_t*>(j->slab) + res;
-          return MR_OK;
-        }
+          hk_partitioned(d.input_bytes / 4, d.hist_bins))
+        alloc_extra(c, j, hk_part_bytes(d.input_bytes / 4, d.hist_bins));
+      // else u32 counters while no bin can reach 2^32; local arrays are few
+      // enough to be added straight into the result
+      const bool wide = d.input_bytes / 4 >= (1ull << 32) || j->container == MR_C_SMEM_ARRAY;
+      const uint64_t cnt = wide ? 0 : align256(nb * 4);
+      uint64_t bytes = res + (j->extra ? 0 : cnt);
+      mr_status st = dev_alloc(c, bytes, &j->slab);
+      if (st == MR_ENOMEM && j->extra) {
+        free_extra(c, j);
+        st = dev_alloc(c, bytes = res + cnt, &j->slab);
       }
-      mr_status st = dev_alloc(c, res + cnt, &j->slab);
       if (st) return st;
-      j->slab_bytes = res + cnt;
+      j->slab_bytes = bytes;
       j->result = j->slab;
       j->result_bytes = nb * 8;
-      j->hk_counters = wide ? nullptr : static_cast<uint8_t*>(j->slab) + res;
+      j->hk_counters = bytes == res ? nullptr : static_cast<uint8_t*>(j->slab) + res;
       return MR_OK;
     }
     case MR_BLOOM_DNA: {
       const uint64_t bytes = align256((d.bloom_bits + 31) / 32 * 4);
-      j->result_bytes = (d.bloom_bits + 7) / 8;
-      // as for the large-key histogram
-      if (d.container == MR_C_AUTO && c->budget == 0 &&
-          bloom_partitioned(d.input_bytes, d.bloom_kmer, d.bloom_bits, d.bloom_hashes)) {
-        const uint64_t scr = align256(bloom_part_bytes(d.input_bytes, d.bloom_kmer, d.bloom_bits, d.bloom_hashes));
-        if (dev_alloc(c, bytes + scr, &j->slab) == MR_OK) {
-          j->slab_bytes = bytes + scr;
-          j->result = j->slab;
-          j->part = static_cast<uint8_t*>(j->slab) + bytes;
-          return MR_OK;
-        }
-      }
       mr_status st = dev_alloc(c, bytes, &j->slab);
       if (st) return st;
       j->slab_bytes = bytes;
       j->result = j->slab;
       j->result_bytes = (d.bloom_bits + 7) / 8;
+      // as for the large-key histogram
+      if (d.container == MR_C_AUTO && c->budget == 0 &&
+          bloom_partitioned(d.input_bytes, d.bloom_kmer, d.bloom_bits, d.bloom_hashes))
+        alloc_extra(c, j, bloom_part_bytes(d.input_bytes, d.bloom_kmer, d.bloom_bits, d.bloom_hashes));
       return MR_OK;
     }
     case MR_KMEANS_F32: {
@@ -448,16 +470,15 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
       // result: centroids [K*D] f32 | assignments [N] i32 | pad to 8 | stats [4] u64
       const uint64_t res_bytes = km_stats_offset(K, D, N) + 32;
       const uint64_t res = align256(res_bytes);
-      // the wide tensor-core pass keeps its centroid operands in scratch, the
-      // filter its bounds; a context without room for them runs without
+      // the wide tensor-core pass keeps its centroid operands in scratch; a
+      // context without room for them runs without
       bool wide = d.km_precision == MR_KM_FP32 && !km_tc_supported(D, K) && km_wide_supported(D, K);
-      bool bounds = !c->budget && !wide && km_tc_supported(D, K) && km_bounds_pay(N, d.km_iters);
-      uint64_t scr = align256(km_scratch_bytes(N, D, K, wide, bounds));
+      uint64_t scr = align256(km_scratch_bytes(N, D, K, wide));
       const uint64_t init_bytes = d.input_on_device ? 0 : align256((uint64_t)K * D * 4);
       mr_status st = dev_alloc(c, res + scr + init_bytes, &j->slab);
-      if ((st == MR_EBUDGET || st == MR_ENOMEM) && (wide || bounds)) {
-        wide = bounds = false;
-        scr = align256(km_scratch_bytes(N, D, K, false, false));
+      if ((st == MR_EBUDGET || st == MR_ENOMEM) && wide) {
+        wide = false;
+        scr = align256(km_scratch_bytes(N, D, K, false));
         st = dev_alloc(c, res + scr + init_bytes, &j->slab);
       }
       if (st) return st;
@@ -469,11 +490,14 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
       j->km.d = D;
       j->km.k = K;
       j->km.precision = (int)d.km_precision;
-      cudaError_t e = km_carve(j->km, p + res, scr, wide, bounds);
+      cudaError_t e = km_carve(j->km, p + res, scr, wide);
       if (e != cudaSuccess) {
         set_last_error("km_carve", e);
         return MR_EINVAL;
       }
+      if (!c->budget && km_tc_supported(D, K) && km_bounds_pay(N, d.km_iters) &&
+          alloc_extra(c, j, km_bounds_bytes(N, K)))
+        km_carve_bounds(j->km, static_cast<uint8_t*>(j->extra));
       if (!d.input_on_device) {
         j->km_init_dev = reinterpret_cast<float*>(p + res + scr);
         MR_CUDA_TRY(cudaMemcpyAsync(j->km_init_dev, d.km_init, (size_t)K * D * 4, cudaMemcpyHostToDevice, c->stream));
@@ -494,6 +518,7 @@ void free_job(mr_ctx* c, Job* j) {
   if (j->t1) c->ev_timing.push_back(j->t1);
   if (j->kt) c->kt_pool.push_back(j->kt);
   if (j->host) c->status_free.push_back(j->host);
+  free_extra(c, j);
   dev_free(c, j->slab, j->slab_bytes);
   dev_free(c, j->in_owned, j->in_owned_bytes);
   delete j;
@@ -516,6 +541,7 @@ int grid_for(const mr_ctx* c, uint64_t bytes, uint64_t bytes_per_block, int max_
 
 mr_status enqueue_plain_on(mr_ctx* c, Job* j, cudaStream_t st) {
   const uint64_t n = j->desc.input_bytes;
+  j->launched = true;
   if (j->t0) MR_CUDA_TRY(cudaEventRecord(j->t0, st));
   if (j->kt) j->kt->n = 0;
   switch (j->desc.kind) {
@@ -548,9 +574,9 @@ mr_status enqueue_plain_on(mr_ctx* c, Job* j, cudaStream_t st) {
                                    c->opt_polls));
       break;
     case MR_HIST_U32:
-      if (j->part) {
+      if (j->extra) {
         MR_CUDA_TRY(launch_hist_keys_part(reinterpret_cast<const uint32_t*>(j->in), n / 4, j->desc.hist_bins,
-                                          j->part, static_cast<unsigned long long*>(j->result), c->di, st,
+                                          static_cast<uint8_t*>(j->extra), static_cast<unsigned long long*>(j->result), c->di, st,
                                           &c->launches, j->kt));
         break;
       }
@@ -559,9 +585,10 @@ mr_status enqueue_plain_on(mr_ctx* c, Job* j, cudaStream_t st) {
                                    static_cast<unsigned long long*>(j->result), c->di, st, &c->launches, j->kt));
       break;
     case MR_BLOOM_DNA:
-      if (j->part) {
-        MR_CUDA_TRY(launch_bloom_part(j->in, n, j->desc.bloom_kmer, j->desc.bloom_bits, j->desc.bloom_hashes, j->part,
-                                      static_cast<uint32_t*>(j->result), c->di, st, &c->launches, j->kt));
+      if (j->extra) {
+        MR_CUDA_TRY(launch_bloom_part(j->in, n, j->desc.bloom_kmer, j->desc.bloom_bits, j->desc.bloom_hashes,
+                                      static_cast<uint8_t*>(j->extra), static_cast<uint32_t*>(j->result), c->di, st,
+                                      &c->launches, j->kt));
         break;
       }
       MR_CUDA_TRY(launch_bloom(j->in, n, j->desc.bloom_kmer, j->desc.bloom_bits, j->desc.bloom_hashes,
@@ -985,6 +1012,7 @@ mr_status wait_job(mr_ctx* c, Job* j, uint64_t* wc_result_bytes = nullptr) {
   }
   if (j->state == JOB_PENDING) return MR_ENOTREADY;
   MR_CUDA_TRY(cudaEventSynchronize(j->done));
+  if (j->extra) free_extra(c, j);
   // the status words the job's last kernel wrote
   const volatile uint64_t* h = j->host;
   if (j->desc.kind == MR_KMEANS_F32) return h[0] ? MR_ETIMEOUT : MR_OK;  // device waits that gave up

@@ -245,10 +245,13 @@ struct KmBuffers {
   uint32_t grid_cap = 0;
   uint32_t stop_copies = 0;
 };
-// wide: with the wide tensor-core pass's operands; bounds: with the points' bounds
-size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide, bool bounds);
+// wide: with the wide tensor-core pass's operands
+size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide);
+cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes, bool wide);
+// the filter's bounds, in memory of their own (after km_carve)
 bool km_bounds_pay(uint32_t n, uint32_t iters);
-cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes, bool wide, bool bounds);
+size_t km_bounds_bytes(uint32_t n, uint32_t k);
+void km_carve_bounds(KmBuffers& b, uint8_t* base);
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,
                           cudaStream_t s, float* out_cent, int32_t* out_assign, unsigned long long* out_stats,
                           uint64_t* nk);

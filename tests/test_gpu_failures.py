@@ -229,3 +229,65 @@ def test_batched_run_allocation_failure_keeps_jobs_pending(mr):
         ctx.release(j)
     ctx.close()
     assert al.live == {}
+
+
+def test_scratch_that_jobs_can_do_without_makes_room(mr):
+    """Grouping and filter scratch is held from mr_add_job until the job is seen
+    to be done, and no longer; a job that finds no memory takes that of jobs
+    which have not been launched, and those run without it."""
+    import torch
+    al = _Alloc()
+    cap = [1 << 40]
+
+    def alloc(n):
+        return al.alloc(n) if sum(al.live.values()) + n <= cap[0] else 0
+
+    seq = synth.dna(2_400_031, seed=71, n_runs=20, max_run=500)
+    keys = synth.keys_u32(1 << 22, 1 << 20, seed=72)
+    x, _, _ = synth.kmeans_points(400_009, 4, 5, seed=73)
+    init = synth.kmeans_init(x, 5, seed=74)
+    dev = {name: torch.from_numpy(a).cuda() for name, a in
+           dict(seq=seq, keys=keys.view(np.int32), x=x, init=init).items()}
+    bloom = (mr.BLOOM_DNA, dev["seq"], dict(bloom_kmer=20, bloom_bits=1 << 24, bloom_hashes=7),
+             oracle.bloom_dna(seq, 20, 1 << 24, 7).tobytes())
+    hist = (mr.HIST_U32, dev["keys"], dict(hist_bins=1 << 20), oracle.hist_u32(keys, 1 << 20).tobytes())
+    km = (mr.KMEANS_F32, dev["x"], dict(km_dims=4, km_k=5, km_iters=6, km_init=dev["init"]), None)
+    big = (mr.HIST_U32, dev["keys"], dict(hist_bins=6_000_000, container=mr.C_GLOBAL_ARRAY),
+           oracle.hist_u32(keys, 6_000_000).tobytes())
+    torch.cuda.synchronize()
+    ctx = mr.Context(allocator=(alloc, al.free))
+    km_want = None
+    for short in (False, True):
+        cap[0] = 1 << 40
+        jobs = []
+        for kind, data, kw, want in (bloom, hist, km):
+            before = ctx.bytes_in_use
+            j = ctx.add_job(kind, data, **kw)
+            jobs.append((j, want, ctx.bytes_in_use - before))
+        if short:
+            # 6 M bins, 72 MB: they fit once the three jobs' scratch is back
+            cap[0] = sum(al.live.values()) + (1 << 20)
+            before = ctx.bytes_in_use
+            kind, data, kw, want = big
+            jobs.append((ctx.add_job(kind, data, **kw), want, 0))
+            assert ctx.bytes_in_use - before < 72 << 20
+        ctx.run()
+        for j, want, held in jobs:
+            before = ctx.bytes_in_use
+            got = ctx.fetch(j)
+            if want is not None:
+                assert got == want
+            elif km_want is None:
+                km_want = got
+            else:
+                assert got[:-32] == km_want[:-32]  # (but for the statistics: more near ties without the filter)
+            if not short:
+                assert ctx.bytes_in_use < before  # (the scratch is back, the result still there)
+                assert ctx.fetch(j) == got
+        for j, _, _ in jobs:
+            ctx.release(j)
+        assert ctx.bytes_in_use == 0
+    c_ref, a_ref = oracle.kmeans(x, init, 6)
+    assert np.array_equal(mr.split_kmeans_result(km_want, 400_009, 4, 5)[1], a_ref)
+    ctx.close()
+    assert not al.live
