@@ -79,8 +79,9 @@ typedef enum {
    * input 4-byte aligned); key k < hist_bins emits (k, 1), any other key
    * (hist_bins, 1).  Output: uint64 bins[hist_bins + 1].  With many keys over
    * many bins MR_C_AUTO groups the keys by ranges of bins first, through 2
-   * bytes of device scratch per key (at most 512 MiB); a context with an HBM
-   * budget, or without memory for it, counts in the global array instead. */
+   * bytes of device scratch per key and tables of a few percent more (at most
+   * 544 MiB, until the job is seen to be done); a context with an HBM budget,
+   * or without memory for it, counts in the global array instead. */
   MR_HIST_U32 = 4,
   /* Bloom-filter build (the paper's Bloom Filter application: k-mers of a
    * chromosome, 30M elements into 300M entries, Sec. IV data sets; array
@@ -91,9 +92,9 @@ typedef enum {
    * mod m and b = 1 + mix(code ^ 0x9E3779B97F4A7C15) mod (m - 1), the element
    * sets bits (a + i*b) mod m for i < bloom_hashes (m = bloom_bits).  Output:
    * ceil(m / 8) bytes, bit j = bit (j mod 8) of byte j / 8.  With many positions
-   * MR_C_AUTO groups them by ranges of bits first, through 4 bytes of device
-   * scratch per position (at most 2 GiB), under the same conditions as the
-   * large-key histogram. */
+   * MR_C_AUTO groups them by ranges of bits first, through about 4 bytes of
+   * device scratch per position (4.4 at most, and 2.1 GiB in all), under the
+   * same conditions as the large-key histogram. */
   MR_BLOOM_DNA = 5
 } mr_kind;
 

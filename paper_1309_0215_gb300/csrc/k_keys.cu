@@ -663,18 +663,21 @@ bloom_kernel(const uint8_t* __restrict__ seq, uint64_t n, uint32_t L, uint64_t m
 // once.  A chunk is as many windows as have at most BCHUNK positions: they are
 // computed once into shared memory (counting them by bucket), then grouped.
 // 4 bytes a position are written and read again; 30M windows into 3e8 bits take
-// 0.85 ms instead of 1.04 in all (grouping 546 us, bound by issue and the
-// shared-memory pipe; setting 255 us), into 1e6 bits 0.83 instead of 2.16.
+// 0.79 ms instead of 1.04 in all (grouping bound by issue and the shared-memory
+// pipe), into 1e6 bits 0.82 instead of 2.16.
 constexpr int BT = 1024;                 // threads of the grouping kernel (two CTAs per SM)
 constexpr uint32_t BCHUNK = 16384;       // positions
 constexpr uint32_t BNF = 512;            // buckets, at most
 constexpr uint32_t BRANGES = 512;        // ranges, at most
 constexpr uint32_t BS = PS + 5;          // log2 of a range's bits
 constexpr uint32_t BNONE = 0xFFFFFFFFu;  // no position (m <= 2^29)
-// windows per chunk: whole rounds of the CTA's threads, or of a warp's
-__host__ __device__ constexpr uint32_t bloom_windows(uint32_t h) {
-  return BCHUNK / h >= (uint32_t)BT ? BCHUNK / h / BT * BT : BCHUNK / h / 32 * 32;
-}
+// Windows per chunk: as many whole warps of them as the chunk has room for, so
+// that its positions take little more than the 4 bytes each that the interface
+// states.  (Whole rounds of the CTA's threads filled chunks of 9 hashes to 56%,
+// 7.2 bytes a position, and were slower: 30M windows into 3e8 bits, us a call,
+// 5 hashes 624 / 608, 6 742 / 695, 7 829 / 788, 9 1,164 / 969, 12 1,302 / 1,243;
+// into 1e6 bits 6 hashes 732 / 761, 9 1,161 / 1,061.)
+__host__ __device__ constexpr uint32_t bloom_windows(uint32_t h) { return BCHUNK / h / 32 * 32; }
 static_assert(bloom_windows(32) >= 32, "a chunk holds windows for every number of hashes");
 struct BitItems {
   using Item = uint32_t;
@@ -973,10 +976,10 @@ cudaError_t launch_bloom(const uint8_t* seq, uint64_t n, uint32_t L, uint64_t m,
 // Partitioned filter: up to 2^29 bits (512 ranges), from 2^24 positions on, with
 // at least 5 hashes (the two 64-bit mixes of a window are paid once) or few
 // ranges, whose words the L2's atomics contend for.  Measured, partitioned
-// against atomicOr on the global array, us a call: 30M windows x 7 into 2.4e8
-// bits 949 / 1,032, x 3 500 / 465 (left to the array), x 3 into 1e6 472 / 944;
+// against atomicOr on the global array, us a call: 30M windows x 7 into 3e8
+// bits 788 / 1,040, x 3 into 2.4e8 500 / 465 (left to the array), x 3 into 1e6 472 / 944;
 // 3M x 7 into 2.4e7 124 / 144; 5.6M x 3 into 1e6 155 / 203.
-constexpr uint64_t BLOOM_ROUND = 1ull << 29;  // positions grouped at a time (4 bytes each of scratch)
+constexpr uint64_t BLOOM_ROUND = 1ull << 29;  // positions grouped at a time (4 bytes each of scratch, and gaps of at most 6%)
 bool bloom_partitioned(uint64_t n, uint32_t L, uint64_t m, uint32_t h) {
   return n >= L && m <= (uint64_t)BRANGES << BS && (n - L + 1) * h >= 1ull << 24 && (h >= 5 || m <= 1ull << 24);
 }

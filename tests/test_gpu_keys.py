@@ -222,3 +222,35 @@ def test_bloom_partitioned_rounds_and_budget(mr):
     want = np.frombuffer(ctx.fetch(j), dtype=np.uint8)
     ctx.close()
     assert np.array_equal(mr.bloom_dna(seq, L, m, h), want)
+
+
+@pytest.mark.parametrize("L,h", [(32, 7), (32, 5), (17, 6), (21, 9), (20, 10), (25, 12), (11, 27), (32, 32)])
+@pytest.mark.parametrize("offset", [0, 1, 3])
+def test_bloom_partitioned_windows_and_scratch(mr, L, h, offset):
+    """The grouped path, seen to be taken by its scratch: at most 4.4 bytes a
+    position whatever the number of hashes (chunks of whole warps of windows),
+    windows of all lengths up to 32 at any start, runs of N."""
+    import torch
+    m = 20_000_003
+    n = ((1 << 24) + 300_000) // h + L
+    seq = synth.dna(n, seed=h + L, n_runs=50, max_run=3000)
+    dev = _dev(seq, offset)
+    torch.cuda.synchronize()
+    with mr.Context() as ctx:
+        j = ctx.add_job(mr.BLOOM_DNA, dev, bloom_kmer=L, bloom_bits=m, bloom_hashes=h)
+        scratch = ctx.bytes_in_use - (m + 7) // 8
+        assert 3.9 <= scratch / ((n - L + 1) * h) <= 4.4
+        ctx.run()
+        assert np.array_equal(np.frombuffer(ctx.fetch(j), dtype=np.uint8), oracle.bloom_dna(seq, L, m, h))
+
+
+@pytest.mark.parametrize("n,nbins", [(1 << 22, 1 << 20), ((1 << 24) + 4_099, 65_535)])
+def test_hist_u32_partitioned_scratch(mr, n, nbins):
+    """The grouped path is seen to be taken, by its 2 bytes a key and its tables."""
+    keys = synth.keys_u32(n, nbins, seed=4)
+    dev = _dev(keys, 4)
+    with mr.Context() as ctx:
+        j = ctx.add_job(mr.HIST_U32, dev, hist_bins=nbins)
+        assert 2.0 <= (ctx.bytes_in_use - 8 * (nbins + 1)) / n <= 2.2
+        ctx.run()
+        assert np.array_equal(np.frombuffer(ctx.fetch(j), dtype=np.uint64), oracle.hist_u32(keys, nbins))
