@@ -2573,7 +2573,9 @@ cudaError_t launch_wordcount_post_multi(const wc::JobDev* jobs, const wc::JobDev
 cudaError_t launch_wordcount(const uint8_t* in, uint64_t n, const WcBuffers& b, const DevInfo& di, cudaStream_t s,
                              uint64_t* nk, bool pipelined, KTimer* kt, long long pipe_polls) {
   cudaError_t e;
-  if (n <= TINY_MAX && b.one_cta && b.cap == TINY_SLOTS && !pipelined) {
+  // (an automatic table of up to TINY_MAX bytes has at most twice the slots; one
+  // that is larger has been regrown, because the text's words did not fit here)
+  if (n <= TINY_MAX && b.one_cta && b.cap <= 2 * TINY_SLOTS && !pipelined) {
     const int smem = (int)sizeof(TinySmem);
     if ((e = cudaFuncSetAttribute(wc_tiny_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess ||
         (e = kt_begin(kt, s)) != cudaSuccess)

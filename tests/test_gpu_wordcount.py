@@ -292,3 +292,33 @@ def test_wc_keys_that_differ_in_the_last_byte_of_each_word(mr):
         i //= 128
     text = text.ravel()
     assert mr.wordcount(_dev(text.tobytes()), wc_slots=1 << 22) == oracle.wordcount(text)
+
+
+@pytest.mark.parametrize("n", [65_534, 65_535, 65_536, 65_537])
+@pytest.mark.parametrize("end", ["word", "space", "one token", "two-byte words", "too many words"])
+def test_wc_largest_text_of_one_cta(mr, n, end):
+    """One launch for texts of up to 65,536 bytes: a word or a delimiter as the
+    last byte, a token of the whole text, as many tokens as there can be; more
+    words than the CTA's table holds take a second attempt."""
+    import torch
+    if end == "one token":
+        text = b"q" * n
+    elif end == "too many words":
+        text = b" ".join(b"%05x" % (i * 7919 % 1048576) for i in range(10_924))[:n]
+    elif end == "two-byte words":
+        text = (b"a b c\nd " * 10_000)[:n]
+    else:
+        zipf, _, _ = synth.wc_text(n, nwords=2000, seed=n)
+        text = bytes(zipf[: n - 9]) + (b" lastword" if end == "word" else b"lastword\n")
+    want = oracle.wordcount(np.frombuffer(text, dtype=np.uint8))
+    with mr.Context() as ctx:
+        for off in (0, 1, 3, 15):
+            buf = torch.full((n + off + 9,), ord("z"), dtype=torch.uint8, device="cuda")
+            buf[off: off + n] = torch.from_numpy(np.frombuffer(text, dtype=np.uint8).copy()).cuda()
+            torch.cuda.synchronize()
+            before = ctx.kernel_launches
+            j = ctx.add_job(mr.WORDCOUNT, buf[off: off + n])
+            ctx.run()
+            assert ctx.fetch(j) == want, off
+            assert (ctx.kernel_launches - before == 1) == (n <= 65_536 and end != "too many words")
+            ctx.release(j)
