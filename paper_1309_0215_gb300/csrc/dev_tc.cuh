@@ -89,9 +89,9 @@ __device__ __forceinline__ void top2_merge(int& a1, int& a2, int b1, int b2) {
 // three-way minimum per key where a running top-2 takes three minima and maxima.
 // cn: the columns' centroid norms, infinite for columns without a centroid (the
 // padding up to a multiple of 16, whose operands are zero); no other column is
-// read.  dbg: null, or where the distances of the first dbg_n columns go.
+// read.  sums: null, or where the columns' raw sums go.
 __device__ __forceinline__ void quarter_keys(uint32_t ta, uint32_t cols, float nxv, const float* cn, int (&col)[GRID],
-                                             int (&row)[GRID], float* dbg, uint32_t dbg_n) {
+                                             int (&row)[GRID], float* sums = nullptr) {
   unsigned long long nx2, m2;
   asm("mov.b64 %0, {%1, %1};" : "=l"(nx2) : "f"(nxv));
   asm("mov.b64 %0, {%1, %1};" : "=l"(m2) : "f"(-2.f));
@@ -117,11 +117,8 @@ __device__ __forceinline__ void quarter_keys(uint32_t ta, uint32_t cols, float n
       key[j] = dist_key(d0, c * CHUNK + j);
       key[j + 1] = dist_key(d1, c * CHUNK + j + 1);
     }
-    if (dbg) {
-      for (int j = 0; j < CHUNK; ++j)
-        if ((uint32_t)(c * CHUNK + j) < dbg_n)
-          dbg[c * CHUNK + j] = fmaf(-2.f, __uint_as_float(acc[j]), nxv) + cn[c * CHUNK + j];
-    }
+    if (sums)
+      for (int j = 0; j < CHUNK; ++j) sums[c * CHUNK + j] = __uint_as_float(acc[j]);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int* k = key + h * GRID;

@@ -40,7 +40,10 @@
 // (one value: |x - hi - lo| <= u_b^2 |x|; sums by Cauchy-Schwarz); a single
 // BF16 product leaves (2 u_b + u_b^2) ||x|| ||c||.  The tensor-core sum of the
 // exact BF16 products is charged (products + 8) * 2^-22 ||x|| ||c|| (four
-// times the round-to-nearest bound, allowing truncating adders), and the FP32
+// times the round-to-nearest bound, allowing truncating adders; how the tensor
+// core rounds is not documented, and the largest error that random and adverse
+// operands show, 192 to 768 products, is 0.05 of the charge:
+// tests/test_gpu_km_sums.py), and the FP32
 // norms and the final fma/add (D + 8) * 2^-24 (||x|| + ||c||)^2 (Higham,
 // eq. 3.5).  Points and centroids are first shifted by the mean m of the
 // initial centroids, x' = fl(x - m) and c' = fl(c - m): distances do not
@@ -118,12 +121,14 @@ __device__ __forceinline__ uint32_t ld_now(const uint32_t* p) {
   return v;
 }
 
-template <int TERMS>
+// SUMS: the tensor core's sums of every point and column go to sums [tiles TM][NMAX]
+// (tests/km_tc_sums.cu measures their error against the charge above).
+template <int TERMS, bool SUMS = false>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, const float* __restrict__ c, uint32_t k,
                     const float* __restrict__ center, const float* __restrict__ cnorm, const unsigned int* cmax_bits, uint32_t* __restrict__ assign, uint32_t* nchg,
                     uint32_t* __restrict__ list, uint32_t* nlist, KmFew* __restrict__ pairs, uint32_t* npairs,
-                    unsigned long long* timeouts, float* dbg, long long polls, uint32_t stop_copies,
+                    unsigned long long* timeouts, float* sums, long long polls, uint32_t stop_copies,
                     unsigned int* maxabs, const uint32_t* __restrict__ act, const uint32_t* nact, KmBounds B) {
   extern __shared__ uint8_t tc_raw[];
   TcSmem& S = *reinterpret_cast<TcSmem*>((reinterpret_cast<uintptr_t>(tc_raw) + 1023) & ~uintptr_t(1023));
@@ -568,10 +573,10 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.nx_free[s]);
       const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * 256u;
-      float* dbg_row = (dbg && tile == 0) ? dbg + (uint64_t)r * NMAX + c_lo : nullptr;
       int w1 = KEY_NONE, w2 = KEY_NONE, lb = KEY_NONE, col[GRID], row[GRID];
       if (c_lo < cols)
-        quarter_keys(ta + c_lo, min(cpq, cols - c_lo), nxv, S.cn + c_lo, col, row, dbg_row, k > c_lo ? k - c_lo : 0);
+        quarter_keys(ta + c_lo, min(cpq, cols - c_lo), nxv, S.cn + c_lo, col, row,
+                     SUMS ? sums + ((uint64_t)tile * TM + r) * NMAX + c_lo : nullptr);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.empty_acc[b]);
@@ -606,29 +611,20 @@ size_t km_tc_smem_bytes() { return sizeof(TcSmem) + 1024; }
 // Raw launch: nchg (null in a job's first round, whose words hold nothing yet)
 // counts the points that changed cluster; list/nlist receive the points to re-check, pairs/npairs the
 // few-candidate points; act/nact (or null) name the points to take; maxabs (when not null) receives the bits of max |x|.
-cudaError_t launch_km_tc_kernel(int terms, const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
+template <int TERMS, bool SUMS = false>
+cudaError_t launch_km_tc_kernel(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                 const float* center, const float* cnorm, const unsigned int* cmax_bits,
-                                uint32_t* assign, uint32_t* nchg, uint32_t* list, uint32_t* nlist, KmFew* pairs, uint32_t* npairs, unsigned long long* timeouts,
-                                float* dbg, int grid, cudaStream_t s, long long polls, uint32_t stop_copies,
-                                unsigned int* maxabs, const uint32_t* act, const uint32_t* nact,
-                                const KmBounds& B) {
+                                uint32_t* assign, uint32_t* nchg, uint32_t* list, uint32_t* nlist, KmFew* pairs,
+                                uint32_t* npairs, unsigned long long* timeouts, float* sums, int grid, cudaStream_t s,
+                                long long polls, uint32_t stop_copies, unsigned int* maxabs, const uint32_t* act,
+                                const uint32_t* nact, const KmBounds& B) {
   const int smem = (int)km_tc_smem_bytes();
-  cudaError_t e;
-  if (terms == 3) {
-    if ((e = cudaFuncSetAttribute(km_tc_assign_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
-        cudaSuccess)
-      return e;
-    return launch_pdl(km_tc_assign_kernel<3>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
-                      cnorm, cmax_bits, assign, nchg, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
-                      maxabs, act, nact, B);
-  } else {
-    if ((e = cudaFuncSetAttribute(km_tc_assign_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) !=
-        cudaSuccess)
-      return e;
-    return launch_pdl(km_tc_assign_kernel<1>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k, center,
-                      cnorm, cmax_bits, assign, nchg, list, nlist, pairs, npairs, timeouts, dbg, polls, stop_copies,
-                      maxabs, act, nact, B);
-  }
+  const cudaError_t e = cudaFuncSetAttribute(km_tc_assign_kernel<TERMS, SUMS>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(km_tc_assign_kernel<TERMS, SUMS>, dim3(grid), dim3(TC_THREADS), (size_t)smem, s, x, n, d, c, k,
+                    center, cnorm, cmax_bits, assign, nchg, list, nlist, pairs, npairs, timeouts, sums, polls,
+                    stop_copies, maxabs, act, nact, B);
 }
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
@@ -638,12 +634,12 @@ cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, cons
   const uint32_t ntiles = (n + TM - 1) / TM;
   uint32_t grid = ntiles < (uint32_t)di.sms ? ntiles : (uint32_t)di.sms;
   if (b.grid_cap && grid > b.grid_cap) grid = b.grid_cap;
-  const int terms = b.precision == MR_KM_BF16X1_TC ? 1 : 3;
+  auto launch = b.precision == MR_KM_BF16X1_TC ? launch_km_tc_kernel<1> : launch_km_tc_kernel<3>;
   cudaError_t e = kt_begin(b.kt, s);
   if (e != cudaSuccess) return e;
-  e = launch_km_tc_kernel(terms, x, n, d, c, k, b.center, b.cnorm, cmax, b.assign, nchg, b.flagged, b.nflag + 1,
-                          b.pairs, b.nflag + 4, b.stats + 3, nullptr, (int)grid, s, b.polls < 0 ? SPIN_LIMIT : b.polls,
-                          b.stop_copies, maxabs ? b.maxabs : nullptr, act, nact, b.bounds);
+  e = launch(x, n, d, c, k, b.center, b.cnorm, cmax, b.assign, nchg, b.flagged, b.nflag + 1, b.pairs, b.nflag + 4,
+             b.stats + 3, nullptr, (int)grid, s, b.polls < 0 ? SPIN_LIMIT : b.polls, b.stop_copies,
+             maxabs ? b.maxabs : nullptr, act, nact, b.bounds);
   if (e != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;
   ++*nk;
   // the caller re-checks the pairs and the listed near ties

@@ -90,12 +90,16 @@ __device__ __forceinline__ void list_insert(int (&t)[KM_CAND_MAX], uint32_t (&c)
   rest = min(rest, key);
 }
 
+// SUMS: the sums of every point and column go to sums [tiles TM][chunks NMAX], for
+// tests.
+template <bool SUMS = false>
 __global__ void __launch_bounds__(WD_THREADS, 1)
 km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint32_t k,
                       const uint8_t* __restrict__ bop, const float* __restrict__ center,
                       const float* __restrict__ cnorm, const unsigned int* cmax_bits, uint32_t* __restrict__ assign,
                       uint32_t* nchg, uint32_t* __restrict__ list, uint32_t* nlist, KmFew* __restrict__ few,
-                      uint32_t* nfew, unsigned long long* timeouts, long long polls, unsigned int* maxabs) {
+                      uint32_t* nfew, unsigned long long* timeouts, float* sums, long long polls,
+                      unsigned int* maxabs) {
   extern __shared__ uint8_t wd_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(wd_raw) + 1023) & ~uintptr_t(1023));
   WideCtl& S = *reinterpret_cast<WideCtl*>(base + OPERANDS);
@@ -414,7 +418,8 @@ km_wide_assign_kernel(const float* __restrict__ x, uint32_t n, uint32_t d, uint3
         const uint32_t c_lo = (uint32_t)quarter * cpq;
         int w1 = KEY_NONE, w2 = KEY_NONE, lb = KEY_NONE, col[GRID], row[GRID];
         if (c_lo < cols)
-          quarter_keys(ta + c_lo, min(cpq, cols - c_lo), nxv, cn + ch * NMAX + c_lo, col, row, nullptr, 0);
+          quarter_keys(ta + c_lo, min(cpq, cols - c_lo), nxv, cn + ch * NMAX + c_lo, col, row,
+                       SUMS ? sums + (((uint64_t)tile * TM + r) * nc + ch) * NMAX + c_lo : nullptr);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.empty_acc[b]);
@@ -456,11 +461,11 @@ cudaError_t launch_kmeans_wide_assign(const float* x, uint32_t n, uint32_t d, ui
   uint32_t grid = ntiles < (uint32_t)di.sms ? ntiles : (uint32_t)di.sms;
   if (b.grid_cap && grid > b.grid_cap) grid = b.grid_cap;
   const size_t smem = wide_smem(k);
-  cudaError_t e = allow_smem<km_wide_assign_kernel>(di);
+  cudaError_t e = allow_smem<km_wide_assign_kernel<>>(di);
   if (e != cudaSuccess || (e = kt_begin(b.kt, s)) != cudaSuccess) return e;
-  e = launch_pdl(km_wide_assign_kernel, dim3(grid), dim3(WD_THREADS), smem, s, x, n, d, k, (const uint8_t*)b.bop,
+  e = launch_pdl(km_wide_assign_kernel<>, dim3(grid), dim3(WD_THREADS), smem, s, x, n, d, k, (const uint8_t*)b.bop,
                  (const float*)b.center, (const float*)b.cnorm, cmax, b.assign, nchg, b.flagged, b.nflag + 1, b.pairs,
-                 b.nflag + 4, b.stats + 3, b.polls < 0 ? SPIN_LIMIT : b.polls,
+                 b.nflag + 4, b.stats + 3, (float*)nullptr, b.polls < 0 ? SPIN_LIMIT : b.polls,
                  maxabs ? b.maxabs : (unsigned int*)nullptr);
   if (e != cudaSuccess || (e = kt_end(b.kt, s)) != cudaSuccess) return e;
   ++*nk;
