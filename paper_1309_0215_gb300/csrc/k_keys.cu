@@ -131,10 +131,12 @@ hk_global_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n, uint3
   }
 }
 
-// Local arrays: nbins + 1 u32 counters per CTA in shared memory.
-template <typename C>
+// Local arrays: nbins + 1 u32 counters per CTA in shared memory, added straight
+// to the u64 result (few enough bins that a u32 array to widen would only add a
+// launch).
 __global__ void __launch_bounds__(HK_SMEM_THREADS)
-hk_smem_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n, uint32_t nbins, C* __restrict__ cnt) {
+hk_smem_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n, uint32_t nbins,
+               unsigned long long* __restrict__ cnt) {
   extern __shared__ uint32_t sh_bins[];
   for (uint32_t i = threadIdx.x; i <= nbins; i += blockDim.x) sh_bins[i] = 0;
   __syncthreads();
@@ -906,9 +908,8 @@ cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbi
 }
 
 cudaError_t launch_hist_keys(const uint32_t* keys, uint64_t n, uint32_t nbins, int container, void* counters,
-                             bool wide, unsigned long long* out, const DevInfo& di, cudaStream_t s, uint64_t* nk,
-                             KTimer* kt) {
-  const bool smem = container == MR_C_SMEM_ARRAY;
+                             unsigned long long* out, const DevInfo& di, cudaStream_t s, uint64_t* nk, KTimer* kt) {
+  const bool smem = container == MR_C_SMEM_ARRAY, wide = smem || !counters;
   const uint64_t nb = (uint64_t)nbins + 1;
   cudaError_t e = cudaMemsetAsync(wide ? (void*)out : counters, 0, nb * (wide ? 8 : 4), s);
   if (e != cudaSuccess) return e;
@@ -924,14 +925,8 @@ cudaError_t launch_hist_keys(const uint32_t* keys, uint64_t n, uint32_t nbins, i
       uint64_t g = (groups + HK_SMEM_THREADS * 16 - 1) / (HK_SMEM_THREADS * 16);
       g = g < 1 ? 1 : g;
       g = g > (uint64_t)di.sms * per_sm ? (uint64_t)di.sms * per_sm : g;
-      if (wide) {
-        if ((e = allow_smem<hk_smem_kernel<unsigned long long>>(di)) != cudaSuccess) return e;
-        hk_smem_kernel<unsigned long long><<<(int)g, HK_SMEM_THREADS, bytes, s>>>(base, off, n, nbins, out);
-      } else {
-        if ((e = allow_smem<hk_smem_kernel<uint32_t>>(di)) != cudaSuccess) return e;
-        hk_smem_kernel<uint32_t><<<(int)g, HK_SMEM_THREADS, bytes, s>>>(base, off, n, nbins,
-                                                                        static_cast<uint32_t*>(counters));
-      }
+      if ((e = allow_smem<hk_smem_kernel>(di)) != cudaSuccess) return e;
+      hk_smem_kernel<<<(int)g, HK_SMEM_THREADS, bytes, s>>>(base, off, n, nbins, out);
     } else if (container == MR_C_CLUSTER_ARRAY) {
       e = wide ? launch_hk_cluster(base, off, n, nbins, out, di, s)
                : launch_hk_cluster(base, off, n, nbins, static_cast<uint32_t*>(counters), di, s);

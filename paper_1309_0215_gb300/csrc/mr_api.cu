@@ -581,8 +581,8 @@ mr_status enqueue_plain_on(mr_ctx* c, Job* j, cudaStream_t st) {
         break;
       }
       MR_CUDA_TRY(launch_hist_keys(reinterpret_cast<const uint32_t*>(j->in), n / 4, j->desc.hist_bins,
-                                   (int)j->container, j->hk_counters, j->hk_counters == nullptr,
-                                   static_cast<unsigned long long*>(j->result), c->di, st, &c->launches, j->kt));
+                                   (int)j->container, j->hk_counters, static_cast<unsigned long long*>(j->result),
+                                   c->di, st, &c->launches, j->kt));
       break;
     case MR_BLOOM_DNA:
       if (j->extra) {

@@ -95,10 +95,11 @@ int hk_cluster_max_bins(const DevInfo& di);
 // Histogram of n u32 keys into out[nbins + 1] (zeroed here).  container:
 // MR_C_SMEM_ARRAY local arrays per CTA, MR_C_CLUSTER_ARRAY local arrays
 // spread over a cluster's shared memory, else atomics on the global array.
-// wide: count straight into the u64 output (needed from 2^32 keys on); else
-// into the u32 counters (nbins + 1 words) and widen at the end.
+// Local arrays of one CTA go straight into the u64 output; the other containers
+// count in the u32 counters (nbins + 1 words) and widen at the end, or straight
+// into the output without counters (null, as from 2^32 keys on).
 cudaError_t launch_hist_keys(const uint32_t* keys, uint64_t n, uint32_t nbins, int container, void* counters,
-                             bool wide, unsigned long long* out, const DevInfo& di, cudaStream_t s, uint64_t* nk,
+                             unsigned long long* out, const DevInfo& di, cudaStream_t s, uint64_t* nk,
                              KTimer* kt = nullptr);
 // The same for many keys over bins beyond one CTA's shared memory
 // (hk_partitioned), through hk_part_bytes of scratch; every bin is written.
