@@ -523,3 +523,108 @@ def test_kmeans_runs_in_as_much_memory_as_ever(mr, n, d, k, precision, limit):
         assert np.array_equal(a, a_ref)
         assert _rel_err(init, c_ref) <= TOL
     assert np.array_equal(a2, a) and np.array_equal(c2, init)
+
+
+@pytest.mark.parametrize("n,d,k,comps,sigma,line", [
+    (30_001, 64, 64, 8, 16.0, 4),     # window-sorted update, 8-byte loads
+    (30_001, 21, 30, 4, 8.0, 4),      # one dimension per lane
+    (30_001, 33, 64, 8, 16.0, 4),     # two dimensions per lane, 4-byte loads
+    (12_001, 96, 16, 8, 4.0, 32),     # row-pipelined update
+    (12_003, 67, 16, 8, 4.0, 32),     # plain local-array update
+    (12_001, 130, 260, 8, 4.0, 8),    # sorted update
+])
+def test_kmeans_full_updates_and_updates_by_changes(mr, n, d, k, comps, sigma, line):
+    """Rounds after the first on both sides of each update's line (n / line moved
+    points): eight rounds in one call equal eight calls of one round, byte for
+    byte."""
+    x, _, _ = synth.kmeans_points(n, d, comps, seed=n + d, sigma=sigma)
+    dx, cur = _dev(x), synth.kmeans_init(x, k, seed=n)
+    c8, a8, _ = mr.kmeans(dx, _dev(cur), 8)
+    moved, last = [], None
+    for _ in range(8):
+        cur, a, _ = mr.kmeans(dx, _dev(cur), 1)
+        if last is not None:
+            moved.append(int((a != last).sum()))
+        last = a
+    assert np.array_equal(a8, last) and np.array_equal(c8, cur)
+    assert any(m > n // line for m in moved) and any(0 < m <= n // line for m in moved), moved
+
+
+@pytest.mark.parametrize("n,d", [(500_009, 64), (450_001, 37)])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_kmeans_skipped_points_not_16_byte_aligned(mr, n, d, precision):
+    """The filter's list over points 4 bytes into a buffer, whose rows the
+    converters load value by value: nine rounds in one call equal nine calls of
+    one round, and the aligned points' result, byte for byte."""
+    import torch
+    x, _, _ = synth.kmeans_points(n, d, 100, seed=n + d)
+    cur = synth.kmeans_init(x, 100, seed=n)
+    buf = torch.zeros(x.size + 1, dtype=torch.float32, device="cuda")
+    buf[1:] = torch.from_numpy(x.ravel()).cuda()
+    off = buf[1:].view(n, d)
+    torch.cuda.synchronize()
+    c9, a9, _ = mr.kmeans(off, _dev(cur), 9, precision)
+    ca, aa, _ = mr.kmeans(_dev(x), _dev(cur), 9, precision)
+    for _ in range(9):
+        cur, a, _ = mr.kmeans(off, _dev(cur), 1, precision)
+    assert np.array_equal(a9, a) and np.array_equal(c9, cur)
+    assert np.array_equal(aa, a) and np.array_equal(ca, cur)
+
+
+@pytest.mark.parametrize("n,d,k,iters", [
+    (400_003, 64, 256, 6),   # tensor-core pass, with the filter
+    (100_003, 37, 100, 6),
+    (60_001, 5, 17, 6),
+    (30_001, 128, 512, 4),   # wide tensor-core pass
+    (20_001, 256, 40, 4),
+    (20_003, 9, 1_500, 4),
+])
+def test_kmeans_tensor_core_and_fp32_passes_agree(mr, n, d, k, iters):
+    """The FP32 SIMT pass (which a context with a wait limit of its own keeps)
+    against the tensor-core passes: the same bytes, since every assignment is the
+    FP64 definition's and the sums are exact."""
+    x, _, _ = synth.kmeans_points(n, d, 60, seed=n + d)
+    init, dx = synth.kmeans_init(x, k, seed=n), _dev(x)
+    with mr.Context() as ctx:
+        ctx.set_option(mr.OPT_WAIT_POLLS, 1 << 20)
+        before = ctx.kernel_launches
+        c32, a32, _ = _run_ctx(mr, ctx, dx, init, iters, 0)
+        simt = ctx.kernel_launches - before
+    with mr.Context() as ctx:
+        before = ctx.kernel_launches
+        c, a, _ = _run_ctx(mr, ctx, dx, init, iters, 0)
+        # (max |x| takes a kernel of its own only beside the SIMT pass)
+        assert ctx.kernel_launches - before != simt
+    assert np.array_equal(a, a32) and np.array_equal(c, c32)
+    if d <= 64 and k <= 256:
+        for precision in (1, 2):
+            c, a, _ = mr.kmeans(dx, _dev(init), iters, precision)
+            assert np.array_equal(a, a32) and np.array_equal(c, c32)
+
+
+@pytest.mark.parametrize("n,d,k,limit", [
+    (3_001, 257, 20, False),     # one dimension past the wide pass
+    (2_003, 300, 300, False),    # SIMT pass with float selection, several threads' centroids in the settling
+    (1_201, 1_024, 64, False),   # the most dimensions
+    (1_024, 1_000, 257, False),
+    (700, 513, 4_096, False),    # the most centroids
+    (4_001, 16, 300, True),      # shapes of the wide pass, kept on the SIMT pass by a wait limit
+    (4_001, 8, 3_000, True),
+])
+@pytest.mark.parametrize("offset", [0.0, 3e4])
+def test_kmeans_fp32_simt_pass_and_settling(mr, n, d, k, limit, offset):
+    """Shapes beyond the tensor-core passes: two rounds, each from the oracle's
+    centroids.  The offset makes near ties of points that FP32 cannot tell."""
+    x, _, _ = synth.kmeans_points(n, d, 16, seed=n + d)
+    x = x + np.float32(offset)
+    cur, dx = x[np.random.default_rng(k).integers(0, n, k)] + np.float32(0.125), _dev(x)
+    with mr.Context() as ctx:
+        if limit:
+            ctx.set_option(mr.OPT_WAIT_POLLS, 1 << 20)
+        for _ in range(2):
+            a_ref = oracle.kmeans_assign(x, cur)
+            c_ref, _ = oracle.kmeans_update(x, a_ref, cur)
+            c, a, st = _run_ctx(mr, ctx, dx, cur, 1, 0)
+            assert np.array_equal(a, a_ref)
+            assert _rel_err(c, c_ref) <= TOL
+            cur = c_ref
