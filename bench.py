@@ -994,7 +994,8 @@ def wordcount_eval(steps: int, warmup: int) -> dict:
 
 def kmeans_eval(steps: int, warmup: int) -> dict:
     """k-means 4M x 64 FP32 points, K = 256, 10 iterations, on the BF16
-    tensor-core paths (three products, one product) and the FP32 path."""
+    tensor-core paths (three products, one product) and as FP32 jobs, which take
+    the first of them."""
     import numpy as np
     import torch
     import oracle
@@ -1049,10 +1050,17 @@ def kmeans_eval(steps: int, warmup: int) -> dict:
         r.update({"tensor_products_per_distance": terms, "tensor_tflops": round(tt, 1),
                   "tensor_frac_of_bf16_peak": round(tt / bf16_peak, 4)})
         out[name] = r
-    # the three paths give identical results (each iteration's assignment is
-    # the FP64 argmin, and the update's integer sums make it order-free)
-    out["bf16_paths_equal_fp32"] = bool(all(np.array_equal(results[p][0], results[0][0]) and
-                                            np.array_equal(results[p][1], results[0][1]) for p in (1, 2)))
+    # every path gives the results of the FP32 SIMT distance pass, which a context
+    # with a wait limit of its own keeps (each iteration's assignment is the FP64
+    # argmin, and the update's integer sums make it order-free)
+    ctx.set_option(mr.OPT_WAIT_POLLS, 1 << 20)
+    j = job(0, KM_ITERS, di)
+    ctx.run()
+    c32, a32, _ = mr.split_kmeans_result(ctx.fetch(j), n, dd, kk)
+    ctx.release(j)
+    ctx.set_option(mr.OPT_WAIT_POLLS, mr.OPT_DEFAULT)
+    out["paths_equal_fp32_simt"] = bool(all(np.array_equal(results[p][0], c32) and
+                                            np.array_equal(results[p][1], a32) for p in results))
     # sampled check of the last iteration against the oracle, on the GPU's ninth centroids
     j = job(1, KM_ITERS - 1, di)
     ctx.run()
