@@ -585,6 +585,7 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
     if (np + nf) atomicAdd(stat, (unsigned long long)np + nf);
   }
   const float widen = rel_bound_widen(d);
+  const bool bounds = km_keeps_bounds(B);
   const bool vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
   const uint64_t rb = ((uint64_t)nf + SET_RP - 1) / SET_RP;
   unsigned long long settled = 0;  // points settled in FP64
@@ -601,7 +602,7 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
       next = load_few(pairs, np, f0 + 4 * ws + (lane >> 3));
       // (loaded with the rows, not after them)
       const uint32_t word = nchg ? assign[e.p] : 0u;
-      const float l = B.ub ? B.lb[e.p] : 0.f;
+      const float l = bounds ? B.lb[e.p] : 0.f;
       const uint32_t nc = e.hi >> 28;
       float fd[KM_CAND_MAX];
       if (__any_sync(0xffffffffu, nc > 2)) few_dists<KM_CAND_MAX>(x, c, d, e, nc, sl, vec, fd);
@@ -640,13 +641,13 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
         }
         if (!clear && sl == 0) {
           settle_put(assign, e.p, bk == 0xffffffffu ? 0u : bk, nchg, word, S);
-          if (B.ub) B.ub[e.p] = INFINITY;  // no bounds: the next round computes it again
+          if (bounds) B.ub[e.p] = INFINITY;  // no bounds: the next round computes it again
           ++settled;
         }
       }
       if (clear && nc && sl == 0) {
         settle_put(assign, e.p, k1, nchg, word, S);
-        if (B.ub) {  // the distance pass left the bound of the other centroids
+        if (bounds) {  // the distance pass left the bound of the other centroids
           km_put_bounds(B, e.p, B.drift[k1], *B.far, m1 * widen + 1e-36f,
                         fminf(m2 * (2.f - widen) - 1e-36f, l * l * 0.999999f));
         }
@@ -725,7 +726,9 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
         const uint32_t p = list[f0 + r];
         if (__uint_as_float(m2) > __uint_as_float(m1) * widen) {
           settle_put(assign, p, k1, nchg, nchg ? assign[p] : 0u, S);
-          if (B.ub) km_put_bounds(B, p, B.drift[k1], *B.far, __uint_as_float(m1) * widen + 1e-36f, __uint_as_float(m2) * (2.f - widen) - 1e-36f);
+          if (bounds)
+            km_put_bounds(B, p, B.drift[k1], *B.far, __uint_as_float(m1) * widen + 1e-36f,
+                          __uint_as_float(m2) * (2.f - widen) - 1e-36f);
         } else {
           S.open[atomicAdd(&S.nopen, 1u)] = p;
         }
@@ -733,7 +736,7 @@ __global__ void __launch_bounds__(SET_T_MAX) km_settle_kernel(
     }
     __syncthreads();
     const uint32_t no = S.nopen;
-    if (B.ub && threadIdx.x < no) B.ub[S.open[threadIdx.x]] = INFINITY;  // no bounds: the next round computes it again
+    if (bounds && threadIdx.x < no) B.ub[S.open[threadIdx.x]] = INFINITY;  // no bounds: the next round computes it again
     for (uint32_t i = 0; i < no; ++i) settle_fp64(x, d, c, ct, k, S.open[i], assign, nchg, prod, xs, dist, cand, S);
     if (threadIdx.x == 0) settled += no;
   }
@@ -1511,6 +1514,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) km_window_sum_kernel(const floa
 // none), each centroid's drift so far and the largest of the round (drift null:
 // not kept) and cleared counters.  first: only the
 // latter, for the initial centroids.
+constexpr uint32_t KM_STATE = 8;  // of the counters: points listed, mode, rounds, length of a rest
+__device__ __forceinline__ void km_next_mode(uint32_t* st, uint32_t n);
 constexpr int RF_THREADS = 256;
 __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long* __restrict__ part, uint32_t g,
                                                                  long long* sums, float* c, uint32_t k, uint32_t d,
@@ -1521,7 +1526,7 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
                                                                  const float* __restrict__ center,
                                                                  float* __restrict__ cn, unsigned int* cmax,
                                                                  float* __restrict__ ct, uint8_t* bop,
-                                                                 float* drift, unsigned int* maxdrift,
+                                                                 float* drift, unsigned int* maxdrift, uint32_t n,
                                                                  uint32_t* nflag, uint32_t first) {
   pdl_wait();
   __shared__ long long red[RF_THREADS / 32][32];
@@ -1582,6 +1587,7 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
       if (kk == 0) {
         nflag[1] = nflag[4] = 0;  // points to re-check, pairs
         *chg_next = 0;
+        if (drift && !first) km_next_mode(nflag + KM_STATE, n);
       }
     }
   }
@@ -1601,21 +1607,51 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
 // skipped point's assignment is the FP64 definition's, by a relative margin of
 // 1e-5.  The listed points go through the distance pass by index.
 //
+// Data without clusters leaves it nothing to skip for many rounds (of normal
+// points in 64 dimensions, K = 256, over 99% are listed in rounds 2 to 7, 93% in
+// round 11; the mixture's 99% are gone after round 3), and a round whose list is
+// not used has paid for it.  So the centroids' kernel decides the next round's mode
+// (km_next_mode): after two rounds that listed all but 1 / 128 of the points
+// the filter rests for three rounds, and no bounds are written; one round then
+// writes them again and the next one filters.  After a rest, one round whose
+// list is not used (km_use_list) starts another, twice as long.
+//
+// st: points listed, mode, rounds (that listed nearly all; of the rest, left), length of the last rest.
+__device__ __forceinline__ void km_next_mode(uint32_t* st, uint32_t n) {
+  const uint32_t listed = st[0];
+  uint32_t mode = st[1], rounds = st[2], rest = st[3];
+  if (mode == KM_REST) {
+    if (--rounds == 0) mode = KM_BOUNDS;
+  } else if (mode == KM_BOUNDS) {
+    mode = KM_FILTER;
+  } else {
+    rounds = listed > n - n / 128 ? rounds + 1 : 0;
+    if (rest ? !tc::km_use_list(listed, n) : rounds == 2) {
+      mode = KM_REST;
+      rounds = rest = rest ? min(2 * rest, 1u << 20) : 3;
+    }
+  }
+  st[1] = mode, st[2] = rounds, st[3] = rest;
+}
+
 // km_half_kernel: half[k], one CTA per centroid, one thread per other centroid;
 // and the largest drift of the round added to the sum of them.
 constexpr int HALF_THREADS = 256;
 __global__ void __launch_bounds__(HALF_THREADS) km_half_kernel(const float* __restrict__ c,
                                                                const float* __restrict__ ct, uint32_t k, uint32_t d,
                                                                float* __restrict__ half, unsigned int* maxdrift,
-                                                               float* far, uint32_t* nact) {
+                                                               float* far, uint32_t n, uint32_t* nact,
+                                                               const uint32_t* mode) {
   pdl_wait();
   __shared__ float own[64], red[HALF_THREADS / 32];
   const uint32_t i = blockIdx.x;
+  const bool on = *mode == KM_FILTER;
   if (i == 0 && threadIdx.x == 0) {
     *far = __fadd_ru(*far, __uint_as_float(*maxdrift));
     *maxdrift = 0;
-    *nact = 0;
+    *nact = on ? 0 : n;
   }
+  if (!on) return;
   for (uint32_t t = threadIdx.x; t < d; t += HALF_THREADS) own[t] = c[(uint64_t)i * d + t];
   __syncthreads();
   float best = INFINITY;
@@ -1642,6 +1678,7 @@ __global__ void __launch_bounds__(FI_THREADS) km_filter_kernel(const uint32_t* _
                                                                uint32_t k, KmBounds B, const float* __restrict__ half,
                                                                uint32_t* __restrict__ act, uint32_t* nact) {
   pdl_wait();
+  if (*B.mode != KM_FILTER) return;
   __shared__ float s_drift[256], s_half[256];
   __shared__ uint32_t wcnt[FI_THREADS / 32], s_base;
   for (uint32_t i = threadIdx.x; i < k; i += FI_THREADS) s_drift[i] = B.drift[i], s_half[i] = half[i];
@@ -1792,15 +1829,32 @@ void km_carve_bounds(KmBuffers& b, uint8_t* p) {
   b.bounds.drift = reinterpret_cast<float*>(take(b.k));
   b.half = reinterpret_cast<float*>(take(b.k));
   b.bounds.far = reinterpret_cast<float*>(b.shift) + 2;
+  b.bounds.mode = b.nflag + KM_STATE + 1;
 }
 
 // The filter pays for its two kernels (10 - 24 us a round) and the bounds the
-// first rounds write for nothing where the distance pass is long enough (its
-// time goes by the points, about 130 us per million whatever D and K) and
-// enough rounds follow.  Ten rounds with / without, us: 200,000 x 37, K = 100
-// 484 / 522, 200,000 x 8 559 / 547, 400,000 x 37 689 / 808, 400,000 x 50 907 /
-// 920, 1.6M x 8 2,169 / 2,528; three rounds at 400,000 x 37 350 / 318.
-bool km_bounds_pay(uint32_t n, uint32_t iters) { return n >= 3u << 17 && iters >= 5; }
+// first rounds write for nothing where the distance pass is long enough and
+// enough rounds follow: ten, or five if it has 10^8 distances.  Calls with /
+// without it, us, of a mixture of 256 Gaussians, and of normal points, which
+// leave it little to skip for many rounds (it rests, see km_next_mode; each round
+// at rest still costs two launches, and without resting the last column's
+// first figures were 2 to 4% higher):
+//                                 mixture            normal
+//   400K x 8,  K = 40   10 rounds   648 / 656        671 / 674
+//   400K x 37, K = 100   5          462 / 435        508 / 471     (left out)
+//                        9          686 / 691        840 / 780     (left out)
+//                       10          725 / 757        916 / 859
+//                       20        1,036 / 1,378    1,668 / 1,613
+//   400K x 64, K = 256   5          487 / 525        615 / 574
+//                       10          747 / 947      1,130 / 1,060
+//   1M x 16,   K = 100   5          734 / 759        839 / 799
+//                       10        1,058 / 1,378    1,432 / 1,474
+//   1M x 64,   K = 256  10        1,161 / 1,764    2,062 / 1,967
+//   4M x 64,   K = 256  10        2,913 / 5,784    6,614 / 6,483
+//                       20        4,099 / 11,091  12,285 / 12,404
+bool km_bounds_pay(uint32_t n, uint32_t k, uint32_t iters) {
+  return n >= 3u << 17 && (iters >= 10 || (iters >= 5 && (uint64_t)n * k >= 100'000'000));
+}
 
 cudaError_t launch_kmeans_tc_assign(const float* x, uint32_t n, uint32_t d, const float* c, uint32_t k,
                                     KmBuffers& b, const unsigned int* cmax, uint32_t* nchg, const DevInfo& di,
@@ -1894,7 +1948,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   float* drift = filter ? const_cast<float*>(b.bounds.drift) : nullptr;
   unsigned int* maxdrift = reinterpret_cast<unsigned int*>(shift) + 1;
   float* far = reinterpret_cast<float*>(shift) + 2;
-  uint32_t* nact = b.nflag + 8;
+  uint32_t* nact = b.nflag + KM_STATE;
   const KmBounds bounds = filter ? b.bounds : KmBounds{};
   const float* center = tc || wide ? b.center : nullptr;
   const uint32_t lim = n / (wsum ? KM_DELTA_WINDOW : local ? KM_DELTA_LOCAL : KM_DELTA_SORTED);  // points moved, at most, in an update by changes
@@ -1906,7 +1960,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
                       b.counts, b.counts + k, it > 1 ? (const uint32_t*)chg_of(it - 1) : (const uint32_t*)nullptr, lim,
                       chg_of(it),
                       (const int*)shift, center, b.cnorm, cmax_of(it), ct, wide ? b.bop : (uint8_t*)nullptr, drift,
-                      maxdrift, b.nflag, first ? 1u : 0u);
+                      maxdrift, n, b.nflag, first ? 1u : 0u);
   };
   if ((e = finalize(0, true)) != cudaSuccess) return e;
   unsigned long long* cnew = b.counts + k;
@@ -1919,7 +1973,7 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
       if (skip) {
         const uint64_t fb = ((uint64_t)n + FI_THREADS * 4 - 1) / (FI_THREADS * 4);
         if ((e = launch_pdl(km_half_kernel, dim3(k), dim3(HALF_THREADS), 0, s, (const float*)b.cent,
-                            (const float*)ct, k, d, b.half, maxdrift, far, nact)) != cudaSuccess ||
+                            (const float*)ct, k, d, b.half, maxdrift, far, n, nact, bounds.mode)) != cudaSuccess ||
             (e = launch_pdl(km_filter_kernel, dim3((unsigned)(fb < 2ull * di.sms ? fb : 2ull * di.sms)),
                             dim3(FI_THREADS), 0, s, (const uint32_t*)b.assign, n, k, bounds, (const float*)b.half,
                             b.act, nact)) != cudaSuccess)

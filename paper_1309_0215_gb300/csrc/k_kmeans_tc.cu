@@ -416,7 +416,8 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
                                      : (2.f * 3.90625e-03f + 1.52587890625e-05f + (float)(KD + 8) * 2.384185791015625e-07f);
     const float eps32 = 1.01f * (float)(d + 12) * 5.9604644775390625e-08f;
     uint32_t moved = 0;  // this lane's points that changed cluster
-    const float far = B.ub ? *B.far : 0.f;
+    const bool bounds = km_keeps_bounds(B);
+    const float far = bounds ? *B.far : 0.f;
     // the points of the next two tiles and the words of the next one, so that no
     // load waits for another
     uint32_t p[FIN_QUADS], word[FIN_QUADS], p1[FIN_QUADS], word1[FIN_QUADS], p2[FIN_QUADS];
@@ -483,7 +484,7 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
             const uint32_t now = (uint32_t)g1 & 0xFFu, o = nchg ? word[h] & 0xffffu : now;
             assign[p[h]] = km_word(now, o);
             moved += now != o;
-            if (B.ub) km_put_bounds(B, p[h], S.drift[now], far, fmaf(d1, 1.00006103515625f, e), d2 - e);
+            if (bounds) km_put_bounds(B, p[h], S.drift[now], far, fmaf(d1, 1.00006103515625f, e), d2 - e);
           } else {
             const uint32_t cpq = quarter_cols(npad);
             // candidates: the quarters' top-2 keys within the margin and what
@@ -514,7 +515,7 @@ km_tc_assign_kernel(const float* __restrict__ x, uint32_t n_all, uint32_t d, con
             const bool few = key_dist(rest) - d1 > gap && nc >= 2 && nc <= KM_CAND_MAX;
             ncand[h] = few ? nc : LISTED;
             // (the settle pass lowers it by the candidates' distances)
-            if (B.ub && few) B.lb[p[h]] = km_sqrt(fmaxf(key_dist(rest) - e, 0.f)) * 0.999999f;
+            if (bounds && few) B.lb[p[h]] = km_sqrt(fmaxf(key_dist(rest) - e, 0.f)) * 0.999999f;
           }
         }
       }

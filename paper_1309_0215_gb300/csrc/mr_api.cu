@@ -495,7 +495,7 @@ mr_status alloc_job_memory(mr_ctx* c, Job* j) {
         set_last_error("km_carve", e);
         return MR_EINVAL;
       }
-      if (!c->budget && km_tc_supported(D, K) && km_bounds_pay(N, d.km_iters) &&
+      if (!c->budget && km_tc_supported(D, K) && km_bounds_pay(N, K, d.km_iters) &&
           alloc_extra(c, j, km_bounds_bytes(N, K)))
         km_carve_bounds(j->km, static_cast<uint8_t*>(j->extra));
       if (!d.input_on_device) {

@@ -180,7 +180,11 @@ struct KmBounds {
   float* lb = nullptr;           // [n] lower bound on the distance to any other, plus the largest drifts so far
   const float* drift = nullptr;  // [k] each centroid's drift so far
   const float* far = nullptr;    // [1] the sum of the rounds' largest drifts
+  const uint32_t* mode = nullptr;  // [1] KM_FILTER, KM_BOUNDS or KM_REST: what the round does
 };
+// The filter at work; the pass over all points with the bounds written, for the
+// filter of the next round; neither (see km_filter_kernel).
+constexpr uint32_t KM_FILTER = 0, KM_BOUNDS = 1, KM_REST = 2;
 
 // A point with 2 to KM_CAND_MAX candidate centroids, 12 bits each (K <= 4096),
 // and their number in the top bits.
@@ -212,6 +216,7 @@ __device__ __forceinline__ void km_put_bounds(const KmBounds& B, uint32_t p, flo
   B.ub[p] = fmaf(km_sqrt(u2), 1.000001f, -drift);
   B.lb[p] = fmaf(km_sqrt(fmaxf(l2, 0.f)), 0.999999f, far);
 }
+__device__ __forceinline__ bool km_keeps_bounds(const KmBounds& B) { return B.ub && *B.mode != KM_REST; }
 __device__ __forceinline__ uint32_t km_summed(uint32_t w, uint32_t k) { return (w >> 16) < k ? w >> 16 : 0u; }
 #endif
 
@@ -250,7 +255,7 @@ struct KmBuffers {
 size_t km_scratch_bytes(uint32_t n, uint32_t d, uint32_t k, bool wide);
 cudaError_t km_carve(KmBuffers& b, uint8_t* base, size_t bytes, bool wide);
 // the filter's bounds, in memory of their own (after km_carve)
-bool km_bounds_pay(uint32_t n, uint32_t iters);
+bool km_bounds_pay(uint32_t n, uint32_t k, uint32_t iters);
 size_t km_bounds_bytes(uint32_t n, uint32_t k);
 void km_carve_bounds(KmBuffers& b, uint8_t* base);
 cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmBuffers& b, const DevInfo& di,

@@ -452,7 +452,7 @@ def test_kmeans_close_centroids_in_the_grid(mr, n, d, k, spread):
     (20_000, 64, 64, 2),    # tensor-core pass, whole tiles in bulk copies
     (6_001, 37, 50, 2),     # values loaded by the converters
     (6_001, 100, 300, 2),   # wide tensor-core pass
-    (400_009, 16, 20, 5),   # with the filter's bounds
+    (400_009, 16, 250, 5),  # with the filter's bounds
     (3_000, 300, 20, 2),    # FP32 SIMT pass
 ])
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, 3e30])
@@ -558,7 +558,7 @@ def test_kmeans_skipped_points_not_16_byte_aligned(mr, n, d, precision):
     one round, and the aligned points' result, byte for byte."""
     import torch
     x, _, _ = synth.kmeans_points(n, d, 100, seed=n + d)
-    cur = synth.kmeans_init(x, 100, seed=n)
+    cur = synth.kmeans_init(x, 230, seed=n)
     buf = torch.zeros(x.size + 1, dtype=torch.float32, device="cuda")
     buf[1:] = torch.from_numpy(x.ravel()).cuda()
     off = buf[1:].view(n, d)
@@ -628,3 +628,21 @@ def test_kmeans_fp32_simt_pass_and_settling(mr, n, d, k, limit, offset):
             assert np.array_equal(a, a_ref)
             assert _rel_err(c, c_ref) <= TOL
             cur = c_ref
+
+
+@pytest.mark.parametrize("n,d,k,rounds", [
+    (400_003, 64, 200, 18),   # nearly every point listed for many rounds: the filter rests twice
+    (400_009, 31, 60, 18),
+    (393_216, 6, 250, 14),
+])
+@pytest.mark.parametrize("precision", [0, 2])
+def test_kmeans_filter_at_rest(mr, n, d, k, rounds, precision):
+    """Points without clusters: rounds with the filter, without it and its bounds,
+    with the bounds alone, and with it again, in one call equal calls of one
+    round, byte for byte."""
+    x = np.random.default_rng(n + d).standard_normal((n, d), dtype=np.float32)
+    dx, cur = _dev(x), synth.kmeans_init(x, k, seed=n)
+    call, a_call, _ = mr.kmeans(dx, _dev(cur), rounds, precision)
+    for _ in range(rounds):
+        cur, a, _ = mr.kmeans(dx, _dev(cur), 1, precision)
+    assert np.array_equal(a_call, a) and np.array_equal(call, cur)
