@@ -125,8 +125,11 @@ typedef enum {
 
 typedef enum {
   MR_KM_FP32 = 0,         /* the library picks the distance pass: split operands on the
-                             tensor cores where they cover the shape, else FP32 SIMT;
-                             exact re-check of near ties */
+                             tensor cores where they cover the shape (D <= 256, K <=
+                             4096), whose bounded waits can end a job with
+                             MR_ETIMEOUT as the other precisions' do; else FP32 SIMT,
+                             which a context with MR_OPT_WAIT_POLLS set takes for
+                             every shape; exact re-check of near ties */
   MR_KM_BF16_TC = 1,      /* BF16 tensor-core distance GEMM (tcgen05, FP32
                              accumulate) on split operands x = hi + lo (three
                              BF16 products), FP32 then FP64 re-check of near
@@ -297,7 +300,8 @@ typedef enum {
    * polls of at most 1 us each) and the ring waits of the pipelined word
    * count (default 2^22 polls of ~128 ns).  value = UINT64_MAX restores the
    * default; 0 gives up at the first wait, so the job's mr_fetch returns
-   * MR_ETIMEOUT.  At most 2^40. */
+   * MR_ETIMEOUT.  At most 2^40.  While it is not the default, MR_KM_FP32 jobs
+   * compute their distances in FP32 on the SIMT units (no waits). */
   MR_OPT_WAIT_POLLS = 0,
   /* Upper bound on the CTAs of the k-means persistent kernels (0 = none: one
    * CTA, or two, per SM), so that a small input runs many tiles per CTA and

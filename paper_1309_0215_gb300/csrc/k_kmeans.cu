@@ -9,22 +9,30 @@
 // Exactness contract: assignments equal the FP64 argmin of
 //   d(x, c) = sum_j ((double)x_j - (double)c_j)^2   (j in order, no FMA),
 // and centroids are the exact-sum means rounded to FP32.
-//  * FP32 pass: d~ = ||x||^2 - 2 x.c + ||c||^2 with FP32 FMAs.  Its error is
-//    at most E = gamma_{D+3} (||x|| + ||c||)^2 (Higham, Accuracy and Stability
-//    of Numerical Algorithms, eq. 3.4 / 3.5 for dot products); we use
-//    E = 1.01 (D + 8) 2^-24 (||x|| + max_k ||c_k||)^2.  If the two smallest
+//
+// A round is: the filter, in jobs where it pays (km_half_kernel,
+// km_filter_kernel: points that provably keep their cluster are left out); the
+// distance pass; the choice of what that left open (km_settle_kernel); the
+// update of the sums; the next centroids (km_finalize_kernel).
+//  * Distance pass: on the tensor cores for BF16 jobs and for FP32 jobs of up to
+//    256 dimensions and 4,096 centroids (k_kmeans_tc.cu, k_kmeans_wide.cu, with
+//    their bounds), else, and in contexts with a wait limit of their own, in
+//    FP32 FMAs here (km_assign_fp32_kernel): d~ = ||x||^2 - 2 x.c + ||c||^2,
+//    whose error is at most E = gamma_{D+3} (||x|| + ||c||)^2 (Higham, Accuracy
+//    and Stability of Numerical Algorithms, eq. 3.4 / 3.5 for dot products); we
+//    use E = 1.01 (D + 8) 2^-24 (||x|| + max_k ||c_k||)^2.  If the two smallest
 //    d~ differ by more than 2E the FP32 winner is the FP64 winner.
-//  * Every other point is re-checked exactly in FP64 with the same operation
-//    order as the definition above, over the centroids that can still win:
-//    FP32 direct-difference distances have relative error at most
-//    g = gamma_{D+3} (Higham, eq. 3.5 on a sum of squares), so centroid k can
-//    be the minimum only if d~_k <= d~_min (1 + g) / (1 - g).
-//  * Sums are accumulated as int64 fixed point q = rint(x * 2^s), with s chosen
-//    from max|x| and N so no sum can overflow; integer addition is exact and
-//    order-independent, so results do not depend on scheduling.  The update
-//    first groups points by cluster (counting sort), so each warp adds runs
-//    of points of one cluster in registers and issues a handful of atomics
-//    per run instead of one per coordinate.
+//  * Every other point is settled by FP32 direct differences, whose relative
+//    error is at most g = gamma_{D+3} (Higham, eq. 3.5 on a sum of squares), and
+//    where those lie within (1 + g) / (1 - g) of each other by the definition in
+//    FP64, with its order of operations.
+//  * Sums are int64 fixed point, q = rint(x * 2^s), with s chosen from max|x| and
+//    N so no sum can overflow; integer addition is exact and order-independent,
+//    so results do not depend on scheduling.  A round in which few points moved
+//    changes the sums by those alone; a full update adds runs of points of one
+//    cluster in registers, after sorting windows of points by cluster in shared
+//    memory (D <= 64) or all of them in global memory (K x D sums beyond one
+//    CTA), or adds every coordinate in shared memory (the other shapes).
 #include <cmath>
 
 #include "dev_tc.cuh"
@@ -1142,7 +1150,7 @@ __global__ void __launch_bounds__(LS_THREADS, 1) km_local_sum_kernel(const float
 // own rows, the ring ran dry and the kernel waited on DRAM latency.)
 //
 // Exact sums without 64-bit shared atomics.  The scale keeps |x 2^s| < 2^39
-// (km_scale_kernel), so q = rint(x 2^s) = hi 2^20 + lo with hi, lo integers
+// (fx_shift_of), so q = rint(x 2^s) = hi 2^20 + lo with hi, lo integers
 // of magnitude <= 2^19, both formed by FP32 adds that are exact (lq_split);
 // each goes into a 32-bit shared-memory array with a non-returning add.
 // Within a window of at most LP_FLUSH_ROWS points no 32-bit sum can overflow,
@@ -1608,9 +1616,9 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
 // 1e-5.  The listed points go through the distance pass by index.
 //
 // Data without clusters leaves it nothing to skip for many rounds (of normal
-// points in 64 dimensions, K = 256, over 99% are listed in rounds 2 to 7, 93% in
-// round 11; the mixture's 99% are gone after round 3), and a round whose list is
-// not used has paid for it.  So the centroids' kernel decides the next round's mode
+// points in 64 dimensions, K = 256, over 99% are listed for six rounds and 93% in
+// the tenth; of the mixture's never more than 82%), and a round whose list is not
+// used has paid for it.  So the centroids' kernel decides the next round's mode
 // (km_next_mode): after two rounds that listed all but 1 / 128 of the points
 // the filter rests for three rounds, and no bounds are written; one round then
 // writes them again and the next one filters.  After a rest, one round whose
@@ -1872,13 +1880,13 @@ cudaError_t launch_kmeans(const float* x, const float* init, uint32_t iters, KmB
   int* shift = b.shift;
   float* ct = out_c;  // [d][k] transposed centroids, until km_finish_kernel writes the result there
   auto cmax_of = [&](uint32_t it) { return b.nflag + 6 + (it & 1); };  // max ||c||, one word per parity of the round
-    // The distance pass only has to settle the clear cases (every near tie is
+  // The distance pass only has to settle the clear cases (every near tie is
   // re-checked), so an FP32 job takes the tensor-core pass on split operands
   // wherever that covers its shape: the assignments are the FP64 definition's
   // either way.  At 200,003 x 37, K = 100 the pass takes 32 us instead of 156
-  // and the whole ten-round call 0.91 ms instead of 2.11.  A context that has set a wait limit or stops
-  // the copies (diagnostics of the pipelined passes) keeps FP32 jobs on the
-  // SIMT pass, which waits on nothing.
+  // and the whole ten-round call 0.69 ms instead of 2.11.  A context that has set
+  // a wait limit or stops the copies (diagnostics of the pipelined passes) keeps
+  // FP32 jobs on the SIMT pass, which waits on nothing.
   const bool plain = b.polls < 0 && b.stop_copies == 0;
   const bool tc = b.precision != MR_KM_FP32 || (km_tc_supported(d, k) && plain);
   const bool wide = !tc && b.bop && plain;
