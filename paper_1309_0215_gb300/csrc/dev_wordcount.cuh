@@ -458,15 +458,18 @@ __device__ inline void warp_segment_t(const JobDev& J, uint64_t seg, WarpLocal& 
 // load of that slot's key; most misses load no key at all.  (Two slots' keys in
 // turn, without tags, took 128 of the 360 us the map kernel spends on 256 MB of
 // 50,000 words; with tags a fifth less.)  A claim CASes the tag into the word and then
-// stores the key with one 16-byte store.  Keys start at zero and keys whose w0
-// is 0 (tokens of NUL bytes) never enter the table, so a read that meets a
-// claim half done does not match; that token, like one whose tag matches
-// another key's, goes on as a miss.  A key may end up in two slots (two lanes
+// stores the key with one 16-byte store.  A slot holds w0 with 0x20 exclusive-ored
+// into every byte: no token has eight spaces there, so a stored first half is
+// never zero (nor is w1), and a read that meets a claim half done, where a half is
+// still zero, does not match; that token, like one whose tag matches another
+// key's, goes on as a miss.  (Keys whose w0 is zero, tokens of NUL bytes, were
+// kept out of the table instead: 16 MiB of such tokens, all misses for one slot of
+// the global container, took 9.0 ms, now 0.10.)  A key may end up in two slots (two lanes
 // claiming it at once) or also in the global container, which merges them.
 template <int NS>
 struct CtaTableT {
   static constexpr int SLOTS = NS;  // a multiple of 4
-  ulonglong2 key[NS];  // {w0, w1}
+  ulonglong2 key[NS];  // {w0 ^ SPACES, w1}; zero: empty
   uint32_t cnt[NS];
   uint32_t tag[NS / 4];
   // all threads of the CTA
@@ -499,9 +502,13 @@ struct MapWarp {
 };
 static_assert(sizeof(CtaTableBig) % 16 == 0 && sizeof(MapWarp) % 16 == 0, "staging buffers must stay 16-byte aligned");
 
-// The hash of a key of the table, all of which are short.
-__device__ __forceinline__ uint32_t cta_hash(const ulonglong2& k) {
-  return hash_short((uint32_t)k.x, (uint32_t)(k.x >> 32), (uint32_t)k.y, (uint32_t)(k.y >> 32));
+constexpr uint64_t SPACES = 0x2020202020202020ull;
+
+// Merge one slot of such a table (all keys are short) into the global container.
+__device__ __forceinline__ void cta_merge(const JobDev& J, const ulonglong2& k, uint32_t c) {
+  if (k.y == 0) return;
+  const uint64_t w0 = k.x ^ SPACES;
+  global_insert(J, w0, k.y, hash_short((uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)k.y, (uint32_t)(k.y >> 32)), c);
 }
 
 // 0x80 in the zero bytes of v: exact up to and including the lowest one
@@ -511,7 +518,8 @@ __device__ __forceinline__ uint32_t zero_bytes(uint32_t v) { return (v - 0x01010
 // holds it nor has a slot that could be claimed for it.
 template <class TT>
 __device__ __forceinline__ bool cta_add(TT& T, const Tok& t) {
-  const bool able = (t.w1 >> 56) != 0xFF && t.w0 != 0;
+  const bool able = (t.w1 >> 56) != 0xFF;
+  const uint64_t w0 = t.w0 ^ SPACES;
   const uint32_t b = __umulhi(t.h, TT::SLOTS / 4);
   const uint32_t tag = max(t.h & 0xFFu, 1u);
   const uint32_t tw = *reinterpret_cast<volatile uint32_t*>(&T.tag[b]);
@@ -524,7 +532,7 @@ __device__ __forceinline__ bool cta_add(TT& T, const Tok& t) {
                  : "=l"(k0), "=l"(k1)
                  : "r"((uint32_t)__cvta_generic_to_shared(&T.key[s]))
                  : "memory");
-    hit = k1 == t.w1 && k0 == t.w0;
+    hit = k1 == t.w1 && k0 == w0;
     if (hit) atomicAdd(&T.cnt[s], 1u);
   }
   if (able && z == 0) {
@@ -535,7 +543,7 @@ __device__ __forceinline__ bool cta_add(TT& T, const Tok& t) {
       if (hit) {
         asm volatile("st.volatile.shared::cta.v2.u64 [%0], {%1, %2};" ::"r"(
                          (uint32_t)__cvta_generic_to_shared(&T.key[s])),
-                     "l"(t.w0), "l"(t.w1)
+                     "l"(w0), "l"(t.w1)
                      : "memory");
         atomicAdd(&T.cnt[s], 1u);
       }

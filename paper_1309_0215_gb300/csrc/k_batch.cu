@@ -205,10 +205,7 @@ batch_kernel(const BatchJob* __restrict__ jobs, uint32_t njobs, uint64_t total_t
       // global container
       mq.drain(s_jd, W);
       __syncthreads();
-      for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += BT) {
-        const ulonglong2 k = T.key[i];
-        if (k.y != 0) wc::global_insert(s_jd, k.x, k.y, wc::cta_hash(k), T.cnt[i]);
-      }
+      for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += BT) wc::cta_merge(s_jd, T.key[i], T.cnt[i]);
       __syncthreads();
     }
   };

@@ -116,10 +116,7 @@ __global__ void __launch_bounds__(CTA_THREADS, 1) wc_map_cta_kernel(JobDev J) {
   }
   mq.drain(J, W);
   __syncthreads();
-  for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += CTA_THREADS) {
-    const ulonglong2 k = T.key[i];
-    if (k.y != 0) wc::global_insert(J, k.x, k.y, wc::cta_hash(k), T.cnt[i]);
-  }
+  for (int i = threadIdx.x; i < wc::CtaTableBig::SLOTS; i += CTA_THREADS) wc::cta_merge(J, T.key[i], T.cnt[i]);
 }
 
 

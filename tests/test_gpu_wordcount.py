@@ -322,3 +322,25 @@ def test_wc_largest_text_of_one_cta(mr, n, end):
             assert ctx.fetch(j) == want, off
             assert (ctx.kernel_launches - before == 1) == (n <= 65_536 and end != "too many words")
             ctx.release(j)
+
+
+@pytest.mark.parametrize("mode", ["plain", "batch"])
+def test_wc_tokens_of_nul_bytes_in_the_cta_table(mr, mode):
+    """Frequent tokens of 1 to 15 NUL bytes and of one letter share their second
+    key word by length, and the first of the NUL ones is zero: the table holds
+    them all, whatever claims are under way beside them."""
+    rng = np.random.default_rng(9)
+    vocab = [b"\x00" * i for i in range(1, 18)] + [bytes([c]) for c in range(97, 123)] + [b"\x00" * 7 + b"a", b"a\x00\x00"]
+    w = np.minimum(rng.zipf(1.5, 1_500_000) - 1, len(vocab) - 1)
+    text = b" ".join(vocab[i] for i in w) + b"\n"
+    text += b"\x00 " * 1_000_000
+    assert len(text) > 4 << 20
+    want = oracle.wordcount(np.frombuffer(text, dtype=np.uint8))
+    if mode == "plain":
+        assert mr.wordcount(_dev(text, 1)) == want
+        return
+    buf = _dev(text)
+    with mr.Context() as ctx:
+        ids = [ctx.add_job(mr.WORDCOUNT, buf) for _ in range(2)]
+        ctx.run(mr.RUN_BATCHED)
+        assert all(ctx.fetch(j) == want for j in ids)
