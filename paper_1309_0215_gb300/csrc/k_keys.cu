@@ -84,14 +84,13 @@ __device__ __forceinline__ uint32_t key_at(const uint4& w, int e) {
 // input's misalignment in keys), and keys outside [0, n) are masked.  A group
 // that holds at least one key lies in the same aligned 16 bytes as that key,
 // so no read leaves the pages of the input.
+// One warp of nwarps.
 template <typename C>
-__global__ void __launch_bounds__(HK_THREADS)
-hk_global_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n, uint32_t nbins, C* __restrict__ cnt) {
+__device__ __forceinline__ void hk_global_warp(const uint4* __restrict__ base, uint32_t off, uint64_t n, uint32_t nbins,
+                                               C* __restrict__ cnt, uint64_t warp, uint64_t nwarps) {
   const int lane = threadIdx.x & 31;
   const uint64_t groups = (n + off + 3) / 4;
   const uint64_t tiles = (groups + 31) / 32;  // one group per lane
-  const uint64_t warp = ((uint64_t)blockIdx.x * HK_THREADS + threadIdx.x) >> 5;
-  const uint64_t nwarps = ((uint64_t)gridDim.x * HK_THREADS) >> 5;
   bool agg = true;
   uint32_t saved = 0, win = 0, off_windows = 0;
   const uint64_t pol_in = l2_policy_evict_first(), pol_cnt = l2_policy_evict_last();
@@ -129,6 +128,13 @@ hk_global_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n, uint3
       }
     }
   }
+}
+
+template <typename C>
+__global__ void __launch_bounds__(HK_THREADS)
+hk_global_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n, uint32_t nbins, C* __restrict__ cnt) {
+  hk_global_warp(base, off, n, nbins, cnt, ((uint64_t)blockIdx.x * HK_THREADS + threadIdx.x) >> 5,
+                 ((uint64_t)gridDim.x * HK_THREADS) >> 5);
 }
 
 // Local arrays: nbins + 1 u32 counters per CTA in shared memory, added straight
@@ -230,6 +236,8 @@ __global__ void hk_widen_kernel(const uint32_t* __restrict__ c32, uint64_t nb, u
 // uniform keys over 16M bins, 12% of the HBM rate), while adds in shared
 // memory run several times faster, so the keys are first grouped by ranges of
 // 2^PS bins ("ranges"), each of which does fit one CTA:
+//   0. hk_look_kernel looks at some of the keys and sends such as sorted ones over
+//      few bins to the global array after all.
 //   1. hk_part_kernel: a CTA takes chunks of PCHUNK consecutive keys, counts
 //      them by bucket (up to 1,024 buckets of 2^F bins, whatever the number of
 //      ranges, so that few ranges do not mean few counters and many conflicts)
@@ -240,8 +248,8 @@ __global__ void hk_widen_kernel(const uint32_t* __restrict__ c32, uint64_t nb, u
 //      in the chunk goes into a table [range][chunk].  Bound by the shared
 //      memory pipe: three random accesses a key, 3.4 wavefronts per warp each.
 //   2. hk_plan_kernel cuts the ranges into units: one, or several over equal
-//      parts of the chunks for a range that holds much more than its share
-//      (skewed keys, or few ranges).
+//      parts of the chunks (or of the keys, where those lie in lumps) for a range
+//      that holds much more than its share (skewed keys, or few ranges).
 //   3. hk_count_kernel: one CTA per unit adds its range's pieces of all chunks
 //      into shared memory and stores the counts (u64, no clearing, no widening)
 //      or, for a range of several units, adds the non-zero ones.
@@ -265,13 +273,16 @@ constexpr uint32_t PUNITS = 256;        // units of an even split
 struct PartArgs {
   void* item;          // [chunks][items of a chunk] grouped offsets within the range
   uint16_t* start;     // [ranges + 1][chunks] first item of each range in each chunk
-  uint32_t* total;     // [ranges] keys of each range; then [0] the counting kernel's cursor, [1] number of units
-  uint4* unit;         // {range, first chunk, end chunk, several}
+  uint32_t* total;     // [ranges] keys of each range
+  uint32_t* most;      // [ranges] its longest piece of a chunk
+  uint32_t* cursor;    // [0] the counting kernel's cursor, [1] number of units, [2] the keys take the global array
+  uint4* unit;         // {range, first chunk, end chunk, UNIT_* and log2 of a piece's parts << 8}
   uint32_t chunks;     // a multiple of PGROUP
   uint32_t ranges, nf, fshift;
   uint32_t step;       // log2 of the buckets per range
-  uint32_t split;      // log2 of the parts a chunk's piece is counted in
 };
+constexpr uint32_t UNIT_SEVERAL = 1;  // one of several units of its range, which add to the result
+constexpr uint32_t UNIT_LUMPS = 2;    // its keys lie in few of its chunks (sorted keys)
 
 // Exclusive scan in place of nf <= T counters by T threads (entry nf: the total).
 template <int T>
@@ -315,28 +326,92 @@ __device__ __forceinline__ void write_starts(const PartArgs& P, const uint16_t* 
       for (uint32_t q = g0 < c0 ? c0 - g0 : 0; q <= c % PGROUP; ++q) t[q] = stage[b * PGROUP + q];
   }
 }
-// The scanned bucket counts of chunk c: where its ranges start, and their totals.
+// The scanned bucket counts of chunk c: where its ranges start, their totals and
+// (MOST) longest pieces ([ranges] each; hashed bit positions lie in no lumps).
+template <bool MOST>
 __device__ __forceinline__ void stage_starts(const PartArgs& P, const uint32_t* cnt, uint16_t* stage, uint32_t* tot,
                                              uint32_t c) {
   for (uint32_t b = threadIdx.x; b <= P.ranges; b += blockDim.x) {
     const uint32_t at = cnt[min(b << P.step, P.nf)];
     stage[b * PGROUP + c % PGROUP] = (uint16_t)at;
-    if (b < P.ranges) tot[b] += cnt[min((b + 1) << P.step, P.nf)] - at;
+    if (b < P.ranges) {
+      const uint32_t len = cnt[min((b + 1) << P.step, P.nf)] - at;
+      tot[b] += len;
+      if (MOST) tot[P.ranges + b] = max(tot[P.ranges + b], len);
+    }
   }
+}
+template <bool MOST>
+__device__ __forceinline__ void add_totals(const PartArgs& P, const uint32_t* tot) {
+  for (uint32_t b = threadIdx.x; b < P.ranges; b += blockDim.x)
+    if (tot[b]) {
+      atomicAdd(P.total + b, tot[b]);
+      if (MOST) atomicMax(P.most + b, tot[P.ranges + b]);
+    }
+}
+
+// Whether grouping pays is for the keys to say.  Sorted keys over few enough bins
+// repeat within a warp's load, and the global-array kernel, which adds equal keys
+// of a warp at once, then reads them little slower than memory gives them: 256M
+// sorted keys over 1M bins take 0.33 ms there and 0.68 grouped, 16M over 60,000
+// 0.048 and 0.165.  So 64
+// groups of 128 consecutive keys are looked at (every CTA the same ones): where
+// they have at most 16 runs of equal keys on average, and at least half of them
+// start with another key than the one before (one hot key would queue at its
+// bin), the result is cleared and the keys take the global array.  This kernel
+// also clears the totals, for which there was a memory operation.
+constexpr int LOOK_T = 1024;
+constexpr uint32_t LOOKS = 64, LOOK_RUNS = 16, LOOK_KEYS = 32;
+__global__ void __launch_bounds__(LOOK_T) hk_look_kernel(const uint4* __restrict__ base, uint64_t n, PartArgs P,
+                                                         uint64_t words, uint32_t add, unsigned long long* __restrict__ out) {
+  __shared__ uint32_t s_first[LOOKS], s_runs;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int PER = LOOKS / (LOOK_T / 32);
+  const uint64_t tiles = n / 128;  // (a later round of a long input may have none: grouped)
+  if (threadIdx.x == 0) s_runs = 0;
+  __syncthreads();
+  uint4 v[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q)
+    v[q] = tiles ? __ldg(base + (PER * warp + q) * tiles / LOOKS * 32 + lane) : make_uint4(0, 1, 2, 3);
+  uint32_t runs = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const uint32_t prev = __shfl_up_sync(0xffffffffu, v[q].w, 1);
+    runs += (lane == 0 || v[q].x != prev) + (v[q].y != v[q].x) + (v[q].z != v[q].y) + (v[q].w != v[q].z);
+    if (lane == 0) s_first[PER * warp + q] = v[q].x;
+  }
+  runs = __reduce_add_sync(0xffffffffu, runs);
+  if (lane == 0) atomicAdd(&s_runs, runs);
+  __syncthreads();
+  const bool other = threadIdx.x && threadIdx.x < LOOKS && s_first[threadIdx.x] != s_first[threadIdx.x - 1];
+  const bool direct = __syncthreads_count(other) >= (int)LOOK_KEYS && s_runs <= LOOK_RUNS * LOOKS;
+  if (blockIdx.x == 0) {
+    for (uint32_t i = threadIdx.x; i < 2 * P.ranges + 2; i += LOOK_T) P.total[i] = 0;
+    if (threadIdx.x == 0) P.cursor[2] = direct;
+  }
+  if (direct && !add)
+    for (uint64_t i = (uint64_t)blockIdx.x * LOOK_T + threadIdx.x; i < words; i += (uint64_t)gridDim.x * LOOK_T) out[i] = 0;
 }
 
 __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict__ base, uint32_t off, uint64_t n,
-                                                        uint32_t nbins, PartArgs P) {
+                                                        uint32_t nbins, PartArgs P, unsigned long long* __restrict__ result) {
+  pdl_wait();
+  if (P.cursor[2]) {
+    hk_global_warp(base, off, n, nbins, result, ((uint64_t)blockIdx.x * PT + threadIdx.x) >> 5,
+                   ((uint64_t)gridDim.x * PT) >> 5);
+    return;
+  }
   extern __shared__ __align__(16) unsigned char hp_sm[];
   uint16_t* buf = reinterpret_cast<uint16_t*>(hp_sm);                 // [PCHUNK]
   uint32_t* cnt = reinterpret_cast<uint32_t*>(buf + PCHUNK);          // [PNF + 1]
-  uint32_t* tot = cnt + PNF + 4;                                      // [PRANGES]
-  uint16_t* stage = reinterpret_cast<uint16_t*>(tot + PRANGES);       // [ranges + 1][PGROUP]
+  uint32_t* tot = cnt + PNF + 4;                                      // [2][ranges]
+  uint16_t* stage = reinterpret_cast<uint16_t*>(tot + 2 * PRANGES);   // [ranges + 1][PGROUP]
   __shared__ uint32_t wsum[32];
   const int lane = threadIdx.x & 31;
   const uint64_t end = n + off;  // items in group space: item i of the stream is key i - off
   const uint32_t fs = P.fshift;
-  for (uint32_t i = threadIdx.x; i < P.ranges; i += PT) tot[i] = 0;
+  for (uint32_t i = threadIdx.x; i < 2 * P.ranges; i += PT) tot[i] = 0;
   const uint32_t per = (P.chunks + gridDim.x - 1) / gridDim.x;
   const uint32_t c0 = blockIdx.x * per, c1 = min(c0 + per, P.chunks);
   for (uint32_t c = c0; c < c1; ++c) {
@@ -367,7 +442,7 @@ __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict_
     }
     __syncthreads();
     block_scan<PT>(cnt, P.nf, wsum);
-    stage_starts(P, cnt, stage, tot, c);
+    stage_starts<true>(P, cnt, stage, tot, c);
     __syncthreads();  // the starts are read; the counters become cursors
     if (whole) {
 #pragma unroll 1
@@ -416,18 +491,30 @@ __global__ void __launch_bounds__(PT, 2) hk_part_kernel(const uint4* __restrict_
     write_starts(P, stage, c, c0, c1);
   }
   __syncthreads();
-  for (uint32_t b = threadIdx.x; b < P.ranges; b += PT)
-    if (tot[b]) atomicAdd(P.total + b, tot[b]);
+  add_totals<true>(P, tot);
 }
 
 // Units of every range (one CTA per range; every CTA scans all ranges' unit
 // counts).  A range of several units starts from zeroed bins (unless the
 // counts add to those of an earlier round).
 // (A range is 2^PS words of the result, words in all.)
+//
+// Units are cut by chunks, and pieces into parts of at least 64 items on
+// average, as long as the range's keys are spread over its chunks.  Where they
+// lie in lumps (a piece several times the average: sorted or sequential keys fill
+// whole chunks with one range) its units are cut at equal numbers of keys
+// instead, to the chunk, and their CTAs share every piece out over all warps;
+// a range without keys is only stored.  (With the cuts by chunks alone one warp
+// of a CTA, or one CTA of a range's, counted nearly all of such an input, and
+// split pieces were walked where there were none.  256M keys over 16M bins,
+// sorted 5.6 ms, in sequence 3.0, all the same 3.0: now 0.73 (0.62 with
+// hk_look_kernel's choice), 0.77 and 0.62; 30M windows of N, 7 hashes into 1e6
+// bits 1.36, now 0.24.)
 template <typename W>
 __global__ void __launch_bounds__(256) hk_plan_kernel(PartArgs P, uint64_t words, uint32_t unit_keys, uint32_t add,
                                                       W* __restrict__ out) {
   pdl_wait();
+  if (P.cursor[2]) return;  // (no units: the cursors are cleared)
   __shared__ uint32_t s_before[8], s_all[8], s_mine;
   const uint32_t b = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -445,26 +532,65 @@ __global__ void __launch_bounds__(256) hk_plan_kernel(PartArgs P, uint64_t words
   __syncthreads();
   before = all = 0;
   for (int w = 0; w < 8; ++w) before += s_before[w], all += s_all[w];
-  const uint32_t parts = s_mine;
-  const uint32_t per = ((P.chunks + parts - 1) / parts + 31) & ~31u;
-  for (uint32_t i = threadIdx.x; i < parts; i += 256)
-    P.unit[before + i] = make_uint4(b, min(i * per, P.chunks), min((i + 1) * per, P.chunks), parts > 1 ? 1u : 0u);
+  const uint32_t parts = s_mine, total = P.total[b], avg = total / P.chunks;
+  uint32_t split = 0;
+  while ((avg >> (split + 1)) >= 64) ++split;
+  const bool lumps = (P.most[b] >> split) > max(4 * (avg >> split), 512u);
+  uint32_t w = parts > 1 ? UNIT_SEVERAL : 0u;
+  if (lumps) w |= UNIT_LUMPS;
+  else w |= split << 8;
+  if (lumps && parts > 1) {
+    // unit i ends with the chunk in which the range's keys reach i + 1 parts of them
+    const uint16_t* s0 = P.start + (uint64_t)b * P.chunks;
+    const uint16_t* s1 = s0 + P.chunks;
+    const uint32_t per = (P.chunks + 255) / 256, c0 = min(threadIdx.x * per, P.chunks), c1 = min(c0 + per, P.chunks);
+    uint32_t sum = 0;
+    for (uint32_t c = c0; c < c1; ++c) sum += s1[c] - s0[c];
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    __syncthreads();  // s_before has been read
+    if (lane == 31) s_before[warp] = incl;
+    __syncthreads();
+    uint64_t at = incl - sum;
+    for (int i = 0; i < warp; ++i) at += s_before[i];
+    for (uint32_t i = threadIdx.x; i < parts; i += 256) P.unit[before + i].x = b, P.unit[before + i].w = w;
+    if (threadIdx.x == 0) P.unit[before].y = 0, P.unit[before + parts - 1].z = P.chunks;
+    for (uint32_t c = c0; c < c1; ++c) {
+      const uint64_t end = at + (s1[c] - s0[c]);
+      // the cuts i with at < i total / parts <= end
+      for (uint64_t i = at * parts / total + 1; i < parts && i * total <= end * parts; ++i) {
+        P.unit[before + i - 1].z = c + 1;
+        P.unit[before + i].y = c + 1;
+      }
+      at = end;
+    }
+  } else {
+    const uint32_t end = total ? P.chunks : 0u;
+    const uint32_t per = ((end + parts - 1) / parts + 31) & ~31u;
+    for (uint32_t i = threadIdx.x; i < parts; i += 256)
+      P.unit[before + i] = make_uint4(b, min(i * per, end), min((i + 1) * per, end), w);
+  }
   if (b == 0 && threadIdx.x == 0) {
-    P.total[P.ranges] = 0;
-    P.total[P.ranges + 1] = all;
+    P.cursor[0] = 0;
+    P.cursor[1] = all;
   }
   if (parts > 1 && !add)
     for (uint64_t i = ((uint64_t)b << PS) + threadIdx.x; i < ((uint64_t)(b + 1) << PS) && i < words; i += 256)
       out[i] = 0;
 }
 
-// A chunk's piece of the range is cut into 2^split parts, so that a unit of few
-// chunks (few ranges, long pieces) has work for every warp.  A warp takes 32
-// parts at a time; they, in quads of four
+// A warp takes 32 parts at a time (a chunk's piece of the range is cut into
+// 2^split parts, so that a unit of few chunks, of few ranges with long pieces,
+// has work for every warp); they, in quads of four
 // offsets (8 aligned bytes), are laid end to end and shared out evenly: quad f
 // belongs to the part whose scanned quad count brackets it (a binary search
 // over the lanes).  CAHEAD quads per lane are in flight (the pieces lie in
-// DRAM).
+// DRAM).  A unit of lumps takes 1,024 pieces at a time, whose quads the whole CTA
+// shares (the search is in shared memory).
 constexpr int CAHEAD = 4;
 // What is grouped, and what a range's words are: keys (16-bit bin numbers, u32
 // counts, u64 results) or bit positions (32 bits, u32 words of a bit array).
@@ -473,6 +599,7 @@ struct KeyItems {
   using Quad = uint2;
   using Word = unsigned long long;
   static constexpr uint32_t CHUNK = PCHUNK;
+  static constexpr bool LUMPS = true;
   static __device__ __forceinline__ void put(uint32_t* w, uint32_t x) { atomicAdd(w + x, 1u); }
   static __device__ __forceinline__ uint32_t item(const Quad& q, int i) {
     return (i & 1) ? (i < 2 ? q.x : q.y) >> 16 : (i < 2 ? q.x : q.y) & 0xffffu;
@@ -480,18 +607,48 @@ struct KeyItems {
   static __device__ __forceinline__ void add(Word* o, uint32_t v) { atomicAdd(o, (Word)v); }
   static __device__ __forceinline__ Word merged(Word o, uint32_t v) { return o + v; }
 };
+// Count CAHEAD quads per lane from quad f0 of `all` on: where(f, start, piece,
+// chunk) gives the first quad, the piece (first offset | end << 16) and the
+// chunk of the part that quad f belongs to; every lane calls it.
+template <class T, class F>
+__device__ __forceinline__ void count_quads(uint32_t* bins, const typename T::Item* items, uint32_t f0, uint32_t all,
+                                            F&& where) {
+  const uint32_t lane = threadIdx.x & 31;
+  typename T::Quad w[CAHEAD];
+  uint32_t r[CAHEAD], len[CAHEAD];  // the quad's first offset relative to its piece, and the piece's length
+#pragma unroll
+  for (int t = 0; t < CAHEAD; ++t) {
+    const uint32_t f = f0 + 32 * t + lane;
+    uint32_t first, pc, chunk;
+    where(f, first, pc, chunk);
+    const uint32_t i = 4 * (f - first) + (pc & 0xfffcu);
+    r[t] = i - (pc & 0xffffu);
+    len[t] = 0;
+    if (f < all) {
+      len[t] = (pc >> 16) - (pc & 0xffffu);
+      w[t] = __ldg(reinterpret_cast<const typename T::Quad*>(items + (uint64_t)chunk * T::CHUNK + i));
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < CAHEAD; ++t) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (r[t] + e < len[t]) T::put(bins, T::item(w[t], e));
+  }
+}
+
 template <class T>
 __global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint64_t words, uint32_t add,
                                                           typename T::Word* __restrict__ out) {
   pdl_wait();
   const typename T::Item* items = static_cast<const typename T::Item*>(P.item);
   extern __shared__ __align__(16) uint32_t hc_bins[];  // [1 << PS]
-  __shared__ uint32_t s_unit;
+  __shared__ uint32_t s_unit, s_ex[T::LUMPS ? PCT + 1 : 1], s_piece[T::LUMPS ? PCT : 1], wsum[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t nunits = P.total[P.ranges + 1];
+  const uint32_t nunits = P.cursor[1];
   for (;;) {
     __syncthreads();  // the previous unit's counts have been stored
-    if (threadIdx.x == 0) s_unit = atomicAdd(P.total + P.ranges, 1u);
+    if (threadIdx.x == 0) s_unit = atomicAdd(P.cursor, 1u);
     for (uint32_t i = threadIdx.x; i < (1u << PS) / 4; i += PCT)
       reinterpret_cast<uint4*>(hc_bins)[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
@@ -499,52 +656,57 @@ __global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint64_t w
     const uint4 u = P.unit[s_unit];
     const uint16_t* s0 = P.start + (uint64_t)u.x * P.chunks;
     const uint16_t* s1 = s0 + P.chunks;
-    const uint32_t nl = (u.z - u.y) << P.split;
-    for (uint32_t l0 = 32 * warp; l0 < nl; l0 += PCT) {
-      // this lane's piece: part `sub` of the quads of chunk c's
-      const uint32_t l = l0 + lane, c = u.y + (l >> P.split), sub = l & ((1u << P.split) - 1);
-      uint32_t piece = 0, nq = 0;  // first and end offset, quads
-      if (l < nl) {
-        const uint32_t a = s0[c], e = s1[c];
-        const uint32_t qa = a >> 2, n4 = e > a ? ((e + 3) >> 2) - qa : 0;
-        const uint32_t q0 = (n4 * sub) >> P.split, q1 = (n4 * (sub + 1)) >> P.split;
-        nq = q1 - q0;
-        if (nq) piece = max(a, 4 * (qa + q0)) | (min(e, 4 * (qa + q1)) << 16);
-      }
-      uint32_t ex = nq;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, ex, o);
-        if (lane >= o) ex += v;
-      }
-      const uint32_t all = __shfl_sync(0xffffffffu, ex, 31);
-      ex -= nq;
-      for (uint32_t f0 = 0; f0 < all; f0 += 32 * CAHEAD) {
-        typename T::Quad w[CAHEAD];
-        uint32_t r[CAHEAD], len[CAHEAD];  // the quad's first offset relative to its piece, and the piece's length
-#pragma unroll
-        for (int t = 0; t < CAHEAD; ++t) {
-          const uint32_t f = f0 + 32 * t + lane;
-          int p = 0;
-#pragma unroll
-          for (int o = 16; o; o >>= 1)
-            if (__shfl_sync(0xffffffffu, ex, p + o) <= f) p += o;
-          const uint32_t pc = __shfl_sync(0xffffffffu, piece, p);
-          const uint32_t i = 4 * (f - __shfl_sync(0xffffffffu, ex, p)) + (pc & 0xfffcu);
-          r[t] = i - (pc & 0xffffu);
-          len[t] = 0;
-          if (f < all) {
-            len[t] = (pc >> 16) - (pc & 0xffffu);
-            const uint32_t cp = u.y + ((l0 + p) >> P.split);
-            w[t] = __ldg(reinterpret_cast<const typename T::Quad*>(items + (uint64_t)cp * T::CHUNK + i));
-          }
+    if (T::LUMPS && (u.w & UNIT_LUMPS)) {
+      for (uint32_t l0 = u.y; l0 < u.z; l0 += PCT) {
+        const uint32_t c = l0 + threadIdx.x;
+        uint32_t nq = 0;
+        if (c < u.z) {
+          const uint32_t a = s0[c], e = s1[c];
+          if (e > a) nq = ((e + 3) >> 2) - (a >> 2), s_piece[threadIdx.x] = a | (e << 16);
         }
+        s_ex[threadIdx.x] = nq;
+        block_scan<PCT>(s_ex, PCT, wsum);
+        const uint32_t all = s_ex[PCT];
+        for (uint32_t f0 = 32 * CAHEAD * warp; f0 < all; f0 += PCT * CAHEAD)
+          count_quads<T>(hc_bins, items, f0, all, [&](uint32_t f, uint32_t& first, uint32_t& pc, uint32_t& chunk) {
+            uint32_t p = 0;  // the last piece that starts at quad f or before it
 #pragma unroll
-        for (int t = 0; t < CAHEAD; ++t) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (r[t] + e < len[t]) T::put(hc_bins, T::item(w[t], e));
+            for (uint32_t o = PCT / 2; o; o >>= 1)
+              if (s_ex[p + o] <= f) p += o;
+            first = s_ex[p], pc = f < all ? s_piece[p] : 0u, chunk = l0 + p;
+          });
+        __syncthreads();  // the pieces are counted
+      }
+    } else {
+      const uint32_t split = u.w >> 8, nl = (u.z - u.y) << split;
+      for (uint32_t l0 = 32 * warp; l0 < nl; l0 += PCT) {
+        // this lane's piece: part `sub` of the quads of chunk c's
+        const uint32_t l = l0 + lane, c = u.y + (l >> split), sub = l & ((1u << split) - 1);
+        uint32_t piece = 0, nq = 0;  // first and end offset, quads
+        if (l < nl) {
+          const uint32_t a = s0[c], e = s1[c];
+          const uint32_t qa = a >> 2, n4 = e > a ? ((e + 3) >> 2) - qa : 0;
+          const uint32_t q0 = (n4 * sub) >> split, q1 = (n4 * (sub + 1)) >> split;
+          nq = q1 - q0;
+          if (nq) piece = max(a, 4 * (qa + q0)) | (min(e, 4 * (qa + q1)) << 16);
         }
+        uint32_t ex = nq;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t v = __shfl_up_sync(0xffffffffu, ex, o);
+          if (lane >= o) ex += v;
+        }
+        const uint32_t all = __shfl_sync(0xffffffffu, ex, 31);
+        ex -= nq;
+        for (uint32_t f0 = 0; f0 < all; f0 += 32 * CAHEAD)
+          count_quads<T>(hc_bins, items, f0, all, [&](uint32_t f, uint32_t& first, uint32_t& pc, uint32_t& chunk) {
+            int p = 0;
+#pragma unroll
+            for (int o = 16; o; o >>= 1)
+              if (__shfl_sync(0xffffffffu, ex, p + o) <= f) p += o;
+            first = __shfl_sync(0xffffffffu, ex, p), pc = __shfl_sync(0xffffffffu, piece, p);
+            chunk = u.y + ((l0 + p) >> split);
+          });
       }
     }
     __syncthreads();
@@ -552,7 +714,7 @@ __global__ void __launch_bounds__(PCT, 1) hk_count_kernel(PartArgs P, uint64_t w
     const uint32_t nb = (uint32_t)min((uint64_t)(1u << PS), words - b0);
     for (uint32_t i = threadIdx.x; i < nb; i += PCT) {
       const uint32_t v = hc_bins[i];
-      if (u.w) {
+      if (u.w & UNIT_SEVERAL) {
         if (v) T::add(out + b0 + i, v);
       } else {
         out[b0 + i] = add ? T::merged(out[b0 + i], v) : v;
@@ -686,6 +848,7 @@ struct BitItems {
   using Quad = uint4;
   using Word = uint32_t;
   static constexpr uint32_t CHUNK = BCHUNK;
+  static constexpr bool LUMPS = false;  // (hashed)
   static __device__ __forceinline__ void put(uint32_t* w, uint32_t x) { atomicOr(w + (x >> 5), 1u << (x & 31)); }
   static __device__ __forceinline__ uint32_t item(const Quad& q, int i) { return key_at(q, i); }
   static __device__ __forceinline__ void add(Word* o, uint32_t v) { atomicOr(o, v); }
@@ -762,7 +925,7 @@ __global__ void __launch_bounds__(BT, 2) bloom_part_kernel(const uint8_t* __rest
     }
     __syncthreads();
     block_scan<BT>(cnt, P.nf, wsum);
-    stage_starts(P, cnt, stage, tot, c);
+    stage_starts<false>(P, cnt, stage, tot, c);
     const uint32_t all = cnt[P.nf], np = count * h;
     // grouped in place, from registers
     uint32_t x[BCHUNK / BT];
@@ -782,8 +945,7 @@ __global__ void __launch_bounds__(BT, 2) bloom_part_kernel(const uint8_t* __rest
     write_starts(P, stage, c, c0, c1);
   }
   __syncthreads();
-  for (uint32_t b = threadIdx.x; b < P.ranges; b += BT)
-    if (tot[b]) atomicAdd(P.total + b, tot[b]);
+  add_totals<false>(P, tot);
 }
 
 }  // namespace
@@ -845,7 +1007,6 @@ static PartArgs part_args(uint64_t chunks, uint32_t chunk_items, size_t item_byt
   PartArgs P{};
   P.chunks = (uint32_t)((chunks + PGROUP - 1) / PGROUP * PGROUP);
   P.ranges = ranges;
-  while ((chunk_items / ranges) >> (P.split + 1) >= 64) ++P.split;  // parts of at least 64 items
   size_t at = 0;
   auto take = [&](size_t sz) {
     uint8_t* r = p + at;
@@ -854,7 +1015,9 @@ static PartArgs part_args(uint64_t chunks, uint32_t chunk_items, size_t item_byt
   };
   P.item = take((size_t)P.chunks * chunk_items * item_bytes);
   P.start = reinterpret_cast<uint16_t*>(take((size_t)(P.ranges + 1) * P.chunks * 2));
-  P.total = reinterpret_cast<uint32_t*>(take((size_t)(P.ranges + 2) * 4));
+  P.total = reinterpret_cast<uint32_t*>(take((size_t)(2 * P.ranges + 3) * 4));
+  P.most = P.total + P.ranges;
+  P.cursor = P.most + P.ranges;
   P.unit = reinterpret_cast<uint4*>(take((size_t)(2 * P.ranges + PUNITS) * 16));
   *bytes = at;
   return P;
@@ -878,7 +1041,7 @@ cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbi
                                   KTimer* kt) {
   size_t bytes = 0;
   const PartArgs P = hk_part_args(n, nbins, scratch, &bytes);
-  const int psm = (int)(PCHUNK * 2 + (PNF + 4 + PRANGES) * 4 + (P.ranges + 1) * PGROUP * 2);
+  const int psm = (int)(PCHUNK * 2 + (PNF + 4 + 2 * PRANGES) * 4 + (P.ranges + 1) * PGROUP * 2);
   const int csm = (1 << PS) * 4;
   cudaError_t e;
   if ((e = allow_smem<hk_part_kernel>(di)) != cudaSuccess ||
@@ -893,16 +1056,17 @@ cudaError_t launch_hist_keys_part(const uint32_t* keys, uint64_t n, uint32_t nbi
     const uint32_t pg = (uint32_t)di.sms * 2;
     const uint64_t uk = m / PUNITS > PUNIT_MIN ? m / PUNITS : PUNIT_MIN;
     const uint32_t add = k0 ? 1u : 0u;
-    if ((e = cudaMemsetAsync(P.total, 0, (P.ranges + 2) * 4, s)) != cudaSuccess) return e;
-    hk_part_kernel<<<P.chunks < pg ? P.chunks : pg, PT, psm, s>>>(base, off, m, nbins, P);
+    hk_look_kernel<<<di.sms, LOOK_T, 0, s>>>(base, m, P, (uint64_t)nbins + 1, add, out);
     if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = launch_pdl(hk_part_kernel, dim3(P.chunks < pg ? P.chunks : pg), dim3(PT), (size_t)psm, s, base, off, m, nbins, P,
+                        out)) != cudaSuccess ||
         (e = launch_pdl(hk_plan_kernel<unsigned long long>, dim3(P.ranges), dim3(256), 0, s, P, (uint64_t)nbins + 1,
                         (uint32_t)uk, add, out)) !=
             cudaSuccess ||
         (e = launch_pdl(hk_count_kernel<KeyItems>, dim3(di.sms), dim3(PCT), (size_t)csm, s, P, (uint64_t)nbins + 1, add,
                         out)) != cudaSuccess)
       return e;
-    *nk += 3;
+    *nk += 4;
   }
   return kt_end(kt, s);
 }
@@ -1009,7 +1173,7 @@ cudaError_t launch_bloom_part(const uint8_t* seq, uint64_t n, uint32_t L, uint64
     const uint64_t w = nwin - w0 < bloom_round(h) ? nwin - w0 : bloom_round(h);
     const uint64_t uk = w * h / PUNITS > PUNIT_MIN ? w * h / PUNITS : PUNIT_MIN;
     const uint32_t add = w0 ? 1u : 0u, pg = (uint32_t)di.sms * 2;
-    if ((e = cudaMemsetAsync(P.total, 0, (P.ranges + 2) * 4, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(P.total, 0, (2 * P.ranges + 3) * 4, s)) != cudaSuccess) return e;
     bloom_part_kernel<<<P.chunks < pg ? P.chunks : pg, BT, psm, s>>>(seq, n, w0, w, bloom_windows(h), L, (uint32_t)m, rm,
                                                                      rm1, h, P);
     if ((e = cudaGetLastError()) != cudaSuccess ||

@@ -254,3 +254,48 @@ def test_hist_u32_partitioned_scratch(mr, n, nbins):
         assert 2.0 <= (ctx.bytes_in_use - 8 * (nbins + 1)) / n <= 2.2
         ctx.run()
         assert np.array_equal(np.frombuffer(ctx.fetch(j), dtype=np.uint64), oracle.hist_u32(keys, nbins))
+
+
+@pytest.mark.parametrize("n,nbins", [
+    (1 << 26, 1 << 20),            # several units a range, cut at equal numbers of keys
+    ((1 << 26) + 4_099, 1 << 24),  # one unit a range, its keys in four chunks
+    (1 << 24, 60_000),             # two ranges, pieces in parts
+    ((1 << 28) + 70_001, 300_000),  # the second round adds to the first
+])
+@pytest.mark.parametrize("kind", ["sorted", "sorted, the end not", "sequence", "reversed", "blocks", "constant",
+                                  "half constant"])
+def test_hist_u32_partitioned_keys_in_lumps(mr, n, nbins, kind):
+    """Keys whose ranges fill whole chunks, or one range all of them; sorted ones
+    repeat enough to take the global array, in one round or both."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n % 1000)
+    if kind in ("sequence", "reversed"):
+        keys = torch.arange(n, device="cuda", dtype=torch.int32).remainder_(nbins + 3)
+        if kind == "reversed":
+            keys = keys.flip(0).contiguous()
+    elif kind == "blocks":  # 100,000 keys of one range at a time, in any order
+        at = torch.randint(0, max(nbins - 1000, 1), (n // 100_000 + 1,), device="cuda", generator=g, dtype=torch.int32)
+        keys = at.repeat_interleave(100_000)[:n] + torch.randint(0, 1000, (n,), device="cuda", generator=g, dtype=torch.int32)
+    else:
+        keys = torch.randint(0, nbins + 9, (n,), device="cuda", generator=g, dtype=torch.int32)
+        if kind == "sorted":
+            keys = keys.sort()[0]
+        elif kind == "sorted, the end not":
+            keys[: n - 70_000] = keys[: n - 70_000].sort()[0]
+        else:
+            keys[: n if kind == "constant" else n // 2] = nbins // 3
+    torch.cuda.synchronize()
+    want = torch.bincount(keys.clamp(max=nbins), minlength=nbins + 1).cpu().numpy().astype(np.uint64)
+    assert np.array_equal(mr.hist_u32(keys, nbins), want)
+
+
+@pytest.mark.parametrize("m,h", [(1_000_003, 7), (300_000_007, 5)])
+@pytest.mark.parametrize("valid", [0, 40, 100_000, 1_000_000])
+def test_bloom_partitioned_few_windows(mr, m, h, valid):
+    """Sequences of which nearly all is N: ranges without a position, and ranges
+    whose positions come from a few chunks."""
+    seq = np.full(5_000_003, ord("N"), dtype=np.uint8)
+    if valid:
+        seq[3_000_001: 3_000_001 + valid] = synth.dna(valid, seed=valid)
+    assert np.array_equal(mr.bloom_dna(_dev(seq, 1), 30, m, h), oracle.bloom_dna(seq, 30, m, h))
