@@ -1525,6 +1525,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) km_window_sum_kernel(const floa
 constexpr uint32_t KM_STATE = 8;  // of the counters: points listed, mode, rounds, length of a rest
 __device__ __forceinline__ void km_next_mode(uint32_t* st, uint32_t n);
 constexpr int RF_THREADS = 256;
+constexpr uint32_t RF_FEW = 8;  // partials
 __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long* __restrict__ part, uint32_t g,
                                                                  long long* sums, float* c, uint32_t k, uint32_t d,
                                                                  unsigned long long* counts,
@@ -1544,11 +1545,21 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
   const unsigned long long cnt = first ? 0 : full ? cnew[kk] : counts[kk];
   const double inv = cnt ? ldexp(1.0, -*shift) : 0.0;
   float nrm = 0.f, moved2 = 0.f;
+  // Many partials are summed by the warps together, 32 dimensions at a time; with
+  // few or none each warp takes 32 dimensions of its own (2,000 x 500, K = 20, two
+  // partials, three rounds: 990 us with the warps in step over every 32 dimensions,
+  // now 936; 20,000 x 300, K = 64, whose sums lie ready after many rounds, 1,630
+  // and 1,511).
+  const bool spread = !(full && cnt && part) || g <= RF_FEW;
+  __shared__ float tails[2][RF_THREADS / 32];
   __syncthreads();  // every thread has read the count that is cleared below
-  for (uint32_t j0 = 0; j0 < d; j0 += 32) {
+  for (uint32_t j0 = spread ? 32 * w : 0; j0 < d; j0 += spread ? RF_THREADS : 32) {
     const uint32_t j = j0 + lane;
     long long a = 0;
-    if (full && cnt && part) {
+    if (full && cnt && part && spread) {
+      if (j < d)
+        for (uint32_t q = 0; q < g; ++q) a += part[(uint64_t)q * kd + row + j];
+    } else if (full && cnt && part) {
       if (j < d) {
 #pragma unroll 4
         for (uint32_t q = w; q < g; q += RF_THREADS / 32) a += part[(uint64_t)q * kd + row + j];
@@ -1557,9 +1568,9 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
       red[w][lane] = a;
       __syncthreads();
     }
-    if (w == 0 && j < d) {
+    if ((spread || w == 0) && j < d) {
       if (full && part) {
-        if (cnt) {
+        if (cnt && !spread) {
 #pragma unroll
           for (int i = 1; i < RF_THREADS / 32; ++i) a += red[i][lane];
         }
@@ -1577,12 +1588,19 @@ __global__ void __launch_bounds__(RF_THREADS) km_finalize_kernel(const long long
       if (bop) tc::put_operand(bop, d, (uint32_t)kk, j, t);
     }
   }
-  if (w == 0) {
+  if (spread || w == 0) {
     for (int o = 16; o; o >>= 1) {
       nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
       moved2 += __shfl_xor_sync(0xffffffffu, moved2, o);
     }
+  }
+  if (spread) {
+    if (lane == 0) tails[0][w] = nrm, tails[1][w] = moved2;
+    __syncthreads();
+  }
+  if (w == 0) {
     if (lane == 0) {
+      for (int i = 1; spread && i < RF_THREADS / 32; ++i) nrm += tails[0][i], moved2 += tails[1][i];
       cn[kk] = nrm;
       if (drift) {
         const float dr = __fmul_ru(__fsqrt_ru(moved2), 1.0001f);  // (the sum's relative error is below 1e-5 at D <= 64)
