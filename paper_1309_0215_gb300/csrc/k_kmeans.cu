@@ -395,7 +395,8 @@ __device__ __forceinline__ int fx_shift_of(float m, uint32_t n) {
 // distance is within the bound of the smallest; the products (x_j - c_j)^2,
 // separately rounded, for all dimensions of a chunk of candidates at once
 // (the FP64 pipe is narrow on this GPU), and one thread per candidate adding
-// them with the dimensions in order.  The lowest index wins an exact tie;
+// them with the dimensions in order.  (A point that equals a centroid needs no
+// such choice: the difference of two unequal floats is not zero.)  The lowest index wins an exact tie;
 // all-NaN distances give index 0, as the definition.
 //
 // Bounded by the FP32 pipe for long lists (2 K D operations a listed point)
@@ -462,21 +463,31 @@ __device__ void settle_fp64(const float* __restrict__ x, uint32_t d, const float
   if (threadIdx.x == 0) S.ncand = 0;
   __syncthreads();
   float m = INFINITY;
+  uint32_t same = 0x7fffffffu;  // the lowest centroid that is the point itself
   for (uint32_t kk = threadIdx.x; kk < k; kk += blockDim.x) {
     float s32 = 0.f;
+    uint32_t bits = 0;
 #pragma unroll 16
     for (uint32_t j = 0; j < d; ++j) {
       const float t = xs[j] - __ldg(ct + (uint64_t)j * k + kk);
       s32 = fmaf(t, t, s32);
+      bits |= __float_as_uint(t);
     }
     dist[kk] = s32;
     m = fminf(m, s32);
+    if (bits == 0) same = min(same, kk);
   }
   for (int o = 16; o; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) S.red_f[warp] = m;
+  same = __reduce_min_sync(0xffffffffu, same);
+  if (lane == 0) S.red_f[warp] = m, S.red_k[warp] = (int)same;
   __syncthreads();
   float m32 = S.red_f[0];
   for (int w = 1; w < nw; ++w) m32 = fminf(m32, S.red_f[w]);
+  for (int w = 0; w < nw; ++w) same = min(same, (uint32_t)S.red_k[w]);
+  if (same != 0x7fffffffu) {  // its distance is zero, and no other's is less
+    if (threadIdx.x == 0) settle_put(assign, p, same, has, has ? assign[p] : 0u, S);
+    return;
+  }
   const float lim = m32 * widen;
   for (uint32_t kk = threadIdx.x; kk < k; kk += blockDim.x)
     if (dist[kk] <= lim || m32 != m32) cand[atomicAdd(&S.ncand, 1u)] = kk;

@@ -646,3 +646,26 @@ def test_kmeans_filter_at_rest(mr, n, d, k, rounds, precision):
     for _ in range(rounds):
         cur, a, _ = mr.kmeans(dx, _dev(cur), 1, precision)
     assert np.array_equal(a_call, a) and np.array_equal(call, cur)
+
+
+@pytest.mark.parametrize("n,d,k", [(3_001, 16, 100), (2_000, 128, 300), (1_500, 300, 20), (1_203, 8, 2_000)])
+def test_kmeans_points_that_are_many_centroids(mr, n, d, k):
+    """Points that equal six and more of the centroids, others that tie among them,
+    and some a least step away from one: the lowest index of a tie."""
+    rng = np.random.default_rng(n)
+    base = rng.normal(0, 1, (3, d)).astype(np.float32)
+    init = base[rng.integers(0, 3, k)]
+    init[k // 2] = rng.normal(0, 1, d)
+    x = base[rng.integers(0, 3, n)].copy()
+    x[::5] += rng.normal(0, 0.1, (len(x[::5]), d)).astype(np.float32)
+    x[1::7, d - 1] = np.nextafter(x[1::7, d - 1], np.float32(9))
+    x[2::7] *= np.float32(1e-22)
+    init[-3:] = np.float32(0)
+    init[-3:, 0] = np.float32(1e-22) * base[0, 0]
+    a_ref = oracle.kmeans_assign(x, init)
+    for precision in (0, 1):
+        if precision and (d > 64 or k > 256):
+            continue
+        _, a, st = _run(mr, x, init, 1, precision)
+        assert np.array_equal(a, a_ref)
+        assert int(st[1]) > 0
